@@ -310,10 +310,10 @@ godec_status godec_profile_trace(godec_ctx* ctx, int32_t cap, int32_t* cls, int3
  *   flags    : 0 or GODEC_BACKWARD_REBUILD
  * The per-iteration factors are recomputed in a forward sweep (checkpointed for the
  * backward sweep), so only the supports are needed from the forward run.  The iterates
- * Z_t and Z_t^T of the forward sweep are kept for the backward sweep when all T of them
- * fit in a quarter of the free device memory (2 T m n floats); with
- * GODEC_BACKWARD_REBUILD, or when they do not fit, one copy is kept and rebuilt from X
- * and the checkpoints in the backward sweep (slower, 2 m n floats).  Scratch is
+ * Z_t of the forward sweep are kept for the backward sweep when all T of them fit in a
+ * quarter of the free device memory (T m n floats); with GODEC_BACKWARD_REBUILD, or when
+ * they do not fit, one copy is kept and rebuilt from X and the checkpoints in the
+ * backward sweep (slower, m n floats).  Scratch is
  * allocated and freed on `stream` (stream-ordered); the call does not synchronise.
  * Float32 arithmetic with the float32-accurate tensor-core products; the sparse products
  * accumulate with float atomics (results may differ in the last bits between runs).

@@ -52,14 +52,11 @@ struct godec_ctx {
   int ev_used = 0;
   int dev = 0, nsm = 0;   // nsm: the SMs this problem's grids are sized for (its budget)
   int nsm_dev = 0;          // SMs of the device
-  size_t npart_cap = 0, npend_cap = 0;   // stream-K buffers (sized for the whole device)
+  size_t npart_cap = 0;     // stream-K buffers (sized for the whole device)
   const float* X = nullptr;
-  float* Z = nullptr;                  // m x ldz   working X - S
+  void* Z = nullptr;                   // m x ldz   working (X - S) s_Z, split (k_prod.cu)
   int64_t ldz = 0;
-  float* Zt = nullptr;                 // n x ldzt  its transpose
-  int64_t ldzt = 0;
-  void* Z16 = nullptr;
-  void* Zt16 = nullptr;
+  bool half = false;                   // precision form: the chain streams the h halves of Z alone
   float* A1 = nullptr;                 // n x RP; columns >= r kept at zero
   float* A1_orig = nullptr;            // n x RP as given (restored by godec_reset)
   float* P = nullptr;                  // max(m,n) x RP
@@ -78,8 +75,8 @@ struct godec_ctx {
   int RPp = 0;
   float* cs = nullptr;                 // [2][RP] output factors: A1's column scales, 1 / kSkinnyScale
   float* rescale_tmp = nullptr;        // 2 floats: factor applied by rescale_z
-  // tensor maps: 0 Z, 1 Z^T, 2-4 bt2[0..2], 5 X, 6-7 Lsplit A, B; precision form: 8 Z16,
-  // 9 Z16^T, 13-14 bt2[3] over K = n and K = m (10-12 unused)
+  // tensor maps: 0 Z for Z B, 1 Z for Z^T C, 2-4 bt2[0..2], 5 X, 6-7 Lsplit A, B; 13-14
+  // bt2[3] over K = n and K = m (8-12 unused)
   alignas(64) unsigned char tmap[16][128];
   // precision form: float32 correction scratch
   float *RA = nullptr, *RB = nullptr, *Wa = nullptr, *Wb = nullptr, *Qa = nullptr, *Qb = nullptr, *Qtmp = nullptr;
@@ -90,7 +87,6 @@ struct godec_ctx {
   TcGeom tg[2];                        // work split of even (Z) and odd (Z^T) products
   float* part = nullptr;               // stream-K partial slots
   unsigned* counters = nullptr;        // per-tile arrival counters
-  int* pend = nullptr;                 // per-CTA lists of deferred tile completions
   int64_t ncounters = 0;
   char* gparts = nullptr;              // per product: tiles x RP x RP Gram partials (double room)
   size_t gpart_stride = 0;
@@ -262,12 +258,6 @@ void join_rank(godec_ctx* c) {
 char* gpart(godec_ctx* c, int i) { return c->gparts + (size_t)i * c->gpart_stride; }
 void* bt2(godec_ctx* c, int b) { return static_cast<char*>(c->bt2) + (size_t)b * 2 * c->RP * c->ldb * 2; }
 
-// The float16 copies of the working matrices (precision form), from Z and Z^T.
-void refresh_z16(godec_ctx* c) {
-  if (!c->Z16) return;
-  launch_to_half(c->Z, c->p.m, c->p.n, c->ldz, c->Z16, c->ldz, c->nsm, c->st);
-  launch_to_half(c->Zt, c->p.n, c->p.m, c->ldzt, c->Zt16, c->ldzt, c->nsm, c->st);
-}
 double* g64(godec_ctx* c, int i) { return c->g64 + (size_t)i * c->RP * c->RP; }
 // The float copy of a Gram in c->g64 (written by the same Gram sum), else null.
 float* g32_of(godec_ctx* c, const double* g) {
@@ -275,7 +265,8 @@ float* g32_of(godec_ctx* c, const double* g) {
   return (c->g32 && g >= c->g64 && g < c->g64 + n) ? c->g32 + (g - c->g64) : nullptr;
 }
 
-// Product i of the chain: even i streams Z (rows m, K n), odd i streams Z^T (rows n, K m).
+// Product i of the chain: Z times its operand for even i (rows m, K n), Z^T for odd i (rows
+// n, K m), both over the same split copy of Z.
 // Its skinny operand is the split transposed output of product i-1 (A1 for i = 0); the
 // rows go to `out` (nullable) and, with want_bt2, to the operand of product i+1.
 void prod(godec_ctx* c, int i, float* out, bool want_bt2, const float* T0, const float* T1, int gram_mode) {
@@ -283,10 +274,8 @@ void prod(godec_ctx* c, int i, float* out, bool want_bt2, const float* T0, const
   TcLaunch l{};
   l.mapA = c->tmap[even ? 0 : 1];
   l.mapB = c->tmap[i == 0 ? 4 : 2 + ((i - 1) & 1)];
-  if (c->Z16) {   // precision form: the chain streams the float16 copies
-    l.half_a = 1;
-    l.mapA = c->tmap[even ? 8 : 9];   // same two-term operand maps as the float32 chain
-  }
+  l.trans = even ? 0 : 1;
+  l.half_a = c->half;
   l.rows = even ? c->p.m : c->p.n;
   l.K = even ? c->p.n : c->p.m;
   l.RP = c->RP;
@@ -300,15 +289,12 @@ void prod(godec_ctx* c, int i, float* out, bool want_bt2, const float* T0, const
   l.Tn[1] = T1;
   l.cscale = c->cs + (i == 0 ? 0 : c->RP);
   l.zscale = c->ctl->zscale;
-  l.prescaled = 1;   // Z and Z^T are stored as (X - S) s_Z
   l.gram_part = gpart(c, i);
   l.gram_mode = gram_mode;
-  l.t_upper = 1;     // slot normalisers are inverses of upper-triangular factors
-  l.pend = c->pend;
   l.ctl = c->ctl;
   l.pdl = 1;
   l.z_prefetch = i > 0;   // within the chain no kernel writes Z (the S-step comes before product 0)
-  PROF(c, 0, c->st, launch_prod_tc(l, c->st));
+  PROF(c, 0, c->st, launch_prod_split(l, c->st));
 }
 
 cudaEvent_t record(godec_ctx* c, cudaStream_t s) {
@@ -383,15 +369,13 @@ void refine(godec_ctx* c) {
   const int64_t m = c->p.m, n = c->p.n;
   cudaStream_t st = c->st;
   const int* ab = &c->ctl->abort;   // an abandoned iteration skips the correction too
-  // A = Z V, B = Z^T U (float32 product kernel on the float32 working copies)
+  // A = Z V, B = Z^T U (both halves of Z)
   TcLaunch l{};
   l.RP = RP;
   l.part = c->part;
   l.counters = c->counters;
   l.cscale = c->cs_ref;
   l.zscale = c->ctl->zscale;
-  l.prescaled = 1;
-  l.pend = c->pend;
   l.ctl = c->ctl;
   launch_split_t(c->V, n, RP, bt2(c, 3), c->ldb, c->cs_ref, st, ab);
   l.mapA = c->tmap[0];
@@ -400,15 +384,16 @@ void refine(godec_ctx* c) {
   l.K = n;
   l.geom = c->tg[0];
   l.out = c->RA;
-  PROF(c, 0, st, launch_prod_tc(l, st));
+  PROF(c, 0, st, launch_prod_split(l, st));
   launch_split_t(c->U, m, RP, bt2(c, 3), c->ldb, c->cs_ref, st, ab);
+  l.trans = 1;
   l.mapA = c->tmap[1];
   l.mapB = c->tmap[14];
   l.rows = n;
   l.K = m;
   l.geom = c->tg[1];
   l.out = c->RB;
-  PROF(c, 0, st, launch_prod_tc(l, st));
+  PROF(c, 0, st, launch_prod_split(l, st));
   // C = U^T A; [U A], [V B] (stride ld, zero padding)
   PROF(c, 10, st, launch_cross_gram(c->U, RP, r, c->RA, RP, r, m, c->rf_part, kRefineParts, c->rf_C, r, st, ab));
   PROF(c, 10, st, launch_concat2(c->U, c->RA, RP, r, m, c->Wa, ld, st, ab));
@@ -457,20 +442,17 @@ void enqueue_lstep(godec_ctx* c, bool fast) {
     const int pi_mode = (i == i_rank) ? 2 : ((i > i_rank && i < last) ? 1 : 0);
     sl.pi_mode = pi_mode;
     if (i == i_rank) {
-      // P = Z Q2 unnormalised, with an exactly accumulated Gram for the rank test.  On the
+      // P = Z Q2 unnormalised, and its exactly accumulated Gram for the rank test.  On the
       // fast path nothing on the critical path needs that Gram: it is formed on the rank
-      // test's stream from P instead of in the product's tile completion.
+      // test's stream.
       const bool aside = fast && i != last;
-      prod(c, i, c->P, false, nullptr, nullptr, aside ? 0 : 2);
-      if (aside) {
-        fork_rank(c);
-        PROF(c, 1, c->rank_st, launch_gram_tiles(c->P, rows, RP, 2, gpart(c, i), c->ctl, c->rank_st));
-        gram_sum(c, gpart(c, i), 1, tiles, g64(c, i), c->rank_st);
-        rank_gram = record(c, c->rank_st);
-      } else {
-        gram_sum(c, gpart(c, i), 1, tiles, g64(c, i), c->st);
-        fork_rank(c);
-      }
+      prod(c, i, c->P, false, nullptr, nullptr, 0);
+      if (aside) fork_rank(c);
+      const cudaStream_t gs = aside ? c->rank_st : c->st;
+      PROF(c, 1, gs, launch_gram_tiles(c->P, rows, RP, 2, gpart(c, i), c->ctl, gs));
+      gram_sum(c, gpart(c, i), 1, tiles, g64(c, i), gs);
+      if (aside) rank_gram = record(c, c->rank_st);
+      else fork_rank(c);
       PROF(c, 5, c->rank_st,
            launch_rank(g64(c, i), c->r, RP, c->p.rank_tol > 0 ? c->p.rank_tol : 1e-4, c->ctl, c->rank_st));
       if (i == last) {   // q = 0: this product is also the last one
@@ -586,10 +568,30 @@ void enqueue_lstep(godec_ctx* c, bool fast) {
   PROF(c, 3, c->rank_st, launch_apply(c->Q2, n, RP, c->Vm, c->Vm, c->V, nullptr, c->ctl, c->rank_st));
   apply(c, c->P, m, c->Um, c->Um, c->U, nullptr);
   join_rank(c);
-  if (c->Z16 && !(c->p.flags & GODEC_FLAG_NO_REFINE)) refine(c);
+  if (c->half && !(c->p.flags & GODEC_FLAG_NO_REFINE)) refine(c);
   // operands of the tensor-core residual pass
   PROF(c, 3, c->st, launch_lsplit(c->U, c->V, c->sigma, m, n, RP, c->r, c->ctl->zscale, c->LA, c->LB, c->st));
   join_side(c);
+}
+
+// The S buffers and the working copy, as the kernels that write Z take them.
+EmitArgs z_args(godec_ctx* c) {
+  EmitArgs ea{};
+  ea.ctl = c->ctl;
+  for (int b = 0; b < 2; ++b) {
+    ea.S_idx[b] = c->S_idx[b];
+    ea.S_val[b] = c->S_val[b];
+  }
+  ea.X = c->X;
+  ea.n = c->p.n;
+  ea.ldx = c->p.ldx;
+  ea.Z = c->Z;
+  ea.ldz = c->ldz;
+  ea.zscale = c->ctl->zscale;
+  ea.max_nnz = c->p.k;
+  ea.sbits = c->sbits;
+  ea.sbits_words = c->sbits_words;
+  return ea;
 }
 
 // S-step of one iteration (Algorithm 1, eq. raw_lss) on the current L factors; r = 0 means L = 0.
@@ -639,29 +641,11 @@ void enqueue_sstep(godec_ctx* c, int r) {
     se.round = round;
     PROF(c, 8, st, launch_select_round(se, c->nsm, st));
   }
-  EmitArgs ea{};
-  ea.ctl = c->ctl;
+  EmitArgs ea = z_args(c);
   ea.cand_key = c->cand_key;
   ea.cand_idx = c->cand_idx;
   ea.cand_val = c->cand_val;
   ea.cand_cap = c->cap;
-  ea.S_idx[0] = c->S_idx[0];
-  ea.S_idx[1] = c->S_idx[1];
-  ea.S_val[0] = c->S_val[0];
-  ea.S_val[1] = c->S_val[1];
-  ea.X = c->X;
-  ea.n = n;
-  ea.ldx = c->p.ldx;
-  ea.Z = c->Z;
-  ea.ldz = c->ldz;
-  ea.Zt = c->Zt;
-  ea.ldzt = c->ldzt;
-  ea.Z16 = c->Z16;
-  ea.Zt16 = c->Zt16;
-  ea.zscale = c->ctl->zscale;
-  ea.max_nnz = c->p.k;
-  ea.sbits = c->sbits;
-  ea.sbits_words = c->sbits_words;
   PROF(c, 8, st, launch_emit(ea, c->nsm, st));
   if (c->Z) PROF(c, 9, st, launch_z_update(ea, c->nsm, st));
 }
@@ -682,13 +666,11 @@ void greb_prod(godec_ctx* c, bool even, int map_b, const float* cscale, float* o
   l.ldb = c->ldb;
   l.cscale = cscale;
   l.zscale = c->ctl->zscale;
-  l.prescaled = 1;
   l.gram_part = gpart(c, gslot);
   l.gram_mode = gram_mode;
-  l.t_upper = 1;
-  l.pend = c->pend;
+  l.trans = even ? 0 : 1;
   l.ctl = c->ctl;
-  launch_prod_tc(l, c->st);
+  launch_prod_split(l, c->st);
 }
 
 // out (m x RP) = D B with D = Z - U W^T (the derivative of eq. GreBsmoD; U = 0 at rank 0);
@@ -815,11 +797,10 @@ godec_status rebuild_sbits(godec_ctx* c) {
   return GODEC_OK;
 }
 
-// X A1 for the chain's first projection (k_sproj.cu): the tensor-core product over X
-// itself, split at Z's scale s_Z (set from max |X|, so X s_Z stays in the split's range).
+// X A1 for the chain's first projection (k_sproj.cu): the product over Z while S = 0.
 void form_xa1(godec_ctx* c) {
   TcLaunch l{};
-  l.mapA = c->tmap[5];
+  l.mapA = c->tmap[0];
   l.mapB = c->tmap[4];
   l.rows = c->p.m;
   l.K = c->p.n;
@@ -830,16 +811,20 @@ void form_xa1(godec_ctx* c) {
   l.out = c->XA1;
   l.cscale = c->cs;
   l.zscale = c->ctl->zscale;
-  l.prescaled = 0;
-  l.pend = c->pend;
   l.ctl = c->ctl;
-  launch_prod_tc(l, c->st);
+  launch_prod_split(l, c->st);
 }
 
 // A product that saw the abort flag part-way leaves tile counters behind.
 godec_status clear_counters(godec_ctx* c) {
   CK(cudaMemsetAsync(c->counters, 0, (size_t)c->ncounters * sizeof(unsigned), c->st));
   return GODEC_OK;
+}
+
+// The working copy Z = X s_Z (S = 0) with s_Z from max |X|; sumsq (nullable): += ||X||^2.
+void refresh_z(godec_ctx* c, double* sumsq) {
+  launch_zscale(c->X, c->p.m, c->p.n, c->p.ldx, &c->ctl->zmax_bits, c->ctl->zscale, c->nsm, c->st, sumsq);
+  launch_split_copy(c->X, c->p.m, c->p.n, c->p.ldx, c->Z, c->ldz, c->ctl->zscale, c->nsm, c->st);
 }
 
 godec_status reset_state(godec_ctx* c) {
@@ -866,13 +851,7 @@ godec_status reset_state(godec_ctx* c) {
   h.tol = -1.0;
   CK(cudaMemcpyAsync(c->ctl, &h, offsetof(Ctl, hist), cudaMemcpyHostToDevice, c->st));
   if (godec_status s = rebuild_sbits(c)) return s;   // S = 0: both bitmaps empty
-  launch_sumsq(c->X, c->p.m, c->p.n, c->p.ldx,
-               reinterpret_cast<double*>(reinterpret_cast<char*>(c->ctl) + offsetof(Ctl, normX2)), c->nsm, c->st);
-  // working copies Z = X s_Z and Z^T, with s_Z from max |X|
-  launch_zscale(c->X, c->p.m, c->p.n, c->p.ldx, &c->ctl->zmax_bits, c->ctl->zscale, c->nsm, c->st);
-  launch_scale_copy(c->X, c->p.m, c->p.n, c->p.ldx, c->Z, c->ldz, c->ctl->zscale, c->nsm, c->st);
-  launch_transpose(c->X, c->p.m, c->p.n, c->p.ldx, c->Zt, c->ldzt, c->st, c->ctl->zscale);
-  refresh_z16(c);
+  refresh_z(c, reinterpret_cast<double*>(reinterpret_cast<char*>(c->ctl) + offsetof(Ctl, normX2)));
   if (c->XA1) form_xa1(c);
   launch_reset_iter(c->ctl, c->st);
   if (c->lingo) {
@@ -912,15 +891,18 @@ godec_status reset_state(godec_ctx* c) {
   return GODEC_OK;
 }
 
-// The S-step wrote an entry of Z beyond the float16 split's range: bring max |Z| back
-// into [2^12, 2^13) by a power of two, exactly, in Z, Z^T and the stored scale.
-godec_status rescale_z(godec_ctx* c) {
-  float* f = c->rescale_tmp;
-  launch_zscale(c->Z, c->p.m, c->p.n, c->ldz, &c->ctl->zmax_bits, f, c->nsm, c->st);
-  launch_scale_copy(c->Z, c->p.m, c->p.n, c->ldz, c->Z, c->ldz, f, c->nsm, c->st);
-  launch_scale_copy(c->Zt, c->p.n, c->p.m, c->ldzt, c->Zt, c->ldzt, f, c->nsm, c->st);
-  launch_scale_update(c->ctl->zscale, f, c->st);
-  refresh_z16(c);
+// The S-step wrote an entry of Z beyond the float16 split's range: a new power-of-two scale
+// from max |X| and max |X - S| over the nnz entries of the committed S, and Z rebuilt from X
+// and S at that scale.  (The candidates of the S-step are spent: their value buffer, at
+// least as large as S, takes X - S.)
+godec_status rescale_z(godec_ctx* c, long long nnz) {
+  EmitArgs ea = z_args(c);
+  ea.max_nnz = nnz;
+  launch_z_values(ea, c->cand_val, c->st);
+  launch_zscale(c->X, c->p.m, c->p.n, c->p.ldx, &c->ctl->zmax_bits, c->ctl->zscale, c->nsm, c->st, nullptr, c->cand_val,
+                nnz);
+  launch_split_copy(c->X, c->p.m, c->p.n, c->p.ldx, c->Z, c->ldz, c->ctl->zscale, c->nsm, c->st);
+  launch_z_apply(ea, c->st);
   CK(cudaGetLastError());
   ++c->rescales;
   return GODEC_OK;
@@ -938,7 +920,7 @@ godec_status handle_abort(godec_ctx* c, const Ctl& h) {
   }
   if (h.range_err && !h.nonfinite) {
     // Z outgrew its scale in the last S-step; the iteration after it was skipped.
-    if ((s = rescale_z(c))) return s;
+    if ((s = rescale_z(c, h.nnz_cur))) return s;
     if ((s = SET_CTL(range_err, 0))) return s;
     launch_reset_iter(c->ctl, c->st);
     CK(cudaGetLastError());
@@ -1072,8 +1054,8 @@ void godec_destroy(godec_ctx* c) {
   if (!c) return;
   if (c->st) cudaStreamSynchronize(c->st);
   free_graphs(c);
-  void* ptrs[] = {c->Z, c->Zt, c->Z16, c->Zt16, c->A1, c->A1_orig, c->P, c->bt2, c->cs, c->rescale_tmp, c->LA, c->LB, c->Q1, c->Q2,
-                  c->U, c->V, c->sigma, c->Um, c->Vm, c->part, c->counters, c->pend, c->gparts, c->RA, c->RB, c->Wa, c->Wb, c->Qa, c->Qb, c->Qtmp, c->Rf,
+  void* ptrs[] = {c->Z, c->A1, c->A1_orig, c->P, c->bt2, c->cs, c->rescale_tmp, c->LA, c->LB, c->Q1, c->Q2,
+                  c->U, c->V, c->sigma, c->Um, c->Vm, c->part, c->counters, c->gparts, c->RA, c->RB, c->Wa, c->Wb, c->Qa, c->Qb, c->Qtmp, c->Rf,
                   c->cs_ref, c->rf_part, c->rf_g, c->rf_C, c->rf_core, c->rf_U, c->rf_V, c->g64, c->g32, c->gscr,
                   c->Rtmp, c->Rslot, c->Tslot, c->Rfin, c->Pi, c->Vprev, c->ctl, c->cand_key, c->cand_idx,
                   c->cand_val, c->S_idx[0], c->S_idx[1], c->S_val[0], c->S_val[1], c->sbits, c->XA1};
@@ -1124,7 +1106,7 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
   CKI(prepare_small_kernels());
   CKI(prepare_select_kernels());
   CKI(prepare_stream_kernels());
-  CKI(prepare_tc_kernels());
+  CKI(prepare_prod_kernels());
   CKI(prepare_resid_kernels());
   CKI(cudaStreamCreateWithFlags(&c->cap_st, cudaStreamNonBlocking));
   CKI(cudaStreamCreateWithFlags(&c->side_st, cudaStreamNonBlocking));
@@ -1134,17 +1116,10 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
   const int RP = c->RP, np = c->nprod;
   const size_t rr = (size_t)RP * RP;
   c->X = X;
-  // rows of the working copies start on 256-byte boundaries: every 128-byte TMA box row
-  // is then one whole cache line (a 40000-byte pitch, say, splits every other one)
-  c->ldz = (n + 63) / 64 * 64;
-  c->ldzt = (m + 63) / 64 * 64;
-  CKI(dalloc(&c->Z, (size_t)m * c->ldz));
-  CKI(dalloc(&c->Zt, (size_t)n * c->ldzt));
-  if (p->precision == GODEC_PREC_BF16_REFINE) {
-    CKI(dalloc(reinterpret_cast<unsigned short**>(&c->Z16), (size_t)m * c->ldz));
-    CKI(dalloc(reinterpret_cast<unsigned short**>(&c->Zt16), (size_t)n * c->ldzt));
-  }
-  if (p->precision == GODEC_PREC_BF16_REFINE || greb || c->naive || c->lingo) {
+  c->half = p->precision == GODEC_PREC_BF16_REFINE;
+  c->ldz = (n + 63) / 64 * 64;   // whole 64-column blocks of the split copy
+  CKI(dalloc(reinterpret_cast<float**>(&c->Z), (size_t)m * c->ldz));
+  if (c->half || greb || c->naive || c->lingo) {
     const size_t W = 64;   // columns of the correction's [U | A] and [V | B] (2r <= 64)
     CKI(dalloc(&c->RA, (size_t)m * RP));
     CKI(dalloc(&c->RB, (size_t)n * RP));
@@ -1166,14 +1141,14 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
   CKI(dalloc(&c->A1, (size_t)n * RP));
   CKI(dalloc(&c->A1_orig, (size_t)n * RP));
   // plain GoDec with a given test matrix, on request: its first projection subtracts S A1
-  // from a cached X A1 (the other forms change A1 or X between L-steps, or stream a float16
-  // copy of Z).  The cost of S A1 grows with k at about the rate of random reads from HBM;
+  // from a cached X A1 (the other forms change A1 or X between L-steps, or stream
+  // half of Z).  The cost of S A1 grows with k at about the rate of random reads from HBM;
   // at m = n = 10^4 it matches the 94 us product near k = m n / 200 and saves 40 us at
   // k = m n / 1000, but over whole iterations at k = m n / 1000 the lagged normalisers'
   // alarm trips more often with it (8 against 2 in 36 iterations), which costs more than
   // it saves, so streaming stays the default.
   const bool sparse_first = (p->flags & GODEC_FLAG_SPARSE_FIRST) != 0;
-  if (A1 && !greb && !c->naive && !c->lingo && !c->Z16 && sparse_first) CKI(dalloc(&c->XA1, (size_t)m * RP));
+  if (A1 && !greb && !c->naive && !c->lingo && !c->half && sparse_first) CKI(dalloc(&c->XA1, (size_t)m * RP));
   CKI(dalloc(&c->P, (size_t)mx * RP));
   CKI(dalloc(&c->Q1, (size_t)m * RP));
   CKI(dalloc(&c->Q2, (size_t)n * RP));
@@ -1192,18 +1167,12 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
     std::vector<float> cs(2 * (size_t)RP, 1.f / kSkinnyScale);
     CKI(cudaMemcpy(c->cs, cs.data(), cs.size() * sizeof(float), cudaMemcpyHostToDevice));
   }
-  c->tg[0] = tc_geometry(m, n, c->nsm);
-  c->tg[1] = tc_geometry(n, m, c->nsm);
+  c->tg[0] = prod_split_geometry(m, n, c->nsm);
+  c->tg[1] = prod_split_geometry(n, m, c->nsm);
   size_t npart = 0;
   for (const TcGeom& g : c->tg) npart = std::max(npart, (size_t)g.tiles * g.maxseg * 128 * RP);
   CKI(dalloc(&c->part, npart));
   c->npart_cap = npart;
-  {
-    size_t npend = 0;
-    for (const TcGeom& g : c->tg) npend = std::max(npend, (size_t)g.G * g.maxpend);
-    CKI(dalloc(&c->pend, npend));
-    c->npend_cap = npend;
-  }
   const int64_t tiles = prod_tiles(mx);
   c->ncounters = tiles;
   CKI(dalloc(&c->counters, (size_t)tiles));
@@ -1214,18 +1183,15 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
     const bool ok = make_tmap_f32(c->tmap[5], X, m, n, p->ldx, 128) &&
                     make_tmap_f16(c->tmap[6], c->LA, m, 128, 128, 128) &&
                     make_tmap_f16(c->tmap[7], c->LB, n, 128, 128, 64) &&
-                    make_tmap_f32(c->tmap[0], c->Z, m, n, c->ldz, 128) &&
-                    make_tmap_f32(c->tmap[1], c->Zt, n, m, c->ldzt, 128) &&
+                    make_tmap_split(c->tmap[0], c->Z, m, c->ldz, 128) &&
+                    make_tmap_split(c->tmap[1], c->Z, m, c->ldz, 64) &&
                     make_tmap_f16(c->tmap[2], bt2(c, 0), 2 * RP, m, c->ldb, 2 * RP) &&
                     make_tmap_f16(c->tmap[3], bt2(c, 1), 2 * RP, n, c->ldb, 2 * RP) &&
                     make_tmap_f16(c->tmap[4], bt2(c, 2), 2 * RP, n, c->ldb, 2 * RP);
-    const bool ok16 = !c->Z16 ||
-                      (make_tmap_f16(c->tmap[8], c->Z16, m, n, c->ldz, 128) &&
-                       make_tmap_f16(c->tmap[9], c->Zt16, n, m, c->ldzt, 128));
-    const bool ok3 = !(c->Z16 || greb || c->naive || c->lingo) ||
+    const bool ok3 = !(c->half || greb || c->naive || c->lingo) ||
                      (make_tmap_f16(c->tmap[13], bt2(c, 3), 2 * RP, n, c->ldb, 2 * RP) &&
                       make_tmap_f16(c->tmap[14], bt2(c, 3), 2 * RP, m, c->ldb, 2 * RP));
-    if (!ok || !ok16 || !ok3) {
+    if (!ok || !ok3) {
       fail(c, GODEC_ERR_CUDA, "tensor map encoding failed");
       return bail(GODEC_ERR_CUDA);
     }
@@ -1664,13 +1630,13 @@ static godec_status mul_common(const float* Z, int64_t m, int64_t n, int64_t ldz
   const int64_t rows = trans ? n : m, K = trans ? m : n;
   int nsm = 0, dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      prepare_tc_kernels() != cudaSuccess) {
+      (trans ? prepare_prod_kernels() : prepare_tc_kernels()) != cudaSuccess) {
     snprintf(g_static_err, sizeof(g_static_err), "godec_mul: no CUDA device");
     return GODEC_ERR_CUDA;
   }
-  const TcGeom geom = tc_geometry(rows, K, nsm);
-  const int64_t ldt = (m + 3) / 4 * 4, ldb = (K + 7) / 8 * 8;
-  float *Bp = nullptr, *part = nullptr, *Yp = nullptr, *Zt = nullptr, *aux = nullptr;
+  const TcGeom geom = trans ? prod_split_geometry(rows, K, nsm) : tc_geometry(rows, K, nsm);
+  const int64_t ldz64 = (n + 63) / 64 * 64, ldb = (K + 7) / 8 * 8;
+  float *Bp = nullptr, *part = nullptr, *Yp = nullptr, *Zs = nullptr, *aux = nullptr;
   void* Bs = nullptr;
   unsigned* cnt = nullptr;
   int* pend = nullptr;
@@ -1683,14 +1649,14 @@ static godec_status mul_common(const float* Z, int64_t m, int64_t n, int64_t ldz
             cudaMallocAsync(reinterpret_cast<void**>(&cnt), (size_t)geom.tiles * sizeof(unsigned), st) == cudaSuccess &&
             cudaMallocAsync(reinterpret_cast<void**>(&pend), (size_t)geom.G * geom.maxpend * sizeof(int), st) ==
                 cudaSuccess &&
-            (!trans || cudaMallocAsync(reinterpret_cast<void**>(&Zt), (size_t)n * ldt * sizeof(float), st) == cudaSuccess);
+            (!trans || cudaMallocAsync(reinterpret_cast<void**>(&Zs), (size_t)m * ldz64 * sizeof(float), st) == cudaSuccess);
   bool mapped = false;
   if (ok) {
     alignas(64) unsigned char mapA[128], mapB[128];
-    mapped = make_tmap_f32(mapA, trans ? Zt : Z, rows, K, trans ? ldt : ldz, 128) &&
+    mapped = (trans ? make_tmap_split(mapA, Zs, m, ldz64, 64) : make_tmap_f32(mapA, Z, rows, K, ldz, 128)) &&
              make_tmap_f16(mapB, Bs, 2 * RP, K, ldb, 2 * RP);
     if (mapped && cudaMemsetAsync(cnt, 0, (size_t)geom.tiles * sizeof(unsigned), st) != cudaSuccess) {
-      for (void* q : {(void*)Bp, Bs, (void*)aux, (void*)part, (void*)Yp, (void*)cnt, (void*)pend, (void*)Zt})
+      for (void* q : {(void*)Bp, Bs, (void*)aux, (void*)part, (void*)Yp, (void*)cnt, (void*)pend, (void*)Zs})
         if (q) cudaFreeAsync(q, st);
       snprintf(g_static_err, sizeof(g_static_err), "godec_mul: clearing the tile counters: %s",
                cudaGetErrorString(cudaGetLastError()));
@@ -1701,7 +1667,7 @@ static godec_status mul_common(const float* Z, int64_t m, int64_t n, int64_t ldz
       launch_zscale(Z, m, n, ldz, reinterpret_cast<unsigned*>(aux + 2), aux, nsm, st);
       launch_pad_copy(B, K, r, r, Bp, RP, st);
       launch_split_t(Bp, K, RP, Bs, ldb, aux + 4, st);
-      if (trans) launch_transpose(Z, m, n, ldz, Zt, ldt, st);
+      if (trans) launch_split_copy(Z, m, n, ldz, Zs, ldz64, aux, nsm, st);   // read M-major: no transpose
       TcLaunch l{};
       l.mapA = mapA;
       l.mapB = mapB;
@@ -1715,11 +1681,13 @@ static godec_status mul_common(const float* Z, int64_t m, int64_t n, int64_t ldz
       l.cscale = aux + 4;
       l.zscale = aux;
       l.pend = pend;
-      launch_prod_tc(l, st);
+      l.trans = trans;
+      if (trans) launch_prod_split(l, st);
+      else launch_prod_tc(l, st);
       launch_unpad_copy(Yp, rows, RP, Y, r, st);
     }
   }
-  void* ptrs[] = {Bp, Bs, aux, part, Yp, cnt, pend, Zt};
+  void* ptrs[] = {Bp, Bs, aux, part, Yp, cnt, pend, Zs};
   for (void* q : ptrs)
     if (q) cudaFreeAsync(q, st);
   if (!ok) {
@@ -1836,24 +1804,7 @@ static void greb_sstep(godec_ctx* c, int ri, unsigned guess, const float* U, flo
   se.sbits_words = c->sbits_words;
   se.lambda = lambda;
   launch_emit_soft(se, c->nsm, st);
-  EmitArgs ea{};
-  ea.ctl = c->ctl;
-  ea.S_idx[0] = c->S_idx[0];
-  ea.S_idx[1] = c->S_idx[1];
-  ea.S_val[0] = c->S_val[0];
-  ea.S_val[1] = c->S_val[1];
-  ea.X = c->X;
-  ea.n = n;
-  ea.ldx = c->p.ldx;
-  ea.Z = c->Z;
-  ea.ldz = c->ldz;
-  ea.Zt = c->Zt;
-  ea.ldzt = c->ldzt;
-  ea.zscale = c->ctl->zscale;
-  ea.max_nnz = c->p.k;
-  ea.sbits = c->sbits;
-  ea.sbits_words = c->sbits_words;
-  launch_z_update(ea, c->nsm, st);
+  launch_z_update(z_args(c), c->nsm, st);
 }
 
 // Grow the S and candidate buffers to hold `need` entries (keeping the committed S).
@@ -2020,7 +1971,7 @@ godec_status godec_lingodec_iterate(godec_ctx* c, int32_t n_iter, double* rel_er
       }
       if (h.abort) return fail(c, GODEC_ERR_STATE, "LinGoDec iteration aborted");
       if (h.range_err) {
-        if ((s = rescale_z(c))) return s;
+        if ((s = rescale_z(c, h.nnz_cur))) return s;
         if ((s = SET_CTL(range_err, 0))) return s;
       }
       if (rel_err) *rel_err = h.rel_err;
@@ -2056,9 +2007,7 @@ static godec_status mse_block_brp(godec_ctx* c, const float* A1, int lda) {
   cudaStream_t st = c->st;
   const int64_t m = c->p.m, n = c->p.n;
   launch_reset_iter(c->ctl, st);
-  launch_zscale(c->X, m, n, c->p.ldx, &c->ctl->zmax_bits, c->ctl->zscale, c->nsm, st);
-  launch_scale_copy(c->X, m, n, c->p.ldx, c->Z, c->ldz, c->ctl->zscale, c->nsm, st);
-  launch_transpose(c->X, m, n, c->p.ldx, c->Zt, c->ldzt, st, c->ctl->zscale);
+  refresh_z(c, nullptr);
   launch_fill_zero(c->A1, (size_t)n * c->RP * sizeof(float), st);
   launch_pad_copy(A1, n, c->p.r, lda, c->A1, c->RP, st);
   launch_split_t(c->A1, n, c->RP, bt2(c, 2), c->ldb, c->cs, st);
@@ -2280,7 +2229,7 @@ godec_status godec_grebsmo_run(godec_ctx* c, int32_t* r_out, double* stage_err, 
         }
         if (h.abort) return fail(c, GODEC_ERR_STATE, "GreBsmo inner step aborted");
         if (h.range_err) {
-          if ((s = rescale_z(c))) return s;
+          if ((s = rescale_z(c, h.nnz_cur))) return s;
           if ((s = SET_CTL(range_err, 0))) return s;
         }
         break;
@@ -2366,13 +2315,10 @@ godec_status bfail(godec_batch* b, godec_status s, const char* fmt, ...) {
 // device at init; a smaller grid never needs more (fewer CTAs split each tile less).
 godec_status set_budget(godec_ctx* c, int B) {
   B = std::max(1, std::min(B, c->nsm_dev));
-  const TcGeom g0 = tc_geometry(c->p.m, c->p.n, B), g1 = tc_geometry(c->p.n, c->p.m, B);
-  size_t npart = 0, npend = 0;
-  for (const TcGeom& g : {g0, g1}) {
-    npart = std::max(npart, (size_t)g.tiles * g.maxseg * 128 * c->RP);
-    npend = std::max(npend, (size_t)g.G * g.maxpend);
-  }
-  if (npart > c->npart_cap || npend > c->npend_cap)
+  const TcGeom g0 = prod_split_geometry(c->p.m, c->p.n, B), g1 = prod_split_geometry(c->p.n, c->p.m, B);
+  size_t npart = 0;
+  for (const TcGeom& g : {g0, g1}) npart = std::max(npart, (size_t)g.tiles * g.maxseg * 128 * c->RP);
+  if (npart > c->npart_cap)
     return fail(c, GODEC_ERR_STATE, "budget %d needs larger stream-K buffers", B);
   c->nsm = B;
   c->tg[0] = g0;

@@ -14,10 +14,10 @@
 //
 // The forward sweep recomputes and checkpoints the per-iteration factors (A2, Y2, Y2p,
 // Q, Z Y2p and L_t on Omega_t; Q an orthonormal basis of range(Y2) from CholeskyQR2);
-// the backward sweep reuses Z_t and Z_t^T kept from the forward sweep when all T of them
-// fit in a quarter of the free device memory, and otherwise rebuilds them from X and the
-// checkpointed values.  Streaming products with Z_t and Z_t^T run on the tensor-core product kernel
-// (float32 accuracy); the r x r solve is the Cholesky kernel of the L-step.
+// the backward sweep reuses the Z_t kept from the forward sweep when all T of them fit in a
+// quarter of the free device memory, and otherwise rebuilds them from X and the checkpointed
+// values.  Each Z_t is held once, split for the tensor cores (k_prod.cu), and serves the
+// products in both directions; the r x r solve is the Cholesky kernel of the L-step.
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
@@ -31,8 +31,8 @@ void launch_spmm(const int64_t* idx, const float* val, int64_t nnz, int64_t n, c
                  int trans, float* out, int64_t ldo, cudaStream_t st);
 void launch_eval_lr(const int64_t* idx, int64_t nnz, int64_t n, const float* U, int64_t ldu, const float* V,
                     int64_t ldv, int K, float* vals, float* D, int64_t ldd, cudaStream_t st);
-void launch_scatter_set(const int64_t* idx, const float* vals, int64_t nnz, int64_t n, float* Z, int64_t ldz,
-                        cudaStream_t st);
+void launch_scatter_split(const int64_t* idx, const float* vals, int64_t nnz, int64_t n, void* Z, int64_t ldz,
+                          const float* scale, cudaStream_t st);
 void launch_outer_acc(const float* U, int64_t ldu, const float* V, int64_t ldv, int K, int64_t m, int64_t n,
                       float beta, float* D, int64_t ldd, cudaStream_t st);
 void launch_axpy(const float* x, float* y, int64_t count, float alpha, cudaStream_t st);
@@ -64,13 +64,11 @@ struct Scratch {
   }
 };
 
-// A float32 source of streaming products (Z_t, Z_t^T or a dense gradient and its
-// transpose) with its tensor map, product geometry and power-of-two scale.
+// A split m x n matrix (k_prod.cu) with its tensor maps and power-of-two scale, the source of
+// products in both directions (index 0: Z B, 1: Z^T C).
 struct Source {
-  alignas(64) unsigned char map[128];
-  const float* p = nullptr;
-  int64_t rows = 0, K = 0, ld = 0;
-  TcGeom geom;
+  alignas(64) unsigned char map[2][128];
+  void* z = nullptr;
   float* zscale = nullptr;     // {s, 1/s} on the device
   unsigned* zmax = nullptr;
 };
@@ -78,48 +76,36 @@ struct Source {
 struct Engine {
   cudaStream_t st;
   int nsm = 0, RP = 0;
+  int64_t dim[2] = {0, 0};                     // m, n
   int64_t ldb = 0;
   void* Bs = nullptr;                          // 2 RP x ldb halves (split transposed operand)
   alignas(64) unsigned char mapB[2][128];      // over Bs with K = n (index 0) and K = m (index 1)
-  int64_t Kb[2] = {0, 0};
+  TcGeom geom[2];
   float *Bp = nullptr, *cscale = nullptr, *part = nullptr, *Yp = nullptr;
   unsigned* cnt = nullptr;
-  int* pend = nullptr;
 
-  // Y (rows x c, dense) = src * B (K x c, dense rows of c)
-  void mul(const Source& s, const float* B, int c, float* Y) {
-    const int bi = (s.K == Kb[0]) ? 0 : 1;
-    launch_pad_copy(B, s.K, c, c, Bp, RP, st);
-    launch_split_t(Bp, s.K, RP, Bs, ldb, cscale, st);
+  // Y (rows x c, dense) = src * B, or src^T * B with trans (B K x c, dense rows of c)
+  void mul(const Source& s, int trans, const float* B, int c, float* Y) {
+    const int64_t rows = dim[trans], K = dim[1 - trans];
+    launch_pad_copy(B, K, c, c, Bp, RP, st);
+    launch_split_t(Bp, K, RP, Bs, ldb, cscale, st);
     TcLaunch l{};
-    l.mapA = s.map;
-    l.mapB = mapB[bi];
-    l.rows = s.rows;
-    l.K = s.K;
+    l.mapA = s.map[trans];
+    l.mapB = mapB[trans];
+    l.rows = rows;
+    l.K = K;
     l.RP = RP;
-    l.geom = s.geom;
+    l.geom = geom[trans];
     l.part = part;
     l.counters = cnt;
     l.out = Yp;
     l.cscale = cscale;
     l.zscale = s.zscale;
-    l.pend = pend;
-    launch_prod_tc(l, st);
-    launch_unpad_copy(Yp, s.rows, RP, Y, c, st);
+    l.trans = trans;
+    launch_prod_split(l, st);
+    launch_unpad_copy(Yp, rows, RP, Y, c, st);
   }
 };
-
-bool setup_source(Source& s, const float* p, int64_t rows, int64_t K, int64_t ld, int nsm, float* zscale,
-                  unsigned* zmax) {
-  s.p = p;
-  s.rows = rows;
-  s.K = K;
-  s.ld = ld;
-  s.geom = tc_geometry(rows, K, nsm);
-  s.zscale = zscale;
-  s.zmax = zmax;
-  return make_tmap_f32(s.map, p, rows, K, ld, 128);
-}
 
 }  // namespace
 
@@ -143,27 +129,22 @@ extern "C" godec_status godec_backward(const float* X, int64_t m, int64_t n, int
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int dev = 0, nsm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      prepare_tc_kernels() != cudaSuccess || prepare_small_kernels() != cudaSuccess) {
+      prepare_prod_kernels() != cudaSuccess || prepare_small_kernels() != cudaSuccess) {
     set_static_error("godec_backward: no CUDA device");
     return GODEC_ERR_CUDA;
   }
   const int RP = (r + 7) / 8 * 8, R3 = 3 * r;
-  const int64_t mx = std::max(m, n), ldz = (n + 63) / 64 * 64, ldzt = (m + 63) / 64 * 64;
+  const int64_t mx = std::max(m, n), ldz = (n + 63) / 64 * 64;
   Scratch sc{st};
-  // Iterates Z_t and Z_t^T: one copy each for all t, rebuilt in the backward sweep, or (when
-  // all T of them fit in a quarter of the free device memory) one per t, kept from the
-  // forward sweep, which saves the backward sweep's copy, scatter, transpose and scale.
+  // Iterates Z_t: one copy for all t, rebuilt in the backward sweep, or (when all T of them
+  // fit in a quarter of the free device memory) one per t, kept from the forward sweep.
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) free_b = 0;
   const bool keep = !(flags & GODEC_BACKWARD_REBUILD) &&
-                    (double)T * (double)(m * ldz + n * ldzt) * sizeof(float) <= 0.25 * (double)free_b;
+                    (double)T * (double)(m * ldz) * sizeof(float) <= 0.25 * (double)free_b;
   const int nzb = keep ? T : 1;
-  std::vector<float*> Zb(nzb), Ztb(nzb);
-  for (int b = 0; b < nzb; ++b) {
-    Zb[b] = sc.get<float>((size_t)m * ldz);
-    Ztb[b] = sc.get<float>((size_t)n * ldzt);
-  }
-  float* Gt = gL ? sc.get<float>((size_t)n * ldzt) : nullptr;      // dense gradient transposed
+  std::vector<Source> src(nzb + (gL ? 1 : 0));   // Z_t copies, then the dense gradient
+  for (Source& q : src) q.z = sc.get<float>((size_t)m * ldz);
   Engine E;
   E.st = st;
   E.nsm = nsm;
@@ -173,10 +154,8 @@ extern "C" godec_status godec_backward(const float* X, int64_t m, int64_t n, int
   E.Bp = sc.get<float>((size_t)mx * RP);
   E.cscale = sc.get<float>(RP);
   E.Yp = sc.get<float>((size_t)mx * RP);
-  float* zsc = sc.get<float>(2 * (size_t)nzb + 2);     // {s, 1/s} of each Z_t copy, then of the dense gradient
-  unsigned* zmax = sc.get<unsigned>((size_t)nzb + 1);
-  std::vector<Source> sZs(nzb), sZts(nzb);
-  Source sG, sGt;
+  float* zsc = sc.get<float>(2 * src.size() + 2);      // {s, 1/s} of each source, then of X
+  unsigned* zmax = sc.get<unsigned>(src.size() + 1);
   // per-iteration checkpoints (forward sweep)
   std::vector<float*> A2(T), Y2(T), Y2p(T), Qk(T), ZY2p(T), Lv(T);
   for (int t = 0; t < T; ++t) {
@@ -202,56 +181,50 @@ extern "C" godec_status godec_backward(const float* X, int64_t m, int64_t n, int
   double* cpart = sc.get<double>((size_t)kCrossParts * GODEC_MAX_RANK * GODEC_MAX_RANK);
   Ctl* ctl = sc.get<Ctl>(1);
   if (sc.ok) {
-    const TcGeom gz = tc_geometry(m, n, nsm), gzt = tc_geometry(n, m, nsm);
-    size_t npart = 0, npend = 0;
-    int64_t tiles = 0;
-    for (const TcGeom& g : {gz, gzt}) {
-      npart = std::max(npart, (size_t)g.tiles * g.maxseg * 128 * RP);
-      npend = std::max(npend, (size_t)g.G * g.maxpend);
-      tiles = std::max(tiles, g.tiles);
-    }
+    E.dim[0] = m;
+    E.dim[1] = n;
+    E.geom[0] = prod_split_geometry(m, n, nsm);
+    E.geom[1] = prod_split_geometry(n, m, nsm);
+    size_t npart = 0;
+    for (const TcGeom& g : E.geom) npart = std::max(npart, (size_t)g.tiles * g.maxseg * 128 * RP);
     E.part = sc.get<float>(npart);
-    E.pend = sc.get<int>(npend);
-    E.cnt = sc.get<unsigned>((size_t)tiles);
+    E.cnt = sc.get<unsigned>((size_t)std::max(E.geom[0].tiles, E.geom[1].tiles));
   }
   if (!sc.ok) {
     set_static_error("godec_backward: out of device memory");
     return GODEC_ERR_OOM;
   }
-  cudaMemsetAsync(E.cnt, 0, (size_t)std::max(tc_geometry(m, n, nsm).tiles, tc_geometry(n, m, nsm).tiles) * sizeof(unsigned), st);
+  cudaMemsetAsync(E.cnt, 0, (size_t)std::max(E.geom[0].tiles, E.geom[1].tiles) * sizeof(unsigned), st);
   cudaMemsetAsync(ctl, 0, sizeof(Ctl), st);
-  E.Kb[0] = n;
-  E.Kb[1] = m;
   bool mapped = make_tmap_f16(E.mapB[0], E.Bs, 2 * RP, n, E.ldb, 2 * RP) &&
                 make_tmap_f16(E.mapB[1], E.Bs, 2 * RP, m, E.ldb, 2 * RP);
-  for (int b = 0; b < nzb; ++b)
-    mapped = mapped && setup_source(sZs[b], Zb[b], m, n, ldz, nsm, zsc + 2 * b, zmax + b) &&
-             setup_source(sZts[b], Ztb[b], n, m, ldzt, nsm, zsc + 2 * b, zmax + b);
-  if (gL) {
-    mapped = mapped && setup_source(sG, gL, m, n, ldg, nsm, zsc + 2 * nzb, zmax + nzb) &&
-             setup_source(sGt, Gt, n, m, ldzt, nsm, zsc + 2 * nzb, zmax + nzb);
+  for (size_t b = 0; b < src.size(); ++b) {
+    src[b].zscale = zsc + 2 * b;
+    src[b].zmax = zmax + b;
+    mapped = mapped && make_tmap_split(src[b].map[0], src[b].z, m, ldz, 128) &&
+             make_tmap_split(src[b].map[1], src[b].z, m, ldz, 64);
   }
   if (!mapped) {
     set_static_error("godec_backward: tensor map encoding failed");
     return GODEC_ERR_CUDA;
   }
   const size_t rowb = sizeof(float);
-  // Z_t = X with L_{t-1} on Omega_{t-1}; Z_t^T; the shared scale of both (copy slot b)
+  // Z_t = X with L_{t-1} on Omega_{t-1}, at a scale that covers both (copy slot b)
+  unsigned* xmax = zmax + src.size();
+  launch_zscale(X, m, n, ldx, xmax, zsc + 2 * src.size(), nsm, st);
   auto build_Z = [&](int t) {
-    const int b = keep ? t : 0;
-    float *Z = Zb[b], *Zt = Ztb[b];
-    cudaMemcpy2DAsync(Z, ldz * rowb, X, ldx * rowb, n * rowb, m, cudaMemcpyDeviceToDevice, st);
-    if (t > 0 && support_nnz[t - 1] > 0) launch_scatter_set(supports[t - 1], Lv[t - 1], support_nnz[t - 1], n, Z, ldz, st);
-    launch_transpose(Z, m, n, ldz, Zt, ldzt, st);
-    launch_zscale(Z, m, n, ldz, zmax + b, zsc + 2 * b, nsm, st);
+    const Source& q = src[keep ? t : 0];
+    const bool sup = t > 0 && support_nnz[t - 1] > 0;
+    launch_zscale_from(xmax, sup ? Lv[t - 1] : nullptr, sup ? support_nnz[t - 1] : 0, q.zmax, q.zscale, nsm, st);
+    launch_split_copy(X, m, n, ldx, q.z, ldz, q.zscale, nsm, st);
+    if (sup) launch_scatter_split(supports[t - 1], Lv[t - 1], support_nnz[t - 1], n, q.z, ldz, q.zscale, st);
   };
   // ---------------- forward sweep: checkpoints ----------------
   for (int t = 0; t < T; ++t) {
     build_Z(t);
-    const Source& sZ = sZs[keep ? t : 0];
-    const Source& sZt = sZts[keep ? t : 0];
-    E.mul(sZ, A1, r, A2[t]);                                   // A2 = Z A1
-    E.mul(sZt, A2[t], r, Y2[t]);                               // Y2 = Z^T A2
+    const Source& sZ = src[keep ? t : 0];
+    E.mul(sZ, 0, A1, r, A2[t]);                                // A2 = Z A1
+    E.mul(sZ, 1, A2[t], r, Y2[t]);                             // Y2 = Z^T A2
     // Y2 = Q R by CholeskyQR2 (R = R2 R1), so that W = (Y2^T Y2)^{-1} = R^{-1} R^{-T} and
     // Y2p = Y2 W = Q T2^T T1^T are formed without squaring Y2's condition number
     const size_t rr = (size_t)RP * RP;
@@ -264,23 +237,23 @@ extern "C" godec_status godec_backward(const float* X, int64_t m, int64_t n, int
     launch_tall_small_f(Y2T, r, r, T2, RP, 0, r, n, 1.f, 0.f, Qk[t], r, st);       // Q = Q1 T2
     launch_tall_small_f(Qk[t], r, r, T2, RP, 1, r, n, 1.f, 0.f, Y2T, r, st);       // Q T2^T
     launch_tall_small_f(Y2T, r, r, T1, RP, 1, r, n, 1.f, 0.f, Y2p[t], r, st);      // ... T1^T
-    E.mul(sZ, Y2p[t], r, ZY2p[t]);                             // Y1 W = Z Y2p
+    E.mul(sZ, 0, Y2p[t], r, ZY2p[t]);                          // Y1 W = Z Y2p
     if (t + 1 < T && support_nnz[t] > 0)                       // L_t on Omega_t
       launch_eval_lr(supports[t], support_nnz[t], n, ZY2p[t], r, Y2[t], r, r, Lv[t], nullptr, 0, st);
   }
   // ---------------- backward sweep ----------------
   if (gL) {
-    launch_transpose(gL, m, n, ldg, Gt, ldzt, st);
-    launch_zscale(gL, m, n, ldg, zmax + nzb, zsc + 2 * nzb, nsm, st);
+    const Source& q = src[nzb];
+    launch_zscale(gL, m, n, ldg, q.zmax, q.zscale, nsm, st);
+    launch_split_copy(gL, m, n, ldg, q.z, ldz, q.zscale, nsm, st);
   }
   for (int t = T - 1; t >= 0; --t) {
     if (!keep) build_Z(t);
-    const Source& sZ = sZs[keep ? t : 0];
-    const Source& sZt = sZts[keep ? t : 0];
+    const Source& sZ = src[keep ? t : 0];
     // a = G Y2p and Wn = b = G^T (Z Y2p)
     if (t == T - 1 && gL) {
-      E.mul(sG, Y2p[t], r, a);
-      E.mul(sGt, ZY2p[t], r, Wn);
+      E.mul(src[nzb], 0, Y2p[t], r, a);
+      E.mul(src[nzb], 1, ZY2p[t], r, Wn);
     } else if (t == T - 1) {
       launch_cross_gram(gV, g_rank, g_rank, Y2p[t], r, r, n, cpart, kCrossParts, Msm, r, st);
       launch_tall_small_d(gU, g_rank, g_rank, Msm, r, 0, r, m, 1.f, 0.f, a, r, st);
@@ -293,11 +266,11 @@ extern "C" godec_status godec_backward(const float* X, int64_t m, int64_t n, int
       launch_spmm(supports[t], gv, support_nnz[t], n, ZY2p[t], r, r, 1, Wn, r, st);
     }
     // Wn += Z^T a;  gY2 = (I - P) Wn = Wn - Y2p (Y2^T Wn)
-    E.mul(sZt, a, r, Y2T);
+    E.mul(sZ, 1, a, r, Y2T);
     launch_axpy(Y2T, Wn, (int64_t)n * r, 1.f, st);
     launch_cross_gram(Qk[t], r, r, Wn, r, r, n, cpart, kCrossParts, Msm, r, st);
     launch_tall_small_d(Qk[t], r, r, Msm, r, 0, r, n, -1.f, 1.f, Wn, r, st);     // Wn = (I - Q Q^T) Wn = gY2
-    E.mul(sZ, Wn, r, Zg);                                       // Z gY2
+    E.mul(sZ, 0, Wn, r, Zg);                                    // Z gY2
     // factors of gZ_t: [a | A2 | Z gY2] [Y2 | gY2 | A1]^T
     cudaMemcpy2DAsync(Uf, R3 * rowb, a, r * rowb, r * rowb, m, cudaMemcpyDeviceToDevice, st);
     cudaMemcpy2DAsync(Uf + r, R3 * rowb, A2[t], r * rowb, r * rowb, m, cudaMemcpyDeviceToDevice, st);

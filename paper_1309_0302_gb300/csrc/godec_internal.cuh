@@ -2,13 +2,15 @@
 //
 // Data layout in HBM (row-major everywhere):
 //   X   m x ldx  float32   borrowed input
-//   Z   m x ldz  float32   working copy of X - S_{t-1}, updated sparsely
+//   Z   m x ldz  4 bytes per element: working copy of (X - S_{t-1}) s_Z in its two-term
+//         float16 split (k_prod.cu), updated sparsely; ldz = n rounded up to 64
 //   skinny m x RP / n x RP float32 factors, RP = r rounded up to 8 (<= 64);
 //         padded columns are kept at zero
 //   S   COO (int64 linear index, float32 value), double-buffered
 //   candidates  (uint32 key, int64 index, float32 value) of the S-step
 #pragma once
 
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -37,6 +39,27 @@ constexpr float kSkinnyScale = 1.f;
 // s_Z puts max |X| in [2^12, 2^13), and an S-step that writes a larger entry flags
 // range_err so Z is rescaled before the next product.
 constexpr float kZRange = 32768.f;
+
+// The split working copy: element (i, j) is z = h + 2^-11 l, its h at zs_at(i, j, ldz) and
+// its l 64 halves further (rows of ldz elements, per 64 columns 64 halves of h, then of l).
+__host__ __device__ __forceinline__ int64_t zs_at(int64_t i, int64_t j, int64_t ldz) {
+  return i * 2 * ldz + (j >> 6) * 128 + (j & 63);
+}
+__device__ __forceinline__ void split_z(float z, __half& h, __half& l) {
+  h = __float2half_rn(z);
+  l = __float2half_rn((z - __half2float(h)) * 2048.f);
+}
+__device__ __forceinline__ void zs_put(__half* Z, int64_t i, int64_t j, int64_t ldz, float z) {
+  __half h, l;
+  split_z(z, h, l);
+  const int64_t o = zs_at(i, j, ldz);
+  Z[o] = h;
+  Z[o + 64] = l;
+}
+__device__ __forceinline__ float zs_get(const __half* Z, int64_t o) {
+  return fmaf(__half2float(Z[o + 64]), 1.f / 2048.f, __half2float(Z[o]));
+}
+
 constexpr int kHistBins = 4096;     // first radix digit: key bits 30..19
 constexpr int kD1Shift = 19;
 constexpr int kNumSelRounds = 7;    // 3 key digits + 4 index digits
@@ -142,7 +165,7 @@ void launch_apply(const float* P, int64_t rows, int RP, const float* T0, const f
 // row stride RP; XA1 and A1 likewise), S read on its support (bitmap ctl->cur of sbits,
 // `words` words per bitmap) as X - Z / s_Z; each row's entries are subtracted in column
 // order.  Like the product, it abandons the iteration when Z is flagged out of range.
-void launch_sproj(const float* XA1, const float* A1, int RP, const float* X, int64_t ldx, const float* Z, int64_t ldz,
+void launch_sproj(const float* XA1, const float* A1, int RP, const float* X, int64_t ldx, const void* Z, int64_t ldz,
                   int64_t m, int64_t n, const unsigned* sbits, long long words, Ctl* ctl, float* P,
                   cudaStream_t st);
 
@@ -153,6 +176,7 @@ struct TcGeom {
   int maxpend = 0;           // completions one CTA may owe (list entries per CTA)
 };
 TcGeom tc_geometry(int64_t rows, int64_t K, int nsm);
+TcGeom prod_split_geometry(int64_t rows, int64_t K, int nsm);
 int tc_rpp(int RP);
 // Float16 split transposed operand of a row-major rows x RP matrix B (2 RP x ldb
 // halves), each column scaled by a power of two; cscale (RP) receives the factors that
@@ -160,19 +184,24 @@ int tc_rpp(int RP);
 void launch_split_t(const float* B, int64_t rows, int RP, void* bt2, int64_t ldb, float* cscale, cudaStream_t st,
                     const int* skip = nullptr);
 // zscale = {s, 1/s}: the power of two with max |Z| s in [2^12, 2^13) (1 if Z is zero or
-// not finite); zmax is scratch.
+// not finite); zmax is scratch.  sumsq (nullable): += sum of Z^2.  extra (nullable): n_extra
+// more values that the maximum covers.
 void launch_zscale(const float* Z, int64_t rows, int64_t cols, int64_t ld, unsigned* zmax, float* zscale, int nsm,
-                   cudaStream_t st);
-// dst = src * scale[0] (rows x cols, strides lds / ldd); dst may equal src.
-void launch_scale_copy(const float* src, int64_t rows, int64_t cols, int64_t lds, float* dst, int64_t ldd,
-                       const float* scale, int nsm, cudaStream_t st);
-// zscale[0..1] *= f[0..1] (one thread).
-void launch_scale_update(float* zscale, const float* f, cudaStream_t st);
+                   cudaStream_t st, double* sumsq = nullptr, const float* extra = nullptr, int64_t n_extra = 0);
+// The same from a maximum already found (float bits) and extra.
+void launch_zscale_from(const unsigned* base, const float* extra, int64_t n_extra, unsigned* zmax, float* zscale, int nsm,
+                        cudaStream_t st);
+// The split matrix Z (m x ldz) of X scale[0]; columns n .. ldz-1 zero.
+void launch_split_copy(const float* X, int64_t m, int64_t n, int64_t ldx, void* Z, int64_t ldz, const float* scale,
+                       int nsm, cudaStream_t st);
+// A tensor map over a split matrix: boxes of one 64-half block x box_rows rows.
+bool make_tmap_split(void* map, const void* base, int64_t rows, int64_t ldz, int box_rows);
 bool make_tmap_f32(void* map, const float* base, int64_t rows, int64_t cols, int64_t ld, int box_rows);
 bool make_tmap_f16(void* map, const void* base, int64_t rows, int64_t cols, int64_t ld, int box_rows);
 cudaError_t prepare_tc_kernels();
 struct TcLaunch {
-  const void* mapA;        // CUtensorMap over Zsrc (rows x K), box 32 x 128
+  const void* mapA;        // launch_prod_tc: CUtensorMap over Zsrc (rows x K float32), box 32 x 128;
+                           // launch_prod_split: over the split matrix (make_tmap_split)
   const void* mapB;        // CUtensorMap over the float16 split operand (2 RP x K), box 64 x 2 RP
   int64_t rows, K;
   int RP;
@@ -182,21 +211,22 @@ struct TcLaunch {
   float* out;              // rows x RP (nullable)
   void* bt2;               // 2 RP x ldb halves (nullable)
   int64_t ldb;
-  const float* Tn[2];
+  const float* Tn[2];      // upper triangular (launch_prod_split)
   const float* cscale;     // per-column output factor (nullable)
   const float* zscale;     // {s_Z, 1/s_Z} on the device (nullable)
-  int prescaled;           // Zsrc already holds x s_Z
-  void* gram_part;
-  int gram_mode;
-  int t_upper;             // Tn upper triangular (inverse of an upper-triangular factor)
-  int half_a;              // mapA is the float16 copy Z16 (box 64 halves x 128 rows)
-  int* pend;               // G x geom.maxpend ints of scratch
+  void* gram_part;         // tiles x RP x RP floats
+  int gram_mode;           // 1: write the Gram partials
+  int trans;               // launch_prod_split: the product with Z^T (mapA's boxes have 64 rows, else 128)
+  int half_a;              // launch_prod_split: the h halves alone
+  int* pend;               // launch_prod_tc: G x geom.maxpend ints of scratch
   Ctl* ctl;
   int pdl = 0;             // programmatic dependent launch on the preceding kernel of the stream
   int z_prefetch = 0;      // the preceding kernels leave Zsrc unchanged: its first stages may be
                            // loaded before the wait on them (with pdl)
 };
-void launch_prod_tc(const TcLaunch& l, cudaStream_t st);
+void launch_prod_tc(const TcLaunch& l, cudaStream_t st);      // float32 source, scaled and split in the kernel
+void launch_prod_split(const TcLaunch& l, cudaStream_t st);   // split source (k_prod.cu)
+cudaError_t prepare_prod_kernels();
 int64_t apply_blocks(int64_t rows);
 
 // r x r kernels (k_small.cu).
@@ -291,13 +321,9 @@ struct EmitArgs {
   float* S_val[2];
   const float* X;
   int64_t n, ldx;
-  float* Z;
+  void* Z;                 // the split working copy
   int64_t ldz;
-  float* Zt;               // transposed copy (n x ldzt), nullable
-  int64_t ldzt;
-  void* Z16;               // nullable bf16 copies (same strides)
-  void* Zt16;
-  const float* zscale;     // Z and Zt are stored scaled by zscale[0]
+  const float* zscale;     // Z is stored scaled by zscale[0]
   long long max_nnz;       // bound on the support of S (k): the z-update grid
   unsigned* sbits;         // two bitmaps of m n bits (nullable), sbits_words words apart: bitmap
   long long sbits_words;   // `cur` holds the support of the committed S, the other one is clear.
@@ -310,6 +336,10 @@ void launch_emit(const EmitArgs& a, int nsm, cudaStream_t st);
 void launch_sbits_rebuild(unsigned* sbits, long long words, long long* const S_idx[2], const Ctl* ctl,
                           long long max_nnz, cudaStream_t st);
 void launch_z_update(const EmitArgs& a, int nsm, cudaStream_t st);
+// Z = (X - S) s_Z on the entries of the committed S (after Z was rebuilt from X alone).
+void launch_z_apply(const EmitArgs& a, cudaStream_t st);
+// out[e] = X - S at entry e of the committed S (for a new scale of Z).
+void launch_z_values(const EmitArgs& a, float* out, cudaStream_t st);
 // Reset the per-iteration S-step state (after an aborted iteration or at start).
 void launch_reset_iter(Ctl* ctl, cudaStream_t st);
 // One bounded wait that nothing completes; flags ctl->timeout / abort when it gives up.
@@ -335,14 +365,12 @@ void launch_tall_small_f(const float* A, int64_t lda, int a, const float* Bm, in
 void launch_tall_small_d(const float* A, int64_t lda, int a, const double* Bm, int ldbm, int trans, int c,
                          int64_t rows, float alpha, float beta, float* C, int64_t ldc, cudaStream_t st,
                          const int* skip = nullptr);
-// Precision form (k_refine.cu): the bases [P | Q] of the correction; float16 copy of a
-// float32 matrix; the 2r x 2r core Ra K Rb^T of the tangent-space correction; SVD of an
-// n x n float64 matrix (n <= 64), leading r triplets.
+// Precision form (k_refine.cu): the bases [P | Q] of the correction; the 2r x 2r core
+// Ra K Rb^T of the tangent-space correction; SVD of an n x n float64 matrix (n <= 64),
+// leading r triplets.
 // W (rows x ld, float32) = [P | Q | 0] for P, Q rows x r with row stride ldp (2r <= ld).
 void launch_concat2(const float* P, const float* Q, int64_t ldp, int r, int64_t rows, float* W, int ld,
                     cudaStream_t st, const int* skip = nullptr);
-void launch_to_half(const float* src, int64_t rows, int64_t cols, int64_t lds, void* dst, int64_t ldd, int nsm,
-                    cudaStream_t st);
 cudaError_t prepare_refine_kernels();
 void launch_refine_core(const float* Ra1, const float* Ra2, const float* Rb1, const float* Rb2, int ld,
                         const double* C, int r, double* core, cudaStream_t st, const int* skip = nullptr);

@@ -124,13 +124,13 @@ __global__ void k_eval_lr(const int64_t* __restrict__ idx, int64_t nnz, int64_t 
   if (D) D[row * ldd + col] -= s;
 }
 
-// Z[row][col] = vals[e] at the COO positions (Z holds a copy of X elsewhere).
-__global__ void k_scatter_set(const int64_t* __restrict__ idx, const float* __restrict__ vals, int64_t nnz, int64_t n,
-                              float* __restrict__ Z, int64_t ldz) {
+// Z[row][col] = vals[e] scale[0] at the COO positions of the split matrix Z.
+__global__ void k_scatter_split(const int64_t* __restrict__ idx, const float* __restrict__ vals, int64_t nnz, int64_t n,
+                                __half* __restrict__ Z, int64_t ldz, const float* __restrict__ scale) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nnz) return;
   const int64_t row = idx[e] / n, col = idx[e] % n;
-  Z[row * ldz + col] = vals[e];
+  zs_put(Z, row, col, ldz, vals[e] * scale[0]);
 }
 
 // D (m x n) = beta D + U V^T, U m x K (ldu), V n x K (ldv), K <= 192: 128 x 128 output
@@ -252,10 +252,10 @@ void launch_eval_lr(const int64_t* idx, int64_t nnz, int64_t n, const float* U, 
   k_eval_lr<<<blocks_for(nnz), BW_THREADS, 0, st>>>(idx, nnz, n, U, ldu, V, ldv, K, vals, D, ldd);
 }
 
-void launch_scatter_set(const int64_t* idx, const float* vals, int64_t nnz, int64_t n, float* Z, int64_t ldz,
-                        cudaStream_t st) {
+void launch_scatter_split(const int64_t* idx, const float* vals, int64_t nnz, int64_t n, void* Z, int64_t ldz,
+                          const float* scale, cudaStream_t st) {
   if (nnz == 0) return;
-  k_scatter_set<<<blocks_for(nnz), BW_THREADS, 0, st>>>(idx, vals, nnz, n, Z, ldz);
+  k_scatter_split<<<blocks_for(nnz), BW_THREADS, 0, st>>>(idx, vals, nnz, n, static_cast<__half*>(Z), ldz, scale);
 }
 
 void launch_axpy(const float* x, float* y, int64_t count, float alpha, cudaStream_t st) {

@@ -1,6 +1,6 @@
 // Kernels of the precision form's float32 correction (reading of the paper's error
-// control for the rounded chain; the oracle is tangent_refine): the 16-bit copies of the
-// working matrix, the 2r x 2r core of the tangent-space re-truncation and its SVD.
+// control for the rounded chain; the oracle is tangent_refine): the bases of the
+// correction, the 2r x 2r core of the tangent-space re-truncation and its SVD.
 #include <cuda_fp16.h>
 
 #include "godec_internal.cuh"
@@ -8,14 +8,6 @@
 namespace godec {
 
 namespace {
-
-// dst (rows x cols, float16, row stride ldd) = src (float32, row stride lds), rounded to
-// nearest (src holds (X - S) s_Z, inside the float16 range).
-__global__ void k_to_half(const float* __restrict__ src, int64_t rows, int64_t cols, int64_t lds,
-                          __half* __restrict__ dst, int64_t ldd) {
-  for (int64_t i = blockIdx.x; i < rows; i += gridDim.x)
-    for (int64_t j = threadIdx.x; j < cols; j += blockDim.x) dst[i * ldd + j] = __float2half_rn(src[i * lds + j]);
-}
 
 // W (rows x ld) = [P | Q | 0]: P and Q rows x r (row stride ldp), zero columns 2r..ld-1.
 __global__ void k_concat2(const float* __restrict__ P, const float* __restrict__ Q, int64_t ldp, int r, int64_t rows,
@@ -190,13 +182,6 @@ __global__ void __launch_bounds__(1024) k_svd_small(const double* __restrict__ A
 }
 
 }  // namespace
-
-void launch_to_half(const float* src, int64_t rows, int64_t cols, int64_t lds, void* dst, int64_t ldd, int nsm,
-                     cudaStream_t st) {
-  int64_t grid = 4LL * nsm;
-  if (grid > rows) grid = rows;
-  if (grid > 0) k_to_half<<<(unsigned)grid, 256, 0, st>>>(src, rows, cols, lds, static_cast<__half*>(dst), ldd);
-}
 
 void launch_concat2(const float* P, const float* Q, int64_t ldp, int r, int64_t rows, float* W, int ld,
                     cudaStream_t st, const int* skip) {

@@ -535,17 +535,14 @@ k_emit(EmitArgs a) {
 }
 
 // Z := X on the entries of S_{t-1}, then Z := X - S_t on the entries of S_t.
-// Z and Zt hold (X - S) zscale[0].  An entry whose scaled magnitude reaches kZRange
+// Z holds (X - S) zscale[0], split.  An entry whose scaled magnitude reaches kZRange
 // flags range_err; the next product sees the flag, abandons that iteration before
-// reading Z, and the caller rescales Z (setting abort here would cut this update short
+// reading Z, and the caller rebuilds Z (setting abort here would cut this update short
 // in blocks that have not started yet).
 __device__ __forceinline__ void z_write(const EmitArgs& a, long long i, long long j, float z, float zs, bool& bad) {
   const float v = z * zs;
   bad |= fabsf(v) >= kZRange && isfinite(v);
-  a.Z[i * a.ldz + j] = v;
-  if (a.Zt) a.Zt[j * a.ldzt + i] = v;
-  if (a.Z16) reinterpret_cast<__half*>(a.Z16)[i * a.ldz + j] = __float2half_rn(v);     // precision form's copies
-  if (a.Zt16) reinterpret_cast<__half*>(a.Zt16)[j * a.ldzt + i] = __float2half_rn(v);
+  zs_put(static_cast<__half*>(a.Z), i, j, a.ldz, v);
 }
 
 __device__ __forceinline__ void z_flag(Ctl* ctl, bool bad) {
@@ -577,7 +574,7 @@ __device__ __forceinline__ void split_idx(long long idx, long long n, float ninv
 // stop the iterations after it), so Z always matches the committed S.
 __device__ __forceinline__ bool z_skip(const Ctl* ctl) { return ctl->abort && !ctl->converged; }
 
-// The update of Z (and its copies) from S_{t-1} to S_t, one launch: entries of Omega_{t-1}
+// The update of Z from S_{t-1} to S_t, one launch: entries of Omega_{t-1}
 // that left the support get Z = X back, and Z = X - S_t on Omega_t.  The two sets are
 // disjoint (the restore skips every entry the emit marked in the bitmap of Omega_t), so
 // thread e does entry e of both lists.  The bitmap of Omega_{t-1} is cleared on the way
@@ -610,6 +607,19 @@ __global__ void k_z_update(EmitArgs a) {
     z_write(a, i, j, a.X[i * a.ldx + j] - a.S_val[cb][e], zs, bad);
   }
   z_flag(ctl, bad);
+}
+
+// Z = (X - S) s_Z on the entries of the committed S (vals null), or their X - S into vals.
+__global__ void k_z_apply(EmitArgs a, float* vals) {
+  Ctl* ctl = a.ctl;
+  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= ctl->nnz_cur) return;
+  const int cb = ctl->cur;
+  long long i, j;
+  split_idx(a.S_idx[cb][e], a.n, 1.f / (float)a.n, i, j);
+  const float z = a.X[i * a.ldx + j] - a.S_val[cb][e];
+  if (vals) vals[e] = z;
+  else zs_put(static_cast<__half*>(a.Z), i, j, a.ldz, z * a.zscale[0]);
 }
 
 // The support bitmap of the committed S (bitmap ctl->cur) from its index list, one entry
@@ -687,6 +697,14 @@ void launch_sbits_rebuild(unsigned* sbits, long long words, long long* const S_i
                           long long max_nnz, cudaStream_t st) {
   const long long nb = (max_nnz + 255) / 256;
   k_sbits_rebuild<<<(unsigned)(nb > 0 ? nb : 1), 256, 0, st>>>(sbits, words, S_idx[0], S_idx[1], ctl);
+}
+
+void launch_z_apply(const EmitArgs& a, cudaStream_t st) {
+  k_z_apply<<<(unsigned)(a.max_nnz > 0 ? (a.max_nnz + 255) / 256 : 1), 256, 0, st>>>(a, nullptr);
+}
+
+void launch_z_values(const EmitArgs& a, float* out, cudaStream_t st) {
+  k_z_apply<<<(unsigned)(a.max_nnz > 0 ? (a.max_nnz + 255) / 256 : 1), 256, 0, st>>>(a, out);
 }
 
 void launch_z_update(const EmitArgs& a, int nsm, cudaStream_t st) {

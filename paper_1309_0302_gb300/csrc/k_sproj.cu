@@ -31,7 +31,7 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
 
 __global__ void __launch_bounds__(SP_WARPS * 32, 18)   // 36 warps, 72 rows per SM
 k_sproj(const float* __restrict__ XA1, const float* __restrict__ A1, int RP, const float* __restrict__ X, int64_t ldx,
-        const float* __restrict__ Z, int64_t ldz, int64_t m, int64_t n, const unsigned* __restrict__ sbits,
+        const __half* __restrict__ Z, int64_t ldz, int64_t m, int64_t n, const unsigned* __restrict__ sbits,
         long long words, Ctl* __restrict__ ctl, float* __restrict__ P) {
   __shared__ unsigned s_w[SP_WARPS * 2][SP_WCAP];
   __shared__ int s_j[SP_WARPS * 2][SP_CAP];
@@ -57,7 +57,7 @@ k_sproj(const float* __restrict__ XA1, const float* __restrict__ A1, int RP, con
   const int64_t nw = live ? ((b1 - 1) >> 5) - w0 + 1 : 0;
   const int64_t nwmax = n / 32 + 2;         // bound on nw for every row (uniform)
   const float* Xr = X + (live ? i : 0) * ldx;
-  const float* Zr = Z + (live ? i : 0) * ldz;
+  const int64_t zr = (live ? i : 0);
   int* lj = s_j[slot];
   float* lv = s_v[slot];
   // Applies the nl listed entries of this row (called by the whole warp).
@@ -73,7 +73,7 @@ k_sproj(const float* __restrict__ XA1, const float* __restrict__ A1, int RP, con
         if (e < nl) {
           const int j = lj[e];
           xv[u] = Xr[j];
-          zv[u] = Zr[j];
+          zv[u] = zs_get(Z, zs_at(zr, j, ldz));
         }
       }
 #pragma unroll
@@ -166,11 +166,12 @@ k_sproj(const float* __restrict__ XA1, const float* __restrict__ A1, int RP, con
 
 }  // namespace
 
-void launch_sproj(const float* XA1, const float* A1, int RP, const float* X, int64_t ldx, const float* Z, int64_t ldz,
+void launch_sproj(const float* XA1, const float* A1, int RP, const float* X, int64_t ldx, const void* Z, int64_t ldz,
                   int64_t m, int64_t n, const unsigned* sbits, long long words, Ctl* ctl, float* P,
                   cudaStream_t st) {
   const unsigned grid = (unsigned)((m + 2 * SP_WARPS - 1) / (2 * SP_WARPS));
-  k_sproj<<<grid, SP_WARPS * 32, 0, st>>>(XA1, A1, RP, X, ldx, Z, ldz, m, n, sbits, words, ctl, P);
+  k_sproj<<<grid, SP_WARPS * 32, 0, st>>>(XA1, A1, RP, X, ldx, static_cast<const __half*>(Z), ldz, m, n, sbits,
+                                          words, ctl, P);
 }
 
 }  // namespace godec

@@ -15,13 +15,12 @@
 // (D[:, :RP] + 2^-11 D[:, RP:2RP]) / (s_Z s_B).  float16 MMAs run at twice the TF32
 // rate with twice the K per instruction.
 //
-// A copier thread moves each landed 128 x 64 float32 tile of Zsrc from shared memory into
-// tensor memory (tcgen05.cp) and frees the shared-memory slot when the copy completes;
-// converter warps then turn the tile into the two packed float16 blocks (h1, h2) in place
-// with TMEM loads and stores.  The working warps thus leave the shared-memory load path
-// to the TMA stream.  Zsrc is either stored already scaled (the working copy of X - S,
-// whose writers keep it inside the float16 range) or scaled here (a caller's matrix,
-// scale from its exact maximum).
+// This kernel serves products with a caller's float32 matrix (k_prod.cu serves the library's
+// own split copies).  A copier thread moves each landed 128 x 64 float32 tile of Zsrc from
+// shared memory into tensor memory (tcgen05.cp) and frees the shared-memory slot when the
+// copy completes; converter warps then scale the tile (s_Z from its exact maximum) and turn
+// it into the two packed float16 blocks (h1, h2) in place with TMEM loads and stores.  The
+// working warps thus leave the shared-memory load path to the TMA stream.
 //
 // Work split: the (128-row tile, 64-wide K stage) iteration space is cut into equal
 // contiguous ranges, one per persistent CTA ("stream-K"), so every SM streams the same
@@ -31,8 +30,7 @@
 // kChunk * 64 terms (its additions are not round-to-nearest, and over thousands of
 // terms of one sign the bias would show).  At a tile boundary the running sum goes to
 // a partial slot.  The last segment of a tile to arrive adds the slots in order
-// (deterministic), unscales, applies the normaliser T, and writes the rows, the next
-// product's split transposed operand and the tile's Gram partial.
+// (deterministic), unscales and writes the rows.
 //
 // Warps: 0 TMA producer of Zsrc tiles, 1 MMA issuer (and TMEM owner), 2-9 converters
 // (two per TMEM lane quarter, one per 32-column half of the tile), 10-13 epilogue,
@@ -50,7 +48,6 @@
 #include <cudaTypedefs.h>
 
 #include "godec_internal.cuh"
-#include "gram_tile.cuh"
 #include "tc_util.cuh"
 
 namespace godec {
@@ -66,16 +63,12 @@ constexpr int NS = 4;              // stage slots: skinny-operand tile in shared
 constexpr int kThreads = 512;
 constexpr int kConvWarps = 8;
 constexpr uint32_t kTmemCols = 512, kTA0 = 256, kTASlot = 64;
-constexpr int EPI_LD = kMaxRP + 1;   // odd stride: row-wise and column-wise accesses are conflict-free
 constexpr size_t kBoxA = (size_t)BM * 32 * 4;               // one 32-column float32 box, 16 KB
 constexpr size_t kStageA = 2 * kBoxA;                       // 32 KB
 constexpr size_t kStageB = (size_t)2 * kMaxRP * BK * 2;     // 16 KB (room for 2 x 64 rows of 64 halves)
 constexpr size_t kOffA = 0;
 constexpr size_t kOffB = kOffA + NA * kStageA;
-// tile completion runs after the stream, in the then idle Zsrc ring
-constexpr size_t kEpiBytes = (size_t)BM * EPI_LD * 4 + (size_t)kMaxRP * kMaxRP * 4;
 constexpr size_t kTcSmem = kOffB + NS * kStageB + 1024;     // + alignment slack
-static_assert(kEpiBytes <= NA * kStageA, "completion staging fits the Zsrc ring");
 constexpr uint32_t kWaitLimit = 1u << 20;
 constexpr float kLoScale = 2048.f, kLoInv = 1.f / 2048.f;
 #ifndef GODEC_TC_CHUNK
@@ -92,20 +85,11 @@ struct TcArgs {
   int maxseg;
   float* part;              // tiles x maxseg x BM x RP
   unsigned* counters;       // tiles
-  float* out;               // rows x RP (nullable)
-  __half* bt2;              // 2 RP x ldb split transposed output (nullable)
-  int64_t ldb;
-  const float* Tn0;
-  const float* Tn1;
+  float* out;               // rows x RP
   const float* cscale;      // per-column output factor 1 / s_B (nullable: 1)
   const float* zscale;      // {s_Z, 1 / s_Z} (nullable: 1)
-  int prescaled;            // Zsrc holds x s_Z already (s_Z then only undone in the epilogue)
-  void* gram_part;
-  int gram_mode;
-  int t_upper;              // the normaliser is upper triangular
   int* pend;                // G x maxpend: tiles each CTA completes, deferred to its end
   int maxpend;
-  int z_prefetch;           // Zsrc's first stages may be loaded before the programmatic wait
   Ctl* ctl;
 };
 
@@ -126,36 +110,19 @@ __device__ __forceinline__ uint32_t pack_h2(float even, float odd) {
   return d;
 }
 
-// Completion of tile t by its last segment, run by nthr threads (u = 0..nthr-1, a
-// multiple of 32) that synchronise on named barrier `bar`: the partial slots are added
-// in slot order (deterministic whoever finishes) and unscaled, the normaliser T applied,
-// the rows and the next product's split transposed operand written, and the tile's Gram
-// partial formed.  Ps (BM x EPI_LD) holds the tile's rows between the phases, Ts (RPp x
-// RPp) a copy of T; csc = per-column output factors 1 / s_B, zi = 1 / s_Z.
-template <int RPp>
-__device__ void tile_finish(const TcArgs& a, int64_t t, int nseg, int u, int nthr, int bar, float* Ps, float* Ts,
-                            const float* csc, float zi, const float* Tn) {
+// Completion of tile t by its last segment, run by the whole block (u = 0 .. nthr-1): the
+// partial slots are added in slot order (deterministic whoever finishes), unscaled and
+// written; csc = per-column output factors 1 / s_B, zi = 1 / s_Z.  Consecutive threads take
+// consecutive float4s (coalesced), four items each and up to four slots of each in flight.
+__device__ void tile_finish(const TcArgs& a, int64_t t, int nseg, int u, int nthr, const float* csc, float zi) {
   const int RP = a.RP, RP4 = RP / 4;
   const int64_t o0 = t * BM;
   const int nrow = (int)(a.rows - o0 < BM ? a.rows - o0 : BM);
   __threadfence();   // the other segments' slots: written before their counter increments
   if (u == 0) a.counters[t] = 0u;
-  // T (chosen at the kernel's start) is loaded together with the slots: one memory round
-  // trip for the whole phase
-  constexpr int kTq = kMaxRP * kMaxRP / 4 / 256;   // float4s of T per thread for nthr >= 256
-  const int nT4 = Tn ? RP * RP4 : 0;
-  float4 tq[kTq];
-#pragma unroll
-  for (int k = 0; k < kTq; ++k) {
-    const int e = u + k * nthr;
-    tq[k] = e < nT4 ? __ldg(reinterpret_cast<const float4*>(Tn) + e) : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  // (1) rows of the tile into Ps: sum of the slots, unscaled.  Consecutive threads take
-  // consecutive float4s of a slot (coalesced); four items per thread and up to four slots
-  // each are in flight at once.
   const float4* part = reinterpret_cast<const float4*>(a.part + t * a.maxseg * (int64_t)BM * RP);
   const int64_t slot4 = (int64_t)BM * RP4;
-  const int nitem = BM * RP4;
+  const int nitem = nrow * RP4;
   for (int it0 = u; it0 < nitem; it0 += 4 * nthr) {
     float4 acc[4];
 #pragma unroll
@@ -183,92 +150,13 @@ __device__ void tile_finish(const TcArgs& a, int64_t t, int nseg, int u, int nth
     for (int q = 0; q < 4; ++q) {
       const int it = it0 + q * nthr;
       if (it < nitem) {
-        const int row = it / RP4, c = (it % RP4) * 4;
-        float* pr = Ps + row * EPI_LD + c;
-        const bool live = row < nrow;
-        pr[0] = live ? acc[q].x * (csc[c] * zi) : 0.f;
-        pr[1] = live ? acc[q].y * (csc[c + 1] * zi) : 0.f;
-        pr[2] = live ? acc[q].z * (csc[c + 2] * zi) : 0.f;
-        pr[3] = live ? acc[q].w * (csc[c + 3] * zi) : 0.f;
+        const int c = (it % RP4) * 4;
+        reinterpret_cast<float4*>(a.out + o0 * RP)[it] =
+            make_float4(acc[q].x * (csc[c] * zi), acc[q].y * (csc[c + 1] * zi), acc[q].z * (csc[c + 2] * zi),
+                        acc[q].w * (csc[c + 3] * zi));
       }
     }
   }
-#pragma unroll
-  for (int k = 0; k < kTq; ++k) {
-    const int e = u + k * nthr;
-    if (e < nT4) *reinterpret_cast<float4*>(Ts + (e / RP4) * RPp + (e % RP4) * 4) = tq[k];
-  }
-  named_sync(bar, nthr);
-  // (2) Y <- Y T.  A warp takes an 8-column group of the output for one half of the rows
-  // (lane: rows lane and lane + 32 of the half), so T is read at warp-uniform addresses;
-  // with T upper triangular the group needs rows c <= its last column only.  Results stay
-  // in registers until every warp has read Y (at most two items per warp for nthr >= 256).
-  if (Tn) {
-    const int lane = u & 31, nw = nthr >> 5, CB = RP / 8, nit = 2 * CB;
-    float acc[2][2][8];
-    int item[2] = {-1, -1};
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int itm = (u >> 5) + k * nw;
-      if (itm < nit) {
-        item[k] = itm;
-        const int cg = itm >> 1, r0 = (itm & 1) * 64 + lane, l0 = cg * 8;
-        const int cend = a.t_upper ? l0 + 8 : RP;
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-          for (int j = 0; j < 8; ++j) acc[k][i][j] = 0.f;
-#pragma unroll 2
-        for (int c = 0; c < cend; ++c) {
-          const float y0 = Ps[r0 * EPI_LD + c], y1 = Ps[(r0 + 32) * EPI_LD + c];
-          const float4 t0 = *reinterpret_cast<const float4*>(Ts + c * RPp + l0);
-          const float4 t1 = *reinterpret_cast<const float4*>(Ts + c * RPp + l0 + 4);
-          const float tv[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            acc[k][0][j] = fmaf(y0, tv[j], acc[k][0][j]);
-            acc[k][1][j] = fmaf(y1, tv[j], acc[k][1][j]);
-          }
-        }
-      }
-    }
-    named_sync(bar, nthr);   // every read of Y done before it is overwritten
-#pragma unroll
-    for (int k = 0; k < 2; ++k)
-      if (item[k] >= 0) {
-        const int cg = item[k] >> 1, r0 = (item[k] & 1) * 64 + lane, l0 = cg * 8;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          Ps[r0 * EPI_LD + l0 + j] = acc[k][0][j];
-          Ps[(r0 + 32) * EPI_LD + l0 + j] = acc[k][1][j];
-        }
-      }
-    named_sync(bar, nthr);
-  }
-  // (3) outputs: rows (float4 per thread), and the split transposed operand (one column
-  // l at a time, consecutive threads on consecutive rows)
-  if (a.out)
-    for (int it = u; it < nrow * RP4; it += nthr) {
-      const int row = it / RP4, c = (it % RP4) * 4;
-      const float* pr = Ps + row * EPI_LD + c;
-      *reinterpret_cast<float4*>(a.out + (o0 + row) * (int64_t)RP + c) = make_float4(pr[0], pr[1], pr[2], pr[3]);
-    }
-  if (a.bt2)
-    for (int it = u; it < RP * BM; it += nthr) {
-      const int l = it / BM, row = it % BM;
-      if (row < nrow) {
-        const float v = Ps[row * EPI_LD + l] * kSkinnyScale;
-        const __half c1 = __float2half_rn(v);
-        a.bt2[(int64_t)l * a.ldb + o0 + row] = c1;
-        a.bt2[(int64_t)(RP + l) * a.ldb + o0 + row] = __float2half_rn((v - __half2float(c1)) * kLoScale);
-      }
-    }
-  // (4) Gram partial Y^T Y of the tile (rows past nrow are zero)
-  if (a.gram_mode) {
-    const size_t esz = a.gram_mode == 2 ? sizeof(double) : sizeof(float);
-    gram_tile(Ps, EPI_LD, RP, a.gram_mode, static_cast<char*>(a.gram_part) + (size_t)t * RP * RP * esz, u, nthr);
-  }
-  named_sync(bar, nthr);   // Ps and Ts free again
 }
 
 // One TMA producer loop over this CTA's stages [g0, g1).  Zsrc stages are two
@@ -276,14 +164,11 @@ __device__ void tile_finish(const TcArgs& a, int64_t t, int nseg, int u, int nth
 // skinny-operand stages are one 64-column float16 box.
 template <bool IS_A>
 __device__ void produce(const CUtensorMap* map, unsigned char* ring, int nslot, size_t slot_bytes, uint32_t box_bytes,
-                        uint64_t* fullb, uint64_t* emptyb, int64_t g0, int64_t g1, int64_t ks, int64_t K, Ctl* ctl,
-                        volatile int* s_err, int64_t npre = 0) {
-  // npre stages were issued already (prefetch_a): continue after them
-  int64_t t = (g0 + npre) / ks, kst = (g0 + npre) % ks;
-  int s = (int)(npre % nslot);
-  uint32_t ph = (uint32_t)((npre / nslot) & 1);
-  int64_t issued = npre;
-  g0 += npre;
+                        uint64_t* fullb, uint64_t* emptyb, int64_t g0, int64_t g1, int64_t ks, Ctl* ctl,
+                        volatile int* s_err) {
+  int64_t t = g0 / ks, kst = g0 % ks, issued = 0;
+  int s = 0;
+  uint32_t ph = 0;
   // Zsrc is streamed once per product and is larger than L2: its lines go first, which
   // leaves L2 to the skinny operand (read by every CTA) and the partial slots
   const uint64_t pol = policy_evict_first();
@@ -308,26 +193,6 @@ __device__ void produce(const CUtensorMap* map, unsigned char* ring, int nslot, 
     if (!mbar_wait(&fullb[(int)(j % nslot)], (uint32_t)((j / nslot) & 1), kWaitLimit)) note_timeout(ctl, s_err);
 }
 
-// The first stages of this CTA's Zsrc range into the empty ring (every slot is free at the
-// start), issued before the programmatic wait on the preceding kernel when that kernel
-// leaves Zsrc unchanged: the stream then starts as soon as the skinny operand lands.
-// Returns the number of stages issued; produce() continues after them and drains them on
-// an abort like its own.
-__device__ int64_t prefetch_a(const CUtensorMap* map, unsigned char* ring, uint64_t* fullb, int64_t g0, int64_t g1,
-                              int64_t ks) {
-  const uint64_t pol = policy_evict_first();
-  const int64_t n = (g1 - g0 < NA) ? g1 - g0 : NA;
-  int64_t t = g0 / ks, kst = g0 % ks;
-  for (int64_t s = 0; s < n; ++s) {
-    unsigned char* dst = ring + (size_t)s * kStageA;
-    mbar_expect_tx(&fullb[s], 2 * (uint32_t)kBoxA);
-    tma_load_2d_hint(dst, map, &fullb[s], (int)(kst * BK), (int)(t * BM), pol);
-    tma_load_2d_hint(dst + kBoxA, map, &fullb[s], (int)(kst * BK + 32), (int)(t * BM), pol);
-    if (++kst == ks) { kst = 0; ++t; }
-  }
-  return n > 0 ? n : 0;
-}
-
 // Warp-uniform bounded wait: lane 0 polls, the warp follows (__syncwarp orders the
 // other lanes' later accesses after lane 0's acquire).
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int lane) {
@@ -338,7 +203,7 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int la
   return ok != 0;
 }
 
-template <int RPp, bool PRESCALED>
+template <int RPp>
 __global__ void __launch_bounds__(kThreads, 1)
 k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, TcArgs a) {
   Ctl* ctl = a.ctl;
@@ -346,8 +211,6 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
   unsigned char* sm = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   unsigned char* sA = sm + kOffA;
   unsigned char* sB = sm + kOffB;
-  float* Ps = reinterpret_cast<float*>(sm + kOffA);   // completion staging: the ring, once idle
-  float* Ts = Ps + BM * EPI_LD;
   __shared__ uint64_t afull[NA], aempty[NA], bfull[NS], tfull[NS], sfree[NS], cpdone[NS];
   __shared__ uint64_t accfull[2], accempty[2], mma_done;
   __shared__ uint32_t tmem_base;
@@ -356,13 +219,11 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
   __shared__ int s_npend;   // tiles this CTA completes (listed in a.pend), done at its end
   __shared__ float s_csc[kMaxRP];
   __shared__ float s_zi;
-  __shared__ const float* s_tn;   // the normaliser of this launch (by slot parity)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int c = blockIdx.x;
-  const int64_t S = a.S, ks = a.ks, K = a.K;
+  const int64_t S = a.S, ks = a.ks;
   const int G = a.G;
   const int64_t g0 = (int64_t)c * S / G, g1 = (int64_t)(c + 1) * S / G;
-  int64_t npre = 0;   // Zsrc stages issued before the programmatic wait (thread 0, the producer)
   if (tid == 0) {
     for (int s = 0; s < NA; ++s) {
       mbar_init(&afull[s], 1);
@@ -380,13 +241,8 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
     }
     mbar_init(&mma_done, 1);
     fence_barrier_init();
-    if (a.z_prefetch) npre = prefetch_a(&mapA, sA, afull, g0, g1, ks);
   }
   if (warp == 1) tmem_alloc(&tmem_base, kTmemCols);
-  // Launched as a programmatic dependent of the previous product: everything above ran
-  // while that product completed its tiles; apart from the prefetch of Zsrc (which the
-  // preceding kernels do not write), no global memory is touched before this.
-  pdl_wait();
   if (tid == 0) {
     // Iteration already abandoned, or Z outgrew its scale in the last S-step (the caller
     // rescales it): do nothing, and make the rest of the iteration skip too.
@@ -394,7 +250,6 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
     if (ctl && ctl->range_err) ctl->abort = 1;
     s_npend = 0;
     s_zi = a.zscale ? a.zscale[1] : 1.f;
-    s_tn = (ctl && ctl->slot_parity) ? a.Tn1 : a.Tn0;
   }
   if (tid < kMaxRP) s_csc[tid] = (tid < a.RP && a.cscale) ? a.cscale[tid] : 1.f;
   __syncthreads();
@@ -404,11 +259,11 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
   if (warp == 0) {
     // ---------------- TMA producer: Zsrc tiles ----------------
     if (lane == 0)
-      produce<true>(&mapA, sA, NA, kStageA, (uint32_t)kBoxA, afull, aempty, g0, g1, ks, K, ctl, &s_err, npre);
+      produce<true>(&mapA, sA, NA, kStageA, (uint32_t)kBoxA, afull, aempty, g0, g1, ks, ctl, &s_err);
   } else if (warp == 14) {
     // ---------------- TMA producer: skinny-operand tiles ----------------
     if (lane == 0)
-      produce<false>(&mapB, sB, NS, kStageB, (uint32_t)(2 * a.RP * BK * 2), bfull, sfree, g0, g1, ks, K, ctl,
+      produce<false>(&mapB, sB, NS, kStageB, (uint32_t)(2 * a.RP * BK * 2), bfull, sfree, g0, g1, ks, ctl,
                      &s_err);
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
@@ -490,7 +345,7 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
     // ---------------- converters: float32 stage in TMEM -> packed (h1, h2) in place ----------------
     const int q = (warp - 2) >> 2;              // 32-column half of the tile handled by this warp
     const uint32_t tlane = (uint32_t)((warp & 3) * 32) << 16;   // this warp's TMEM lane quarter
-    const float zs = (!PRESCALED && a.zscale) ? a.zscale[0] : 1.f;
+    const float zs = a.zscale ? a.zscale[0] : 1.f;
     int st = 0;
     uint32_t ph = 0;
     for (int64_t g = g0; g < g1; ++g) {
@@ -507,10 +362,8 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
 #pragma unroll
       for (int k = 0; k < 16; ++k) {
         float x0 = xs[2 * k], x1 = xs[2 * k + 1];
-        if (!PRESCALED) {
-          x0 *= zs;
-          x1 *= zs;
-        }
+        x0 *= zs;
+        x1 *= zs;
         const float h0 = __uint_as_float(__float_as_uint(x0) & 0xFFFFE000u);
         const float h1 = __uint_as_float(__float_as_uint(x1) & 0xFFFFE000u);
         h[k] = pack_h2(h0, h1);
@@ -601,7 +454,6 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
 
   tc_fence_before();
   __syncthreads();
-  pdl_launch_dependents();   // the stream is done: the next product may start its prologue
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tbase, kTmemCols);
@@ -612,241 +464,7 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
     const int64_t t = a.pend[(int64_t)c * a.maxpend + k];
     const int64_t c_first = cta_of(t * ks, S, G);
     const int nseg = (int)(cta_of((t + 1) * ks - 1, S, G) - c_first + 1);
-    tile_finish<RPp>(a, t, nseg, tid, kThreads, 0, Ps, Ts, s_csc, s_zi, s_tn);
-  }
-}
-
-// ---- 16-bit streaming product (precision form) -------------------------------------------
-// part/out = Z16 (rows x K, float16 copy of (X - S) s_Z, rounded) * B with B in its two-term
-// split c1 + 2^-11 c2 (rows 0..2RP-1 of bt2): one float16 MMA of N = 2 RP per stage gives
-// Z16 c1 and Z16 c2 side by side in tensor memory, summed as hi + 2^-11 lo in the
-// epilogue, float32 accumulation.  Z16 carries about 2^-12 relative rounding per element
-// (fixed for the whole chain); B is exact to about 2^-22, so the chain's error is that of
-// X's rounding alone (rounding B to one float16 term as well adds a fresh 2^-12 per
-// product, which the float32 correction pass can no longer remove when sigma_r and
-// sigma_{r+1} are close).  The Z16 tile of a stage is one 128-row x 64-column box that
-// the MMA reads straight from shared memory (no conversion), so the stream moves half
-// the bytes of the float32 kernel.  Same stream-K split, partial slots and deferred tile
-// completion as k_prod_tc.  RP <= 32 (the precision form's bound on r).
-// Warps: 0 TMA producer of Z16 tiles, 1 MMA issuer (TMEM owner), 2-5 epilogue, 6 TMA
-// producer of the skinny operand, 7 spare (completion only).
-constexpr int NA16 = 10, NS16 = 6, kThreads16 = 256;
-constexpr size_t kStageA16 = (size_t)BM * 128;                 // 64 halves x 128 rows = 16 KB
-constexpr int kMaxRP16 = 32;                                   // RP bound of the 16-bit kernel
-constexpr size_t kStageB16 = (size_t)2 * kMaxRP16 * 128;       // up to 2 x 32 rows of 64 halves = 8 KB
-constexpr size_t kOffB16 = NA16 * kStageA16;
-constexpr size_t kTc16Smem = kOffB16 + NS16 * kStageB16 + 1024;
-static_assert(kEpiBytes <= NA16 * kStageA16, "completion staging fits the 16-bit ring");
-static_assert(kTc16Smem <= 232448 - 1024, "shared memory of the 16-bit product");
-
-template <int RPp>
-__global__ void __launch_bounds__(kThreads16, 1)
-k_prod_h16(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, TcArgs a) {
-  Ctl* ctl = a.ctl;
-  extern __shared__ unsigned char smem_raw[];
-  unsigned char* sm = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  unsigned char* sA = sm;
-  unsigned char* sB = sm + kOffB16;
-  float* Ps = reinterpret_cast<float*>(sm);   // completion staging: the ring, once idle
-  float* Ts = Ps + BM * EPI_LD;
-  __shared__ uint64_t afull[NA16], aempty[NA16], bfull[NS16], bempty[NS16];
-  __shared__ uint64_t accfull[2], accempty[2], mma_done;
-  __shared__ uint32_t tmem_base;
-  __shared__ volatile int s_err;
-  __shared__ int s_stop, s_last, s_npend;
-  __shared__ float s_csc[kMaxRP];
-  __shared__ float s_zi;
-  __shared__ const float* s_tn;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int c = blockIdx.x;
-  const int64_t S = a.S, ks = a.ks;
-  const int G = a.G;
-  const int64_t g0 = (int64_t)c * S / G, g1 = (int64_t)(c + 1) * S / G;
-  static_assert(RPp <= kMaxRP16, "16-bit kernel: RP <= 32");
-  const uint32_t bbytes = (uint32_t)(2 * a.RP * 128);   // c1 and c2 rows of the stage
-  if (tid == 0) {
-    for (int s = 0; s < NA16; ++s) {
-      mbar_init(&afull[s], 1);
-      mbar_init(&aempty[s], 1);
-    }
-    for (int s = 0; s < NS16; ++s) {
-      mbar_init(&bfull[s], 1);
-      mbar_init(&bempty[s], 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&accfull[b], 1);
-      mbar_init(&accempty[b], 4);
-    }
-    mbar_init(&mma_done, 1);
-    fence_barrier_init();
-  }
-  if (warp == 1) tmem_alloc(&tmem_base, 128);
-  pdl_wait();   // see k_prod_tc
-  if (tid == 0) {
-    s_err = (ctl && (ctl->abort || ctl->range_err)) ? 2 : 0;
-    if (ctl && ctl->range_err) ctl->abort = 1;
-    s_npend = 0;
-    s_zi = a.zscale ? a.zscale[1] : 1.f;
-    s_tn = (ctl && ctl->slot_parity) ? a.Tn1 : a.Tn0;
-  }
-  if (tid < kMaxRP) s_csc[tid] = (tid < a.RP && a.cscale) ? a.cscale[tid] : 1.f;
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tbase = tmem_base;
-
-  if (warp == 0 || warp == 6) {
-    // ---------------- TMA producers: Z16 tiles (warp 0), skinny-operand tiles (warp 6) ----------
-    if (lane == 0) {
-      const bool isA = warp == 0;
-      const int nslot = isA ? NA16 : NS16;
-      uint64_t* fullb = isA ? afull : bfull;
-      uint64_t* emptyb = isA ? aempty : bempty;
-      int64_t t = g0 / ks, kst = g0 % ks, issued = 0;
-      int s = 0;
-      uint32_t ph = 0;
-      const uint64_t pol = policy_evict_first();   // Z16 streamed once per product
-      for (int64_t g = g0; g < g1 && !s_err; ++g) {
-        if (!mbar_wait(&emptyb[s], ph ^ 1u, kWaitLimit)) { note_timeout(ctl, &s_err); break; }
-        if (isA) {
-          mbar_expect_tx(&fullb[s], (uint32_t)kStageA16);
-          tma_load_2d_hint(sA + (size_t)s * kStageA16, &mapA, &fullb[s], (int)(kst * BK), (int)(t * BM), pol);
-        } else {
-          mbar_expect_tx(&fullb[s], bbytes);
-          tma_load_2d(sB + (size_t)s * kStageB16, &mapB, &fullb[s], (int)(kst * BK), 0);
-        }
-        ++issued;
-        if (++kst == ks) { kst = 0; ++t; }
-        if (++s == nslot) { s = 0; ph ^= 1u; }
-      }
-      for (int64_t j = (issued > nslot ? issued - nslot : 0); j < issued; ++j)
-        if (!mbar_wait(&fullb[(int)(j % nslot)], (uint32_t)((j / nslot) & 1), kWaitLimit)) note_timeout(ctl, &s_err);
-    }
-  } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      const uint32_t id = idesc_f16(BM, 2 * a.RP);   // [Z16 c1 | Z16 c2], RP multiple of 8
-      int ch = 0, sa = 0, sb = 0;
-      uint32_t pha = 0, phb = 0;
-      int64_t kst = g0 % ks, g = g0;
-      while (g < g1 && !s_err) {
-        int64_t n = ks - kst;
-        if (n > kChunk) n = kChunk;
-        if (n > g1 - g) n = g1 - g;
-        const int b = ch & 1;
-        if (!mbar_wait(&accempty[b], (uint32_t)(((ch >> 1) & 1) ^ 1), kWaitLimit)) { note_timeout(ctl, &s_err); break; }
-        tc_fence_after();
-        const uint32_t dcol = tbase + (uint32_t)(b * 64);
-        uint32_t acc = 0;
-        for (int64_t e = 0; e < n; ++e) {
-          if (!mbar_wait(&afull[sa], pha, kWaitLimit) || !mbar_wait(&bfull[sb], phb, kWaitLimit)) {
-            note_timeout(ctl, &s_err);
-            break;
-          }
-          tc_fence_after();
-          const uint64_t da = sdesc_k128(sA + (size_t)sa * kStageA16), db = sdesc_k128(sB + (size_t)sb * kStageB16);
-#pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk) {
-            const uint64_t off = (uint64_t)((kk * 16 * 2) >> 4);   // 32 bytes per 16-wide K step
-            mma_bf16(dcol, da + off, db + off, id, acc);
-            acc = 1u;
-          }
-          mma_commit(&aempty[sa]);
-          mma_commit(&bempty[sb]);
-          if (++sa == NA16) { sa = 0; pha ^= 1u; }
-          if (++sb == NS16) { sb = 0; phb ^= 1u; }
-        }
-        if (s_err) break;
-        mma_commit(&accfull[b]);
-        ++ch;
-        g += n;
-        kst += n;
-        if (kst == ks) kst = 0;
-      }
-      mma_commit(&mma_done);
-      if (!mbar_wait(&mma_done, 0, kWaitLimit)) note_timeout(ctl, &s_err);
-    }
-  } else if (warp >= 2 && warp < 6) {
-    // ---------------- epilogue: TMEM -> running sums -> partial slot ----------------
-    const int et = tid - 64;
-    const int q4 = warp & 3;
-    const int row = q4 * 32 + lane;
-    const uint32_t tlane = (uint32_t)(q4 * 32) << 16;
-    int ch = 0, npend = 0;
-    int64_t g = g0;
-    for (;;) {
-      named_sync(1, BM);
-      if (et == 0) s_stop = (g >= g1) || s_err;
-      named_sync(1, BM);
-      if (s_stop) break;
-      const int64_t t = g / ks;
-      const int64_t tend = ((t + 1) * ks < g1) ? (t + 1) * ks : g1;
-      float y[RPp];
-#pragma unroll
-      for (int l = 0; l < RPp; ++l) y[l] = 0.f;
-      bool failed = false;
-      for (; g < tend; g = (g + kChunk < tend) ? g + kChunk : tend, ++ch) {
-        if (failed) continue;
-        const int b = ch & 1;
-        if (!__all_sync(0xffffffffu, mbar_wait(&accfull[b], (uint32_t)((ch >> 1) & 1), kWaitLimit))) {
-          if (lane == 0) note_timeout(ctl, &s_err);
-          failed = true;
-          continue;
-        }
-        tc_fence_after();
-        const uint32_t taddr = tbase + (uint32_t)(b * 64) + tlane;
-#pragma unroll
-        for (int c0 = 0; c0 < RPp; c0 += 8) {
-          if (c0 < a.RP) {
-            float vh[8], vl[8];
-            tmem_ld8(taddr + c0, vh);
-            tmem_ld8(taddr + a.RP + c0, vl);
-#pragma unroll
-            for (int l = 0; l < 8; ++l) y[c0 + l] += fmaf(vl[l], kLoInv, vh[l]);
-          }
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&accempty[b]);
-      }
-      named_sync(1, BM);
-      if (et == 0) s_stop = s_err;
-      named_sync(1, BM);
-      if (s_stop) break;
-      const int64_t c_first = cta_of(t * ks, S, G);
-      const int nseg = (int)(cta_of((t + 1) * ks - 1, S, G) - c_first + 1);
-      const int slot = (int)(c - c_first);
-      float* p = a.part + ((t * a.maxseg + slot) * BM + row) * (int64_t)a.RP;
-#pragma unroll
-      for (int l = 0; l < RPp; l += 4)
-        if (l < a.RP) *reinterpret_cast<float4*>(p + l) = make_float4(y[l], y[l + 1], y[l + 2], y[l + 3]);
-      __threadfence();
-      named_sync(1, BM);
-      if (et == 0) s_last = (atomicAdd(&a.counters[t], 1u) == (unsigned)(nseg - 1));
-      named_sync(1, BM);
-      if (s_last) {
-        if (et == 0) {
-          if (npend < a.maxpend) a.pend[(int64_t)c * a.maxpend + npend] = (int)t;
-          else if (ctl) ctl->abort = 1;
-        }
-        ++npend;
-      }
-    }
-    if (et == 0) s_npend = npend;
-  }
-
-  tc_fence_before();
-  __syncthreads();
-  pdl_launch_dependents();
-  if (warp == 1) {
-    tc_fence_after();
-    tmem_dealloc(tbase, 128);
-  }
-  const int np = s_err ? 0 : (s_npend < a.maxpend ? s_npend : a.maxpend);
-  for (int k = 0; k < np; ++k) {
-    const int64_t t = a.pend[(int64_t)c * a.maxpend + k];
-    const int64_t c_first = cta_of(t * ks, S, G);
-    const int nseg = (int)(cta_of((t + 1) * ks - 1, S, G) - c_first + 1);
-    tile_finish<RPp>(a, t, nseg, tid, kThreads16, 0, Ps, Ts, s_csc, s_zi, s_tn);
+    tile_finish(a, t, nseg, tid, kThreads, s_csc, s_zi);
   }
 }
 
@@ -925,6 +543,18 @@ bool make_tmap_f16(void* map, const void* base, int64_t rows, int64_t cols, int6
   return make_tmap(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, base, rows, cols, ld, box_rows);
 }
 
+bool make_tmap_split(void* map, const void* base, int64_t rows, int64_t ldz, int box_rows) {
+  PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[3] = {64, (cuuint64_t)(ldz / 32), (cuuint64_t)rows};
+  cuuint64_t strides[2] = {128, (cuuint64_t)ldz * 4};
+  cuuint32_t box[3] = {64, 1, (cuuint32_t)box_rows};
+  cuuint32_t es[3] = {1, 1, 1};
+  return fn(reinterpret_cast<CUtensorMap*>(map), CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(base), dims, strides,
+            box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 int tc_rpp(int RP) { return (RP + 15) / 16 * 16; }
 
 void launch_split_t(const float* B, int64_t rows, int RP, void* bt2, int64_t ldb, float* cscale, cudaStream_t st,
@@ -955,48 +585,11 @@ TcGeom tc_geometry(int64_t rows, int64_t K, int nsm) {
   return g;
 }
 
-template <int RPp, bool PS>
-static cudaError_t prep_one() {
-  return cudaFuncSetAttribute(k_prod_tc<RPp, PS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
-}
-
-template <int RPp>
-static cudaError_t prep16() {
-  return cudaFuncSetAttribute(k_prod_h16<RPp>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTc16Smem);
-}
-
 cudaError_t prepare_tc_kernels() {
   cudaError_t e = cudaSuccess;
-  if (e == cudaSuccess) e = prep16<16>();
-  if (e == cudaSuccess) e = prep16<32>();
-  if (e == cudaSuccess) e = prep_one<16, false>();
-  if (e == cudaSuccess) e = prep_one<32, false>();
-  if (e == cudaSuccess) e = prep_one<48, false>();
-  if (e == cudaSuccess) e = prep_one<64, false>();
-  if (e == cudaSuccess) e = prep_one<16, true>();
-  if (e == cudaSuccess) e = prep_one<32, true>();
-  if (e == cudaSuccess) e = prep_one<48, true>();
-  if (e == cudaSuccess) e = prep_one<64, true>();
+  for (auto k : {k_prod_tc<16>, k_prod_tc<32>, k_prod_tc<48>, k_prod_tc<64>})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
   return e;
-}
-
-// Launch with the programmatic-stream-serialization attribute when pdl is set: the kernel
-// may begin (barrier set-up, tensor-memory allocation) while the preceding kernel of the
-// stream finishes, and waits for it in pdl_wait() before its first global access.
-template <typename Kern>
-static void launch_tc(Kern kern, unsigned grid, unsigned block, size_t smem, cudaStream_t st, bool pdl,
-                      const CUtensorMap& A, const CUtensorMap& B, const TcArgs& a) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  cudaLaunchKernelEx(&cfg, kern, A, B, a);
 }
 
 void launch_prod_tc(const TcLaunch& l, cudaStream_t st) {
@@ -1011,45 +604,18 @@ void launch_prod_tc(const TcLaunch& l, cudaStream_t st) {
   a.part = l.part;
   a.counters = l.counters;
   a.out = l.out;
-  a.bt2 = reinterpret_cast<__half*>(l.bt2);
-  a.ldb = l.ldb;
-  a.Tn0 = l.Tn[0];
-  a.Tn1 = l.Tn[1];
   a.cscale = l.cscale;
   a.zscale = l.zscale;
-  a.gram_part = l.gram_part;
-  a.gram_mode = l.gram_mode;
-  a.z_prefetch = l.z_prefetch;
-  a.t_upper = l.t_upper;
   a.pend = l.pend;
   a.maxpend = l.geom.maxpend;
   a.ctl = l.ctl;
   const CUtensorMap& A = *reinterpret_cast<const CUtensorMap*>(l.mapA);
   const CUtensorMap& B = *reinterpret_cast<const CUtensorMap*>(l.mapB);
-  a.prescaled = l.prescaled;
-  const int rpp = tc_rpp(l.RP);
-  const bool pdl = l.pdl != 0;
-  const unsigned G = (unsigned)a.G;
-  if (l.half_a) {
-    switch (rpp) {
-      case 16: launch_tc(k_prod_h16<16>, G, kThreads16, kTc16Smem, st, pdl, A, B, a); break;
-      case 32: launch_tc(k_prod_h16<32>, G, kThreads16, kTc16Smem, st, pdl, A, B, a); break;
-      default: if (l.ctl) cudaMemsetAsync(&l.ctl->abort, 0xff, sizeof(int), st); break;   // RP > 32: rejected at init
-    }
-  } else if (l.prescaled) {
-    switch (rpp) {
-      case 16: launch_tc(k_prod_tc<16, true>, G, kThreads, kTcSmem, st, pdl, A, B, a); break;
-      case 32: launch_tc(k_prod_tc<32, true>, G, kThreads, kTcSmem, st, pdl, A, B, a); break;
-      case 48: launch_tc(k_prod_tc<48, true>, G, kThreads, kTcSmem, st, pdl, A, B, a); break;
-      default: launch_tc(k_prod_tc<64, true>, G, kThreads, kTcSmem, st, pdl, A, B, a); break;
-    }
-  } else {
-    switch (rpp) {
-      case 16: launch_tc(k_prod_tc<16, false>, G, kThreads, kTcSmem, st, pdl, A, B, a); break;
-      case 32: launch_tc(k_prod_tc<32, false>, G, kThreads, kTcSmem, st, pdl, A, B, a); break;
-      case 48: launch_tc(k_prod_tc<48, false>, G, kThreads, kTcSmem, st, pdl, A, B, a); break;
-      default: launch_tc(k_prod_tc<64, false>, G, kThreads, kTcSmem, st, pdl, A, B, a); break;
-    }
+  switch (tc_rpp(l.RP)) {
+    case 16: k_prod_tc<16><<<a.G, kThreads, kTcSmem, st>>>(A, B, a); break;
+    case 32: k_prod_tc<32><<<a.G, kThreads, kTcSmem, st>>>(A, B, a); break;
+    case 48: k_prod_tc<48><<<a.G, kThreads, kTcSmem, st>>>(A, B, a); break;
+    default: k_prod_tc<64><<<a.G, kThreads, kTcSmem, st>>>(A, B, a); break;
   }
 }
 

@@ -49,45 +49,58 @@ __global__ void k_unpad_copy(const float* src, int64_t rows, int RP, float* dst,
   }
 }
 
-__global__ void k_sumsq(const float* X, int64_t m, int64_t n, int64_t ldx, double* out) {
-  double acc = 0.0;
-  const int64_t total = m * n;
-  for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 16; base < total;
-       base += (int64_t)gridDim.x * blockDim.x * 16) {
-    float f = 0.f;
-    for (int64_t e = base; e < min(total, base + 16); ++e) {
-      int64_t i = e / n, j = e % n;
-      float v = X[i * ldx + j];
-      f = fmaf(v, v, f);
-    }
-    acc += (double)f;
-  }
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(out, acc);
-}
-
 // ---- LSD radix sort, 4-bit digits, items owned contiguously by threads (stable) ------
 constexpr int SORT_THREADS = 256, SORT_ITEMS = 16, SORT_TILE = SORT_THREADS * SORT_ITEMS;
 
-__global__ void k_scale_copy(const float* src, int64_t rows, int64_t cols, int64_t lds, float* dst, int64_t ldd,
-                             const float* scale) {
-  const float sc = scale[0];
-  for (int64_t r = blockIdx.x; r < rows; r += gridDim.x)
-    for (int64_t c = threadIdx.x; c < cols; c += blockDim.x) dst[r * ldd + c] = src[r * lds + c] * sc;
-}
-
-__global__ void k_scale_update(float* zscale, const float* f) {
-  zscale[0] *= f[0];
-  zscale[1] *= f[1];
-}
-
-// max |Z| over the matrix (non-negative floats order like their bit patterns).
-__global__ void k_maxabs(const float* Z, int64_t rows, int64_t cols, int64_t ld, unsigned* out) {
+// max |Z| over the matrix (non-negative floats order like their bit patterns) and, with
+// sumsq, += sum of Z^2 in the same pass: float4 loads, four in flight per thread, float
+// sums of sixteen squares added up in float64.  Bound: 4 rows cols bytes read from HBM.
+__global__ void __launch_bounds__(256)
+k_maxabs(const float* __restrict__ Z, int64_t rows, int64_t cols, int64_t ld, unsigned* out, double* sumsq, int vec) {
   float m = 0.f;
-  for (int64_t r = blockIdx.x; r < rows; r += gridDim.x)
-    for (int64_t c = threadIdx.x; c < cols; c += blockDim.x) m = fmaxf(m, fabsf(Z[r * ld + c]));
-  for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(m));
+  double acc = 0.0;
+  const int64_t per = (cols + 15) / 16, total = rows * per;   // runs of 16 columns
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = e / per, j = (e - i * per) * 16;
+    const float* z = Z + i * ld + j;
+    float v[16];
+    if (vec && j + 16 <= cols) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float4 q = __ldg(reinterpret_cast<const float4*>(z) + u);
+        v[4 * u] = q.x; v[4 * u + 1] = q.y; v[4 * u + 2] = q.z; v[4 * u + 3] = q.w;
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < 16; ++u) v[u] = j + u < cols ? z[u] : 0.f;
+    }
+    float f = 0.f;
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      m = fmaxf(m, fabsf(v[u]));
+      f = fmaf(v[u], v[u], f);
+    }
+    if (sumsq) acc += (double)f;
+  }
+  for (int o = 16; o; o >>= 1) {
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (sumsq) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  }
+  __shared__ float sm[8];
+  __shared__ double sa[8];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (lane == 0) {
+    sm[w] = m;
+    sa[w] = acc;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int k = 1; k < 8; ++k) {
+    m = fmaxf(m, sm[k]);
+    acc += sa[k];
+  }
+  if (out) atomicMax(out, __float_as_uint(m));
+  if (sumsq) atomicAdd(sumsq, acc);
 }
 
 __global__ void k_make_zscale(const unsigned* mx, float* zscale) {
@@ -244,33 +257,37 @@ void launch_unpad_copy(const float* src, int64_t rows, int RP, float* dst, int c
   if (grid) k_unpad_copy<<<grid, 256, 0, st>>>(src, rows, RP, dst, cols);
 }
 
-void launch_sumsq(const float* X, int64_t m, int64_t n, int64_t ldx, double* out, int nsm,
-                  cudaStream_t st) {
-  k_sumsq<<<(unsigned)(4 * nsm), 256, 0, st>>>(X, m, n, ldx, out);
-}
-
 size_t sort_coo_scratch(long long nnz) {
   long long nblk = (nnz + SORT_TILE - 1) / SORT_TILE;
   return (size_t)nnz * (sizeof(long long) + sizeof(float)) + (size_t)(16 * nblk + 16) * sizeof(unsigned) + 256;
 }
 
-void launch_zscale(const float* Z, int64_t rows, int64_t cols, int64_t ld, unsigned* zmax, float* zscale, int nsm,
-                   cudaStream_t st) {
-  cudaMemsetAsync(zmax, 0, sizeof(unsigned), st);
-  int64_t grid = 4LL * nsm;
-  if (grid > rows) grid = rows;
-  k_maxabs<<<(unsigned)grid, 256, 0, st>>>(Z, rows, cols, ld, zmax);
+static void launch_maxabs(const float* Z, int64_t rows, int64_t cols, int64_t ld, unsigned* mx, double* sumsq, int nsm,
+                          cudaStream_t st) {
+  int64_t grid = (rows * ((cols + 15) / 16) + 255) / 256;
+  if (grid > 8LL * nsm) grid = 8LL * nsm;
+  const int vec = (ld % 4 == 0) && (reinterpret_cast<uintptr_t>(Z) % 16 == 0);
+  k_maxabs<<<(unsigned)(grid > 0 ? grid : 1), 256, 0, st>>>(Z, rows, cols, ld, mx, sumsq, vec);
+}
+
+void launch_zscale_from(const unsigned* base, const float* extra, int64_t n_extra, unsigned* zmax, float* zscale, int nsm,
+                        cudaStream_t st) {
+  cudaMemcpyAsync(zmax, base, sizeof(unsigned), cudaMemcpyDeviceToDevice, st);
+  if (extra && n_extra > 0) launch_maxabs(extra, 1, n_extra, n_extra, zmax, nullptr, nsm, st);
   k_make_zscale<<<1, 1, 0, st>>>(zmax, zscale);
 }
 
-void launch_scale_copy(const float* src, int64_t rows, int64_t cols, int64_t lds, float* dst, int64_t ldd,
-                       const float* scale, int nsm, cudaStream_t st) {
-  int64_t grid = 4LL * nsm;
-  if (grid > rows) grid = rows;
-  k_scale_copy<<<(unsigned)grid, 256, 0, st>>>(src, rows, cols, lds, dst, ldd, scale);
+void launch_sumsq(const float* X, int64_t m, int64_t n, int64_t ldx, double* out, int nsm, cudaStream_t st) {
+  launch_maxabs(X, m, n, ldx, nullptr, out, nsm, st);
 }
 
-void launch_scale_update(float* zscale, const float* f, cudaStream_t st) { k_scale_update<<<1, 1, 0, st>>>(zscale, f); }
+void launch_zscale(const float* Z, int64_t rows, int64_t cols, int64_t ld, unsigned* zmax, float* zscale, int nsm,
+                   cudaStream_t st, double* sumsq, const float* extra, int64_t n_extra) {
+  cudaMemsetAsync(zmax, 0, sizeof(unsigned), st);
+  launch_maxabs(Z, rows, cols, ld, zmax, sumsq, nsm, st);
+  if (extra && n_extra > 0) launch_maxabs(extra, 1, n_extra, n_extra, zmax, nullptr, nsm, st);
+  k_make_zscale<<<1, 1, 0, st>>>(zmax, zscale);
+}
 
 void launch_sort_coo(long long* idx, float* val, long long nnz, void* scratch, size_t scratch_bytes,
                      int idx_bits, cudaStream_t st) {

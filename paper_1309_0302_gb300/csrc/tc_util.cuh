@@ -280,6 +280,30 @@ __device__ __forceinline__ void tmem_ld16x2(uint32_t ta, uint32_t tb, float* va,
   }
 }
 
+// Columns ta .. ta+15 and tb .. tb+15 (ta, tb multiples of 8) of this warp's lanes: four
+// 8-column loads and a single wait.
+__device__ __forceinline__ void tmem_ld8x4(uint32_t ta, uint32_t tb, float* va, float* vb) {
+  uint32_t r[32];
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[8 * k]), "=r"(r[8 * k + 1]), "=r"(r[8 * k + 2]), "=r"(r[8 * k + 3]), "=r"(r[8 * k + 4]),
+                   "=r"(r[8 * k + 5]), "=r"(r[8 * k + 6]), "=r"(r[8 * k + 7])
+                 : "r"((k < 2 ? ta : tb) + 8u * (k & 1)));
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+                 "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
+                 "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+               :
+               : "memory");
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    va[j] = __uint_as_float(r[j]);
+    vb[j] = __uint_as_float(r[16 + j]);
+  }
+}
+
 // Programmatic dependent launch: wait until the preceding kernel of the stream has
 // completed and its memory is visible (returns at once when this launch has no
 // programmatic dependency), and let the next kernel of the stream start its prologue
