@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <cmath>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "godec_internal.cuh"
@@ -52,6 +53,8 @@ struct godec_ctx {
   int ev_used = 0;
   int dev = 0, nsm = 0;   // nsm: the SMs this problem's grids are sized for (its budget)
   int nsm_dev = 0;          // SMs of the device
+  char* arena = nullptr;                 // one allocation for every buffer of the context
+  size_t arena_bytes = 0;
   size_t npart_cap = 0;     // stream-K buffers (sized for the whole device)
   const float* X = nullptr;
   void* Z = nullptr;                   // m x ldz   working (X - S) s_Z, split (k_prod.cu)
@@ -116,6 +119,8 @@ struct godec_ctx {
   int graph_r[2] = {-1, -1};
   unsigned graph_epoch = 0;   // bumped whenever captured graphs become invalid (buffers, geometry)
   int graph_nodes = 0;
+  int exact_direct = 3;       // exact iterations still launched directly before a graph of them is captured
+  int fast_run = 0;           // fast iterations since the start or the last alarm
   bool need_exact = true;
   int exact_left = 0;   // exact iterations still owed after an alarm of the lagged normalisers
   int backoff = 1;      // exact iterations owed at the next alarm (doubles while alarms repeat)
@@ -208,10 +213,16 @@ void free_graphs(godec_ctx* c) {
   }
 }
 
+// A buffer of the context: part of its arena, or (candidates and S grown later) its own.
+void ctx_free(godec_ctx* c, void* p) {
+  char* q = static_cast<char*>(p);
+  if (q && !(q >= c->arena && q < c->arena + c->arena_bytes)) cudaFree(p);
+}
+
 godec_status alloc_candidates(godec_ctx* c, unsigned long long cap) {
-  cudaFree(c->cand_key);
-  cudaFree(c->cand_idx);
-  cudaFree(c->cand_val);
+  ctx_free(c, c->cand_key);
+  ctx_free(c, c->cand_idx);
+  ctx_free(c, c->cand_val);
   c->cand_key = nullptr;
   c->cand_idx = nullptr;
   c->cand_val = nullptr;
@@ -225,14 +236,20 @@ godec_status alloc_candidates(godec_ctx* c, unsigned long long cap) {
 // ---------------------------------------------------------------------------------
 // Launch helpers
 // ---------------------------------------------------------------------------------
+cudaEvent_t next_event(godec_ctx* c) {
+  cudaEvent_t& e = c->ev[c->ev_used++ % kEvents];
+  if (!e) cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
+  return e;
+}
+
 void fork_side(godec_ctx* c) {
-  cudaEvent_t e = c->ev[c->ev_used++ % kEvents];
+  cudaEvent_t e = next_event(c);
   cudaEventRecord(e, c->st);
   cudaStreamWaitEvent(c->side_st, e, 0);
 }
 
 void join_side(godec_ctx* c) {
-  cudaEvent_t e = c->ev[c->ev_used++ % kEvents];
+  cudaEvent_t e = next_event(c);
   cudaEventRecord(e, c->side_st);
   cudaStreamWaitEvent(c->st, e, 0);
 }
@@ -241,7 +258,7 @@ void join_side(godec_ctx* c) {
 // iteration) is needed only before the S-step commits, so it overlaps the rest of the
 // chain instead of delaying the lagged-normaliser updates queued behind it.
 void fork_rank(godec_ctx* c) {
-  cudaEvent_t e = c->ev[c->ev_used++ % kEvents];
+  cudaEvent_t e = next_event(c);
   cudaEventRecord(e, c->st);
   cudaStreamWaitEvent(c->rank_st, e, 0);
   c->rank_forked = true;
@@ -249,7 +266,7 @@ void fork_rank(godec_ctx* c) {
 
 void join_rank(godec_ctx* c) {
   if (!c->rank_forked) return;
-  cudaEvent_t e = c->ev[c->ev_used++ % kEvents];
+  cudaEvent_t e = next_event(c);
   cudaEventRecord(e, c->rank_st);
   cudaStreamWaitEvent(c->st, e, 0);
   c->rank_forked = false;
@@ -298,7 +315,7 @@ void prod(godec_ctx* c, int i, float* out, bool want_bt2, const float* T0, const
 }
 
 cudaEvent_t record(godec_ctx* c, cudaStream_t s) {
-  cudaEvent_t e = c->ev[c->ev_used++ % kEvents];
+  cudaEvent_t e = next_event(c);
   cudaEventRecord(e, s);
   return e;
 }
@@ -828,8 +845,8 @@ void refresh_z(godec_ctx* c, double* sumsq) {
 }
 
 godec_status reset_state(godec_ctx* c) {
-  free_graphs(c);
-  c->r = c->p.r;
+  c->r = c->p.r;   // captured graphs stay: buffers and geometry are the same, and graph_r tells a rank drop
+  c->fast_run = 0;
   c->rank_drops = 0;
   c->need_exact = true;
   c->exact_left = 0;
@@ -941,6 +958,7 @@ godec_status handle_abort(godec_ctx* c, const Ctl& h) {
     // the lagged normalisers no longer condition the chain (its subspaces moved): stay on
     // the exact path for `backoff` iterations, twice as many at each repeated alarm
     c->need_exact = true;
+    c->fast_run = 0;
     c->exact_left = c->backoff;
     c->backoff = std::min(2 * c->backoff, kMaxBackoff);
   } else if (h.need_bigger_cand) {
@@ -964,6 +982,7 @@ void note_done(godec_ctx* c, bool fast, int k) {
   if (k <= 0) return;
   if (fast) {
     c->backoff = 1;
+    c->fast_run += k;
     return;
   }
   c->exact_iters += k;
@@ -985,14 +1004,25 @@ godec_status run_iterations(godec_ctx* c, int n_iter, double tol) {
     if ((s = SET_CTL(tol, tol))) return s;
   }
   int guard = 0, done = 0;
-  int chunk = tol >= 0.0 ? 1 : n_iter;
+  // Launches ahead of the host's look at the result: an abandoned iteration turns those queued
+  // behind it into empty launches (about 100 us each at 10^4 x 10^4), and an alarm is likeliest
+  // in the first fast iterations, so these go two, four, ... at a time.
+  int chunk = tol >= 0.0 ? 1 : std::max(2, c->fast_run);
   while (done < n_iter) {
     const int mode = c->need_exact ? 0 : 1;
-    if (!c->gexec[mode] || c->graph_r[mode] != c->r) {
-      if ((s = build_graph(c, mode))) return s;
-    }
     const int want = std::min(mode == 0 ? std::max(c->exact_left, 1) : chunk, n_iter - done);
-    for (int i = 0; i < want; ++i) CK(cudaGraphLaunch(c->gexec[mode], c->st));
+    for (int i = 0; i < want; ++i) {
+      bool have = c->gexec[mode] && c->graph_r[mode] == c->r;
+      if (!have && mode == 0 && c->exact_direct > 0) {
+        // most runs take the exact path once or twice: a graph of it would not pay
+        --c->exact_direct;
+        enqueue_iteration(c, false);
+        CK(cudaGetLastError());
+        continue;
+      }
+      if (!have && (s = build_graph(c, mode))) return s;
+      CK(cudaGraphLaunch(c->gexec[mode], c->st));
+    }
     if ((s = read_ctl(c, &h))) return s;
     const int before = done;
     done = h.iter - start;
@@ -1000,10 +1030,12 @@ godec_status run_iterations(godec_ctx* c, int n_iter, double tol) {
     if (h.abort) {
       if (h.converged) return GODEC_OK;
       if ((s = handle_abort(c, h))) return s;
+      if (tol < 0.0) chunk = 2;
       if (++guard > 64) return fail(c, GODEC_ERR_STATE, "too many aborted iterations");
       continue;
     }
-    if (tol >= 0.0 && chunk < 8) chunk *= 2;
+    if (mode == 1) chunk = tol >= 0.0 ? std::min(2 * chunk, 8) : 2 * chunk;
+    if (chunk > n_iter) chunk = std::max(n_iter, 1);
   }
   return GODEC_OK;
 }
@@ -1054,12 +1086,10 @@ void godec_destroy(godec_ctx* c) {
   if (!c) return;
   if (c->st) cudaStreamSynchronize(c->st);
   free_graphs(c);
-  void* ptrs[] = {c->Z, c->A1, c->A1_orig, c->P, c->bt2, c->cs, c->rescale_tmp, c->LA, c->LB, c->Q1, c->Q2,
-                  c->U, c->V, c->sigma, c->Um, c->Vm, c->part, c->counters, c->gparts, c->RA, c->RB, c->Wa, c->Wb, c->Qa, c->Qb, c->Qtmp, c->Rf,
-                  c->cs_ref, c->rf_part, c->rf_g, c->rf_C, c->rf_core, c->rf_U, c->rf_V, c->g64, c->g32, c->gscr,
-                  c->Rtmp, c->Rslot, c->Tslot, c->Rfin, c->Pi, c->Vprev, c->ctl, c->cand_key, c->cand_idx,
-                  c->cand_val, c->S_idx[0], c->S_idx[1], c->S_val[0], c->S_val[1], c->sbits, c->XA1};
-  for (void* p : ptrs) cudaFree(p);
+  for (void* p : {(void*)c->cand_key, (void*)c->cand_idx, (void*)c->cand_val, (void*)c->S_idx[0], (void*)c->S_idx[1],
+                  (void*)c->S_val[0], (void*)c->S_val[1]})
+    ctx_free(c, p);
+  cudaFree(c->arena);
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
   for (cudaEvent_t e : c->ev)
     if (e) cudaEventDestroy(e);
@@ -1111,35 +1141,42 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
   CKI(cudaStreamCreateWithFlags(&c->cap_st, cudaStreamNonBlocking));
   CKI(cudaStreamCreateWithFlags(&c->side_st, cudaStreamNonBlocking));
   CKI(cudaStreamCreateWithFlags(&c->rank_st, cudaStreamNonBlocking));
-  for (int k = 0; k < kEvents; ++k) CKI(cudaEventCreateWithFlags(&c->ev[k], cudaEventDisableTiming));
   const int64_t m = p->m, n = p->n, mx = std::max(m, n);
   const int RP = c->RP, np = c->nprod;
   const size_t rr = (size_t)RP * RP;
   c->X = X;
   c->half = p->precision == GODEC_PREC_BF16_REFINE;
+  // every buffer's address and size, 256-byte aligned, for one allocation (39 calls of about
+  // 20 us, and as many frees, were a quarter of a decomposition of a 3001 x 2047 matrix)
+  std::vector<std::pair<void**, size_t>> plan;
+  auto want = [&](auto** q, size_t elems) {
+    *q = nullptr;
+    plan.emplace_back(reinterpret_cast<void**>(q), c->arena_bytes);
+    c->arena_bytes += (std::max<size_t>(elems, 1) * sizeof(**q) + 255) & ~size_t(255);
+  };
   c->ldz = (n + 63) / 64 * 64;   // whole 64-column blocks of the split copy
-  CKI(dalloc(reinterpret_cast<float**>(&c->Z), (size_t)m * c->ldz));
+  want(reinterpret_cast<float**>(&c->Z), (size_t)m * c->ldz);
   if (c->half || greb || c->naive || c->lingo) {
     const size_t W = 64;   // columns of the correction's [U | A] and [V | B] (2r <= 64)
-    CKI(dalloc(&c->RA, (size_t)m * RP));
-    CKI(dalloc(&c->RB, (size_t)n * RP));
-    CKI(dalloc(&c->Wa, (size_t)m * W));
-    CKI(dalloc(&c->Wb, (size_t)n * W));
-    CKI(dalloc(&c->Qa, (size_t)m * W));
-    CKI(dalloc(&c->Qb, (size_t)n * W));
-    CKI(dalloc(&c->Qtmp, (size_t)mx * W));
-    CKI(dalloc(&c->Rf, (size_t)8 * W * W));
-    CKI(dalloc(&c->cs_ref, (size_t)RP));
-    CKI(dalloc(&c->rf_part, (size_t)kRefineParts * W * W));
-    CKI(dalloc(&c->rf_g, W * W));
-    CKI(dalloc(&c->rf_C, W * W));
-    CKI(dalloc(&c->rf_core, W * W));
-    CKI(dalloc(&c->rf_U, W * W));
-    CKI(dalloc(&c->rf_V, W * W));
+    want(&c->RA, (size_t)m * RP);
+    want(&c->RB, (size_t)n * RP);
+    want(&c->Wa, (size_t)m * W);
+    want(&c->Wb, (size_t)n * W);
+    want(&c->Qa, (size_t)m * W);
+    want(&c->Qb, (size_t)n * W);
+    want(&c->Qtmp, (size_t)mx * W);
+    want(&c->Rf, (size_t)8 * W * W);
+    want(&c->cs_ref, (size_t)RP);
+    want(&c->rf_part, (size_t)kRefineParts * W * W);
+    want(&c->rf_g, W * W);
+    want(&c->rf_C, W * W);
+    want(&c->rf_core, W * W);
+    want(&c->rf_U, W * W);
+    want(&c->rf_V, W * W);
     CKI(prepare_refine_kernels());
   }
-  CKI(dalloc(&c->A1, (size_t)n * RP));
-  CKI(dalloc(&c->A1_orig, (size_t)n * RP));
+  want(&c->A1, (size_t)n * RP);
+  want(&c->A1_orig, (size_t)n * RP);
   // plain GoDec with a given test matrix, on request: its first projection subtracts S A1
   // from a cached X A1 (the other forms change A1 or X between L-steps, or stream
   // half of Z).  The cost of S A1 grows with k at about the rate of random reads from HBM;
@@ -1148,37 +1185,70 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
   // alarm trips more often with it (8 against 2 in 36 iterations), which costs more than
   // it saves, so streaming stays the default.
   const bool sparse_first = (p->flags & GODEC_FLAG_SPARSE_FIRST) != 0;
-  if (A1 && !greb && !c->naive && !c->lingo && !c->half && sparse_first) CKI(dalloc(&c->XA1, (size_t)m * RP));
-  CKI(dalloc(&c->P, (size_t)mx * RP));
-  CKI(dalloc(&c->Q1, (size_t)m * RP));
-  CKI(dalloc(&c->Q2, (size_t)n * RP));
-  CKI(dalloc(&c->U, (size_t)m * RP));
-  CKI(dalloc(&c->V, (size_t)n * RP));
-  CKI(dalloc(&c->sigma, (size_t)RP));
-  CKI(dalloc(&c->Um, rr));
-  CKI(dalloc(&c->Vm, rr));
+  if (A1 && !greb && !c->naive && !c->lingo && !c->half && sparse_first) want(&c->XA1, (size_t)m * RP);
+  want(&c->P, (size_t)mx * RP);
+  want(&c->Q1, (size_t)m * RP);
+  want(&c->Q2, (size_t)n * RP);
+  want(&c->U, (size_t)m * RP);
+  want(&c->V, (size_t)n * RP);
+  want(&c->sigma, (size_t)RP);
+  want(&c->Um, rr);
+  want(&c->Vm, rr);
   c->RPp = tc_rpp(RP);
   c->ldb = (mx + 7) / 8 * 8;
-  CKI(dalloc(reinterpret_cast<unsigned short**>(&c->bt2), (size_t)4 * 2 * RP * c->ldb));
-  CKI(cudaMemsetAsync(c->bt2, 0, (size_t)4 * 2 * RP * c->ldb * 2, c->st));
-  CKI(dalloc(&c->cs, (size_t)2 * RP));
-  CKI(dalloc(&c->rescale_tmp, 2));
-  {
-    std::vector<float> cs(2 * (size_t)RP, 1.f / kSkinnyScale);
-    CKI(cudaMemcpy(c->cs, cs.data(), cs.size() * sizeof(float), cudaMemcpyHostToDevice));
-  }
+  want(reinterpret_cast<unsigned short**>(&c->bt2), (size_t)4 * 2 * RP * c->ldb);
+  want(&c->cs, (size_t)2 * RP);
+  want(&c->rescale_tmp, 2);
   c->tg[0] = prod_split_geometry(m, n, c->nsm);
   c->tg[1] = prod_split_geometry(n, m, c->nsm);
   size_t npart = 0;
   for (const TcGeom& g : c->tg) npart = std::max(npart, (size_t)g.tiles * g.maxseg * 128 * RP);
-  CKI(dalloc(&c->part, npart));
+  want(&c->part, npart);
   c->npart_cap = npart;
   const int64_t tiles = prod_tiles(mx);
   c->ncounters = tiles;
-  CKI(dalloc(&c->counters, (size_t)tiles));
+  want(&c->counters, (size_t)tiles);
+  want(reinterpret_cast<unsigned short**>(&c->LA), (size_t)m * 128);
+  want(reinterpret_cast<unsigned short**>(&c->LB), (size_t)n * 128);
+  c->gpart_stride = ((size_t)tiles * rr * sizeof(double) + 255) & ~size_t(255);
+  want(&c->gparts, c->gpart_stride * np);
+  want(&c->g64, (size_t)(np + 2) * rr);
+  want(&c->g32, (size_t)(np + 2) * rr);
+  want(&c->gscr, (size_t)apply_blocks(mx) * rr);
+  want(&c->Rtmp, (size_t)np * 2 * rr);
+  want(&c->Rslot, (size_t)2 * np * rr);
+  want(&c->Tslot, (size_t)2 * np * rr);
+  want(&c->Rfin, 8 * rr);
+  want(&c->Pi, rr);
+  want(&c->Vprev, rr);
+  want(reinterpret_cast<char**>(&c->ctl), sizeof(Ctl));
+  const unsigned long long mn = (unsigned long long)(m * n);
+  unsigned long long cap = 2ull * (unsigned long long)p->k + 65536ull;
+  if (cap > mn) cap = mn;
+  c->cap = cap;
+  want(&c->cand_key, cap);
+  want(&c->cand_idx, cap);
+  want(&c->cand_val, cap);
+  for (int b = 0; b < 2; ++b) {
+    want(&c->S_idx[b], (size_t)p->k);
+    want(&c->S_val[b], (size_t)p->k);
+  }
+  c->sbits_words = ((long long)((mn + 31) / 32) + 31) / 32 * 32;   // each bitmap 128-byte aligned
+  c->sbits_bytes = 2 * (size_t)c->sbits_words * sizeof(unsigned);
+  want(reinterpret_cast<char**>(&c->sbits), c->sbits_bytes);
+  {
+    const size_t total = c->arena_bytes;
+    c->arena_bytes = 0;
+    CKI(cudaMalloc(reinterpret_cast<void**>(&c->arena), total));
+    c->arena_bytes = total;
+    for (auto& q : plan) *q.first = c->arena + q.second;
+  }
+  CKI(cudaMemsetAsync(c->bt2, 0, (size_t)4 * 2 * RP * c->ldb * 2, c->st));
+  {
+    std::vector<float> cs(2 * (size_t)RP, 1.f / kSkinnyScale);
+    CKI(cudaMemcpyAsync(c->cs, cs.data(), cs.size() * sizeof(float), cudaMemcpyHostToDevice, c->st));
+  }
   CKI(cudaMemsetAsync(c->counters, 0, (size_t)tiles * sizeof(unsigned), c->st));
-  CKI(dalloc(reinterpret_cast<unsigned short**>(&c->LA), (size_t)m * 128));
-  CKI(dalloc(reinterpret_cast<unsigned short**>(&c->LB), (size_t)n * 128));
   {
     const bool ok = make_tmap_f32(c->tmap[5], X, m, n, p->ldx, 128) &&
                     make_tmap_f16(c->tmap[6], c->LA, m, 128, 128, 128) &&
@@ -1196,30 +1266,7 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
       return bail(GODEC_ERR_CUDA);
     }
   }
-  c->gpart_stride = ((size_t)tiles * rr * sizeof(double) + 255) & ~size_t(255);
-  CKI(dalloc(&c->gparts, c->gpart_stride * np));
-  CKI(dalloc(&c->g64, (size_t)(np + 2) * rr));
-  CKI(dalloc(&c->g32, (size_t)(np + 2) * rr));
-  CKI(dalloc(&c->gscr, (size_t)apply_blocks(mx) * rr));
-  CKI(dalloc(&c->Rtmp, (size_t)np * 2 * rr));
-  CKI(dalloc(&c->Rslot, (size_t)2 * np * rr));
-  CKI(dalloc(&c->Tslot, (size_t)2 * np * rr));
-  CKI(dalloc(&c->Rfin, 8 * rr));
-  CKI(dalloc(&c->Pi, rr));
-  CKI(dalloc(&c->Vprev, rr));
-  CKI(dalloc(reinterpret_cast<char**>(&c->ctl), sizeof(Ctl)));
   CKI(cudaMemsetAsync(c->ctl, 0, sizeof(Ctl), c->st));
-  const unsigned long long mn = (unsigned long long)(m * n);
-  unsigned long long cap = 2ull * (unsigned long long)p->k + 65536ull;
-  if (cap > mn) cap = mn;
-  if (alloc_candidates(c, cap)) return bail(GODEC_ERR_OOM);
-  for (int b = 0; b < 2; ++b) {
-    CKI(dalloc(&c->S_idx[b], (size_t)p->k));
-    CKI(dalloc(&c->S_val[b], (size_t)p->k));
-  }
-  c->sbits_words = ((long long)((mn + 31) / 32) + 31) / 32 * 32;   // each bitmap 128-byte aligned
-  c->sbits_bytes = 2 * (size_t)c->sbits_words * sizeof(unsigned);
-  CKI(dalloc(reinterpret_cast<char**>(&c->sbits), c->sbits_bytes));
   c->idx_bits = 1;
   while ((1ull << c->idx_bits) < mn) ++c->idx_bits;
   launch_fill_zero(c->Q1, (size_t)m * RP * sizeof(float), c->st);
@@ -1824,8 +1871,8 @@ static godec_status greb_grow(godec_ctx* c, const Ctl& h, unsigned long long nee
       CK(cudaMemcpyAsync(nv, c->S_val[b], (size_t)h.nnz_cur * sizeof(float), cudaMemcpyDeviceToDevice, c->st));
     }
     CK(cudaStreamSynchronize(c->st));
-    cudaFree(c->S_idx[b]);
-    cudaFree(c->S_val[b]);
+    ctx_free(c, c->S_idx[b]);
+    ctx_free(c, c->S_val[b]);
     c->S_idx[b] = ni;
     c->S_val[b] = nv;
   }
