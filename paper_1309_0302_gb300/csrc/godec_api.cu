@@ -19,6 +19,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 #include <new>
 #include <utility>
 #include <vector>
@@ -26,6 +27,40 @@
 #include "godec_internal.cuh"
 
 using namespace godec;
+
+namespace {
+// Stream-ordered scratch from a pool of the library's own (one per device): blocks come back
+// to the pool in stream order and up to 256 MB stay in it between calls, so that a call need
+// not map memory anew (a device-wide operation of tens of microseconds each).
+constexpr int kPoolDevices = 64;
+constexpr uint64_t kPoolKeep = 256ull << 20;
+cudaMemPool_t scratch_pool(int dev) {
+  static std::mutex mu;
+  static cudaMemPool_t pools[kPoolDevices] = {};
+  if (dev < 0 || dev >= kPoolDevices) return nullptr;
+  std::lock_guard<std::mutex> lock(mu);
+  if (!pools[dev]) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p = nullptr;
+    uint64_t keep = kPoolKeep;
+    if (cudaMemPoolCreate(&p, &props) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+    pools[dev] = p;
+  }
+  return pools[dev];
+}
+}
+
+cudaError_t godec::scratch_alloc(void** p, size_t bytes, int dev, cudaStream_t st) {
+  cudaMemPool_t pool = scratch_pool(dev);
+  return pool ? cudaMallocFromPoolAsync(p, bytes, pool, st) : cudaMallocAsync(p, bytes, st);
+}
 
 namespace {
 constexpr int kEvents = 160;
@@ -110,6 +145,7 @@ struct godec_ctx {
   unsigned* sbits = nullptr;           // two bitmaps of m n bits: the support of the committed S (bitmap
   long long sbits_words = 0;           // ctl->cur) and a clear one the next S-step marks its support in
   size_t sbits_bytes = 0;
+  unsigned* order = nullptr;           // scratch of the ordered export of S
   float* XA1 = nullptr;                // m x RP: X A1, the cached part of the first projection (null: the
                                        // first product streams Z)
   long long* S_idx[2] = {nullptr, nullptr};
@@ -611,7 +647,7 @@ EmitArgs z_args(godec_ctx* c) {
   return ea;
 }
 
-// S-step of one iteration (Algorithm 1, eq. raw_lss) on the current L factors; r = 0 means L = 0.
+// S-step of one iteration (Algorithm 1, eq. raw_lss) on the current L factors.
 void enqueue_sstep(godec_ctx* c, int r) {
   const int64_t m = c->p.m, n = c->p.n;
   cudaStream_t st = c->st;
@@ -632,18 +668,14 @@ void enqueue_sstep(godec_ctx* c, int r) {
   ra.cand_cap = c->cap;
   for (int pass = 0; pass < 3; ++pass) {
     ra.pass = pass;
-    if (c->LA && r > 0) {
-      ResidTcLaunch rl{};
-      rl.ra = ra;
-      rl.mapX = c->tmap[5];
-      rl.mapA = c->tmap[6];
-      rl.mapB = c->tmap[7];
-      rl.zscale = c->ctl->zscale;
-      rl.nsm = c->nsm;
-      PROF(c, 7, st, launch_resid_tc(rl, st));
-    } else {
-      PROF(c, 7, st, launch_residual(ra, c->nsm, st));
-    }
+    ResidTcLaunch rl{};
+    rl.ra = ra;
+    rl.mapX = c->tmap[5];
+    rl.mapA = c->tmap[6];
+    rl.mapB = c->tmap[7];
+    rl.zscale = c->ctl->zscale;
+    rl.nsm = c->nsm;
+    PROF(c, 7, st, launch_resid_tc(rl, st));
     PROF(c, 8, st, launch_after_pass(c->ctl, pass, c->p.k, c->cap, st));
   }
   SelectArgs se{};
@@ -664,7 +696,7 @@ void enqueue_sstep(godec_ctx* c, int r) {
   ea.cand_val = c->cand_val;
   ea.cand_cap = c->cap;
   PROF(c, 8, st, launch_emit(ea, c->nsm, st));
-  if (c->Z) PROF(c, 9, st, launch_z_update(ea, c->nsm, st));
+  PROF(c, 9, st, launch_z_update(ea, c->nsm, st));
 }
 
 // Product over Z (even: m rows, K = n) or Z^T (odd: n rows, K = m) with the operand of
@@ -1134,7 +1166,6 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
   CKI(cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->dev));
   c->nsm_dev = c->nsm;
   CKI(prepare_small_kernels());
-  CKI(prepare_select_kernels());
   CKI(prepare_stream_kernels());
   CKI(prepare_prod_kernels());
   CKI(prepare_resid_kernels());
@@ -1236,6 +1267,7 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
   c->sbits_words = ((long long)((mn + 31) / 32) + 31) / 32 * 32;   // each bitmap 128-byte aligned
   c->sbits_bytes = 2 * (size_t)c->sbits_words * sizeof(unsigned);
   want(reinterpret_cast<char**>(&c->sbits), c->sbits_bytes);
+  want(reinterpret_cast<char**>(&c->order), order_scratch(c->sbits_words));
   {
     const size_t total = c->arena_bytes;
     c->arena_bytes = 0;
@@ -1505,15 +1537,9 @@ godec_status godec_get_S(godec_ctx* c, int64_t* idx, float* val, int64_t cap, in
   const long long k = h.nnz_cur;
   if (k == 0) return GODEC_OK;
   if (!idx || !val) return fail(c, GODEC_ERR_ARG, "idx and val must be non-NULL");
-  // sort a copy by linear index, in place in the caller's buffers
-  size_t scratch = sort_coo_scratch(k);
-  void* tmp = nullptr;
-  CK(cudaMallocAsync(&tmp, scratch, c->st));
-  CK(cudaMemcpyAsync(idx, c->S_idx[h.cur], k * sizeof(long long), cudaMemcpyDeviceToDevice, c->st));
-  CK(cudaMemcpyAsync(val, c->S_val[h.cur], k * sizeof(float), cudaMemcpyDeviceToDevice, c->st));
-  launch_sort_coo(reinterpret_cast<long long*>(idx), val, k, tmp, scratch, c->idx_bits, c->st);
+  launch_order(c->sbits + (size_t)h.cur * (size_t)c->sbits_words, c->sbits_words, c->order, reinterpret_cast<long long*>(idx),
+               val, k, nullptr, c->p.n, 0, c->S_idx[h.cur], c->S_val[h.cur], k, nullptr, c->st);
   CK(cudaGetLastError());
-  CK(cudaFreeAsync(tmp, c->st));
   CK(cudaStreamSynchronize(c->st));
   return GODEC_OK;
 }
@@ -1596,72 +1622,90 @@ done:
 
 godec_status godec_hard_threshold(const float* R, int64_t m, int64_t n, int64_t ldr, int64_t k,
                                   int64_t* idx, float* val, int64_t cap, int64_t* nnz, void* stream) {
-  // A context with r = 0 (L = 0) and no working copy of X - S: only the S-step runs.
   if (!R || m < 1 || n < 1 || ldr < n || (ldr * 4) % 16 || k < 0 || k > m * n ||
       (double)m * (double)n >= 4294967296.0 || (reinterpret_cast<uintptr_t>(R) & 15)) {
     snprintf(g_static_err, sizeof(g_static_err), "godec_hard_threshold: invalid argument");
     return GODEC_ERR_ARG;
   }
-  godec_ctx* c = new (std::nothrow) godec_ctx;
-  if (!c) return GODEC_ERR_OOM;
-  godec_status s = GODEC_OK;
-  c->st = reinterpret_cast<cudaStream_t>(stream);
-  c->p.m = m;
-  c->p.n = n;
-  c->p.ldx = ldr;
-  c->p.k = k;
-  c->p.r = 0;
-  c->RP = 8;
-  c->X = R;
-  do {
-    if (cudaGetDevice(&c->dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->dev) != cudaSuccess ||
-        prepare_select_kernels() != cudaSuccess) {
-      s = fail(c, GODEC_ERR_CUDA, "no CUDA device");
-      break;
+  auto out = [](godec_status s, const char* why) {
+    snprintf(g_static_err, sizeof(g_static_err), "godec_hard_threshold: %.200s", why);
+    return s;
+  };
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  int dev = 0, nsm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return out(GODEC_ERR_CUDA, "no CUDA device");
+  const unsigned long long mn = (unsigned long long)(m * n);
+  const long long words = ((long long)((mn + 31) / 32) + 31) / 32 * 32;
+  unsigned long long cap0 = std::min<unsigned long long>(2ull * (unsigned long long)k + 65536ull, mn);
+  for (;;) {
+    // one scratch block: control block, bitmap, ordering scratch, candidates
+    auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
+    const size_t b_ctl = up(sizeof(Ctl)), b_bits = up((size_t)words * 4), b_ord = up(order_scratch(words)),
+                 b_tot = up(sizeof(unsigned)), b_idx = up(cap0 * 8), b_val = up(cap0 * 4);
+    char* mem = nullptr;
+    if (scratch_alloc(reinterpret_cast<void**>(&mem), b_ctl + b_bits + b_ord + b_tot + b_idx + 2 * b_val, dev, st) !=
+        cudaSuccess) {
+      cudaGetLastError();
+      return out(GODEC_ERR_OOM, "out of device memory");
     }
-    const unsigned long long mn = (unsigned long long)(m * n);
-    unsigned long long cap0 = 2ull * (unsigned long long)k + 65536ull;
-    if (cap0 > mn) cap0 = mn;
-    if (dalloc(&c->ctl, 1) != cudaSuccess || dalloc(&c->U, (size_t)m * 8) != cudaSuccess ||
-        dalloc(&c->V, (size_t)n * 8) != cudaSuccess || dalloc(&c->sigma, 8) != cudaSuccess ||
-        dalloc(&c->S_idx[0], (size_t)k) != cudaSuccess || dalloc(&c->S_idx[1], (size_t)k) != cudaSuccess ||
-        dalloc(&c->S_val[0], (size_t)k) != cudaSuccess || dalloc(&c->S_val[1], (size_t)k) != cudaSuccess) {
-      s = fail(c, GODEC_ERR_OOM, "out of device memory");
-      break;
+    SelectArgs se{};
+    se.ctl = reinterpret_cast<Ctl*>(mem);
+    unsigned* bits = reinterpret_cast<unsigned*>(mem + b_ctl);
+    unsigned* order = reinterpret_cast<unsigned*>(mem + b_ctl + b_bits);
+    unsigned* total = reinterpret_cast<unsigned*>(mem + b_ctl + b_bits + b_ord);
+    long long* cidx = reinterpret_cast<long long*>(mem + b_ctl + b_bits + b_ord + b_tot);
+    float* cval = reinterpret_cast<float*>(mem + b_ctl + b_bits + b_ord + b_tot + b_idx);
+    unsigned* ckey = reinterpret_cast<unsigned*>(mem + b_ctl + b_bits + b_ord + b_tot + b_idx + b_val);
+    se.cand_key = ckey;
+    se.cand_idx = cidx;
+    se.cand_val = cval;
+    se.cand_cap = cap0;
+    se.k = k;
+    se.idx_bits = 1;
+    while ((1ull << se.idx_bits) < mn) ++se.idx_bits;
+    cudaMemsetAsync(mem, 0, b_ctl + b_bits, st);
+    launch_start_select(se.ctl, k, st);
+    ResidualArgs ra{};
+    ra.X = R;
+    ra.m = m;
+    ra.n = n;
+    ra.ldx = ldr;
+    ra.ctl = se.ctl;
+    ra.cand_key = ckey;
+    ra.cand_idx = cidx;
+    ra.cand_val = cval;
+    ra.cand_cap = cap0;
+    for (ra.pass = 0; ra.pass < 2; ++ra.pass) {   // histogram, then the candidates above its bin
+      launch_thresh_pass(ra, nsm, st);
+      launch_after_pass(se.ctl, ra.pass, k, cap0, st);
     }
-    if ((s = alloc_candidates(c, cap0))) break;
-    c->idx_bits = 1;
-    while ((1ull << c->idx_bits) < mn) ++c->idx_bits;
-    if (cudaMemsetAsync(c->ctl, 0, sizeof(Ctl), c->st) != cudaSuccess) {
-      s = fail(c, GODEC_ERR_CUDA, "memset");
-      break;
+    for (int round = 0; round < 7; ++round) {
+      se.round = round;
+      launch_select_round(se, nsm, st);
     }
+    launch_mark(se, bits, nsm, st);
+    launch_order(bits, words, order, reinterpret_cast<long long*>(idx), val, (idx && val) ? cap : 0, R, n, ldr, nullptr,
+                 nullptr, 0, total, st);
+    cudaError_t e = cudaGetLastError();
     Ctl h;
-    memset(&h, 0, offsetof(Ctl, hist));
-    h.k_req = k;
-    h.k_eff = k;
-    h.tol = -1.0;
-    h.normX2 = 1.0;
-    cudaMemcpyAsync(c->ctl, &h, offsetof(Ctl, hist), cudaMemcpyHostToDevice, c->st);
-    launch_reset_iter(c->ctl, c->st);
-    for (int attempt = 0; attempt < 8; ++attempt) {
-      enqueue_sstep(c, 0);
-      Ctl hh;
-      if ((s = read_ctl(c, &hh))) break;
-      if (hh.nonfinite) { s = fail(c, GODEC_ERR_NONFINITE, "non-finite values in R"); break; }
-      if (!hh.abort) break;
-      if (!hh.need_bigger_cand) { s = fail(c, GODEC_ERR_STATE, "selection aborted"); break; }
-      unsigned long long cap2 = std::min<unsigned long long>(c->cap * 2, mn);
-      if ((s = alloc_candidates(c, cap2))) break;
-      launch_reset_iter(c->ctl, c->st);
+    unsigned got = 0;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, se.ctl, offsetof(Ctl, hist), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&got, total, sizeof(got), cudaMemcpyDeviceToHost, st);
+    cudaFreeAsync(mem, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return out(GODEC_ERR_CUDA, cudaGetErrorString(e));
+    if (h.nonfinite) return out(GODEC_ERR_NONFINITE, "non-finite values in R");
+    if (h.abort && h.need_bigger_cand && cap0 < mn) {   // one bin of the histogram outgrew the candidates
+      cap0 = std::min<unsigned long long>(cap0 * 2, mn);
+      continue;
     }
-    if (s) break;
-    s = godec_get_S(c, idx, val, cap, nnz);
-  } while (0);
-  if (s) snprintf(g_static_err, sizeof(g_static_err), "godec_hard_threshold: %.200s", c->err);
-  godec_destroy(c);
-  return s;
+    if (h.abort) return out(GODEC_ERR_STATE, "selection aborted");
+    if (nnz) *nnz = (int64_t)got;
+    if (cap < (int64_t)got) return out(GODEC_ERR_ARG, "cap is smaller than the result");
+    if (got > 0 && (!idx || !val)) return out(GODEC_ERR_ARG, "idx and val must be non-NULL");
+    return GODEC_OK;
+  }
 }
 
 // ---- streaming primitives ----------------------------------------------------------------

@@ -47,12 +47,13 @@ constexpr int kCrossParts = 256;
 // Stream-ordered scratch of one call; freed (stream-ordered) on destruction.
 struct Scratch {
   cudaStream_t st;
+  int dev;
   std::vector<void*> ptrs;
   bool ok = true;
   template <typename T>
   T* get(size_t elems) {
     void* p = nullptr;
-    if (!ok || cudaMallocAsync(&p, std::max<size_t>(elems, 1) * sizeof(T), st) != cudaSuccess) {
+    if (!ok || scratch_alloc(&p, std::max<size_t>(elems, 1) * sizeof(T), dev, st) != cudaSuccess) {
       ok = false;
       return nullptr;
     }
@@ -135,7 +136,7 @@ extern "C" godec_status godec_backward(const float* X, int64_t m, int64_t n, int
   }
   const int RP = (r + 7) / 8 * 8, R3 = 3 * r;
   const int64_t mx = std::max(m, n), ldz = (n + 63) / 64 * 64;
-  Scratch sc{st};
+  Scratch sc{st, dev};
   // Iterates Z_t: one copy for all t, rebuilt in the backward sweep, or (when all T of them
   // fit in a quarter of the free device memory) one per t, kept from the forward sweep.
   size_t free_b = 0, total_b = 0;

@@ -278,7 +278,7 @@ struct ResidualArgs {
   float* cand_val;
   unsigned long long cand_cap;
 };
-void launch_residual(const ResidualArgs& a, int nsm, cudaStream_t st);
+void launch_thresh_pass(const ResidualArgs& a, int nsm, cudaStream_t st);   // R = X (no low-rank part)
 
 // Tensor-core residual pass (k_resid.cu).  A and B hold the float16 split of
 // U diag(sqrt(sigma s_Z)) and V diag(sqrt(sigma s_Z)), rows of 128 halves (64 high,
@@ -310,6 +310,16 @@ struct SelectArgs {
   int idx_bits;            // bits needed for linear indices (<= 42)
 };
 void launch_select_round(const SelectArgs& a, int nsm, cudaStream_t st);
+// The selected candidates' bits set in a clear bitmap of m n bits.
+void launch_mark(const SelectArgs& a, unsigned* bits, int nsm, cudaStream_t st);
+// Indices (ascending, below cap) of a bitmap's set bits, and their values: from R (row stride
+// ldr) or, with R null, from the unordered list S_idx / S_val of nnz entries.  words: a
+// multiple of 32, bits 16-byte aligned; total (device, nullable) receives their number.
+constexpr int kOrderWords = 1024;    // words a block of these kernels takes
+size_t order_scratch(long long words);
+void launch_order(const unsigned* bits, long long words, unsigned* scratch, long long* idx, float* val, long long cap,
+                  const float* R, int64_t n, int64_t ldr, const long long* S_idx, const float* S_val, long long nnz,
+                  unsigned* total, cudaStream_t st);
 
 struct EmitArgs {
   Ctl* ctl;
@@ -345,12 +355,15 @@ void launch_reset_iter(Ctl* ctl, cudaStream_t st);
 // One bounded wait that nothing completes; flags ctl->timeout / abort when it gives up.
 void launch_wait_check(Ctl* ctl, uint32_t polls, cudaStream_t st);
 
+// Stream-ordered scratch (freed with cudaFreeAsync) from the library's own memory pool.
+cudaError_t scratch_alloc(void** p, size_t bytes, int dev, cudaStream_t st);
+// Ctl of a selection over a dense matrix alone (zeroed before): k, one full pass first.
+void launch_start_select(Ctl* ctl, long long k, cudaStream_t st);
 // Error text returned by godec_last_error(NULL) for calls without a context.
 void set_static_error(const char* fmt, ...);
 
 // Kernel attributes (dynamic shared memory limits); call before launching or capturing.
 cudaError_t prepare_small_kernels();
-cudaError_t prepare_select_kernels();
 
 // Tall x small and sparse kernels (k_backward.cu), shared by the differentiated form and
 // the precision form's correction.
@@ -439,8 +452,4 @@ void launch_unpad_copy(const float* src, int64_t rows, int RP, float* dst, int c
 // *out += sum of X^2 (float64 atomics: clear *out first for a fresh sum)
 void launch_sumsq(const float* X, int64_t m, int64_t n, int64_t ldx, double* out, int nsm,
                   cudaStream_t st);
-void launch_sort_coo(long long* idx, float* val, long long nnz, void* scratch, size_t scratch_bytes,
-                     int idx_bits, cudaStream_t st);
-size_t sort_coo_scratch(long long nnz);
-
 }  // namespace godec

@@ -1,7 +1,7 @@
 // S-step of Algorithm 1 (eq. raw_lss): S_t = P_Omega(X - L_t) with Omega
 // the nonzero subset of the k largest |X - L_t|, ties by ascending linear index.
 //
-// One pass over X rebuilds R = X - U diag(sigma) V^T tile by tile.  Magnitudes
+// One pass over X rebuilds R = X - U diag(sigma) V^T tile by tile (k_resid.cu).  Magnitudes
 // are compared through their float bit patterns (monotone for |R| >= 0).  In
 // candidate mode the pass keeps every entry whose key reaches a threshold
 // guessed from the previous iteration; in full mode it builds a 4096-bin
@@ -18,12 +18,27 @@ namespace godec {
 
 namespace {
 
-constexpr int RT_M = 128, RT_N = 64, RES_THREADS = 128;
-constexpr int RES_US_STRIDE = RT_M + 4, RES_VS_STRIDE = RT_N + 4;
-constexpr size_t kResSmem = (size_t)kMaxRP * (RES_US_STRIDE + RES_VS_STRIDE) * sizeof(float) +
-                            kHistBins * sizeof(unsigned);
-
 __device__ __forceinline__ unsigned key_of(float v) { return __float_as_uint(v) & 0x7fffffffu; }
+
+// Row and column of a linear index (idx = i n + j): a float estimate of the quotient,
+// refined once from the remainder and then corrected exactly in integers (no 64-bit
+// division; the estimate is off by at most a couple of units for any size).
+__device__ __forceinline__ void split_idx(long long idx, long long n, float ninv, long long& i, long long& j) {
+  long long q = (long long)((float)idx * ninv);
+  long long r = idx - q * n;
+  q += (long long)((float)r * ninv);
+  r = idx - q * n;
+  while (r < 0) {
+    --q;
+    r += n;
+  }
+  while (r >= n) {
+    ++q;
+    r -= n;
+  }
+  i = q;
+  j = r;
+}
 
 // Block-wide exclusive scan of one unsigned per thread (any blockDim multiple of 32).
 __device__ unsigned block_excl_scan(unsigned v, unsigned* total) {
@@ -68,135 +83,241 @@ __device__ double block_sum_double(double v) {
 }
 
 // --------------------------------------------------------------------------------------
-// Residual pass
+// Pass over a dense residual R (hard threshold without L): the histogram of the top key bits
+// (full mode) or the candidates with key >= guess, staged per block and written with one
+// global atomic per full buffer.  Eight columns per thread and step as two 16-byte loads.
+// Bound: 4 m n bytes read (4001 x 2999: 24 -> 9 us a pass against the tiled kernel with the
+// general X - U V^T arithmetic that this replaces).
 // --------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(RES_THREADS)
-k_residual(ResidualArgs a) {
-  Ctl* ctl = a.ctl;
+constexpr int TH_THREADS = 512, TH_STAGE = 2048;
+
+__global__ void __launch_bounds__(TH_THREADS)
+k_thresh_pass(const float* __restrict__ R, int64_t m, int64_t n, int64_t ldr, int pass, Ctl* ctl,
+              unsigned* __restrict__ cand_key, long long* __restrict__ cand_idx, float* __restrict__ cand_val,
+              unsigned long long cand_cap) {
   if (ctl->abort) return;
-  const int mode = ctl->plan[a.pass];
+  const int mode = ctl->plan[pass];
   if (mode == PASS_NONE) return;
-  const unsigned guess = ctl->guess[a.pass];
-  extern __shared__ __align__(16) float res_smem[];
-  float* Us = res_smem;                                  // [RP][RES_US_STRIDE]
-  float* Vs = Us + kMaxRP * RES_US_STRIDE;               // [RP][RES_VS_STRIDE]
-  unsigned* hist = reinterpret_cast<unsigned*>(Vs + kMaxRP * RES_VS_STRIDE);
-
+  const unsigned guess = max(ctl->guess[pass], 1u);   // exact zeros are never candidates
+  __shared__ unsigned hist[kHistBins];                // candidate mode: the staged linear indices (low words)
+  __shared__ float sval[TH_STAGE];
+  __shared__ unsigned s_cnt;
+  __shared__ unsigned long long s_base;
+  static_assert(TH_STAGE <= kHistBins, "staged indices fit the histogram");
   const int tid = threadIdx.x;
-  const int ty = tid >> 3, tx = tid & 7;
-  const int r = a.r, RP = a.RP;
-  const int64_t m = a.m, n = a.n, ldx = a.ldx;
-  const int64_t tiles_n = (n + RT_N - 1) / RT_N;
-  const int64_t ntiles = ((m + RT_M - 1) / RT_M) * tiles_n;
-
   if (mode == PASS_FULL)
-    for (int b = tid; b < kHistBins; b += RES_THREADS) hist[b] = 0u;
-
-  double dsum = 0.0;
-  int bad = 0;
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t i0 = (tile / tiles_n) * RT_M;
-    const int64_t j0 = (tile % tiles_n) * RT_N;
-    __syncthreads();
-    for (int e = tid; e < RT_M * r; e += RES_THREADS) {
-      int ii = e / r, l = e % r;
-      int64_t i = i0 + ii;
-      Us[l * RES_US_STRIDE + ii] = (i < m) ? a.U[i * RP + l] * a.sigma[l] : 0.f;
-    }
-    for (int e = tid; e < RT_N * r; e += RES_THREADS) {
-      int jj = e / r, l = e % r;
-      int64_t j = j0 + jj;
-      Vs[l * RES_VS_STRIDE + jj] = (j < n) ? a.V[j * RP + l] : 0.f;
-    }
-    __syncthreads();
-    float acc[8][8];
+    for (int b = tid; b < kHistBins; b += TH_THREADS) hist[b] = 0u;
+  if (tid == 0) s_cnt = 0u;
+  __syncthreads();
+  const int64_t per = (n + 7) / 8, total = m * per;
+  bool bad = false;
+  // every thread takes the same number of steps (the staging has block-wide barriers)
+  for (int64_t e0 = (int64_t)blockIdx.x * TH_THREADS; e0 < total; e0 += (int64_t)gridDim.x * TH_THREADS) {
+    const int64_t e = e0 + tid;
+    float v[8];
+    int64_t i = 0, j = 0;
 #pragma unroll
-    for (int p = 0; p < 8; ++p)
-#pragma unroll
-      for (int q = 0; q < 8; ++q) acc[p][q] = 0.f;
-    for (int l = 0; l < r; ++l) {
-      float4 u0 = *reinterpret_cast<const float4*>(&Us[l * RES_US_STRIDE + ty * 8]);
-      float4 u1 = *reinterpret_cast<const float4*>(&Us[l * RES_US_STRIDE + ty * 8 + 4]);
-      float4 v0 = *reinterpret_cast<const float4*>(&Vs[l * RES_VS_STRIDE + tx * 8]);
-      float4 v1 = *reinterpret_cast<const float4*>(&Vs[l * RES_VS_STRIDE + tx * 8 + 4]);
-      float uv[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
-      float vv[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-#pragma unroll
-      for (int p = 0; p < 8; ++p)
-#pragma unroll
-        for (int q = 0; q < 8; ++q) acc[p][q] = fmaf(uv[p], vv[q], acc[p][q]);
-    }
-    // residual R = X - L on the 8 x 8 register tile
-    const int64_t jb = j0 + tx * 8;
-    unsigned ncand = 0;
-    float fsum = 0.f;
-#pragma unroll
-    for (int p = 0; p < 8; ++p) {
-      const int64_t i = i0 + ty * 8 + p;
-      float xv[8];
-      if (i < m && jb + 8 <= n) {
-        const float4* xp = reinterpret_cast<const float4*>(a.X + i * ldx + jb);
-        float4 x0 = xp[0], x1 = xp[1];
-        xv[0] = x0.x; xv[1] = x0.y; xv[2] = x0.z; xv[3] = x0.w;
-        xv[4] = x1.x; xv[5] = x1.y; xv[6] = x1.z; xv[7] = x1.w;
+    for (int u = 0; u < 8; ++u) v[u] = 0.f;
+    if (e < total) {
+      i = e / per;
+      j = (e - i * per) * 8;
+      const float* r = R + i * ldr + j;   // rows and R are 16-byte aligned
+      if (j + 8 <= n) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(r)), b = __ldg(reinterpret_cast<const float4*>(r) + 1);
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+        v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
       } else {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) xv[q] = (i < m && jb + q < n) ? a.X[i * ldx + jb + q] : 0.f;
-      }
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const bool in = (i < m) && (jb + q < n);
-        float res = in ? xv[q] - acc[p][q] : 0.f;
-        acc[p][q] = res;
-        unsigned key = key_of(res);
-        if (key >= 0x7f800000u) bad = 1;
-        if (mode == PASS_FULL) {
-          fsum = fmaf(res, res, fsum);
-          if (key) atomicAdd(&hist[key >> kD1Shift], 1u);
-        } else if (key != 0u && key >= guess) {
-          ++ncand;
-        } else {
-          fsum = fmaf(res, res, fsum);
-        }
+        for (int u = 0; u < 8; ++u)
+          if (j + u < n) v[u] = r[u];
       }
     }
-    dsum += (double)fsum;
-    if (mode == PASS_CAND) {
-      unsigned total;
-      unsigned off = block_excl_scan(ncand, &total);
-      __shared__ unsigned long long s_base;
-      if (tid == 0) s_base = total ? atomicAdd(&ctl->cand_count, (unsigned long long)total) : 0ull;
-      __syncthreads();
-      if (ncand) {
-        unsigned long long pos = s_base + off;
+    if (mode == PASS_FULL) {
 #pragma unroll
-        for (int p = 0; p < 8; ++p) {
-          const int64_t i = i0 + ty * 8 + p;
+      for (int u = 0; u < 8; ++u) {
+        const unsigned key = key_of(v[u]);
+        bad |= key >= 0x7f800000u;
+        if (key) atomicAdd(&hist[key >> kD1Shift], 1u);
+      }
+      continue;
+    }
+    unsigned cm = 0u;
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            float res = acc[p][q];
-            unsigned key = key_of(res);
-            if (key != 0u && key >= guess) {
-              if (pos < a.cand_cap) {
-                a.cand_key[pos] = key;
-                a.cand_idx[pos] = (long long)(i * n + jb + q);
-                a.cand_val[pos] = res;
-              }
-              ++pos;
-            }
+    for (int u = 0; u < 8; ++u) {
+      const unsigned key = key_of(v[u]);
+      bad |= key >= 0x7f800000u;
+      if (key >= guess) cm |= 1u << u;
+    }
+    // stage; when a step's candidates do not fit, the buffer goes out first (a step has at
+    // most 8 TH_THREADS of them, taken TH_STAGE at a time)
+    const int cnt = __popc(cm);
+    unsigned tot;
+    const unsigned off = block_excl_scan((unsigned)cnt, &tot);
+    for (unsigned lo = 0; lo < tot; lo += TH_STAGE) {
+      const unsigned have = s_cnt, part = min(tot - lo, (unsigned)TH_STAGE);
+      if (have + part > TH_STAGE) {
+        __syncthreads();
+        if (tid == 0) s_base = atomicAdd(&ctl->cand_count, (unsigned long long)have);
+        __syncthreads();
+        for (unsigned q = tid; q < have; q += TH_THREADS)
+          if (s_base + q < cand_cap) {
+            cand_key[s_base + q] = key_of(sval[q]);
+            cand_idx[s_base + q] = (long long)hist[q];
+            cand_val[s_base + q] = sval[q];
           }
-        }
+        __syncthreads();
+        if (tid == 0) s_cnt = 0u;
+        __syncthreads();
       }
+      const unsigned at = s_cnt;
+      unsigned pos = off;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (cm & (1u << u)) {
+          if (pos >= lo && pos < lo + part) {
+            sval[at + pos - lo] = v[u];
+            hist[at + pos - lo] = (unsigned)(i * n + j + u);   // m n < 2^32
+          }
+          ++pos;
+        }
+      __syncthreads();
+      if (tid == 0) s_cnt = at + part;
+      __syncthreads();
     }
+  }
+  __syncthreads();
+  if (mode == PASS_FULL) {
+    for (int b = tid; b < kHistBins; b += TH_THREADS)
+      if (hist[b]) atomicAdd(&ctl->hist[b], hist[b]);
+  } else if (s_cnt) {
+    if (tid == 0) s_base = atomicAdd(&ctl->cand_count, (unsigned long long)s_cnt);
+    __syncthreads();
+    for (unsigned q = tid; q < s_cnt; q += TH_THREADS)
+      if (s_base + q < cand_cap) {
+        cand_key[s_base + q] = key_of(sval[q]);
+        cand_idx[s_base + q] = (long long)hist[q];
+        cand_val[s_base + q] = sval[q];
+      }
   }
   if (bad) ctl->nonfinite = 1;
-  double t = block_sum_double(dsum);
-  if (tid == 0) atomicAdd(mode == PASS_FULL ? &ctl->sumsq_full : &ctl->sumsq_noncand, t);
-  if (mode == PASS_FULL) {
-    __syncthreads();
-    for (int b = tid; b < kHistBins; b += RES_THREADS)
-      if (hist[b]) atomicAdd(&ctl->hist[b], hist[b]);
+}
+
+// Bits of the selected candidates (bitmap of m n bits, clear before).
+__global__ void __launch_bounds__(256)
+k_mark(Ctl* ctl, const unsigned* __restrict__ cand_key, const long long* __restrict__ cand_idx,
+       unsigned long long cand_cap, unsigned* __restrict__ bits) {
+  if (ctl->abort || !ctl->ready || ctl->need <= 0) return;
+  const unsigned long long ncand = min(ctl->cand_count, cand_cap);
+  const unsigned tau = ctl->tau_key;
+  const unsigned long long cut = ctl->idx_cut;
+  for (unsigned long long c = (unsigned long long)blockIdx.x * 256 + threadIdx.x; c < ncand;
+       c += (unsigned long long)gridDim.x * 256) {
+    const unsigned key = cand_key[c];
+    if (key < tau) continue;
+    const unsigned long long idx = (unsigned long long)cand_idx[c];
+    if (key > tau || idx <= cut) atomicOr(&bits[idx >> 5], 1u << (idx & 31));
   }
+}
+
+// --------------------------------------------------------------------------------------
+// The support in ascending order from its bitmap: the entries' positions are ranks in the
+// bitmap, so no sort is needed.  A block takes OB_WORDS words; per group of eight words
+// (256 bits, one 32-byte sector) the write pass also leaves the rank of its first bit.
+// Bound: m n / 8 bytes read twice, 12 bytes written per entry, and one random read and write
+// per entry where the values come from an unordered list (10^4 x 10^4, 10^6 entries: 300 us
+// as eight passes of a radix sort before).
+// --------------------------------------------------------------------------------------
+constexpr int OB_THREADS = 256, OB_WORDS = kOrderWords;
+
+__global__ void __launch_bounds__(OB_THREADS)
+k_bits_count(const unsigned* __restrict__ bits, long long words, unsigned* __restrict__ blocksum) {
+  const long long w0 = (long long)blockIdx.x * OB_WORDS;
+  unsigned c = 0;
+#pragma unroll
+  for (int k = 0; k < OB_WORDS / OB_THREADS / 4; ++k) {   // words: a multiple of 32, OB_WORDS of 1024
+    const long long w = w0 + 4 * ((long long)k * OB_THREADS + threadIdx.x);
+    if (w < words) {
+      const uint4 q = __ldg(reinterpret_cast<const uint4*>(bits + w));
+      c += __popc(q.x) + __popc(q.y) + __popc(q.z) + __popc(q.w);
+    }
+  }
+  unsigned tot;
+  block_excl_scan(c, &tot);
+  if (threadIdx.x == 0) blocksum[blockIdx.x] = tot;
+}
+
+// blocksum := its exclusive prefix sums (one block of 1024 threads); *total = their sum.
+__global__ void __launch_bounds__(1024) k_bits_scan(unsigned* __restrict__ blocksum, int nblk, unsigned* total) {
+  unsigned carry = 0;
+  for (int b = 0; b < nblk; b += 1024) {
+    const int i = b + threadIdx.x;
+    const unsigned v = i < nblk ? blocksum[i] : 0u;
+    unsigned tot;
+    const unsigned x = block_excl_scan(v, &tot);
+    if (i < nblk) blocksum[i] = carry + x;
+    carry += tot;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0 && total) *total = carry;
+}
+
+// idx[rank] = linear index of every set bit, below cap; with R, val[rank] = R there; rank0
+// (nullable) the rank of each 256-bit group's first bit.
+__global__ void __launch_bounds__(OB_THREADS)
+k_bits_write(const unsigned* __restrict__ bits, long long words, const unsigned* __restrict__ blocksum,
+             long long* __restrict__ idx, float* __restrict__ val, long long cap, const float* __restrict__ R, int64_t n,
+             int64_t ldr, unsigned* __restrict__ rank0) {
+  constexpr int WT = OB_WORDS / OB_THREADS;   // words per thread, consecutive
+  const long long w0 = (long long)blockIdx.x * OB_WORDS + (long long)threadIdx.x * WT;
+  unsigned w[WT];
+  unsigned c = 0;
+#pragma unroll
+  for (int k = 0; k < WT; k += 4) {
+    const uint4 q = w0 + k < words ? __ldg(reinterpret_cast<const uint4*>(bits + w0 + k)) : make_uint4(0, 0, 0, 0);
+    w[k] = q.x;
+    w[k + 1] = q.y;
+    w[k + 2] = q.z;
+    w[k + 3] = q.w;
+    c += __popc(q.x) + __popc(q.y) + __popc(q.z) + __popc(q.w);
+  }
+  unsigned tot;
+  long long pos = (long long)blocksum[blockIdx.x] + block_excl_scan(c, &tot);
+  const float ninv = 1.f / (float)n;
+#pragma unroll
+  for (int k = 0; k < WT; ++k) {
+    if (rank0 && ((w0 + k) & 7) == 0 && w0 + k < words) rank0[(w0 + k) >> 3] = (unsigned)pos;
+    unsigned x = w[k];
+    while (x) {
+      const int b = __ffs(x) - 1;
+      x &= x - 1u;
+      const long long id = (w0 + k) * 32 + b;
+      if (pos < cap) {
+        idx[pos] = id;
+        if (R) {
+          long long i, j;
+          split_idx(id, n, ninv, i, j);
+          val[pos] = R[i * ldr + j];
+        }
+      }
+      ++pos;
+    }
+  }
+}
+
+// val[rank of idx[e]] = v[e].
+__global__ void __launch_bounds__(256)
+k_val_order(const long long* __restrict__ idx, const float* __restrict__ v, long long nnz,
+            const unsigned* __restrict__ bits, const unsigned* __restrict__ rank0, float* __restrict__ val) {
+  const long long e = (long long)blockIdx.x * 256 + threadIdx.x;
+  if (e >= nnz) return;
+  const long long id = idx[e], w = id >> 5, g = w >> 3;
+  const uint4 a = __ldg(reinterpret_cast<const uint4*>(bits + 8 * g)), b = __ldg(reinterpret_cast<const uint4*>(bits + 8 * g) + 1);
+  const unsigned q[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+  unsigned r = __ldg(rank0 + g);
+  const int k = (int)(w & 7);
+#pragma unroll
+  for (int u = 0; u < 8; ++u) r += u < k ? __popc(q[u]) : (u == k ? __popc(q[u] & ((1u << (id & 31)) - 1u)) : 0u);
+  val[r] = v[e];
 }
 
 // --------------------------------------------------------------------------------------
@@ -549,26 +670,6 @@ __device__ __forceinline__ void z_flag(Ctl* ctl, bool bad) {
   if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) ctl->range_err = 1;
 }
 
-// Row and column of a linear index (idx = i n + j): a float estimate of the quotient,
-// refined once from the remainder and then corrected exactly in integers (no 64-bit
-// division; the estimate is off by at most a couple of units for any size).
-__device__ __forceinline__ void split_idx(long long idx, long long n, float ninv, long long& i, long long& j) {
-  long long q = (long long)((float)idx * ninv);
-  long long r = idx - q * n;
-  q += (long long)((float)r * ninv);
-  r = idx - q * n;
-  while (r < 0) {
-    --q;
-    r += n;
-  }
-  while (r >= n) {
-    ++q;
-    r -= n;
-  }
-  i = q;
-  j = r;
-}
-
 // One entry per thread (the grid covers the largest possible support, k).  The update
 // also runs after the iteration that met the stop test (converged sets abort only to
 // stop the iterations after it), so Z always matches the committed S.
@@ -632,6 +733,13 @@ __global__ void k_sbits_rebuild(unsigned* sbits, long long words, long long* S0,
   atomicOr(&sbits[(size_t)cb * (size_t)words + (size_t)(idx >> 5)], 1u << (idx & 31));
 }
 
+// Start of a selection over a dense matrix alone, from a zeroed control block.
+__global__ void k_start_select(Ctl* ctl, long long k) {
+  ctl->plan[0] = PASS_FULL;
+  ctl->k_req = ctl->k_eff = k;
+  ctl->tol = -1.0;
+}
+
 // Per-iteration S-step state back to "start of an iteration" (one thread).
 __global__ void k_reset_iter(Ctl* ctl) {
   for (int b = threadIdx.x; b < kHistBins; b += blockDim.x) {
@@ -668,17 +776,34 @@ __global__ void k_reset_iter(Ctl* ctl) {
 
 }  // namespace
 
-cudaError_t prepare_select_kernels() {
-  return cudaFuncSetAttribute(k_residual, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmem);
-}
+void launch_start_select(Ctl* ctl, long long k, cudaStream_t st) { k_start_select<<<1, 1, 0, st>>>(ctl, k); }
 
 void launch_reset_iter(Ctl* ctl, cudaStream_t st) { k_reset_iter<<<1, 256, 0, st>>>(ctl); }
 
-void launch_residual(const ResidualArgs& a, int nsm, cudaStream_t st) {
-  const int64_t ntiles = ((a.m + RT_M - 1) / RT_M) * ((a.n + RT_N - 1) / RT_N);
-  int64_t grid = 3LL * nsm;
-  if (grid > ntiles) grid = ntiles;
-  k_residual<<<(unsigned)grid, RES_THREADS, kResSmem, st>>>(a);
+void launch_thresh_pass(const ResidualArgs& a, int nsm, cudaStream_t st) {
+  int64_t grid = (a.m * ((a.n + 7) / 8) + TH_THREADS - 1) / TH_THREADS;
+  if (grid > 4LL * nsm) grid = 4LL * nsm;
+  k_thresh_pass<<<(unsigned)grid, TH_THREADS, 0, st>>>(a.X, a.m, a.n, a.ldx, a.pass, a.ctl, a.cand_key, a.cand_idx,
+                                                       a.cand_val, a.cand_cap);
+}
+
+void launch_mark(const SelectArgs& a, unsigned* bits, int nsm, cudaStream_t st) {
+  k_mark<<<(unsigned)(4 * nsm), 256, 0, st>>>(a.ctl, a.cand_key, a.cand_idx, a.cand_cap, bits);
+}
+
+size_t order_scratch(long long words) {
+  return (size_t)((words + OB_WORDS - 1) / OB_WORDS + 1 + words / 8) * sizeof(unsigned);
+}
+
+void launch_order(const unsigned* bits, long long words, unsigned* scratch, long long* idx, float* val, long long cap,
+                  const float* R, int64_t n, int64_t ldr, const long long* S_idx, const float* S_val, long long nnz,
+                  unsigned* total, cudaStream_t st) {
+  const int nblk = (int)((words + OB_WORDS - 1) / OB_WORDS);
+  unsigned* rank0 = R ? nullptr : scratch + nblk + 1;
+  k_bits_count<<<nblk, OB_THREADS, 0, st>>>(bits, words, scratch);
+  k_bits_scan<<<1, 1024, 0, st>>>(scratch, nblk, total);
+  k_bits_write<<<nblk, OB_THREADS, 0, st>>>(bits, words, scratch, idx, val, cap, R, n, ldr, rank0);
+  if (!R && nnz > 0) k_val_order<<<(unsigned)((nnz + 255) / 256), 256, 0, st>>>(S_idx, S_val, nnz, bits, rank0, val);
 }
 
 void launch_after_pass(Ctl* ctl, int pass, long long k, unsigned long long cap, cudaStream_t st) {

@@ -1,5 +1,4 @@
-// Small helpers: zero fill, padded copies of tall factors, ||X||_F^2 and a
-// stable LSD radix sort of the COO of S by linear index (export order).
+// Small helpers: zero fill, padded copies of tall factors, the scale of a matrix and ||X||_F^2.
 #include <algorithm>
 
 #include "godec_internal.cuh"
@@ -48,9 +47,6 @@ __global__ void k_unpad_copy(const float* src, int64_t rows, int RP, float* dst,
     dst[e] = src[i * RP + c];
   }
 }
-
-// ---- LSD radix sort, 4-bit digits, items owned contiguously by threads (stable) ------
-constexpr int SORT_THREADS = 256, SORT_ITEMS = 16, SORT_TILE = SORT_THREADS * SORT_ITEMS;
 
 // max |Z| over the matrix (non-negative floats order like their bit patterns) and, with
 // sumsq, += sum of Z^2 in the same pass: float4 loads, four in flight per thread, float
@@ -116,101 +112,6 @@ __global__ void k_make_zscale(const unsigned* mx, float* zscale) {
   zscale[1] = ldexpf(1.f, -e);
 }
 
-__global__ void k_sort_hist(const long long* keys, long long n, int shift, unsigned* cnt, int nblk) {
-  __shared__ unsigned h[16];
-  if (threadIdx.x < 16) h[threadIdx.x] = 0;
-  __syncthreads();
-  const long long base = (long long)blockIdx.x * SORT_TILE;
-  for (int j = threadIdx.x; j < SORT_TILE; j += SORT_THREADS) {
-    long long e = base + j;
-    if (e < n) atomicAdd(&h[(keys[e] >> shift) & 15], 1u);
-  }
-  __syncthreads();
-  if (threadIdx.x < 16) cnt[threadIdx.x * nblk + blockIdx.x] = h[threadIdx.x];
-}
-
-__global__ void k_sort_scan(unsigned* cnt, int total) {
-  // single block exclusive scan of `total` counts (digit-major), 1024 threads
-  __shared__ unsigned carry;
-  __shared__ unsigned ws[32];
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  for (int base = 0; base < total; base += 1024) {
-    int i = base + threadIdx.x;
-    unsigned v = i < total ? cnt[i] : 0u;
-    unsigned x = v;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int o = 1; o < 32; o <<= 1) {
-      unsigned y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) ws[w] = x;
-    __syncthreads();
-    if (w == 0) {
-      unsigned s = ws[lane];
-      for (int o = 1; o < 32; o <<= 1) {
-        unsigned y = __shfl_up_sync(0xffffffffu, s, o);
-        if (lane >= o) s += y;
-      }
-      ws[lane] = s;
-    }
-    __syncthreads();
-    unsigned excl = carry + (w ? ws[w - 1] : 0u) + x - v;
-    if (i < total) cnt[i] = excl;
-    __syncthreads();
-    if (threadIdx.x == 1023) carry = excl + v;
-    __syncthreads();
-  }
-}
-
-__global__ void k_sort_scatter(const long long* kin, const float* vin, long long* kout, float* vout,
-                               long long n, int shift, const unsigned* off, int nblk) {
-  __shared__ unsigned tab[16][SORT_THREADS + 1];
-  const int t = threadIdx.x;
-  const long long base = (long long)blockIdx.x * SORT_TILE + (long long)t * SORT_ITEMS;
-  unsigned c[16];
-#pragma unroll
-  for (int d = 0; d < 16; ++d) c[d] = 0;
-  long long kk[SORT_ITEMS];
-#pragma unroll
-  for (int j = 0; j < SORT_ITEMS; ++j) {
-    long long e = base + j;
-    kk[j] = e < n ? kin[e] : -1;
-    if (e < n) c[(kk[j] >> shift) & 15]++;
-  }
-#pragma unroll
-  for (int d = 0; d < 16; ++d) tab[d][t] = c[d];
-  __syncthreads();
-  // exclusive scan of each digit row across the 256 threads: warp w scans rows 2w, 2w+1
-  const int lane = t & 31, w = t >> 5;
-  for (int d = 2 * w; d < 2 * w + 2; ++d) {
-    unsigned run = 0;
-    unsigned vals[8];
-    for (int j = 0; j < 8; ++j) { vals[j] = tab[d][lane * 8 + j]; run += vals[j]; }
-    unsigned x = run;
-    for (int o = 1; o < 32; o <<= 1) {
-      unsigned y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    unsigned e = x - run;
-    for (int j = 0; j < 8; ++j) { tab[d][lane * 8 + j] = e; e += vals[j]; }
-  }
-  __syncthreads();
-  unsigned pos[16];
-#pragma unroll
-  for (int d = 0; d < 16; ++d) pos[d] = off[d * nblk + blockIdx.x] + tab[d][t];
-#pragma unroll
-  for (int j = 0; j < SORT_ITEMS; ++j) {
-    long long e = base + j;
-    if (e < n) {
-      int d = (int)((kk[j] >> shift) & 15);
-      unsigned p = pos[d]++;
-      kout[p] = kk[j];
-      vout[p] = vin[e];
-    }
-  }
-}
-
 // Self-test of the timeout path: thread 0 waits, with the pipelines' bounded polling
 // helper, on a fresh mbarrier that nothing arrives on, and gives up after `polls` polls
 // (each at most tc::kPollNs) as a pipeline wait does: it flags the context (timeout,
@@ -257,11 +158,6 @@ void launch_unpad_copy(const float* src, int64_t rows, int RP, float* dst, int c
   if (grid) k_unpad_copy<<<grid, 256, 0, st>>>(src, rows, RP, dst, cols);
 }
 
-size_t sort_coo_scratch(long long nnz) {
-  long long nblk = (nnz + SORT_TILE - 1) / SORT_TILE;
-  return (size_t)nnz * (sizeof(long long) + sizeof(float)) + (size_t)(16 * nblk + 16) * sizeof(unsigned) + 256;
-}
-
 static void launch_maxabs(const float* Z, int64_t rows, int64_t cols, int64_t ld, unsigned* mx, double* sumsq, int nsm,
                           cudaStream_t st) {
   int64_t grid = (rows * ((cols + 15) / 16) + 255) / 256;
@@ -287,33 +183,6 @@ void launch_zscale(const float* Z, int64_t rows, int64_t cols, int64_t ld, unsig
   launch_maxabs(Z, rows, cols, ld, zmax, sumsq, nsm, st);
   if (extra && n_extra > 0) launch_maxabs(extra, 1, n_extra, n_extra, zmax, nullptr, nsm, st);
   k_make_zscale<<<1, 1, 0, st>>>(zmax, zscale);
-}
-
-void launch_sort_coo(long long* idx, float* val, long long nnz, void* scratch, size_t scratch_bytes,
-                     int idx_bits, cudaStream_t st) {
-  if (nnz <= 1) return;
-  const int nblk = (int)((nnz + SORT_TILE - 1) / SORT_TILE);
-  char* p = reinterpret_cast<char*>(scratch);
-  long long* k2 = reinterpret_cast<long long*>(p);
-  float* v2 = reinterpret_cast<float*>(p + (size_t)nnz * sizeof(long long));
-  size_t offb = (size_t)nnz * (sizeof(long long) + sizeof(float));
-  offb = (offb + 255) & ~size_t(255);
-  unsigned* cnt = reinterpret_cast<unsigned*>(p + offb);
-  (void)scratch_bytes;
-  long long* ka = idx;
-  float* va = val;
-  long long* kb = k2;
-  float* vb = v2;
-  int passes = (idx_bits + 3) / 4;
-  if (passes & 1) ++passes;                  // even count: result lands back in idx/val
-  for (int ps = 0; ps < passes; ++ps) {
-    const int shift = 4 * ps;
-    k_sort_hist<<<nblk, SORT_THREADS, 0, st>>>(ka, nnz, shift, cnt, nblk);
-    k_sort_scan<<<1, 1024, 0, st>>>(cnt, 16 * nblk);
-    k_sort_scatter<<<nblk, SORT_THREADS, 0, st>>>(ka, va, kb, vb, nnz, shift, cnt, nblk);
-    long long* tk = ka; ka = kb; kb = tk;
-    float* tv = va; va = vb; vb = tv;
-  }
 }
 
 }  // namespace godec
