@@ -1716,84 +1716,72 @@ static godec_status mul_common(const float* Z, int64_t m, int64_t n, int64_t ldz
     snprintf(g_static_err, sizeof(g_static_err), "godec_mul: invalid argument");
     return GODEC_ERR_ARG;
   }
+  auto out = [](godec_status s, const char* why) {
+    snprintf(g_static_err, sizeof(g_static_err), "godec_mul: %.200s", why);
+    return s;
+  };
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int RP = round_up(r, 8);
   const int64_t rows = trans ? n : m, K = trans ? m : n;
   int nsm = 0, dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      (trans ? prepare_prod_kernels() : prepare_tc_kernels()) != cudaSuccess) {
-    snprintf(g_static_err, sizeof(g_static_err), "godec_mul: no CUDA device");
-    return GODEC_ERR_CUDA;
-  }
+      (trans ? prepare_prod_kernels() : prepare_tc_kernels()) != cudaSuccess)
+    return out(GODEC_ERR_CUDA, "no CUDA device");
   const TcGeom geom = trans ? prod_split_geometry(rows, K, nsm) : tc_geometry(rows, K, nsm);
   const int64_t ldz64 = (n + 63) / 64 * 64, ldb = (K + 7) / 8 * 8;
-  float *Bp = nullptr, *part = nullptr, *Yp = nullptr, *Zs = nullptr, *aux = nullptr;
-  void* Bs = nullptr;
-  unsigned* cnt = nullptr;
-  int* pend = nullptr;
-  bool ok = cudaMallocAsync(reinterpret_cast<void**>(&Bp), (size_t)K * RP * sizeof(float), st) == cudaSuccess &&
-            cudaMallocAsync(&Bs, (size_t)2 * RP * ldb * 2, st) == cudaSuccess &&
-            cudaMallocAsync(reinterpret_cast<void**>(&aux), (size_t)(4 + RP) * sizeof(float), st) == cudaSuccess &&
-            cudaMallocAsync(reinterpret_cast<void**>(&part), (size_t)geom.tiles * geom.maxseg * 128 * RP * sizeof(float),
-                            st) == cudaSuccess &&
-            cudaMallocAsync(reinterpret_cast<void**>(&Yp), (size_t)rows * RP * sizeof(float), st) == cudaSuccess &&
-            cudaMallocAsync(reinterpret_cast<void**>(&cnt), (size_t)geom.tiles * sizeof(unsigned), st) == cudaSuccess &&
-            cudaMallocAsync(reinterpret_cast<void**>(&pend), (size_t)geom.G * geom.maxpend * sizeof(int), st) ==
-                cudaSuccess &&
-            (!trans || cudaMallocAsync(reinterpret_cast<void**>(&Zs), (size_t)m * ldz64 * sizeof(float), st) == cudaSuccess);
-  bool mapped = false;
-  if (ok) {
-    alignas(64) unsigned char mapA[128], mapB[128];
-    mapped = (trans ? make_tmap_split(mapA, Zs, m, ldz64, 64) : make_tmap_f32(mapA, Z, rows, K, ldz, 128)) &&
-             make_tmap_f16(mapB, Bs, 2 * RP, K, ldb, 2 * RP);
-    if (mapped && cudaMemsetAsync(cnt, 0, (size_t)geom.tiles * sizeof(unsigned), st) != cudaSuccess) {
-      for (void* q : {(void*)Bp, Bs, (void*)aux, (void*)part, (void*)Yp, (void*)cnt, (void*)pend, (void*)Zs})
-        if (q) cudaFreeAsync(q, st);
-      snprintf(g_static_err, sizeof(g_static_err), "godec_mul: clearing the tile counters: %s",
-               cudaGetErrorString(cudaGetLastError()));
-      return GODEC_ERR_CUDA;
-    }
-    if (mapped) {
-      // aux: {s_Z, 1/s_Z}, max-|Z| scratch, pad, then RP column factors of B
-      launch_zscale(Z, m, n, ldz, reinterpret_cast<unsigned*>(aux + 2), aux, nsm, st);
-      launch_pad_copy(B, K, r, r, Bp, RP, st);
-      launch_split_t(Bp, K, RP, Bs, ldb, aux + 4, st);
-      if (trans) launch_split_copy(Z, m, n, ldz, Zs, ldz64, aux, nsm, st);   // read M-major: no transpose
-      TcLaunch l{};
-      l.mapA = mapA;
-      l.mapB = mapB;
-      l.rows = rows;
-      l.K = K;
-      l.RP = RP;
-      l.geom = geom;
-      l.part = part;
-      l.counters = cnt;
-      l.out = Yp;
-      l.cscale = aux + 4;
-      l.zscale = aux;
-      l.pend = pend;
-      l.trans = trans;
-      if (trans) launch_prod_split(l, st);
-      else launch_prod_tc(l, st);
-      launch_unpad_copy(Yp, rows, RP, Y, r, st);
-    }
+  // one scratch block: cleared part (maxima, tile counters), scales, split operand, partial
+  // slots, deferred completions, the split copy that Z^T C reads M-major
+  size_t total = 0;
+  auto place = [&](size_t bytes) {
+    const size_t at = total;
+    total += (bytes + 255) & ~size_t(255);
+    return at;
+  };
+  const size_t o_max = place((1 + (size_t)RP) * sizeof(unsigned)), o_cnt = place((size_t)geom.tiles * sizeof(unsigned)),
+               b_clear = total, o_sc = place((2 + (size_t)RP) * sizeof(float)), o_bs = place((size_t)2 * RP * ldb * 2),
+               o_part = place((size_t)geom.tiles * geom.maxseg * 128 * RP * sizeof(float)),
+               o_pend = place((size_t)geom.G * geom.maxpend * sizeof(int)),
+               o_zs = place(trans ? (size_t)m * ldz64 * sizeof(float) : 0);
+  char* mem = nullptr;
+  if (scratch_alloc(reinterpret_cast<void**>(&mem), total, dev, st) != cudaSuccess) {
+    cudaGetLastError();
+    return out(GODEC_ERR_OOM, "out of device memory");
   }
-  void* ptrs[] = {Bp, Bs, aux, part, Yp, cnt, pend, Zs};
-  for (void* q : ptrs)
-    if (q) cudaFreeAsync(q, st);
-  if (!ok) {
-    snprintf(g_static_err, sizeof(g_static_err), "godec_mul: out of device memory");
-    return GODEC_ERR_OOM;
-  }
+  unsigned* mx = reinterpret_cast<unsigned*>(mem + o_max);   // max |Z|, then max |B| by column
+  float* sc = reinterpret_cast<float*>(mem + o_sc);          // s_Z, 1 / s_Z, then the columns' factors
+  alignas(64) unsigned char mapA[128], mapB[128];
+  const bool mapped = (trans ? make_tmap_split(mapA, mem + o_zs, m, ldz64, 64) : make_tmap_f32(mapA, Z, rows, K, ldz, 128)) &&
+                      make_tmap_f16(mapB, mem + o_bs, 2 * RP, K, ldb, 2 * RP);
   if (!mapped) {
-    snprintf(g_static_err, sizeof(g_static_err), "godec_mul: tensor map encoding failed");
-    return GODEC_ERR_CUDA;
+    cudaFreeAsync(mem, st);
+    return out(GODEC_ERR_CUDA, "tensor map encoding failed");
   }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) {
-    snprintf(g_static_err, sizeof(g_static_err), "godec_mul: %s", cudaGetErrorString(e));
-    return GODEC_ERR_CUDA;
+  cudaError_t e = cudaMemsetAsync(mem, 0, b_clear, st);
+  if (e == cudaSuccess) {
+    launch_mul_stats(Z, m, n, ldz, B, K, r, mx, nsm, st);
+    launch_split_b(B, K, r, RP, mx + 1, mem + o_bs, ldb, sc + 2, mx, sc, st);
+    if (trans) launch_split_copy(Z, m, n, ldz, mem + o_zs, ldz64, sc, nsm, st);
+    TcLaunch l{};
+    l.mapA = mapA;
+    l.mapB = mapB;
+    l.rows = rows;
+    l.K = K;
+    l.RP = RP;
+    l.geom = geom;
+    l.part = reinterpret_cast<float*>(mem + o_part);
+    l.counters = reinterpret_cast<unsigned*>(mem + o_cnt);
+    l.out = Y;
+    l.out_cols = r;
+    l.cscale = sc + 2;
+    l.zscale = sc;
+    l.pend = reinterpret_cast<int*>(mem + o_pend);
+    l.trans = trans;
+    if (trans) launch_prod_split(l, st);
+    else launch_prod_tc(l, st);
+    e = cudaGetLastError();
   }
+  cudaFreeAsync(mem, st);
+  if (e != cudaSuccess) return out(GODEC_ERR_CUDA, cudaGetErrorString(e));
   return GODEC_OK;
 }
 

@@ -82,14 +82,16 @@ struct Engine {
   void* Bs = nullptr;                          // 2 RP x ldb halves (split transposed operand)
   alignas(64) unsigned char mapB[2][128];      // over Bs with K = n (index 0) and K = m (index 1)
   TcGeom geom[2];
-  float *Bp = nullptr, *cscale = nullptr, *part = nullptr, *Yp = nullptr;
+  float *cscale = nullptr, *part = nullptr;
+  unsigned* cmax = nullptr;
   unsigned* cnt = nullptr;
 
   // Y (rows x c, dense) = src * B, or src^T * B with trans (B K x c, dense rows of c)
   void mul(const Source& s, int trans, const float* B, int c, float* Y) {
     const int64_t rows = dim[trans], K = dim[1 - trans];
-    launch_pad_copy(B, K, c, c, Bp, RP, st);
-    launch_split_t(Bp, K, RP, Bs, ldb, cscale, st);
+    cudaMemsetAsync(cmax, 0, (size_t)(1 + RP) * sizeof(unsigned), st);
+    launch_mul_stats(nullptr, 0, 0, 0, B, K, c, cmax, nsm, st);
+    launch_split_b(B, K, c, RP, cmax + 1, Bs, ldb, cscale, nullptr, nullptr, st);
     TcLaunch l{};
     l.mapA = s.map[trans];
     l.mapB = mapB[trans];
@@ -99,12 +101,12 @@ struct Engine {
     l.geom = geom[trans];
     l.part = part;
     l.counters = cnt;
-    l.out = Yp;
+    l.out = Y;
+    l.out_cols = c;
     l.cscale = cscale;
     l.zscale = s.zscale;
     l.trans = trans;
     launch_prod_split(l, st);
-    launch_unpad_copy(Yp, rows, RP, Y, c, st);
   }
 };
 
@@ -152,9 +154,8 @@ extern "C" godec_status godec_backward(const float* X, int64_t m, int64_t n, int
   E.RP = RP;
   E.ldb = (mx + 7) / 8 * 8;
   E.Bs = sc.get<unsigned short>((size_t)2 * RP * E.ldb);
-  E.Bp = sc.get<float>((size_t)mx * RP);
+  E.cmax = sc.get<unsigned>(1 + (size_t)RP);
   E.cscale = sc.get<float>(RP);
-  E.Yp = sc.get<float>((size_t)mx * RP);
   float* zsc = sc.get<float>(2 * src.size() + 2);      // {s, 1/s} of each source, then of X
   unsigned* zmax = sc.get<unsigned>(src.size() + 1);
   // per-iteration checkpoints (forward sweep)

@@ -183,6 +183,13 @@ int tc_rpp(int RP);
 // undo the scaling.
 void launch_split_t(const float* B, int64_t rows, int RP, void* bt2, int64_t ldb, float* cscale, cudaStream_t st,
                     const int* skip = nullptr);
+// The operand of a product with a K x r matrix B: column maxima (and max |Z| when Z is given)
+// into mx = {max |Z|, max |B[:, 0]|, ...} (cleared before), then the split form with its column
+// factors cscale; with zmax also zscale.
+void launch_mul_stats(const float* Z, int64_t m, int64_t n, int64_t ldz, const float* B, int64_t K, int r, unsigned* mx,
+                      int nsm, cudaStream_t st);
+void launch_split_b(const float* B, int64_t K, int r, int RP, const unsigned* cmax, void* bt2, int64_t ldb, float* cscale,
+                    const unsigned* zmax, float* zscale, cudaStream_t st);
 // zscale = {s, 1/s}: the power of two with max |Z| s in [2^12, 2^13) (1 if Z is zero or
 // not finite); zmax is scratch.  sumsq (nullable): += sum of Z^2.  extra (nullable): n_extra
 // more values that the maximum covers.
@@ -208,7 +215,8 @@ struct TcLaunch {
   TcGeom geom;
   float* part;             // tiles x maxseg x 128 x RP
   unsigned* counters;      // tiles, zero
-  float* out;              // rows x RP (nullable)
+  float* out;              // rows x out_cols (nullable)
+  int out_cols;            // <= RP; 0: RP
   void* bt2;               // 2 RP x ldb halves (nullable)
   int64_t ldb;
   const float* Tn[2];      // upper triangular (launch_prod_split)

@@ -85,7 +85,8 @@ struct PArgs {
   int pin;                  // of kPinOf classes of blocks, those kept in L2 (< 0: no cache hints)
   float* part;              // tiles x maxseg x RP x BM
   unsigned* counters;       // tiles
-  float* out;               // rows x RP (nullable)
+  float* out;               // rows x oc, oc <= RP (nullable)
+  int oc;
   __half* bt2;              // 2 RP x ldb split transposed output (nullable)
   int64_t ldb;
   const float* Tn0;
@@ -309,11 +310,11 @@ __device__ __forceinline__ void finish_tile(const PArgs& a, int64_t t, int nseg,
     named_sync(2, kHelpers);
   }
   if (a.out) {
-    const int q4 = RP / 4;
-    for (int it = u; it < nrow * q4; it += kHelpers) {
-      const int r = it / q4, l = (it - r * q4) * 4;
-      const float* p = Ps + r * LD + l;
-      *reinterpret_cast<float4*>(a.out + (o0 + r) * (int64_t)RP + l) = make_float4(p[0], p[1], p[2], p[3]);
+    const int oc = a.oc;   // consecutive threads on consecutive floats of the output rows
+    float* o = a.out + o0 * oc;
+    for (int it = u; it < nrow * oc; it += kHelpers) {
+      const int r = it / oc;
+      o[it] = Ps[r * LD + it - r * oc];
     }
   }
   if (a.bt2) {
@@ -679,6 +680,7 @@ void launch_prod_split(const TcLaunch& l, cudaStream_t st) {
   a.part = l.part;
   a.counters = l.counters;
   a.out = l.out;
+  a.oc = l.out_cols ? l.out_cols : l.RP;
   a.bt2 = reinterpret_cast<__half*>(l.bt2);
   a.ldb = l.ldb;
   a.Tn0 = l.Tn[0];

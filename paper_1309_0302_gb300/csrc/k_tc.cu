@@ -85,7 +85,8 @@ struct TcArgs {
   int maxseg;
   float* part;              // tiles x maxseg x BM x RP
   unsigned* counters;       // tiles
-  float* out;               // rows x RP
+  float* out;               // rows x oc, oc <= RP
+  int oc;
   const float* cscale;      // per-column output factor 1 / s_B (nullable: 1)
   const float* zscale;      // {s_Z, 1 / s_Z} (nullable: 1)
   int* pend;                // G x maxpend: tiles each CTA completes, deferred to its end
@@ -151,9 +152,12 @@ __device__ void tile_finish(const TcArgs& a, int64_t t, int nseg, int u, int nth
       const int it = it0 + q * nthr;
       if (it < nitem) {
         const int c = (it % RP4) * 4;
-        reinterpret_cast<float4*>(a.out + o0 * RP)[it] =
-            make_float4(acc[q].x * (csc[c] * zi), acc[q].y * (csc[c + 1] * zi), acc[q].z * (csc[c + 2] * zi),
-                        acc[q].w * (csc[c + 3] * zi));
+        const float w[4] = {acc[q].x * (csc[c] * zi), acc[q].y * (csc[c + 1] * zi), acc[q].z * (csc[c + 2] * zi),
+                            acc[q].w * (csc[c + 3] * zi)};
+        float* o = a.out + (o0 + it / RP4) * a.oc + c;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (c + k < a.oc) o[k] = w[k];
       }
     }
   }
@@ -506,6 +510,90 @@ __global__ void k_split_t(const float* __restrict__ B, int64_t rows, int RP, __h
   }
 }
 
+// The power of two that brings a maximum (float bits) into [2^(top-1), 2^top): its exponent.
+__device__ __forceinline__ int scale_exp(unsigned mx, int top) {
+  const float m = __uint_as_float(mx);
+  if (!(m > 0.f) || !isfinite(m)) return 0;
+  int ex;
+  frexpf(m, &ex);   // m in [2^(ex-1), 2^ex)
+  const int e = top - ex;
+  return e < -120 ? -120 : (e > 120 ? 120 : e);
+}
+
+// max |Z| into mx[0] (blocks below gz) and max |B[:, c]| into mx[1 + c] (the others, 256 rows
+// of the K x r operand each), atomic maxima of float bits.
+__global__ void __launch_bounds__(256)
+k_mul_stats(const float* __restrict__ Z, int64_t m, int64_t n, int64_t ldz, int gz, const float* __restrict__ B, int64_t K,
+            int r, unsigned* __restrict__ mx) {
+  __shared__ unsigned sm[kMaxRP];
+  const int tid = threadIdx.x;
+  if (tid < kMaxRP) sm[tid] = 0u;
+  __syncthreads();
+  if ((int)blockIdx.x >= gz) {
+    const int64_t r0 = (int64_t)(blockIdx.x - gz) * 256;
+    const int cnt = (int)((K - r0 < 256 ? K - r0 : 256) * r);
+    const float* b = B + r0 * r;
+    for (int e = tid; e < cnt; e += 256) atomicMax(&sm[e % r], __float_as_uint(fmaxf(0.f, fabsf(b[e]))));
+    __syncthreads();
+    if (tid < r) atomicMax(&mx[1 + tid], sm[tid]);
+    return;
+  }
+  float v = 0.f;
+  const int64_t per = (n + 15) / 16, total = m * per;   // runs of 16 columns; rows are 16-byte aligned
+  for (int64_t e = (int64_t)blockIdx.x * 256 + tid; e < total; e += (int64_t)gz * 256) {
+    const int64_t i = e / per, j = (e - i * per) * 16;
+    const float* z = Z + i * ldz + j;
+    if (j + 16 <= n) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float4 q = __ldg(reinterpret_cast<const float4*>(z) + u);
+        v = fmaxf(v, fmaxf(fmaxf(fabsf(q.x), fabsf(q.y)), fmaxf(fabsf(q.z), fabsf(q.w))));
+      }
+    } else {
+      for (int u = 0; j + u < n; ++u) v = fmaxf(v, fabsf(z[u]));
+    }
+  }
+  for (int o = 16; o; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  if ((tid & 31) == 0) atomicMax(&sm[0], __float_as_uint(v));
+  __syncthreads();
+  if (tid == 0) atomicMax(&mx[0], sm[0]);
+}
+
+// The split transposed operand (2 RP x ldb halves) of a K x r matrix B from its column maxima
+// cmax, 64 rows per block through shared memory (both sides coalesced): column c scaled by the
+// power of two that brings its maximum into [2^9, 2^10), cscale[c] undoing it; columns r ..
+// RP-1 zero.  zmax (nullable): block 0 also forms zscale = {s, 1/s} from it.
+constexpr int SB_ROWS = 64;
+__global__ void __launch_bounds__(256)
+k_split_b(const float* __restrict__ B, int64_t K, int r, int RP, const unsigned* __restrict__ cmax, __half* __restrict__ bt2,
+          int64_t ldb, float* __restrict__ cscale, const unsigned* __restrict__ zmax, float* __restrict__ zscale) {
+  __shared__ float t[SB_ROWS][kMaxRP + 1];
+  __shared__ float s_sc[kMaxRP];
+  const int tid = threadIdx.x;
+  const int64_t r0 = (int64_t)blockIdx.x * SB_ROWS;
+  const int nr = (int)(K - r0 < SB_ROWS ? K - r0 : SB_ROWS);
+  if (tid < RP) {
+    const int e = tid < r ? scale_exp(cmax[tid], 10) : 0;
+    s_sc[tid] = ldexpf(1.f, e);
+    if (blockIdx.x == 0) cscale[tid] = ldexpf(1.f, -e);
+  }
+  if (blockIdx.x == 0 && tid == 0 && zmax) {
+    const int e = scale_exp(zmax[0], 13);
+    zscale[0] = ldexpf(1.f, e);
+    zscale[1] = ldexpf(1.f, -e);
+  }
+  for (int e = tid; e < nr * r; e += 256) t[e / r][e % r] = B[r0 * r + e];
+  __syncthreads();
+  const int row = tid & 63;
+  if (row < nr)
+    for (int c = tid >> 6; c < RP; c += 4) {
+      const float v = c < r ? t[row][c] * s_sc[c] : 0.f;
+      const __half c1 = __float2half_rn(v);
+      bt2[(int64_t)c * ldb + r0 + row] = c1;
+      bt2[(int64_t)(RP + c) * ldb + r0 + row] = __float2half_rn((v - __half2float(c1)) * kLoScale);
+    }
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   if (!fn) {
@@ -562,6 +650,19 @@ void launch_split_t(const float* B, int64_t rows, int RP, void* bt2, int64_t ldb
   k_split_t<<<RP, 256, 0, st>>>(B, rows, RP, reinterpret_cast<__half*>(bt2), ldb, cscale, skip);
 }
 
+void launch_mul_stats(const float* Z, int64_t m, int64_t n, int64_t ldz, const float* B, int64_t K, int r, unsigned* mx,
+                      int nsm, cudaStream_t st) {
+  int64_t gz = Z ? (m * ((n + 15) / 16) + 255) / 256 : 0;
+  if (gz > 8LL * nsm) gz = 8LL * nsm;
+  k_mul_stats<<<(unsigned)(gz + (K + 255) / 256), 256, 0, st>>>(Z, m, n, ldz, (int)gz, B, K, r, mx);
+}
+
+void launch_split_b(const float* B, int64_t K, int r, int RP, const unsigned* cmax, void* bt2, int64_t ldb, float* cscale,
+                    const unsigned* zmax, float* zscale, cudaStream_t st) {
+  k_split_b<<<(unsigned)((K + SB_ROWS - 1) / SB_ROWS), 256, 0, st>>>(B, K, r, RP, cmax, static_cast<__half*>(bt2), ldb,
+                                                                    cscale, zmax, zscale);
+}
+
 TcGeom tc_geometry(int64_t rows, int64_t K, int nsm) {
   TcGeom g;
   g.tiles = (rows + BM - 1) / BM;
@@ -604,6 +705,7 @@ void launch_prod_tc(const TcLaunch& l, cudaStream_t st) {
   a.part = l.part;
   a.counters = l.counters;
   a.out = l.out;
+  a.oc = l.out_cols ? l.out_cols : l.RP;
   a.cscale = l.cscale;
   a.zscale = l.zscale;
   a.pend = l.pend;
