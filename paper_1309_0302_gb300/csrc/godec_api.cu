@@ -146,6 +146,7 @@ struct godec_ctx {
   long long sbits_words = 0;           // ctl->cur) and a clear one the next S-step marks its support in
   size_t sbits_bytes = 0;
   unsigned* order = nullptr;           // scratch of the ordered export of S
+  float* svd_warm = nullptr;           // naive GoDec, LinGoDec: right basis of the last small SVD
   float* XA1 = nullptr;                // m x RP: X A1, the cached part of the first projection (null: the
                                        // first product streams Z)
   long long* S_idx[2] = {nullptr, nullptr};
@@ -765,7 +766,7 @@ void enqueue_naive_lstep(godec_ctx* c) {
   cqr2(c, c->P, m, p, RP, c->Qa, R1, T1, R2m, T2);
   const int* ab = &c->ctl->abort;   // an abandoned iteration leaves U, V and the basis as they were
   launch_rmul(R2m, R1, RP, p, c->rf_core, 0, nullptr, st, ab);
-  launch_svd_small(c->rf_core, p, r, c->rf_U, c->sigma, c->rf_V, st, ab, true);
+  launch_svd_small(c->rf_core, p, r, c->rf_U, c->sigma, c->rf_V, st, ab, true, c->svd_warm);
   launch_tall_small_d(c->Qa, RP, p, c->rf_U, r, 0, r, m, 1.f, 0.f, c->U, RP, st, ab);
   launch_tall_small_d(c->Qb, RP, p, c->rf_V, r, 0, r, n, 1.f, 0.f, c->V, RP, st, ab);
   launch_lsplit(c->U, c->V, c->sigma, m, n, RP, r, c->ctl->zscale, c->LA, c->LB, st, ab);
@@ -903,6 +904,12 @@ godec_status reset_state(godec_ctx* c) {
   refresh_z(c, reinterpret_cast<double*>(reinterpret_cast<char*>(c->ctl) + offsetof(Ctl, normX2)));
   if (c->XA1) form_xa1(c);
   launch_reset_iter(c->ctl, c->st);
+  if (c->lingo || c->naive) {
+    const int d = c->lingo ? c->lg_d : c->np_cols;
+    std::vector<float> id((size_t)d * d, 0.f);
+    for (int i = 0; i < d; ++i) id[(size_t)i * d + i] = 1.f;
+    CK(cudaMemcpyAsync(c->svd_warm, id.data(), id.size() * sizeof(float), cudaMemcpyHostToDevice, c->st));
+  }
   if (c->lingo) {
     // the features' basis Qf = orth(F) (F was copied into A1) and its split operand, fixed
     // for the whole run; Rf keeps F = Qf R2 R1 for the final W
@@ -1204,6 +1211,7 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
     want(&c->rf_core, W * W);
     want(&c->rf_U, W * W);
     want(&c->rf_V, W * W);
+    want(&c->svd_warm, W * W);
     CKI(prepare_refine_kernels());
   }
   want(&c->A1, (size_t)n * RP);
@@ -1996,7 +2004,7 @@ static void lingo_lstep(godec_ctx* c) {
   final_cqr2(c, m, g64(c, 0), c->Rfin, c->Rfin + 2 * rr, c->Q1, g64(c, 2), nullptr);   // Y Qf = Qy Rb Ra
   c->r = r;
   launch_rmul(c->Rfin + 2 * rr, c->Rfin, RP, d, c->rf_core, 0, nullptr, st, ab);
-  launch_svd_small(c->rf_core, d, r, c->rf_U, c->sigma, c->rf_V, st, ab, true);
+  launch_svd_small(c->rf_core, d, r, c->rf_U, c->sigma, c->rf_V, st, ab, true, c->svd_warm);
   launch_tall_small_d(c->Q1, RP, d, c->rf_U, r, 0, r, m, 1.f, 0.f, c->U, RP, st, ab);
   launch_tall_small_d(c->Q2, RP, d, c->rf_V, r, 0, r, n, 1.f, 0.f, c->V, RP, st, ab);
 }

@@ -61,6 +61,7 @@ __global__ void k_refine_core(const float* __restrict__ Ra1, const float* __rest
 }
 
 constexpr double kJacobiTol = 1e-14;
+constexpr int kWarmItems = 5;   // n^2 / (32 ceil(n / 2)) entries a thread for n <= 64, rounded up
 
 // SVD of an n x n float64 matrix (n <= 64) by one-sided Jacobi (Hestenes): columns of
 // W = A V are rotated pairwise until orthogonal.  Round-robin ordering: each round the
@@ -76,13 +77,17 @@ constexpr double kJacobiQuad = 1e-7;
 constexpr float kJacobiTolF = 2e-6f;
 constexpr double kJacobiQuadF = 0.0;
 
+// warm (nullable, n x n floats, in and out): an orthonormal V to start from, the one the last
+// call of the same iteration ended with.  The core of the next iteration differs little, so
+// two or three sweeps follow where a start from I takes ten (50 x 50: 594 us cold).
+//
 // T = double, or float for the larger cores of the subspace iterations (GB300 issues a
 // warp's float64 instruction over many cycles: a float64 sweep over 58 columns costs
 // hundreds of microseconds); float32 rotates down to kJacobiTolF.
 template <typename T>
 __global__ void __launch_bounds__(1024) k_svd_small(const double* __restrict__ A, int n, int r, double* __restrict__ Uo,
                                                     float* __restrict__ sigma, double* __restrict__ Vo,
-                                                    const int* skip) {
+                                                    const int* skip, float* __restrict__ warm) {
   if (block_skip(skip)) return;
   extern __shared__ double smd[];   // W, V: 2 x 64 x 65 values (dynamic)
   T (*W)[kMaxRP + 1] = reinterpret_cast<T (*)[kMaxRP + 1]>(smd);
@@ -95,7 +100,34 @@ __global__ void __launch_bounds__(1024) k_svd_small(const double* __restrict__ A
   for (int e = tid; e < n * n; e += nt) {
     const int i = e / n, j = e % n;
     W[i][j] = (T)A[e];
-    V[i][j] = (i == j) ? (T)1 : (T)0;
+    V[i][j] = warm ? (T)warm[e] : (i == j ? (T)1 : (T)0);
+  }
+  if (warm) {
+    // V := V (3 I - V^T V) / 2 removes what rounding cost the last call's basis, then W = A V;
+    // the products go through registers (at most five entries a thread) and S = V^T V's block
+    T (*S)[kMaxRP + 1] = V + kMaxRP;
+    __syncthreads();
+    auto mm = [&](auto&& left, const T (*R)[kMaxRP + 1], T (*out)[kMaxRP + 1], bool newton) {
+      T acc[kWarmItems];
+#pragma unroll
+      for (int u = 0; u < kWarmItems; ++u) {
+        const int e = tid + u * nt, i = e / n, j = e % n;
+        T s = 0;
+        if (e < n * n)
+          for (int k = 0; k < n; ++k) s += left(i, k) * R[k][j];
+        acc[u] = newton ? ((i == j) ? (T)1.5 : (T)0) - (T)0.5 * s : s;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < kWarmItems; ++u) {
+        const int e = tid + u * nt;
+        if (e < n * n) out[e / n][e % n] = acc[u];
+      }
+      __syncthreads();
+    };
+    mm([&](int i, int k) { return V[k][i]; }, V, S, true);    // S = (3 I - V^T V) / 2
+    mm([&](int i, int k) { return V[i][k]; }, S, V, false);   // V = V S
+    mm([&](int i, int k) { return W[i][k]; }, V, W, false);   // W = A V
   }
   const int np = (n + 1) & ~1, npairs = np / 2;
   for (int sweep = 0; sweep < 40; ++sweep) {
@@ -179,6 +211,8 @@ __global__ void __launch_bounds__(1024) k_svd_small(const double* __restrict__ A
     Vo[i * r + j] = (double)V[i][col];
   }
   for (int j = tid; j < r; j += nt) sigma[j] = (float)nrm[order[j]];
+  if (warm)
+    for (int e = tid; e < n * n; e += nt) warm[e] = (float)V[e / n][e % n];
 }
 
 }  // namespace
@@ -190,7 +224,7 @@ void launch_concat2(const float* P, const float* Q, int64_t ldp, int r, int64_t 
 }
 
 constexpr size_t kCoreSmem = 3 * kMaxRP * (kMaxRP + 1) * sizeof(double);
-constexpr size_t kSvdSmem = 2 * kMaxRP * (kMaxRP + 1) * sizeof(double);
+constexpr size_t kSvdSmem = 2 * kMaxRP * (kMaxRP + 1) * sizeof(double);   // also three blocks of floats
 
 cudaError_t prepare_refine_kernels() {
   cudaError_t e = cudaFuncSetAttribute(k_refine_core, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoreSmem);
@@ -205,9 +239,9 @@ void launch_refine_core(const float* Ra1, const float* Ra2, const float* Rb1, co
 }
 
 void launch_svd_small(const double* A, int n, int r, double* U, float* sigma, double* V, cudaStream_t st,
-                      const int* skip, bool f32) {
-  if (f32) k_svd_small<float><<<1, 32 * ((n + 1) / 2), kSvdSmem, st>>>(A, n, r, U, sigma, V, skip);
-  else k_svd_small<double><<<1, 32 * ((n + 1) / 2), kSvdSmem, st>>>(A, n, r, U, sigma, V, skip);
+                      const int* skip, bool f32, float* warm) {
+  if (f32) k_svd_small<float><<<1, 32 * ((n + 1) / 2), kSvdSmem, st>>>(A, n, r, U, sigma, V, skip, warm);
+  else k_svd_small<double><<<1, 32 * ((n + 1) / 2), kSvdSmem, st>>>(A, n, r, U, sigma, V, skip, nullptr);
 }
 
 }  // namespace godec
