@@ -146,7 +146,8 @@ struct godec_ctx {
   long long sbits_words = 0;           // ctl->cur) and a clear one the next S-step marks its support in
   size_t sbits_bytes = 0;
   unsigned* order = nullptr;           // scratch of the ordered export of S
-  float* svd_warm = nullptr;           // naive GoDec, LinGoDec: right basis of the last small SVD
+  double* svd_warm = nullptr;          // right basis of the last small SVD (floats but in the precision form)
+  unsigned* cmax = nullptr;            // column maxima of an operand being split
   float* XA1 = nullptr;                // m x RP: X A1, the cached part of the first projection (null: the
                                        // first product streams Z)
   long long* S_idx[2] = {nullptr, nullptr};
@@ -395,6 +396,19 @@ void slot(godec_ctx* c, SlotLaunch& sl) {
   PROF(c, 4, c->side_st, launch_slot(sl, c->side_st));
 }
 
+// The split operand bt2[3] of B (rows x RP) with its column factors cs_ref.  Tall operands
+// take two passes over row blocks (38400 x 8: 17 -> 6 us); the one-launch form with a block per
+// column is the faster one below about 8000 rows.
+void split_operand(godec_ctx* c, const float* B, int64_t rows) {
+  if (rows < 8192) {
+    launch_split_t(B, rows, c->RP, bt2(c, 3), c->ldb, c->cs_ref, c->st, &c->ctl->abort);
+    return;
+  }
+  cudaMemsetAsync(c->cmax, 0, (1 + (size_t)c->RP) * sizeof(unsigned), c->st);
+  launch_mul_stats(nullptr, 0, 0, 0, B, rows, c->RP, c->cmax, c->nsm, c->st);
+  launch_split_b(B, rows, c->RP, c->RP, c->cmax + 1, bt2(c, 3), c->ldb, c->cs_ref, nullptr, nullptr, c->st);
+}
+
 // ---------------------------------------------------------------------------------
 // Precision form: one float32 correction of the L factors from the float16 chain
 // (reading of the error control for the rounded chain).  With U, V orthonormal, one
@@ -431,7 +445,7 @@ void refine(godec_ctx* c) {
   l.cscale = c->cs_ref;
   l.zscale = c->ctl->zscale;
   l.ctl = c->ctl;
-  launch_split_t(c->V, n, RP, bt2(c, 3), c->ldb, c->cs_ref, st, ab);
+  split_operand(c, c->V, n);
   l.mapA = c->tmap[0];
   l.mapB = c->tmap[13];
   l.rows = m;
@@ -439,7 +453,7 @@ void refine(godec_ctx* c) {
   l.geom = c->tg[0];
   l.out = c->RA;
   PROF(c, 0, st, launch_prod_split(l, st));
-  launch_split_t(c->U, m, RP, bt2(c, 3), c->ldb, c->cs_ref, st, ab);
+  split_operand(c, c->U, m);
   l.trans = 1;
   l.mapA = c->tmap[1];
   l.mapB = c->tmap[14];
@@ -458,7 +472,7 @@ void refine(godec_ctx* c) {
   cqr2(c, c->Wa, m, R2, ld, c->Qa, Ra1, Ta1, Ra2, Ta2);
   cqr2(c, c->Wb, n, R2, ld, c->Qb, Rb1, Tb1, Rb2, Tb2);
   PROF(c, 10, st, launch_refine_core(Ra1, Ra2, Rb1, Rb2, ld, c->rf_C, r, c->rf_core, st, ab));
-  PROF(c, 10, st, launch_svd_small(c->rf_core, R2, r, c->rf_U, c->sigma, c->rf_V, st, ab));
+  PROF(c, 10, st, launch_svd_small(c->rf_core, R2, r, c->rf_U, c->sigma, c->rf_V, st, ab, false, c->svd_warm));
   PROF(c, 10, st, launch_tall_small_d(c->Qa, ld, R2, c->rf_U, r, 0, r, m, 1.f, 0.f, c->U, RP, st, ab));
   PROF(c, 10, st, launch_tall_small_d(c->Qb, ld, R2, c->rf_V, r, 0, r, n, 1.f, 0.f, c->V, RP, st, ab));
 }
@@ -727,7 +741,7 @@ void greb_prod(godec_ctx* c, bool even, int map_b, const float* cscale, float* o
 // B (n x RP) has p nonzero columns.
 void greb_apply_D(godec_ctx* c, int ri, int p, const float* B, float* out) {
   const int RP = c->RP;
-  launch_split_t(B, c->p.n, RP, bt2(c, 3), c->ldb, c->cs_ref, c->st, &c->ctl->abort);
+  split_operand(c, B, c->p.n);
   greb_prod(c, true, 13, c->cs_ref, out, 0, 0);
   if (ri > 0) {
     launch_cross_gram(c->Q2, RP, ri, B, RP, p, c->p.n, c->rf_part, kRefineParts, c->rf_C, RP, c->st, &c->ctl->abort);
@@ -738,7 +752,7 @@ void greb_apply_D(godec_ctx* c, int ri, int p, const float* B, float* out) {
 // out (n x RP) = D^T Y for Y (m x RP) with p nonzero columns.
 void greb_apply_Dt(godec_ctx* c, int ri, int p, const float* Y, float* out) {
   const int RP = c->RP;
-  launch_split_t(Y, c->p.m, RP, bt2(c, 3), c->ldb, c->cs_ref, c->st, &c->ctl->abort);
+  split_operand(c, Y, c->p.m);
   greb_prod(c, false, 14, c->cs_ref, out, 0, 0);
   if (ri > 0) {
     launch_cross_gram(c->Q1, RP, ri, Y, RP, p, c->p.m, c->rf_part, kRefineParts, c->rf_C, RP, c->st, &c->ctl->abort);
@@ -904,11 +918,14 @@ godec_status reset_state(godec_ctx* c) {
   refresh_z(c, reinterpret_cast<double*>(reinterpret_cast<char*>(c->ctl) + offsetof(Ctl, normX2)));
   if (c->XA1) form_xa1(c);
   launch_reset_iter(c->ctl, c->st);
-  if (c->lingo || c->naive) {
-    const int d = c->lingo ? c->lg_d : c->np_cols;
-    std::vector<float> id((size_t)d * d, 0.f);
-    for (int i = 0; i < d; ++i) id[(size_t)i * d + i] = 1.f;
-    CK(cudaMemcpyAsync(c->svd_warm, id.data(), id.size() * sizeof(float), cudaMemcpyHostToDevice, c->st));
+  if (c->half || c->lingo || c->naive) {
+    const int d = c->lingo ? c->lg_d : (c->naive ? c->np_cols : 2 * c->r);
+    std::vector<double> id((size_t)d * d, 0.0);
+    for (int i = 0; i < d; ++i) {
+      if (c->half) id[(size_t)i * d + i] = 1.0;
+      else reinterpret_cast<float*>(id.data())[(size_t)i * d + i] = 1.f;
+    }
+    CK(cudaMemcpyAsync(c->svd_warm, id.data(), id.size() * sizeof(double), cudaMemcpyHostToDevice, c->st));
   }
   if (c->lingo) {
     // the features' basis Qf = orth(F) (F was copied into A1) and its split operand, fixed
@@ -992,6 +1009,12 @@ godec_status handle_abort(godec_ctx* c, const Ctl& h) {
     c->need_exact = true;
     if (c->r <= 0) return fail(c, GODEC_ERR_UNSUPPORTED, "rank test found rank 0 (X - S is zero)");
     if ((s = drop_columns(c))) return s;
+    if (c->half) {   // the correction's core shrank with the rank
+      const int d = 2 * c->r;
+      std::vector<double> id((size_t)d * d, 0.0);
+      for (int i = 0; i < d; ++i) id[(size_t)i * d + i] = 1.0;
+      CK(cudaMemcpyAsync(c->svd_warm, id.data(), id.size() * sizeof(double), cudaMemcpyHostToDevice, c->st));
+    }
   } else if (h.alarm) {
     ++c->alarms;
     // the lagged normalisers no longer condition the chain (its subspaces moved): stay on
@@ -1212,6 +1235,7 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
     want(&c->rf_U, W * W);
     want(&c->rf_V, W * W);
     want(&c->svd_warm, W * W);
+    want(&c->cmax, 1 + W);
     CKI(prepare_refine_kernels());
   }
   want(&c->A1, (size_t)n * RP);

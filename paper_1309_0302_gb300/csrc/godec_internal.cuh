@@ -396,10 +396,10 @@ cudaError_t prepare_refine_kernels();
 void launch_refine_core(const float* Ra1, const float* Ra2, const float* Rb1, const float* Rb2, int ld,
                         const double* C, int r, double* core, cudaStream_t st, const int* skip = nullptr);
 // SVD of an n x n float64 matrix (n <= 64), leading r triplets, computed in float64 or,
-// with f32, in float32 (one-sided Jacobi either way).  warm (f32 only): an n x n orthonormal
-// right basis to start from, replaced by the one found.
+// with f32, in float32 (one-sided Jacobi either way).  warm: an n x n orthonormal (float
+// with f32, else double) right basis to start from, replaced by the one found.
 void launch_svd_small(const double* A, int n, int r, double* U, float* sigma, double* V, cudaStream_t st,
-                      const int* skip = nullptr, bool f32 = false, float* warm = nullptr);
+                      const int* skip = nullptr, bool f32 = false, void* warm = nullptr);
 
 // GreBsmo (k_grebsmo.cu): the S-step's plan (one candidate pass at the key of lambda + 1
 // ulp), the soft-threshold emit S = R - lambda sgn R over every candidate, column norms

@@ -77,9 +77,10 @@ constexpr double kJacobiQuad = 1e-7;
 constexpr float kJacobiTolF = 2e-6f;
 constexpr double kJacobiQuadF = 0.0;
 
-// warm (nullable, n x n floats, in and out): an orthonormal V to start from, the one the last
+// warm (nullable, n x n, in and out): an orthonormal V to start from, the one the last
 // call of the same iteration ended with.  The core of the next iteration differs little, so
-// two or three sweeps follow where a start from I takes ten (50 x 50: 594 us cold).
+// two or three sweeps follow where a start from I takes ten (50 x 50 in float32: 594 us cold;
+// 12 x 12 in float64: 129 us cold).
 //
 // T = double, or float for the larger cores of the subspace iterations (GB300 issues a
 // warp's float64 instruction over many cycles: a float64 sweep over 58 columns costs
@@ -87,9 +88,9 @@ constexpr double kJacobiQuadF = 0.0;
 template <typename T>
 __global__ void __launch_bounds__(1024) k_svd_small(const double* __restrict__ A, int n, int r, double* __restrict__ Uo,
                                                     float* __restrict__ sigma, double* __restrict__ Vo,
-                                                    const int* skip, float* __restrict__ warm) {
+                                                    const int* skip, T* __restrict__ warm) {
   if (block_skip(skip)) return;
-  extern __shared__ double smd[];   // W, V: 2 x 64 x 65 values (dynamic)
+  extern __shared__ double smd[];   // W, V, S: 3 x 64 x 65 values (dynamic)
   T (*W)[kMaxRP + 1] = reinterpret_cast<T (*)[kMaxRP + 1]>(smd);
   T (*V)[kMaxRP + 1] = W + kMaxRP;
   __shared__ T nrm[kMaxRP];
@@ -100,7 +101,7 @@ __global__ void __launch_bounds__(1024) k_svd_small(const double* __restrict__ A
   for (int e = tid; e < n * n; e += nt) {
     const int i = e / n, j = e % n;
     W[i][j] = (T)A[e];
-    V[i][j] = warm ? (T)warm[e] : (i == j ? (T)1 : (T)0);
+    V[i][j] = warm ? warm[e] : (i == j ? (T)1 : (T)0);
   }
   if (warm) {
     // V := V (3 I - V^T V) / 2 removes what rounding cost the last call's basis, then W = A V;
@@ -212,7 +213,7 @@ __global__ void __launch_bounds__(1024) k_svd_small(const double* __restrict__ A
   }
   for (int j = tid; j < r; j += nt) sigma[j] = (float)nrm[order[j]];
   if (warm)
-    for (int e = tid; e < n * n; e += nt) warm[e] = (float)V[e / n][e % n];
+    for (int e = tid; e < n * n; e += nt) warm[e] = V[e / n][e % n];
 }
 
 }  // namespace
@@ -224,7 +225,7 @@ void launch_concat2(const float* P, const float* Q, int64_t ldp, int r, int64_t 
 }
 
 constexpr size_t kCoreSmem = 3 * kMaxRP * (kMaxRP + 1) * sizeof(double);
-constexpr size_t kSvdSmem = 2 * kMaxRP * (kMaxRP + 1) * sizeof(double);   // also three blocks of floats
+constexpr size_t kSvdSmem = 3 * kMaxRP * (kMaxRP + 1) * sizeof(double);   // W, V and the warm start's products
 
 cudaError_t prepare_refine_kernels() {
   cudaError_t e = cudaFuncSetAttribute(k_refine_core, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoreSmem);
@@ -239,9 +240,9 @@ void launch_refine_core(const float* Ra1, const float* Ra2, const float* Rb1, co
 }
 
 void launch_svd_small(const double* A, int n, int r, double* U, float* sigma, double* V, cudaStream_t st,
-                      const int* skip, bool f32, float* warm) {
-  if (f32) k_svd_small<float><<<1, 32 * ((n + 1) / 2), kSvdSmem, st>>>(A, n, r, U, sigma, V, skip, warm);
-  else k_svd_small<double><<<1, 32 * ((n + 1) / 2), kSvdSmem, st>>>(A, n, r, U, sigma, V, skip, nullptr);
+                      const int* skip, bool f32, void* warm) {
+  if (f32) k_svd_small<float><<<1, 32 * ((n + 1) / 2), kSvdSmem, st>>>(A, n, r, U, sigma, V, skip, static_cast<float*>(warm));
+  else k_svd_small<double><<<1, 32 * ((n + 1) / 2), kSvdSmem, st>>>(A, n, r, U, sigma, V, skip, static_cast<double*>(warm));
 }
 
 }  // namespace godec
