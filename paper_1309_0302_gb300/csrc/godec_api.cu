@@ -887,8 +887,8 @@ godec_status clear_counters(godec_ctx* c) {
 
 // The working copy Z = X s_Z (S = 0) with s_Z from max |X|; sumsq (nullable): += ||X||^2.
 void refresh_z(godec_ctx* c, double* sumsq) {
-  launch_zscale(c->X, c->p.m, c->p.n, c->p.ldx, &c->ctl->zmax_bits, c->ctl->zscale, c->nsm, c->st, sumsq);
-  launch_split_copy(c->X, c->p.m, c->p.n, c->p.ldx, c->Z, c->ldz, c->ctl->zscale, c->nsm, c->st);
+  launch_zscale(c->X, c->p.m, c->p.n, c->p.ldx, &c->ctl->zmax_bits, c->ctl->zscale, c->nsm_dev, c->st, sumsq);
+  launch_split_copy(c->X, c->p.m, c->p.n, c->p.ldx, c->Z, c->ldz, c->ctl->zscale, c->nsm_dev, c->st);
 }
 
 godec_status reset_state(godec_ctx* c) {
@@ -1518,6 +1518,25 @@ godec_status godec_get_L(godec_ctx* c, float* U, float* sigma, float* V, int32_t
   return GODEC_OK;
 }
 
+// The residual pass in its dump mode on the current factors: R, or L alone.
+static void dump_pass(godec_ctx* c, float* out, int64_t ldo, bool l_only) {
+  launch_lsplit(c->U, c->V, c->sigma, c->p.m, c->p.n, c->RP, c->r, c->ctl->zscale, c->LA, c->LB, c->st);
+  ResidTcLaunch rl{};
+  rl.ra.X = c->X;
+  rl.ra.m = c->p.m;
+  rl.ra.n = c->p.n;
+  rl.ra.ctl = c->ctl;
+  rl.mapX = c->tmap[5];
+  rl.mapA = c->tmap[6];
+  rl.mapB = c->tmap[7];
+  rl.zscale = c->ctl->zscale;
+  rl.dump = out;
+  rl.ldd = ldo;
+  rl.dump_l = l_only ? 1 : 0;
+  rl.nsm = c->nsm_dev;   // alone on the device, whatever the problem's budget
+  launch_resid_tc(rl, c->st);
+}
+
 godec_status godec_get_L_dense(godec_ctx* c, float* L, int64_t ldl) {
   if (!c) return GODEC_ERR_ARG;
   if (!L || ldl < c->p.n) return fail(c, GODEC_ERR_ARG, "godec_get_L_dense: L must be non-NULL with ldl >= n");
@@ -1525,7 +1544,7 @@ godec_status godec_get_L_dense(godec_ctx* c, float* L, int64_t ldl) {
   godec_status s = read_ctl(c, &h);
   if (s) return s;
   if (h.iter == 0) return fail(c, GODEC_ERR_STATE, "no iteration has run yet");
-  launch_lowrank_dense(c->U, c->RP, c->sigma, c->V, c->RP, c->p.m, c->p.n, c->r, L, ldl, c->st);
+  dump_pass(c, L, ldl, true);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(c->st));
   return GODEC_OK;
@@ -1540,20 +1559,7 @@ godec_status godec_residual(godec_ctx* c, float* R, int64_t ldr) {
   godec_status s = read_ctl(c, &h);
   if (s) return s;
   if (h.iter < 1) return fail(c, GODEC_ERR_STATE, "no iteration has run yet");
-  launch_lsplit(c->U, c->V, c->sigma, c->p.m, c->p.n, c->RP, c->r, c->ctl->zscale, c->LA, c->LB, c->st);
-  ResidTcLaunch rl{};
-  rl.ra.X = c->X;
-  rl.ra.m = c->p.m;
-  rl.ra.n = c->p.n;
-  rl.ra.ctl = c->ctl;
-  rl.mapX = c->tmap[5];
-  rl.mapA = c->tmap[6];
-  rl.mapB = c->tmap[7];
-  rl.zscale = c->ctl->zscale;
-  rl.dump = R;
-  rl.ldd = ldr;
-  rl.nsm = c->nsm;
-  launch_resid_tc(rl, c->st);
+  dump_pass(c, R, ldr, false);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(c->st));
   return GODEC_OK;

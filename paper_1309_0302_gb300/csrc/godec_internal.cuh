@@ -300,6 +300,7 @@ struct ResidTcLaunch {
   const void* mapB;        // over B (n x 128 halves), box 64 x 64
   const float* zscale;     // {s_Z, 1/s_Z}
   float* dump;             // non-null: write R densely (row stride ldd) instead of selecting
+  int dump_l;              // ... or L alone
   int64_t ldd;
   int nsm;
 };
@@ -443,10 +444,6 @@ void launch_mse_init(const float* X, int64_t ldx, const float* invD, int64_t row
                      int nsm, cudaStream_t st);
 void launch_sub(const float* X, int64_t ldx, const float* R, int64_t ldr, int64_t rows, int64_t p, float* out,
                 int64_t ldo, int nsm, cudaStream_t st);
-
-// L (m x n, row stride ldl) = U diag(sigma) V^T, U m x r (ldu), V n x r (ldv) (k_dense.cu).
-void launch_lowrank_dense(const float* U, int64_t ldu, const float* sigma, const float* V, int64_t ldv, int64_t m,
-                          int64_t n, int r, float* L, int64_t ldl, cudaStream_t st);
 
 // Small helpers.
 void launch_fill_zero(void* p, size_t bytes, cudaStream_t st);

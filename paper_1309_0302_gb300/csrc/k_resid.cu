@@ -4,18 +4,20 @@
 //   A = U diag(sqrt(sigma s_Z)),  B = V diag(sqrt(sigma s_Z))
 //
 // A and B (m x RP, n x RP) are split once per iteration into two float16 terms each
-// (x = h + 2^-11 l, h cut to 11 significant bits, l rounded), stored as rows of 128
+// (x = h + 2^-11 l, both rounded to nearest), stored as rows of 128
 // halves: 64 of h (K zero-padded to 64) then 64 of l.  Per 128 x 64 tile of R:
 //   D[:, 0:128]  = A_h [B_h; B_l]^T      (N = 128, K = 64)
 //   D[:, 64:128] += A_l B_h^T           (N = 64)
 // so L = (D[:, :64] + 2^-11 D[:, 64:]) / s_Z to float32 accuracy (the dropped A_l B_l
-// term is 2^-22 relative).  s_Z, the scale of the working copy of X - S, bounds
+// term is 2^-24 relative).  s_Z, the scale of the working copy of X - S, bounds
 // sigma s_Z and keeps A and B inside the float16 range.
 //
 // The epilogue forms R from the accumulator and the X tile (TMA-staged), and does
 // what k_residual does: a 4096-bin histogram of the top key bits (full mode) or the
 // candidates with key >= guess (candidate mode), the float64 sums of R^2, and the
-// non-finite check.  A dump mode writes R densely (testing).  Candidates are staged
+// non-finite check.  A dump mode writes R densely, or L alone (godec_get_L_dense: bound by
+// the 4 m n bytes written; 10^4 x 10^4, r = 50: 562 us before as float32 fmas on the CUDA
+// cores).  Candidates are staged
 // per warp in shared memory (the histogram's space) and written out with one global
 // atomic per full buffer, so no tile waits on a contended atomic.
 //
@@ -73,6 +75,7 @@ struct RTArgs {
   unsigned long long cand_cap;
   const float* zscale;      // zscale[1] = 1 / s_Z
   float* dump;              // dump mode when non-null: R into dump (row stride ldd)
+  int dump_l;               // dump mode writes L = X - R instead (X is not read)
   int64_t ldd;
 };
 
@@ -173,7 +176,7 @@ k_resid_tc(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUt
       uint32_t phx = 0;
       int64_t nx = 0;
       const uint64_t pol = policy_evict_first();
-      for (int64_t g = g0; g < g1 && !s_err; ++g) {
+      for (int64_t g = a.dump_l ? g1 : g0; g < g1 && !s_err; ++g) {
         if (!mbar_wait(&xempty[sx], phx ^ 1u, kRWait)) { rtimeout(ctl, &s_err); break; }
         // both boxes always: columns past n (and rows past m) are zero-filled, and so are
         // the rows of A and B past m and n, which makes R exactly 0 there
@@ -266,6 +269,7 @@ k_resid_tc(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUt
     const int f4b = (cq & 1) * 4;           // this quarter's first float4 in its 128-byte box row
     const uint32_t tlane = (uint32_t)(q4 * 32) << 16;
     const float zinv = a.zscale[1], zlo = zinv * kLoInv;
+    const bool vec4 = a.dump && (a.ldd & 3) == 0 && (reinterpret_cast<uintptr_t>(a.dump) & 15) == 0;
     // candidate iff key >= max(guess, 1); for a non-NaN value that is |R| >= gf (a NaN
     // fails the compare, lands in the sum and is caught there)
     const float gf = __uint_as_float(guess > 1u ? guess : 1u);
@@ -300,7 +304,7 @@ k_resid_tc(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUt
     for (int64_t g = g0; g < g1; ++g) {
       if (__any_sync(0xffffffffu, s_err != 0)) break;
       const int b = ai % kAcc;
-      if (!wwait(&accfull[b], (uint32_t)((ai / kAcc) & 1), lane) || !wwait(&xfull[sx], phx, lane)) {
+      if (!wwait(&accfull[b], (uint32_t)((ai / kAcc) & 1), lane) || (!a.dump_l && !wwait(&xfull[sx], phx, lane))) {
         if (lane == 0) rtimeout(ctl, &s_err);
         break;
       }
@@ -395,6 +399,23 @@ k_resid_tc(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUt
             if (key) atomicAdd(&hist[key >> kD1Shift], 1u);
           }
         }
+      } else if (a.dump_l) {   // L: a thread writes 64 contiguous bytes of its row
+        const int64_t i = ib * RM + row, j0 = jb * RNC + cq * kECols;
+        float* d = a.dump + i * a.ldd + j0;
+        float l[kECols];
+#pragma unroll
+        for (int q = 0; q < kECols; ++q) l[q] = fmaf(vl[q], zlo, vh[q] * zinv);
+        if (i < m) {
+          if (vec4 && j0 + kECols <= n) {
+#pragma unroll
+            for (int u = 0; u < kECols / 4; ++u)
+              *reinterpret_cast<float4*>(d + 4 * u) = make_float4(l[4 * u], l[4 * u + 1], l[4 * u + 2], l[4 * u + 3]);
+          } else {
+#pragma unroll
+            for (int q = 0; q < kECols; ++q)
+              if (j0 + q < n) d[q] = l[q];
+          }
+        }
       } else {   // dump
         const int64_t i = ib * RM + row, j0 = jb * RNC + cq * kECols;
 #pragma unroll
@@ -468,7 +489,7 @@ __global__ void k_lsplit(const float* __restrict__ U, const float* __restrict__ 
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       v[e] = (l + e < r) ? src[l + e] * sq[l + e] : 0.f;
-      h[e] = __uint_as_float(__float_as_uint(v[e]) & 0xFFFFE000u);
+      h[e] = __half2float(__float2half_rn(v[e]));
       lo[e] = (v[e] - h[e]) * 2048.f;
     }
     dst[lane] = __floats2half2_rn(h[0], h[1]);
@@ -504,6 +525,7 @@ void launch_resid_tc(const ResidTcLaunch& l, cudaStream_t st) {
   a.cand_cap = l.ra.cand_cap;
   a.zscale = l.zscale;
   a.dump = l.dump;
+  a.dump_l = l.dump_l;
   a.ldd = l.ldd;
   const int64_t T = ((a.m + RM - 1) / RM) * ((a.n + RNC - 1) / RNC);
   const int G = (int)(T < l.nsm ? T : l.nsm);
