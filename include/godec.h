@@ -248,6 +248,15 @@ godec_status godec_mul_ZtC(const float* Z, int64_t m, int64_t n, int64_t ldz,
                            const float* C, int32_t r, float* W, void* stream);
 
 /*
+ * Copy an m x n float32 matrix to another row stride: src (device, any row stride lds >= n)
+ * to dst (device, 16-byte aligned, ldd >= n, ldd*4 a multiple of 16 bytes; columns n .. ldd-1
+ * are left as they are).  What a caller whose rows are not 16-byte aligned does before the
+ * calls that need it.  Does not synchronise.
+ */
+godec_status godec_copy_rows(const float* src, int64_t m, int64_t n, int64_t lds, float* dst, int64_t ldd,
+                             void* stream);
+
+/*
  * Kernel-level timing: run n_iter real iterations (they advance the state like
  * godec_iterate) launching each kernel directly on the context stream with a
  * CUDA event before and after it, and accumulate per kernel class:

@@ -74,6 +74,7 @@ def _declare(lib):
         "godec_check_timeout": ([_P, C.c_uint32], C.c_int),
         "godec_hard_threshold": ([_P, C.c_int64, C.c_int64, C.c_int64, C.c_int64, _P, _P, C.c_int64, i64p, _P],
                                  C.c_int),
+        "godec_copy_rows": ([_P, C.c_int64, C.c_int64, C.c_int64, _P, C.c_int64, _P], C.c_int),
         "godec_mul_ZB": ([_P, C.c_int64, C.c_int64, C.c_int64, _P, C.c_int32, _P, _P], C.c_int),
         "godec_backward": ([_P, C.c_int64, C.c_int64, C.c_int64, _P, C.c_int32, C.c_int32, C.POINTER(_P), i64p,
                             _P, _P, C.c_int32, _P, C.c_int64, _P, C.c_int64, C.c_int32, _P], C.c_int),
@@ -146,6 +147,21 @@ def _stream_ptr(stream):
     return C.c_void_p(s.cuda_stream)
 
 
+def _pitched(A):
+    """A copy of a 2-D CUDA float32 tensor whose row stride is a multiple of 4 elements."""
+    torch = _torch()
+    m, n = A.shape
+    Ap = torch.empty((m, (n + 3) // 4 * 4), dtype=torch.float32, device=A.device)
+    if (A.dtype != torch.float32 or not A.is_cuda or A.stride(1) != 1 or A.stride(0) < n or m < 1 or n < 1 or
+            A.device.index != torch.cuda.current_device()):
+        Ap[:, :n] = A
+    else:
+        # on the current stream, as the allocation and the tensor's own work
+        _check(library().godec_copy_rows(_ptr(A), m, n, A.stride(0), _ptr(Ap), Ap.stride(0), _stream_ptr(None)),
+               "godec_copy_rows")
+    return Ap
+
+
 def _ptr(t):
     return C.c_void_p(t.data_ptr()) if t is not None else None
 
@@ -166,9 +182,7 @@ class GoDec:
             raise ValueError("X must be a 2-D CUDA float32 tensor")
         m, n = X.shape
         if X.stride(1) != 1 or X.stride(0) % 4 or X.stride(0) < n or X.data_ptr() % 16:
-            Xp = torch.zeros((m, (n + 3) // 4 * 4), dtype=torch.float32, device=X.device)
-            Xp[:, :n] = X
-            X = Xp
+            X = _pitched(X)
         self._X = X
         self._A1 = A1.contiguous().to(torch.float32)
         self.m, self.n, self.r, self.k, self.q = m, n, int(r), int(k), int(q)
@@ -295,9 +309,7 @@ class NaiveGoDec(GoDec):
             raise ValueError("X must be a 2-D CUDA float32 tensor")
         m, n = X.shape
         if X.stride(1) != 1 or X.stride(0) % 4 or X.stride(0) < n or X.data_ptr() % 16:
-            Xp = torch.zeros((m, (n + 3) // 4 * 4), dtype=torch.float32, device=X.device)
-            Xp[:, :n] = X
-            X = Xp
+            X = _pitched(X)
         p_cols = naive_columns(m, n, r)
         if tuple(omega.shape) != (n, p_cols):
             raise ValueError(f"omega must be ({n}, {p_cols})")
@@ -325,9 +337,7 @@ class LinGoDec(GoDec):
             raise ValueError("X must be a 2-D CUDA float32 tensor")
         m, n = X.shape
         if X.stride(1) != 1 or X.stride(0) % 4 or X.stride(0) < n or X.data_ptr() % 16:
-            Xp = torch.zeros((m, (n + 3) // 4 * 4), dtype=torch.float32, device=X.device)
-            Xp[:, :n] = X
-            X = Xp
+            X = _pitched(X)
         if F.dim() != 2 or F.shape[0] != n:
             raise ValueError("F must be (n, d)")
         self._X = X
@@ -376,9 +386,7 @@ class GreBsmo(GoDec):
             raise ValueError("X must be a 2-D CUDA float32 tensor")
         m, n = X.shape
         if X.stride(1) != 1 or X.stride(0) % 4 or X.stride(0) < n or X.data_ptr() % 16:
-            Xp = torch.zeros((m, (n + 3) // 4 * 4), dtype=torch.float32, device=X.device)
-            Xp[:, :n] = X
-            X = Xp
+            X = _pitched(X)
         p_cols = int(dr) + int(oversample)
         if omegas.dim() != 3 or omegas.shape[1] != n or omegas.shape[2] != p_cols:
             raise ValueError("omegas must be (stages, n, dr + oversample)")
@@ -426,9 +434,7 @@ def mse_train(X, labels, ranks, K: int, iters: int, A1s, stream=None):
         raise ValueError("X must be a 2-D CUDA float32 tensor")
     n, p = X.shape
     if X.stride(1) != 1 or X.stride(0) % 4 or X.stride(0) < p or X.data_ptr() % 16:
-        Xp = torch.zeros((n, (p + 3) // 4 * 4), dtype=torch.float32, device=X.device)
-        Xp[:, :p] = X
-        X = Xp
+        X = _pitched(X)
     lab = np.ascontiguousarray(np.asarray(labels) != 0, dtype=np.int32)
     k = lab.shape[1]
     rk = np.ascontiguousarray(ranks, dtype=np.int32)
@@ -455,9 +461,7 @@ def _mul(name, Z, B, stream=None):
         raise ValueError("Z and B must be CUDA float32")
     m, n = Z.shape
     if Z.stride(1) != 1 or Z.stride(0) % 4 or Z.data_ptr() % 16:
-        Zp = torch.zeros((m, (n + 3) // 4 * 4), dtype=torch.float32, device=Z.device)
-        Zp[:, :n] = Z
-        Z = Zp
+        Z = _pitched(Z)
     B = B.contiguous()
     r = B.shape[1]
     out = torch.empty(((n if name == "godec_mul_ZtC" else m), r), dtype=torch.float32, device=Z.device)
@@ -474,9 +478,7 @@ def hard_threshold(R, k: int, stream=None):
     torch = _torch()
     m, n = R.shape
     if R.stride(1) != 1 or R.stride(0) % 4 or R.data_ptr() % 16:
-        Rp = torch.zeros((m, (n + 3) // 4 * 4), dtype=torch.float32, device=R.device)
-        Rp[:, :n] = R
-        R = Rp
+        R = _pitched(R)
     cap = max(1, min(int(k), m * n))
     idx = torch.empty((cap,), dtype=torch.int64, device=R.device)
     val = torch.empty((cap,), dtype=torch.float32, device=R.device)
@@ -539,9 +541,7 @@ def _pad_rows(A):
     torch = _torch()
     m, n = A.shape
     if A.stride(1) != 1 or A.stride(0) % 4 or A.data_ptr() % 16:
-        Ap = torch.zeros((m, (n + 3) // 4 * 4), dtype=torch.float32, device=A.device)
-        Ap[:, :n] = A
-        return Ap
+        return _pitched(A)
     return A
 
 
@@ -589,9 +589,7 @@ def _padded(X):
         raise ValueError("X must be a 2-D CUDA float32 tensor")
     m, n = X.shape
     if X.stride(1) != 1 or X.stride(0) % 4 or X.stride(0) < n or X.data_ptr() % 16:
-        Xp = torch.zeros((m, (n + 3) // 4 * 4), dtype=torch.float32, device=X.device)
-        Xp[:, :n] = X
-        return Xp
+        return _pitched(X)
     return X
 
 

@@ -1823,6 +1823,23 @@ static godec_status mul_common(const float* Z, int64_t m, int64_t n, int64_t ldz
   return GODEC_OK;
 }
 
+godec_status godec_copy_rows(const float* src, int64_t m, int64_t n, int64_t lds, float* dst, int64_t ldd, void* stream) {
+  int dev = 0, nsm = 0;
+  if (!src || !dst || m < 1 || n < 1 || lds < n || ldd < n || (ldd * 4) % 16 || (reinterpret_cast<uintptr_t>(dst) & 15)) {
+    snprintf(g_static_err, sizeof(g_static_err), "godec_copy_rows: invalid argument");
+    return GODEC_ERR_ARG;
+  }
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    snprintf(g_static_err, sizeof(g_static_err), "godec_copy_rows: no CUDA device");
+    return GODEC_ERR_CUDA;
+  }
+  launch_copy_rows(src, m, n, lds, dst, ldd, nsm, reinterpret_cast<cudaStream_t>(stream));
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) return GODEC_OK;
+  snprintf(g_static_err, sizeof(g_static_err), "godec_copy_rows: %s", cudaGetErrorString(e));
+  return GODEC_ERR_CUDA;
+}
+
 godec_status godec_mul_ZB(const float* Z, int64_t m, int64_t n, int64_t ldz, const float* B, int32_t r,
                           float* Y, void* stream) {
   return mul_common(Z, m, n, ldz, B, r, Y, stream, 0);

@@ -451,6 +451,8 @@ void launch_fill_zero(void* p, size_t bytes, cudaStream_t st);
 // dst = src^T, optionally times scale[0]
 void launch_transpose(const float* src, int64_t m, int64_t n, int64_t lds, float* dst, int64_t ldd,
                       cudaStream_t st, const float* scale = nullptr);
+void launch_copy_rows(const float* src, int64_t m, int64_t n, int64_t lds, float* dst, int64_t ldd, int nsm,
+                      cudaStream_t st);
 void launch_pad_copy(const float* src, int64_t rows, int cols, int64_t lds, float* dst, int RP,
                      cudaStream_t st);
 void launch_unpad_copy(const float* src, int64_t rows, int RP, float* dst, int cols,

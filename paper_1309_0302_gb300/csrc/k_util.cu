@@ -30,6 +30,26 @@ __global__ void k_transpose(const float* __restrict__ src, int64_t m, int64_t n,
   }
 }
 
+// dst (row stride ldd, 16-byte aligned rows) = src (row stride lds): four columns per thread,
+// scalar loads (rows of src start anywhere; neighbouring lanes share their sectors), one
+// 16-byte store.  Bound: 8 m n bytes (20011 x 3003: 90 us against 185 us as a zero fill and a
+// strided copy).
+__global__ void __launch_bounds__(256)
+k_copy_rows(const float* __restrict__ src, int64_t m, int64_t n, int64_t lds, float* __restrict__ dst, int64_t ldd) {
+  const int64_t per = (n + 3) / 4, total = m * per;
+  for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < total; e += (int64_t)gridDim.x * 256) {
+    const int64_t i = e / per, j = (e - i * per) * 4;
+    const float* s = src + i * lds + j;
+    float* d = dst + i * ldd + j;
+    if (j + 4 <= n) {
+      const float a = s[0], b = s[1], c = s[2], f = s[3];
+      *reinterpret_cast<float4*>(d) = make_float4(a, b, c, f);
+    } else {
+      for (int u = 0; j + u < n; ++u) d[u] = s[u];
+    }
+  }
+}
+
 __global__ void k_pad_copy(const float* src, int64_t rows, int cols, int64_t lds, float* dst, int RP) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < rows * RP;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -143,6 +163,13 @@ void launch_transpose(const float* src, int64_t m, int64_t n, int64_t lds, float
                       cudaStream_t st, const float* scale) {
   dim3 grid((unsigned)((n + 31) / 32), (unsigned)((m + 31) / 32));
   k_transpose<<<grid, dim3(32, 8), 0, st>>>(src, m, n, lds, dst, ldd, scale);
+}
+
+void launch_copy_rows(const float* src, int64_t m, int64_t n, int64_t lds, float* dst, int64_t ldd, int nsm,
+                      cudaStream_t st) {
+  int64_t grid = (m * ((n + 3) / 4) + 255) / 256;
+  if (grid > 32LL * nsm) grid = 32LL * nsm;
+  k_copy_rows<<<(unsigned)grid, 256, 0, st>>>(src, m, n, lds, dst, ldd);
 }
 
 void launch_pad_copy(const float* src, int64_t rows, int cols, int64_t lds, float* dst, int RP,
