@@ -84,6 +84,7 @@ struct godec_ctx {
   cudaStream_t side_st = nullptr;   // off-critical-path work of the power chain
   cudaStream_t rank_st = nullptr;   // the rank test, joined before the S-step commits
   bool rank_forked = false;
+  bool chain_only = false;          // capturing for a batch: every iteration is exact, no slot is read later
   cudaEvent_t ev[kEvents] = {};
   int ev_used = 0;
   int dev = 0, nsm = 0;   // nsm: the SMs this problem's grids are sized for (its budget)
@@ -388,6 +389,10 @@ void final_cqr2(godec_ctx* c, int64_t rows, const double* g1, float* Ra, float* 
 }
 
 void slot(godec_ctx* c, SlotLaunch& sl) {
+  // a batch's iterations never take the fast path: only the core's factor is needed (64 uneven
+  // problems, q = 1: six of nine slot updates of every iteration are not launched)
+  if (c->chain_only && sl.pi_mode == 0) return;
+  sl.pi_only = c->chain_only;
   sl.g32 = g32_of(c, sl.g64);
   sl.r = c->r;
   sl.RP = c->RP;
@@ -891,7 +896,7 @@ void refresh_z(godec_ctx* c, double* sumsq) {
   launch_split_copy(c->X, c->p.m, c->p.n, c->p.ldx, c->Z, c->ldz, c->ctl->zscale, c->nsm_dev, c->st);
 }
 
-godec_status reset_state(godec_ctx* c) {
+godec_status reset_state(godec_ctx* c, bool sync = true) {
   c->r = c->p.r;   // captured graphs stay: buffers and geometry are the same, and graph_r tells a rank drop
   c->fast_run = 0;
   c->rank_drops = 0;
@@ -960,7 +965,7 @@ godec_status reset_state(godec_ctx* c) {
     }
   }
   CK(cudaGetLastError());
-  CK(cudaStreamSynchronize(c->st));
+  if (sync) CK(cudaStreamSynchronize(c->st));
   return GODEC_OK;
 }
 
@@ -2514,7 +2519,9 @@ godec_status build_batch_graph(godec_batch* b) {
     c->st = c->cap_st;
     e = cudaStreamWaitEvent(c->st, b->fork, 0);
     if (e == cudaSuccess) {
+      c->chain_only = true;
       enqueue_iteration(c, false);
+      c->chain_only = false;
       e = cudaEventRecord(b->join[i], c->st);
     }
     if (e == cudaSuccess) e = cudaStreamWaitEvent(b->cap_st, b->join[i], 0);
@@ -2552,9 +2559,11 @@ godec_status read_all(godec_batch* b) {
 
 godec_status batch_reset(godec_batch* b) {
   for (size_t i = 0; i < b->ctx.size(); ++i) {
-    godec_status s = reset_state(b->ctx[i]);
+    godec_status s = reset_state(b->ctx[i], false);
     if (s) return bfail(b, s, "problem %zu: %s", i, b->ctx[i]->err);
   }
+  if (cudaStreamSynchronize(b->st) != cudaSuccess)
+    return bfail(b, GODEC_ERR_CUDA, "batch reset: %s", cudaGetErrorString(cudaGetLastError()));
   return GODEC_OK;
 }
 
@@ -2576,6 +2585,10 @@ godec_status batch_iterate(godec_batch* b, int n_iter) {
     rebuild = rebuild || b->graph_r[i] != b->ctx[i]->r || b->graph_epoch[i] != b->ctx[i]->graph_epoch;
   }
   if (rebuild && (s = build_batch_graph(b))) return s;
+  for (godec_ctx* c : b->ctx) {   // the batch graph forms no lagged normalisers
+    c->need_exact = true;
+    c->fast_run = 0;
+  }
   for (int t = 0; t < n_iter; ++t)
     if (cudaGraphLaunch(b->gexec, b->st) != cudaSuccess) return bfail(b, GODEC_ERR_CUDA, "batch graph launch failed");
   if ((s = read_all(b))) return s;

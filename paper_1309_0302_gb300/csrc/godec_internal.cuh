@@ -259,6 +259,7 @@ struct SlotLaunch {
   float* T_next[2] = {nullptr, nullptr};
   float* Pi = nullptr;
   int pi_mode = 0;
+  int pi_only = 0;           // the core's factor Pi alone: no normaliser for the next iteration
   int fast = 0;
   int r = 0, RP = 0;
   float alarm_ratio = 30.f;

@@ -605,6 +605,7 @@ struct SlotArgs {
   float* R_next[2];        // written at index 1 - parity
   float* T_next[2];
   float* Pi;               // RP x RP, nullable
+  int pi_only;             // no normaliser for the next iteration is formed
   int pi_mode;             // 0 none, 1 Pi := R_app Pi, 2 Pi := R_app
   int fast;                // compute chol(Gram of Q~)
   int r, RP;
@@ -683,9 +684,11 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_slot(SlotArgs a) {
     for (int e = threadIdx.x; e < kMaxRP * kMaxRP; e += SMALL_THREADS) A[e / kMaxRP][e % kMaxRP] = B[e / kMaxRP][e % kMaxRP];
     __syncthreads();
   }
-  store_mat(a.R_next[nxt], A, RP);
-  tri_inverse(A, C, RP, nullptr);
-  store_mat(a.T_next[nxt], C, RP);
+  if (!a.pi_only) {
+    store_mat(a.R_next[nxt], A, RP);
+    tri_inverse(A, C, RP, nullptr);
+    store_mat(a.T_next[nxt], C, RP);
+  }
   if (a.pi_mode == 2) {
     normalise_into(B, a.Pi, RP, ctl, true);
   } else if (a.pi_mode == 1) {
@@ -1112,6 +1115,7 @@ void launch_slot(const SlotLaunch& l, cudaStream_t st) {
   a.L2 = l.L2;
   a.Pi = l.Pi;
   a.pi_mode = l.pi_mode;
+  a.pi_only = l.pi_only;
   a.fast = l.fast;
   a.r = l.r;
   a.RP = l.RP;
