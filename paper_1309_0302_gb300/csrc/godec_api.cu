@@ -686,6 +686,7 @@ void enqueue_sstep(godec_ctx* c, int r) {
   ra.cand_idx = c->cand_idx;
   ra.cand_val = c->cand_val;
   ra.cand_cap = c->cap;
+  ra.k = c->p.k;
   for (int pass = 0; pass < 3; ++pass) {
     ra.pass = pass;
     ResidTcLaunch rl{};
@@ -696,7 +697,6 @@ void enqueue_sstep(godec_ctx* c, int r) {
     rl.zscale = c->ctl->zscale;
     rl.nsm = c->nsm;
     PROF(c, 7, st, launch_resid_tc(rl, st));
-    PROF(c, 8, st, launch_after_pass(c->ctl, pass, c->p.k, c->cap, st));
   }
   SelectArgs se{};
   se.ctl = c->ctl;
@@ -706,10 +706,7 @@ void enqueue_sstep(godec_ctx* c, int r) {
   se.cand_cap = c->cap;
   se.k = c->p.k;
   se.idx_bits = c->idx_bits;
-  for (int round = 0; round < 7; ++round) {
-    se.round = round;
-    PROF(c, 8, st, launch_select_round(se, c->nsm, st));
-  }
+  PROF(c, 8, st, launch_select(se, c->nsm, st));
   EmitArgs ea = z_args(c);
   ea.cand_key = c->cand_key;
   ea.cand_idx = c->cand_idx;
@@ -1719,14 +1716,10 @@ godec_status godec_hard_threshold(const float* R, int64_t m, int64_t n, int64_t 
     ra.cand_idx = cidx;
     ra.cand_val = cval;
     ra.cand_cap = cap0;
-    for (ra.pass = 0; ra.pass < 2; ++ra.pass) {   // histogram, then the candidates above its bin
+    ra.k = k;
+    for (ra.pass = 0; ra.pass < 2; ++ra.pass)   // histogram, then the candidates above its bin
       launch_thresh_pass(ra, nsm, st);
-      launch_after_pass(se.ctl, ra.pass, k, cap0, st);
-    }
-    for (int round = 0; round < 7; ++round) {
-      se.round = round;
-      launch_select_round(se, nsm, st);
-    }
+    launch_select(se, nsm, st);
     launch_mark(se, bits, nsm, st);
     launch_order(bits, words, order, reinterpret_cast<long long*>(idx), val, (idx && val) ? cap : 0, R, n, ldr, nullptr,
                  nullptr, 0, total, st);

@@ -286,6 +286,7 @@ struct ResidualArgs {
   long long* cand_idx;
   float* cand_val;
   unsigned long long cand_cap;
+  long long k = -1;        // select the k largest (-1: the pass alone)
 };
 void launch_thresh_pass(const ResidualArgs& a, int nsm, cudaStream_t st);   // R = X (no low-rank part)
 
@@ -307,7 +308,6 @@ struct ResidTcLaunch {
 };
 void launch_resid_tc(const ResidTcLaunch& l, cudaStream_t st);
 cudaError_t prepare_resid_kernels();
-void launch_after_pass(Ctl* ctl, int pass, long long k, unsigned long long cap, cudaStream_t st);
 
 struct SelectArgs {
   Ctl* ctl;
@@ -319,7 +319,8 @@ struct SelectArgs {
   int round;
   int idx_bits;            // bits needed for linear indices (<= 42)
 };
-void launch_select_round(const SelectArgs& a, int nsm, cudaStream_t st);
+// All rounds, each launched where it can have something to do.
+void launch_select(SelectArgs a, int nsm, cudaStream_t st);
 // The selected candidates' bits set in a clear bitmap of m n bits.
 void launch_mark(const SelectArgs& a, unsigned* bits, int nsm, cudaStream_t st);
 // Indices (ascending, below cap) of a bitmap's set bits, and their values: from R (row stride

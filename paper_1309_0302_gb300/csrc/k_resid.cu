@@ -34,6 +34,7 @@
 #include <cuda_fp16.h>
 
 #include "godec_internal.cuh"
+#include "select_util.cuh"
 #include "tc_util.cuh"
 
 namespace godec {
@@ -73,6 +74,7 @@ struct RTArgs {
   long long* cand_idx;
   float* cand_val;
   unsigned long long cand_cap;
+  long long k;              // selecting for the k largest (-1: the caller ends the pass itself)
   const float* zscale;      // zscale[1] = 1 / s_Z
   float* dump;              // dump mode when non-null: R into dump (row stride ldd)
   int dump_l;               // dump mode writes L = X - R instead (X is not read)
@@ -462,6 +464,7 @@ k_resid_tc(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUt
     tc_fence_after();
     tmem_dealloc(tbase, 128 * kAcc);
   }
+  if (mode != PASS_DUMP && a.k >= 0) after_pass<kRThreads>(ctl, a.pass, mode, a.k, a.cand_cap);
 }
 
 // Rows of A (i < m) and B (i >= m): 64 halves of h (K padded to 64), then 64 of l.
@@ -523,6 +526,7 @@ void launch_resid_tc(const ResidTcLaunch& l, cudaStream_t st) {
   a.cand_idx = l.ra.cand_idx;
   a.cand_val = l.ra.cand_val;
   a.cand_cap = l.ra.cand_cap;
+  a.k = l.ra.k;
   a.zscale = l.zscale;
   a.dump = l.dump;
   a.dump_l = l.dump_l;

@@ -13,6 +13,7 @@
 #include <cuda_fp16.h>
 
 #include "godec_internal.cuh"
+#include "select_util.cuh"
 
 namespace godec {
 
@@ -38,34 +39,6 @@ __device__ __forceinline__ void split_idx(long long idx, long long n, float ninv
   }
   i = q;
   j = r;
-}
-
-// Block-wide exclusive scan of one unsigned per thread (any blockDim multiple of 32).
-__device__ unsigned block_excl_scan(unsigned v, unsigned* total) {
-  __shared__ unsigned wsum[32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  unsigned x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    unsigned y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  __syncthreads();
-  if (lane == 31) wsum[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    unsigned w = lane < nw ? wsum[lane] : 0u;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      unsigned y = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += y;
-    }
-    if (lane < nw) wsum[lane] = w;
-  }
-  __syncthreads();
-  unsigned before = warp ? wsum[warp - 1] : 0u;
-  *total = wsum[nw - 1];
-  return before + x - v;
 }
 
 __device__ double block_sum_double(double v) {
@@ -94,7 +67,7 @@ constexpr int TH_THREADS = 512, TH_STAGE = 2048;
 __global__ void __launch_bounds__(TH_THREADS)
 k_thresh_pass(const float* __restrict__ R, int64_t m, int64_t n, int64_t ldr, int pass, Ctl* ctl,
               unsigned* __restrict__ cand_key, long long* __restrict__ cand_idx, float* __restrict__ cand_val,
-              unsigned long long cand_cap) {
+              unsigned long long cand_cap, long long k) {
   if (ctl->abort) return;
   const int mode = ctl->plan[pass];
   if (mode == PASS_NONE) return;
@@ -200,6 +173,7 @@ k_thresh_pass(const float* __restrict__ R, int64_t m, int64_t n, int64_t ldr, in
       }
   }
   if (bad) ctl->nonfinite = 1;
+  after_pass<TH_THREADS>(ctl, pass, mode, k, cand_cap);
 }
 
 // Bits of the selected candidates (bitmap of m n bits, clear before).
@@ -321,115 +295,11 @@ k_val_order(const long long* __restrict__ idx, const float* __restrict__ v, long
 }
 
 // --------------------------------------------------------------------------------------
-// Pass control (one block of 1024 threads): decide what the next residual pass does.
-// --------------------------------------------------------------------------------------
-constexpr int CTL_THREADS = 1024;
-
-// Find the bin holding the `need`-th largest (from_top) or smallest (!from_top) element of a
-// histogram of `nb` bins (nb <= 4096).  Returns the bin; *above = elements strictly before it
-// in that order, *in_bin = its count.  All threads get the result.
-__device__ int block_find_bin(const unsigned* h, int nb, unsigned long long need, bool from_top,
-                              unsigned long long* before, unsigned* in_bin,
-                              unsigned long long* total_out) {
-  __shared__ int s_bin;
-  __shared__ unsigned long long s_before;
-  __shared__ unsigned s_in;
-  __shared__ unsigned long long s_total;
-  const int per = (nb + CTL_THREADS - 1) / CTL_THREADS;   // bins per thread (<= 4)
-  const int t = threadIdx.x;
-  // thread t owns ordered positions [t*per, t*per+per); position o maps to bin
-  // from_top ? nb-1-o : o
-  unsigned loc = 0;
-  for (int o = t * per; o < min(nb, t * per + per); ++o) loc += h[from_top ? nb - 1 - o : o];
-  unsigned tot32;
-  unsigned excl = block_excl_scan(loc, &tot32);
-  if (t == 0) { s_bin = -1; s_total = tot32; }
-  __syncthreads();
-  unsigned long long run = excl;
-  for (int o = t * per; o < min(nb, t * per + per); ++o) {
-    int b = from_top ? nb - 1 - o : o;
-    unsigned c = h[b];
-    if (run < need && run + c >= need) {
-      s_bin = b;
-      s_before = run;
-      s_in = c;
-    }
-    run += c;
-  }
-  __syncthreads();
-  *before = s_before;
-  *in_bin = s_in;
-  *total_out = s_total;
-  return s_bin;
-}
-
-__global__ void __launch_bounds__(CTL_THREADS)
-k_after_pass(Ctl* ctl, int pass, long long k, unsigned long long cap) {
-  if (ctl->abort) return;
-  const int mode = ctl->plan[pass];
-  if (mode == PASS_NONE || ctl->ready) return;
-  const int t = threadIdx.x;
-  if (mode == PASS_FULL) {
-    unsigned long long before, total;
-    unsigned in_bin;
-    // total count first (need = 1 finds the top non-empty bin; we only want the total)
-    block_find_bin(ctl->hist, kHistBins, 1ull, true, &before, &in_bin, &total);
-    long long keff = (long long)((unsigned long long)k < total ? (unsigned long long)k : total);
-    int bin = -1;
-    if (keff > 0) bin = block_find_bin(ctl->hist, kHistBins, (unsigned long long)keff, true,
-                                       &before, &in_bin, &total);
-    __syncthreads();
-    for (int b = t; b < kHistBins; b += CTL_THREADS) ctl->hist[b] = 0u;
-    if (t == 0) {
-      ctl->k_eff = keff;
-      if (ctl->nonfinite) {
-        ctl->abort = 1;
-      } else if (keff == 0) {
-        ctl->ready = 1;
-        ctl->need = 0;
-        ctl->cand_count = 0;
-        ctl->sumsq_noncand = ctl->sumsq_full;
-      } else {
-        unsigned long long ge = before + in_bin;   // keys in bins >= bin
-        if (ge > cap) {
-          ctl->need_bigger_cand = 1;
-          ctl->abort = 1;
-        } else if (pass < 2) {
-          ctl->plan[pass + 1] = PASS_CAND;
-          unsigned g = (unsigned)bin << kD1Shift;
-          ctl->guess[pass + 1] = g ? g : 1u;
-          ctl->cand_count = 0;
-          ctl->sumsq_noncand = 0.0;
-        } else {
-          ctl->abort = 1;                          // cannot happen: FULL is never last
-        }
-      }
-    }
-  } else if (t == 0) {   // PASS_CAND
-    unsigned long long cc = ctl->cand_count;
-    if (ctl->nonfinite) {
-      ctl->abort = 1;
-    } else if (cc <= cap && (long long)cc >= ctl->k_eff) {
-      ctl->ready = 1;
-      ctl->need = ctl->k_eff;
-    } else if (pass < 2) {
-      ctl->plan[pass + 1] = PASS_FULL;
-      ctl->cand_count = 0;
-      ctl->sumsq_full = 0.0;
-    } else {
-      ctl->need_bigger_cand = 1;
-      ctl->abort = 1;
-    }
-  }
-  if (t == 0) ctl->passes_run = pass + 1;
-}
-
-// --------------------------------------------------------------------------------------
 // Radix select rounds over the candidates.  Round 0..2: key digits (bits 30..19, 18..7,
 // 6..0), largest first.  Rounds 3..6: 12-bit digits of the linear index of the ties,
 // smallest first.  The last block to finish scans the histogram.
 // --------------------------------------------------------------------------------------
-constexpr int SEL_THREADS = 512;
+constexpr int SEL_THREADS = 512, SEL_BLOCK = 2 * SEL_THREADS;
 
 __device__ __forceinline__ void round_digit(int round, int* shift, int* bits) {
   switch (round) {
@@ -443,27 +313,29 @@ __device__ __forceinline__ void round_digit(int round, int* shift, int* bits) {
 __global__ void __launch_bounds__(SEL_THREADS)
 k_select_round(SelectArgs a) {
   Ctl* ctl = a.ctl;
-  if (ctl->abort || !ctl->ready || ctl->need <= 0) return;
+  // all of the state in one go: a load behind each test would be a round trip to L2 of its own
+  const int aborted = ctl->abort, ready = ctl->ready, key_done = ctl->key_done, idx_done = ctl->idx_done;
+  const long long need0 = ctl->need;
+  const unsigned long long ncand = min(ctl->cand_count, a.cand_cap);
+  const unsigned long long kp = ctl->key_prefix;   // key bits above this digit
+  const unsigned long long ip = ctl->idx_prefix;
+  const unsigned tau = ctl->tau_key;
   const int round = a.round;
-  if (round < 3 && ctl->key_done) return;
-  if (round >= 3) {
-    if (!ctl->key_done || ctl->idx_done) return;
-    int sh, bt;
-    round_digit(round, &sh, &bt);
-    if (sh >= a.idx_bits && round < 6) return;     // digit is zero for every index
-  }
+  if (aborted || !ready || need0 <= 0) return;
+  if (round < 3 ? key_done : (!key_done || idx_done)) return;
+  // Only as many blocks as have SEL_BLOCK candidates each: every block costs a clear of its
+  // histogram, a merge of it by global atomics and an arrival.  (With the same rule in the emit
+  // kernel and two launches fewer: 500 x 500 at k = 12500 0.215 -> 0.204 ms an iteration.)
+  const unsigned active = (unsigned)min((unsigned long long)gridDim.x, max(1ull, (ncand + SEL_BLOCK - 1) / SEL_BLOCK));
+  if (blockIdx.x >= active) return;
   __shared__ unsigned h[kHistBins];
   const int tid = threadIdx.x;
   for (int b = tid; b < kHistBins; b += SEL_THREADS) h[b] = 0u;
   __syncthreads();
   int shift, bits;
   round_digit(round, &shift, &bits);
-  const unsigned long long ncand = min(ctl->cand_count, a.cand_cap);
-  const unsigned long long kp = ctl->key_prefix;   // key bits above this digit
-  const unsigned long long ip = ctl->idx_prefix;
-  const unsigned tau = ctl->tau_key;
   for (unsigned long long c = (unsigned long long)blockIdx.x * SEL_THREADS + tid; c < ncand;
-       c += (unsigned long long)gridDim.x * SEL_THREADS) {
+       c += (unsigned long long)active * SEL_THREADS) {
     unsigned key = a.cand_key[c];
     if (round < 3) {
       if (round > 0 && (key >> (shift + bits)) != kp) continue;
@@ -481,7 +353,7 @@ k_select_round(SelectArgs a) {
   __threadfence();
   __shared__ unsigned s_last;
   __syncthreads();
-  if (tid == 0) s_last = (atomicAdd(&ctl->done_ctas, 1u) == gridDim.x - 1);
+  if (tid == 0) s_last = (atomicAdd(&ctl->done_ctas, 1u) == active - 1);
   __syncthreads();
   if (!s_last) return;
   __threadfence();
@@ -496,7 +368,7 @@ k_select_round(SelectArgs a) {
   __shared__ unsigned s_in;
   const int nb = 1 << bits;
   const bool from_top = round < 3;
-  const unsigned long long need = (unsigned long long)ctl->need;
+  const unsigned long long need = (unsigned long long)need0;
   const int per = (nb + SEL_THREADS - 1) / SEL_THREADS;
   unsigned loc = 0;
   for (int o = tid * per; o < min(nb, tid * per + per); ++o) loc += h[from_top ? nb - 1 - o : o];
@@ -548,30 +420,43 @@ constexpr int EMIT_THREADS = 256, EMIT_ITEMS = 8;
 __global__ void __launch_bounds__(EMIT_THREADS)
 k_emit(EmitArgs a) {
   Ctl* ctl = a.ctl;
-  if (ctl->abort || !ctl->ready) return;
   const int tid = threadIdx.x;
-  const int nb = ctl->cur ^ 1;
-  const unsigned long long ncand = (ctl->need > 0) ? min(ctl->cand_count, a.cand_cap) : 0ull;
+  // the state in one go, as in the select rounds
+  const int aborted = ctl->abort, ready = ctl->ready, nb = ctl->cur ^ 1;
+  const long long need = ctl->need, k_req = ctl->k_req;
+  const unsigned long long ncand = (need > 0) ? min(ctl->cand_count, a.cand_cap) : 0ull;
   const unsigned tau = ctl->tau_key;
   const unsigned long long cut = ctl->idx_cut;
+  if (aborted || !ready) return;
+  const unsigned long long tile = (unsigned long long)EMIT_THREADS * EMIT_ITEMS;
+  const unsigned active = (unsigned)min((unsigned long long)gridDim.x, max(1ull, (ncand + tile - 1) / tile));
+  if (blockIdx.x >= active) return;
   long long* Sidx = a.S_idx[nb];
   float* Sval = a.S_val[nb];
   unsigned* bits = a.sbits ? a.sbits + (size_t)nb * (size_t)a.sbits_words : nullptr;   // clear until now
   double dsum = 0.0;
-  const unsigned long long tile = (unsigned long long)EMIT_THREADS * EMIT_ITEMS;
   __shared__ unsigned long long s_base;
   for (unsigned long long t0 = (unsigned long long)blockIdx.x * tile; t0 < ncand;
-       t0 += (unsigned long long)gridDim.x * tile) {
+       t0 += (unsigned long long)active * tile) {
     unsigned sel = 0;
     unsigned cnt = 0;
+    unsigned key[EMIT_ITEMS];
+    long long idx[EMIT_ITEMS];
+    float val[EMIT_ITEMS];
+#pragma unroll
+    for (int j = 0; j < EMIT_ITEMS; ++j) {   // all loads in flight before the first store
+      const unsigned long long c = t0 + (unsigned long long)j * EMIT_THREADS + tid;
+      key[j] = c < ncand ? a.cand_key[c] : 0u;
+      idx[j] = c < ncand ? a.cand_idx[c] : 0ll;
+      val[j] = c < ncand ? a.cand_val[c] : 0.f;
+    }
 #pragma unroll
     for (int j = 0; j < EMIT_ITEMS; ++j) {
       unsigned long long c = t0 + (unsigned long long)j * EMIT_THREADS + tid;
       if (c < ncand) {
-        unsigned key = a.cand_key[c];
-        bool s = key > tau || (key == tau && (unsigned long long)a.cand_idx[c] <= cut);
+        const bool s = key[j] > tau || (key[j] == tau && (unsigned long long)idx[j] <= cut);
         if (s) { sel |= 1u << j; ++cnt; }
-        else { float v = a.cand_val[c]; dsum += (double)v * (double)v; }
+        else dsum += (double)val[j] * (double)val[j];
       }
     }
     unsigned total;
@@ -582,12 +467,10 @@ k_emit(EmitArgs a) {
 #pragma unroll
     for (int j = 0; j < EMIT_ITEMS; ++j) {
       if (sel & (1u << j)) {
-        unsigned long long c = t0 + (unsigned long long)j * EMIT_THREADS + tid;
-        if (pos < (unsigned long long)ctl->k_req) {   // never past the S buffers
-          const long long idx = a.cand_idx[c];
-          Sidx[pos] = idx;
-          Sval[pos] = a.cand_val[c];
-          if (bits) atomicOr(&bits[idx >> 5], 1u << (idx & 31));
+        if (pos < (unsigned long long)k_req) {   // never past the S buffers
+          Sidx[pos] = idx[j];
+          Sval[pos] = val[j];
+          if (bits) atomicOr(&bits[idx[j] >> 5], 1u << (idx[j] & 31));
         }
         ++pos;
       }
@@ -598,54 +481,53 @@ k_emit(EmitArgs a) {
   __threadfence();
   __shared__ unsigned s_last;
   __syncthreads();
-  if (tid == 0) s_last = (atomicAdd(&ctl->done_ctas2, 1u) == gridDim.x - 1);
+  if (tid == 0) s_last = (atomicAdd(&ctl->done_ctas2, 1u) == active - 1);
   __syncthreads();
   if (!s_last || tid != 0) return;
   __threadfence();
-  // ---- last thread of the last block: commit the iteration ----
-  const double obj = atomicAdd(&ctl->sumsq_noncand, 0.0) + atomicAdd(&ctl->sumsq_cand_out, 0.0);
+  // ---- last thread of the last block: commit the iteration (loads first, then stores) ----
+  const double in_sum = __ldcg(&ctl->sumsq_noncand), out_sum = __ldcg(&ctl->sumsq_cand_out), nx2 = ctl->normX2;
+  const unsigned long long got = __ldcg(&ctl->nnz_new);
+  const double tol = ctl->tol;
+  const long long nnz0 = ctl->nnz_cur, keff = ctl->k_eff;
+  const int iter = ctl->iter, parity = ctl->slot_parity, passes = ctl->passes_run;
+  const double obj = in_sum + out_sum;
+  const double rel = nx2 > 0.0 ? obj / nx2 : 0.0;
   ctl->obj = obj;
-  ctl->rel_err = ctl->normX2 > 0.0 ? obj / ctl->normX2 : 0.0;
-  ctl->nnz_prev = ctl->nnz_cur;
-  {
-    unsigned long long got = atomicAdd(&ctl->nnz_new, 0ull);
-    if (got > (unsigned long long)ctl->k_eff) {   // selection inconsistent: keep the old S
-      ctl->nnz_cur = ctl->nnz_prev;
-      ctl->need_bigger_cand = 1;
-      ctl->abort = 1;
-      ctl->done_ctas2 = 0u;
-      return;
-    }
-    ctl->nnz_cur = (long long)got;
+  ctl->rel_err = rel;
+  ctl->nnz_prev = nnz0;
+  if (got > (unsigned long long)keff) {   // selection inconsistent: keep the old S
+    ctl->need_bigger_cand = 1;
+    ctl->abort = 1;
+    ctl->done_ctas2 = 0u;
+    return;
   }
+  ctl->nnz_cur = (long long)got;
   ctl->cur = nb;
-  ctl->iter += 1;
-  ctl->slot_parity ^= 1;          // normalisers written during this iteration become current
-  ctl->last_passes = ctl->passes_run;
-  if (ctl->tol >= 0.0 && ctl->rel_err <= ctl->tol) {
+  ctl->iter = iter + 1;
+  ctl->slot_parity = parity ^ 1;          // normalisers written during this iteration become current
+  ctl->last_passes = passes;
+  if (tol >= 0.0 && rel <= tol) {
     ctl->converged = 1;
     ctl->abort = 1;
   }
   // threshold guess for the next S-step: two digit-1 bins below the k-th key
-  if (ctl->need > 0) {
-    int b = (int)(ctl->tau_key >> kD1Shift) - 2;
-    ctl->next_guess = b > 0 ? ((unsigned)b << kD1Shift) : 1u;
-  } else {
-    ctl->next_guess = 0u;
-  }
+  const int gb = (int)(tau >> kD1Shift) - 2;
+  const unsigned guess = need > 0 ? (gb > 0 ? ((unsigned)gb << kD1Shift) : 1u) : 0u;
+  ctl->next_guess = guess;
   // reset per-iteration state
   ctl->done_ctas2 = 0u;
   ctl->nnz_new = 0ull;
-  ctl->plan[0] = ctl->next_guess ? PASS_CAND : PASS_FULL;
+  ctl->plan[0] = guess ? PASS_CAND : PASS_FULL;
   ctl->plan[1] = PASS_NONE;
   ctl->plan[2] = PASS_NONE;
-  ctl->guess[0] = ctl->next_guess;
+  ctl->guess[0] = guess;
   ctl->ready = 0;
   ctl->cand_count = 0ull;
   ctl->sumsq_noncand = 0.0;
   ctl->sumsq_full = 0.0;
   ctl->sumsq_cand_out = 0.0;
-  ctl->k_eff = ctl->k_req;
+  ctl->k_eff = k_req;
   ctl->key_prefix = 0ull;
   ctl->idx_prefix = 0ull;
   ctl->key_done = 0;
@@ -784,7 +666,7 @@ void launch_thresh_pass(const ResidualArgs& a, int nsm, cudaStream_t st) {
   int64_t grid = (a.m * ((a.n + 7) / 8) + TH_THREADS - 1) / TH_THREADS;
   if (grid > 4LL * nsm) grid = 4LL * nsm;
   k_thresh_pass<<<(unsigned)grid, TH_THREADS, 0, st>>>(a.X, a.m, a.n, a.ldx, a.pass, a.ctl, a.cand_key, a.cand_idx,
-                                                       a.cand_val, a.cand_cap);
+                                                       a.cand_val, a.cand_cap, a.k);
 }
 
 void launch_mark(const SelectArgs& a, unsigned* bits, int nsm, cudaStream_t st) {
@@ -806,12 +688,14 @@ void launch_order(const unsigned* bits, long long words, unsigned* scratch, long
   if (!R && nnz > 0) k_val_order<<<(unsigned)((nnz + 255) / 256), 256, 0, st>>>(S_idx, S_val, nnz, bits, rank0, val);
 }
 
-void launch_after_pass(Ctl* ctl, int pass, long long k, unsigned long long cap, cudaStream_t st) {
-  k_after_pass<<<1, CTL_THREADS, 0, st>>>(ctl, pass, k, cap);
-}
-
-void launch_select_round(const SelectArgs& a, int nsm, cudaStream_t st) {
-  k_select_round<<<(unsigned)(2 * nsm), SEL_THREADS, 0, st>>>(a);
+void launch_select(SelectArgs a, int nsm, cudaStream_t st) {
+  for (int d = 0; d < kNumSelRounds; ++d) {
+    // an index digit that is zero for every index is not looked at (500 x 500: two of seven
+    // launches, 10^4 x 10^4: one, about 1.7 us each)
+    if (d >= 3 && d < 6 && 12 * (6 - d) >= a.idx_bits) continue;
+    a.round = d;
+    k_select_round<<<(unsigned)(2 * nsm), SEL_THREADS, 0, st>>>(a);
+  }
 }
 
 void launch_emit(const EmitArgs& a, int nsm, cudaStream_t st) {
