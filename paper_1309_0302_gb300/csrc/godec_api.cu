@@ -113,7 +113,6 @@ struct godec_ctx {
   int64_t ldb = 0;
   int RPp = 0;
   float* cs = nullptr;                 // [2][RP] output factors: A1's column scales, 1 / kSkinnyScale
-  float* rescale_tmp = nullptr;        // 2 floats: factor applied by rescale_z
   // tensor maps: 0 Z for Z B, 1 Z for Z^T C, 2-4 bt2[0..2], 5 X, 6-7 Lsplit A, B; 13-14
   // bt2[3] over K = n and K = m (8-12 unused)
   alignas(64) unsigned char tmap[16][128];
@@ -1263,7 +1262,6 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
   c->ldb = (mx + 7) / 8 * 8;
   want(reinterpret_cast<unsigned short**>(&c->bt2), (size_t)4 * 2 * RP * c->ldb);
   want(&c->cs, (size_t)2 * RP);
-  want(&c->rescale_tmp, 2);
   c->tg[0] = prod_split_geometry(m, n, c->nsm);
   c->tg[1] = prod_split_geometry(n, m, c->nsm);
   size_t npart = 0;
