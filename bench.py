@@ -124,11 +124,11 @@ def peaks():
 
 def pass_traffic():
     """DRAM bytes per launch of the streaming product (dram__bytes_read.sum +
-    dram__bytes_write.sum of one ncu capture, scaled to the benchmark's size) from the
+    dram__bytes_write.sum of one ncu capture at the benchmark's size) from the
     committed summary, if it was taken on the current kernel source; else None."""
     import hashlib
-    src = os.path.join(ROOT, "paper_1309_0302_gb300", "csrc", "k_tc.cu")
-    p = os.path.join(ROOT, "profiles", "k_prod_tc_traffic.txt")
+    src = os.path.join(ROOT, "paper_1309_0302_gb300", "csrc", "k_prod.cu")
+    p = os.path.join(ROOT, "profiles", "k_prod_split_traffic.txt")
     if not os.path.exists(p):
         return None
     kv = dict(line.strip().split("=", 1) for line in open(p) if "=" in line and not line.startswith("#"))
