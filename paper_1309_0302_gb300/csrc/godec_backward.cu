@@ -35,6 +35,8 @@ void launch_scatter_split(const int64_t* idx, const float* vals, int64_t nnz, in
                           const float* scale, cudaStream_t st);
 void launch_outer_acc(const float* U, int64_t ldu, const float* V, int64_t ldv, int K, int64_t m, int64_t n,
                       float beta, float* D, int64_t ldd, cudaStream_t st);
+void launch_pack3(const float* const u[3], const float* const v[3], int64_t m, int64_t n, int r, float* U, float* V,
+                  int ld, cudaStream_t st);
 void launch_axpy(const float* x, float* y, int64_t count, float alpha, cudaStream_t st);
 }  // namespace godec
 
@@ -43,6 +45,7 @@ namespace {
 using namespace godec;
 
 constexpr int kCrossParts = 256;
+constexpr int kMaxSlots = 32;
 
 // Stream-ordered scratch of one call; freed (stream-ordered) on destruction.
 struct Scratch {
@@ -83,15 +86,18 @@ struct Engine {
   alignas(64) unsigned char mapB[2][128];      // over Bs with K = n (index 0) and K = m (index 1)
   TcGeom geom[2];
   float *cscale = nullptr, *part = nullptr;
-  unsigned* cmax = nullptr;
+  unsigned* cmax = nullptr;                    // kMaxSlots column maxima, cleared together (one
+  int slot = 0;                                // memset per kMaxSlots products, not one each)
   unsigned* cnt = nullptr;
 
   // Y (rows x c, dense) = src * B, or src^T * B with trans (B K x c, dense rows of c)
   void mul(const Source& s, int trans, const float* B, int c, float* Y) {
     const int64_t rows = dim[trans], K = dim[1 - trans];
-    cudaMemsetAsync(cmax, 0, (size_t)(1 + RP) * sizeof(unsigned), st);
-    launch_mul_stats(nullptr, 0, 0, 0, B, K, c, cmax, nsm, st);
-    launch_split_b(B, K, c, RP, cmax + 1, Bs, ldb, cscale, nullptr, nullptr, st);
+    if (slot == 0) cudaMemsetAsync(cmax, 0, (size_t)kMaxSlots * (1 + RP) * sizeof(unsigned), st);
+    unsigned* mx = cmax + (size_t)slot * (1 + RP);
+    slot = (slot + 1) % kMaxSlots;
+    launch_mul_stats(nullptr, 0, 0, 0, B, K, c, mx, nsm, st);
+    launch_split_b(B, K, c, RP, mx + 1, Bs, ldb, cscale, nullptr, nullptr, st);
     TcLaunch l{};
     l.mapA = s.map[trans];
     l.mapB = mapB[trans];
@@ -136,7 +142,7 @@ extern "C" godec_status godec_backward(const float* X, int64_t m, int64_t n, int
     set_static_error("godec_backward: no CUDA device");
     return GODEC_ERR_CUDA;
   }
-  const int RP = (r + 7) / 8 * 8, R3 = 3 * r;
+  const int RP = (r + 7) / 8 * 8, R3 = 3 * r, ldf = (R3 + 3) / 4 * 4;
   const int64_t mx = std::max(m, n), ldz = (n + 63) / 64 * 64;
   Scratch sc{st, dev};
   // Iterates Z_t: one copy for all t, rebuilt in the backward sweep, or (when all T of them
@@ -154,7 +160,7 @@ extern "C" godec_status godec_backward(const float* X, int64_t m, int64_t n, int
   E.RP = RP;
   E.ldb = (mx + 7) / 8 * 8;
   E.Bs = sc.get<unsigned short>((size_t)2 * RP * E.ldb);
-  E.cmax = sc.get<unsigned>(1 + (size_t)RP);
+  E.cmax = sc.get<unsigned>(kMaxSlots * (1 + (size_t)RP));
   E.cscale = sc.get<float>(RP);
   float* zsc = sc.get<float>(2 * src.size() + 2);      // {s, 1/s} of each source, then of X
   unsigned* zmax = sc.get<unsigned>(src.size() + 1);
@@ -175,8 +181,8 @@ extern "C" godec_status godec_backward(const float* X, int64_t m, int64_t n, int
   float* a = sc.get<float>((size_t)m * r);
   float* Wn = sc.get<float>((size_t)n * r);
   float* Zg = sc.get<float>((size_t)m * r);
-  float* Uf = sc.get<float>((size_t)m * R3);
-  float* Vf = sc.get<float>((size_t)n * R3);
+  float* Uf = sc.get<float>((size_t)m * ldf);
+  float* Vf = sc.get<float>((size_t)n * ldf);
   float* Rm = sc.get<float>((size_t)RP * RP * 4);                  // R1, T1, R2, T2 of CholeskyQR2
   double* g64 = sc.get<double>((size_t)RP * RP);
   double* Msm = sc.get<double>((size_t)GODEC_MAX_RANK * GODEC_MAX_RANK);
@@ -210,7 +216,6 @@ extern "C" godec_status godec_backward(const float* X, int64_t m, int64_t n, int
     set_static_error("godec_backward: tensor map encoding failed");
     return GODEC_ERR_CUDA;
   }
-  const size_t rowb = sizeof(float);
   // Z_t = X with L_{t-1} on Omega_{t-1}, at a scale that covers both (copy slot b)
   unsigned* xmax = zmax + src.size();
   launch_zscale(X, m, n, ldx, xmax, zsc + 2 * src.size(), nsm, st);
@@ -274,16 +279,12 @@ extern "C" godec_status godec_backward(const float* X, int64_t m, int64_t n, int
     launch_tall_small_d(Qk[t], r, r, Msm, r, 0, r, n, -1.f, 1.f, Wn, r, st);     // Wn = (I - Q Q^T) Wn = gY2
     E.mul(sZ, 0, Wn, r, Zg);                                    // Z gY2
     // factors of gZ_t: [a | A2 | Z gY2] [Y2 | gY2 | A1]^T
-    cudaMemcpy2DAsync(Uf, R3 * rowb, a, r * rowb, r * rowb, m, cudaMemcpyDeviceToDevice, st);
-    cudaMemcpy2DAsync(Uf + r, R3 * rowb, A2[t], r * rowb, r * rowb, m, cudaMemcpyDeviceToDevice, st);
-    cudaMemcpy2DAsync(Uf + 2 * r, R3 * rowb, Zg, r * rowb, r * rowb, m, cudaMemcpyDeviceToDevice, st);
-    cudaMemcpy2DAsync(Vf, R3 * rowb, Y2[t], r * rowb, r * rowb, n, cudaMemcpyDeviceToDevice, st);
-    cudaMemcpy2DAsync(Vf + r, R3 * rowb, Wn, r * rowb, r * rowb, n, cudaMemcpyDeviceToDevice, st);
-    cudaMemcpy2DAsync(Vf + 2 * r, R3 * rowb, A1, r * rowb, r * rowb, n, cudaMemcpyDeviceToDevice, st);
-    launch_outer_acc(Uf, R3, Vf, R3, R3, m, n, t == T - 1 ? 0.f : 1.f, dX, lddx, st);
+    const float *const us[3] = {a, A2[t], Zg}, *const vs[3] = {Y2[t], Wn, A1};
+    launch_pack3(us, vs, m, n, r, Uf, Vf, ldf, st);
+    launch_outer_acc(Uf, ldf, Vf, ldf, R3, m, n, t == T - 1 ? 0.f : 1.f, dX, lddx, st);
     // on Omega_{t-1}: gZ_t goes to L_{t-1} (next G) instead of X
     if (t > 0 && support_nnz[t - 1] > 0)
-      launch_eval_lr(supports[t - 1], support_nnz[t - 1], n, Uf, R3, Vf, R3, R3, gv, dX, lddx, st);
+      launch_eval_lr(supports[t - 1], support_nnz[t - 1], n, Uf, ldf, Vf, ldf, R3, gv, dX, lddx, st);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {

@@ -60,6 +60,26 @@ __device__ __forceinline__ float zs_get(const __half* Z, int64_t o) {
   return fmaf(__half2float(Z[o + 64]), 1.f / 2048.f, __half2float(Z[o]));
 }
 
+// Row and column of a linear index (idx = i n + j): a float estimate of the quotient,
+// refined once from the remainder and then corrected exactly in integers (no 64-bit
+// division; the estimate is off by at most a couple of units for any size).
+__device__ __forceinline__ void split_idx(long long idx, long long n, float ninv, long long& i, long long& j) {
+  long long q = (long long)((float)idx * ninv);
+  long long r = idx - q * n;
+  q += (long long)((float)r * ninv);
+  r = idx - q * n;
+  while (r < 0) {
+    --q;
+    r += n;
+  }
+  while (r >= n) {
+    ++q;
+    r -= n;
+  }
+  i = q;
+  j = r;
+}
+
 constexpr int kHistBins = 4096;     // first radix digit: key bits 30..19
 constexpr int kD1Shift = 19;
 constexpr int kNumSelRounds = 7;    // 3 key digits + 4 index digits

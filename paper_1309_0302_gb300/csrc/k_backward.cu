@@ -94,32 +94,53 @@ k_tall_small(const float* __restrict__ A, int64_t lda, int a, const TB* __restri
 }
 
 // out[row][c] += v_e B[col][c] (or, transposed, out[col][c] += v_e B[row][c]) for the COO
-// entries e (linear index row * n + col); float atomics.
-__global__ void k_spmm(const int64_t* __restrict__ idx, const float* __restrict__ val, int64_t nnz, int64_t n,
-                       const float* __restrict__ B, int64_t ldb, int c, int trans, float* __restrict__ out,
-                       int64_t ldo) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nnz * c) return;
-  const int64_t e = t / c;
-  const int cc = (int)(t % c);
-  const int64_t row = idx[e] / n, col = idx[e] % n;
+// entries e (linear index row * n + col); float atomics.  blockDim.x threads per entry, four
+// columns each: one row and column per thread without 64-bit divisions, and (vec: rows of B and
+// out 16-byte aligned) one 16-byte load and one four-wide atomic.  Bound: the atomics in L2.
+// nnz = 335 000, c = 20: 29.2 -> 14.9 us (before: a thread per column, four 64-bit divisions each).
+__global__ void __launch_bounds__(BW_THREADS)
+k_spmm(const int64_t* __restrict__ idx, const float* __restrict__ val, int64_t nnz, int64_t n, float ninv,
+       const float* __restrict__ B, int64_t ldb, int c, int trans, float* __restrict__ out, int64_t ldo, int vec) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
+  if (e >= nnz) return;
+  long long row, col;
+  split_idx(idx[e], n, ninv, row, col);
   const float v = val[e];
-  if (trans) atomicAdd(out + col * ldo + cc, v * B[row * ldb + cc]);
-  else atomicAdd(out + row * ldo + cc, v * B[col * ldb + cc]);
+  const int c0 = 4 * threadIdx.x;
+  const float* b = B + (trans ? row : col) * ldb + c0;
+  float* o = out + (trans ? col : row) * ldo + c0;
+  if (vec && c0 + 4 <= c) {
+    const float4 q = *reinterpret_cast<const float4*>(b);
+    atomicAdd(reinterpret_cast<float4*>(o), make_float4(v * q.x, v * q.y, v * q.z, v * q.w));
+  } else {
+    for (int u = 0; u < 4 && c0 + u < c; ++u) atomicAdd(o + u, v * b[u]);
+  }
 }
 
 // vals[e] = sum_c U[row][c] V[col][c] at the COO positions; with sub, also
-// D[row][col] -= vals[e].
-__global__ void k_eval_lr(const int64_t* __restrict__ idx, int64_t nnz, int64_t n, const float* __restrict__ U,
-                          int64_t ldu, const float* __restrict__ V, int64_t ldv, int K, float* __restrict__ vals,
-                          float* __restrict__ D, int64_t ldd) {
+// D[row][col] -= vals[e].  vec: rows of U and V are 16-byte aligned, four columns a load (the
+// sum keeps its order).  Bound: the gathers of V's rows from L2.  nnz = 335 000, K = 20 and 60: 25.0 -> 14.1 us
+// (before: scalar loads, 64-bit divisions).
+__global__ void k_eval_lr(const int64_t* __restrict__ idx, int64_t nnz, int64_t n, float ninv,
+                          const float* __restrict__ U, int64_t ldu, const float* __restrict__ V, int64_t ldv, int K,
+                          float* __restrict__ vals, float* __restrict__ D, int64_t ldd, int vec) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nnz) return;
-  const int64_t row = idx[e] / n, col = idx[e] % n;
+  long long row, col;
+  split_idx(idx[e], n, ninv, row, col);
   const float* u = U + row * ldu;
   const float* v = V + col * ldv;
   float s = 0.f;
-  for (int c = 0; c < K; ++c) s = fmaf(u[c], v[c], s);
+  int c = 0;
+  if (vec)
+    for (; c + 4 <= K; c += 4) {
+      const float4 p = *reinterpret_cast<const float4*>(u + c), q = *reinterpret_cast<const float4*>(v + c);
+      s = fmaf(p.x, q.x, s);
+      s = fmaf(p.y, q.y, s);
+      s = fmaf(p.z, q.z, s);
+      s = fmaf(p.w, q.w, s);
+    }
+  for (; c < K; ++c) s = fmaf(u[c], v[c], s);
   if (vals) vals[e] = s;
   if (D) D[row * ldd + col] -= s;
 }
@@ -204,11 +225,37 @@ k_outer_acc(const float* __restrict__ U, int64_t ldu, const float* __restrict__ 
   }
 }
 
+// Factors of gZ_t side by side: U (m x 3r) = [u0 | u1 | u2], V (n x 3r) = [v0 | v1 | v2] with rows
+// of ld, every source dense rows of r; one warp per row.  Bound: latency (8 (m + n) 3r bytes, 4 MB at
+// m = n = 4096, r = 20); one launch where six strided copies took 3.2 us each and a gap.
+__global__ void __launch_bounds__(BW_THREADS)
+k_pack3(const float* __restrict__ u0, const float* __restrict__ u1, const float* __restrict__ u2,
+        const float* __restrict__ v0, const float* __restrict__ v1, const float* __restrict__ v2, int64_t m, int64_t n,
+        int r, float* __restrict__ U, float* __restrict__ V, int ld) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * (BW_THREADS / 32);
+  for (int64_t w = (int64_t)blockIdx.x * (BW_THREADS / 32) + (threadIdx.x >> 5); w < m + n; w += warps) {
+    const bool up = w < m;
+    const int64_t i = up ? w : w - m;
+    const float *s0 = (up ? u0 : v0) + i * r, *s1 = (up ? u1 : v1) + i * r, *s2 = (up ? u2 : v2) + i * r;
+    float* o = (up ? U : V) + i * ld;
+    for (int c = lane; c < r; c += 32) {
+      const float a = s0[c], b = s1[c], d = s2[c];
+      o[c] = a;
+      o[r + c] = b;
+      o[2 * r + c] = d;
+    }
+  }
+}
+
 // y += alpha x
 __global__ void k_axpy(const float* __restrict__ x, float* __restrict__ y, int64_t count, float alpha) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < count) y[i] = fmaf(alpha, x[i], y[i]);
 }
+
+// Every row of a row-major float matrix starts on 16 bytes.
+bool rows16(const float* p, int64_t ld) { return ld % 4 == 0 && reinterpret_cast<uintptr_t>(p) % 16 == 0; }
 
 unsigned blocks_for(int64_t n) { return (unsigned)((n + BW_THREADS - 1) / BW_THREADS); }
 
@@ -243,19 +290,30 @@ void launch_tall_small_d(const float* A, int64_t lda, int a, const double* Bm, i
 void launch_spmm(const int64_t* idx, const float* val, int64_t nnz, int64_t n, const float* B, int64_t ldb, int c,
                  int trans, float* out, int64_t ldo, cudaStream_t st) {
   if (nnz * c == 0) return;
-  k_spmm<<<blocks_for(nnz * c), BW_THREADS, 0, st>>>(idx, val, nnz, n, B, ldb, c, trans, out, ldo);
+  const int cq = (c + 3) / 4;
+  const dim3 block((unsigned)cq, (unsigned)(BW_THREADS / cq));
+  k_spmm<<<(unsigned)((nnz + block.y - 1) / block.y), block, 0, st>>>(idx, val, nnz, n, 1.f / (float)n, B, ldb, c, trans,
+                                                                      out, ldo, rows16(B, ldb) && rows16(out, ldo));
 }
 
 void launch_eval_lr(const int64_t* idx, int64_t nnz, int64_t n, const float* U, int64_t ldu, const float* V,
                     int64_t ldv, int K, float* vals, float* D, int64_t ldd, cudaStream_t st) {
   if (nnz == 0) return;
-  k_eval_lr<<<blocks_for(nnz), BW_THREADS, 0, st>>>(idx, nnz, n, U, ldu, V, ldv, K, vals, D, ldd);
+  k_eval_lr<<<blocks_for(nnz), BW_THREADS, 0, st>>>(idx, nnz, n, 1.f / (float)n, U, ldu, V, ldv, K, vals, D, ldd,
+                                                    rows16(U, ldu) && rows16(V, ldv));
 }
 
 void launch_scatter_split(const int64_t* idx, const float* vals, int64_t nnz, int64_t n, void* Z, int64_t ldz,
                           const float* scale, cudaStream_t st) {
   if (nnz == 0) return;
   k_scatter_split<<<blocks_for(nnz), BW_THREADS, 0, st>>>(idx, vals, nnz, n, static_cast<__half*>(Z), ldz, scale);
+}
+
+void launch_pack3(const float* const u[3], const float* const v[3], int64_t m, int64_t n, int r, float* U, float* V,
+                  int ld, cudaStream_t st) {
+  const int64_t blocks = (m + n + BW_THREADS / 32 - 1) / (BW_THREADS / 32);
+  k_pack3<<<(unsigned)(blocks < 4096 ? blocks : 4096), BW_THREADS, 0, st>>>(u[0], u[1], u[2], v[0], v[1], v[2], m, n, r,
+                                                                            U, V, ld);
 }
 
 void launch_axpy(const float* x, float* y, int64_t count, float alpha, cudaStream_t st) {

@@ -21,26 +21,6 @@ namespace {
 
 __device__ __forceinline__ unsigned key_of(float v) { return __float_as_uint(v) & 0x7fffffffu; }
 
-// Row and column of a linear index (idx = i n + j): a float estimate of the quotient,
-// refined once from the remainder and then corrected exactly in integers (no 64-bit
-// division; the estimate is off by at most a couple of units for any size).
-__device__ __forceinline__ void split_idx(long long idx, long long n, float ninv, long long& i, long long& j) {
-  long long q = (long long)((float)idx * ninv);
-  long long r = idx - q * n;
-  q += (long long)((float)r * ninv);
-  r = idx - q * n;
-  while (r < 0) {
-    --q;
-    r += n;
-  }
-  while (r >= n) {
-    ++q;
-    r -= n;
-  }
-  i = q;
-  j = r;
-}
-
 __device__ double block_sum_double(double v) {
   __shared__ double ws[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
