@@ -327,6 +327,10 @@ struct ResidTcLaunch {
   int nsm;
 };
 void launch_resid_tc(const ResidTcLaunch& l, cudaStream_t st);
+// L = U diag(sigma) V^T densely, r <= kDenseSmall.
+constexpr int kDenseSmall = 8;
+void launch_dense_small(const float* U, const float* V, const float* sigma, int64_t m, int64_t n, int RP, int r, float* L,
+                        int64_t ldl, cudaStream_t st);
 cudaError_t prepare_resid_kernels();
 
 struct SelectArgs {

@@ -501,6 +501,47 @@ __global__ void k_lsplit(const float* __restrict__ U, const float* __restrict__ 
   }
 }
 
+// Dense L = U diag(sigma) V^T for r <= RT <= 8: float32 fmas, a thread keeps four rows of V in
+// registers and takes eight rows of U from shared memory.  Bound: the 4 m n bytes written.  At
+// these ranks the fmas are the more exact side (error against 64 bits 4.4e-8 against 1.2e-7 on the
+// tensor cores at r = 3, 5.5e-8 against 1.1e-7 at r = 6).  A call at
+// 76800 x 1000, r = 3: 186 -> 156 us; at 38400 x 600, r = 6: 86 -> 106 us; 16 columns of registers
+// (r = 16 at 10^4 x 10^4: 206 -> 818 us) are too many, so the line is at 8.
+template <int RT>
+__global__ void __launch_bounds__(256)
+k_dense_small(const float* __restrict__ U, const float* __restrict__ V, const float* __restrict__ sigma, int64_t m,
+              int64_t n, int RP, int r, float* __restrict__ L, int64_t ldl, int vec) {
+  constexpr int TM = 64;
+  __shared__ float sU[TM][RT];
+  const int64_t i0 = (int64_t)blockIdx.x * TM;
+  for (int e = threadIdx.x; e < TM * RT; e += 256) {
+    const int i = e / RT, l = e % RT;
+    sU[i][l] = (i0 + i < m && l < r) ? U[(i0 + i) * RP + l] * sigma[l] : 0.f;
+  }
+  __syncthreads();
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (int64_t j = (int64_t)blockIdx.y * 128 + tx * 4; j < n; j += (int64_t)gridDim.y * 128) {
+    float v[4][RT];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int l = 0; l < RT; ++l) v[q][l] = (j + q < n && l < r) ? V[(j + q) * RP + l] : 0.f;
+    for (int i = ty; i < TM && i0 + i < m; i += 8) {
+      float a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int l = 0; l < RT; ++l) {
+        const float u = sU[i][l];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) a[q] = fmaf(u, v[q][l], a[q]);
+      }
+      float* o = L + (i0 + i) * ldl + j;
+      if (vec && j + 4 <= n) *reinterpret_cast<float4*>(o) = make_float4(a[0], a[1], a[2], a[3]);
+      else
+        for (int q = 0; q < 4 && j + q < n; ++q) o[q] = a[q];
+    }
+  }
+}
+
 }  // namespace
 
 cudaError_t prepare_resid_kernels() {
@@ -515,6 +556,15 @@ void launch_lsplit(const float* U, const float* V, const float* sigma, int64_t m
   k_lsplit<<<(unsigned)blocks, 256, 0, st>>>(U, V, sigma, m, n, RP, r, zscale,
                                                           reinterpret_cast<__half*>(A), reinterpret_cast<__half*>(B),
                                                           skip);
+}
+
+void launch_dense_small(const float* U, const float* V, const float* sigma, int64_t m, int64_t n, int RP, int r, float* L,
+                        int64_t ldl, cudaStream_t st) {
+  const int vec = ldl % 4 == 0 && reinterpret_cast<uintptr_t>(L) % 16 == 0;
+  const int64_t cols = (n + 127) / 128;
+  const dim3 grid((unsigned)((m + 63) / 64), (unsigned)(cols < 65535 ? cols : 65535));
+  if (r <= 4) k_dense_small<4><<<grid, 256, 0, st>>>(U, V, sigma, m, n, RP, r, L, ldl, vec);
+  else k_dense_small<8><<<grid, 256, 0, st>>>(U, V, sigma, m, n, RP, r, L, ldl, vec);
 }
 
 void launch_resid_tc(const ResidTcLaunch& l, cudaStream_t st) {
