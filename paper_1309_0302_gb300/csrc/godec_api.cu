@@ -251,7 +251,8 @@ void free_graphs(godec_ctx* c) {
   }
 }
 
-// A buffer of the context: part of its arena, or (candidates and S grown later) its own.
+// A buffer of the context: part of its arena, or (candidates, S and partial slots grown later)
+// its own.
 void ctx_free(godec_ctx* c, void* p) {
   char* q = static_cast<char*>(p);
   if (q && !(q >= c->arena && q < c->arena + c->arena_bytes)) cudaFree(p);
@@ -1150,7 +1151,7 @@ void godec_destroy(godec_ctx* c) {
   if (c->st) cudaStreamSynchronize(c->st);
   free_graphs(c);
   for (void* p : {(void*)c->cand_key, (void*)c->cand_idx, (void*)c->cand_val, (void*)c->S_idx[0], (void*)c->S_idx[1],
-                  (void*)c->S_val[0], (void*)c->S_val[1]})
+                  (void*)c->S_val[0], (void*)c->S_val[1], (void*)c->part})
     ctx_free(c, p);
   cudaFree(c->arena);
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
@@ -2443,15 +2444,24 @@ godec_status bfail(godec_batch* b, godec_status s, const char* fmt, ...) {
 }
 
 // Size every grid of problem c for B SMs (the stream-K geometry of both product
-// orientations and the S-step's grids).  The stream-K buffers were sized for the whole
-// device at init; a smaller grid never needs more (fewer CTAs split each tile less).
+// orientations and the S-step's grids).  The partial slots were sized for the whole device
+// at init.  A smaller grid can need more of them: where the CTAs' ranges end at tile ends
+// (128 tiles over 128 CTAs) every tile has one slot, and over 72 CTAs two, so they grow here.
 godec_status set_budget(godec_ctx* c, int B) {
   B = std::max(1, std::min(B, c->nsm_dev));
   const TcGeom g0 = prod_split_geometry(c->p.m, c->p.n, B), g1 = prod_split_geometry(c->p.n, c->p.m, B);
   size_t npart = 0;
   for (const TcGeom& g : {g0, g1}) npart = std::max(npart, (size_t)g.tiles * g.maxseg * 128 * c->RP);
-  if (npart > c->npart_cap)
-    return fail(c, GODEC_ERR_STATE, "budget %d needs larger stream-K buffers", B);
+  if (npart > c->npart_cap) {
+    float* part = nullptr;
+    if (dalloc(&part, npart) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(c, GODEC_ERR_OOM, "partial slots of a budget of %d SMs: out of device memory", B);
+    }
+    ctx_free(c, c->part);
+    c->part = part;
+    c->npart_cap = npart;
+  }
   c->nsm = B;
   c->tg[0] = g0;
   c->tg[1] = g1;
