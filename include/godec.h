@@ -576,14 +576,21 @@ godec_status godec_batch_budgets(int32_t count, const int64_t* m, const int64_t*
                                  int32_t* sm);
 
 /*
- * Stream-K geometry of the tensor-core product over a rows x K operand on nsm SMs, host
- * logic only (no device work).  out (host, 6 entries) receives: row tiles of 128,
+ * Stream-K geometry of the tensor-core product with a caller's rows x K matrix on nsm SMs,
+ * host logic only (no device work).  out (host, 6 entries) receives: row tiles of 128,
  * K-stages of 64 per tile, stages S = tiles x stages, CTAs G (all SMs, or four fewer
  * above 16, at most S; CTA c owns stages [c S / G, (c+1) S / G)), the most CTAs that
  * share one tile (partial slots per tile), and the most tiles one CTA's range touches
  * (completions it may owe).  GODEC_ERR_ARG on a bad argument.
  */
 godec_status godec_tc_geometry(int64_t rows, int64_t K, int32_t nsm, int64_t* out);
+
+/*
+ * The same for the product over the library's own working copy (the power chain, Z^T C, the
+ * gradient): as above, on max(nsm - 20, min(nsm, 100)) SMs, which leaves SMs to the small
+ * kernels beside a chain.  Never fewer CTAs for more SMs from 17 SMs on.
+ */
+godec_status godec_prod_geometry(int64_t rows, int64_t K, int32_t nsm, int64_t* out);
 
 #ifdef __cplusplus
 }

@@ -89,6 +89,7 @@ def _declare(lib):
         "godec_batch_last_error": ([_P], C.c_char_p),
         "godec_batch_budgets": ([C.c_int32, i64p, i64p, C.c_int32, C.c_int32, i32p], C.c_int),
         "godec_tc_geometry": ([C.c_int64, C.c_int64, C.c_int32, i64p], C.c_int),
+        "godec_prod_geometry": ([C.c_int64, C.c_int64, C.c_int32, i64p], C.c_int),
         "godec_grebsmo_init": ([C.POINTER(_P), C.POINTER(GrebsmoParams), _P, _P, _P], C.c_int),
         "godec_naive_init": ([C.POINTER(_P), C.POINTER(GodecParams), _P, _P, _P], C.c_int),
         "godec_lingodec_init": ([C.POINTER(_P), C.POINTER(GodecParams), C.c_double, _P, _P, C.c_int32, _P], C.c_int),
@@ -689,8 +690,17 @@ def batch_budgets(shapes, nsm: int, policy: int):
     return list(out)
 
 
-def tc_geometry(rows: int, K: int, nsm: int) -> dict:
-    """Stream-K geometry of the tensor-core product (host logic, no device work)."""
+def _geometry(name, rows, K, nsm) -> dict:
     out = (C.c_int64 * 6)()
-    _check(library().godec_tc_geometry(int(rows), int(K), int(nsm), out), "godec_tc_geometry")
+    _check(getattr(library(), name)(int(rows), int(K), int(nsm), out), name)
     return dict(zip(("tiles", "ks", "S", "G", "maxseg", "maxpend"), list(out)))
+
+
+def tc_geometry(rows: int, K: int, nsm: int) -> dict:
+    """Stream-K geometry of the product with a caller's matrix (host logic, no device work)."""
+    return _geometry("godec_tc_geometry", rows, K, nsm)
+
+
+def prod_geometry(rows: int, K: int, nsm: int) -> dict:
+    """Stream-K geometry of the product over the working copy (host logic, no device work)."""
+    return _geometry("godec_prod_geometry", rows, K, nsm)

@@ -2755,9 +2755,7 @@ godec_status godec_batch_budgets(int32_t count, const int64_t* m, const int64_t*
   return GODEC_OK;
 }
 
-godec_status godec_tc_geometry(int64_t rows, int64_t K, int32_t nsm, int64_t* out) {
-  if (rows < 1 || K < 1 || nsm < 1 || !out) return GODEC_ERR_ARG;
-  const TcGeom g = tc_geometry(rows, K, nsm);
+static godec_status report_geometry(const TcGeom& g, int64_t* out) {
   out[0] = g.tiles;
   out[1] = g.ks;
   out[2] = g.S;
@@ -2765,6 +2763,16 @@ godec_status godec_tc_geometry(int64_t rows, int64_t K, int32_t nsm, int64_t* ou
   out[4] = g.maxseg;
   out[5] = g.maxpend;
   return GODEC_OK;
+}
+
+godec_status godec_tc_geometry(int64_t rows, int64_t K, int32_t nsm, int64_t* out) {
+  if (rows < 1 || K < 1 || nsm < 1 || !out) return GODEC_ERR_ARG;
+  return report_geometry(tc_geometry(rows, K, nsm), out);
+}
+
+godec_status godec_prod_geometry(int64_t rows, int64_t K, int32_t nsm, int64_t* out) {
+  if (rows < 1 || K < 1 || nsm < 1 || !out) return GODEC_ERR_ARG;
+  return report_geometry(prod_split_geometry(rows, K, nsm), out);
 }
 
 const char* godec_batch_last_error(godec_batch* b) { return b ? b->err : g_static_err; }

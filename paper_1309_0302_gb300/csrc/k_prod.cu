@@ -46,6 +46,8 @@
 #include <cuda.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
+
 #include "godec_internal.cuh"
 #include "tc_util.cuh"
 
@@ -661,11 +663,16 @@ static int prod_pin(double bytes) {
   return (int)(kPinOf * 44e6 / bytes);
 }
 
-// The split product's work split: 20 SMs fewer than the general rule on a whole device.  From
+// The split product's work split: on a whole device 20 SMs fewer than the general rule.  From
 // about 110 CTAs on the stream is bound by HBM (10^4 x 10^4, r = 50: the same time at 148, 136
 // and 120 CTAs), and the SMs left over run the r x r kernels of the side streams, which
 // otherwise outlast the products (one iteration: 1.76 ms with 4 SMs left, 1.61 ms with 24).
-TcGeom prod_split_geometry(int64_t rows, int64_t K, int nsm) { return tc_geometry(rows, K, nsm > 100 ? nsm - 20 : nsm); }
+// A share of the device (a batch problem's budget) up to 100 SMs follows the general rule, one
+// of 100 to 120 keeps the 96 CTAs of 100, so that more SMs never get fewer CTAs.  The line was
+// measured on chains of a whole device alone.
+TcGeom prod_split_geometry(int64_t rows, int64_t K, int nsm) {
+  return tc_geometry(rows, K, std::max(nsm - 20, std::min(nsm, 100)));
+}
 
 void launch_prod_split(const TcLaunch& l, cudaStream_t st) {
   PArgs a;
