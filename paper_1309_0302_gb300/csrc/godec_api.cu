@@ -31,7 +31,9 @@ using namespace godec;
 namespace {
 // Stream-ordered scratch from a pool of the library's own (one per device): blocks come back
 // to the pool in stream order and up to 256 MB stay in it between calls, so that a call need
-// not map memory anew (a device-wide operation of tens of microseconds each).
+// not map memory anew (a device-wide operation of tens of microseconds each).  The first call
+// creates the pool, which may be a call that a stream capture records: creating a pool is no
+// stream work, so it is exempted from the capture's check, which would end the capture.
 constexpr int kPoolDevices = 64;
 constexpr uint64_t kPoolKeep = 256ull << 20;
 cudaMemPool_t scratch_pool(int dev) {
@@ -46,11 +48,16 @@ cudaMemPool_t scratch_pool(int dev) {
     props.location.id = dev;
     cudaMemPool_t p = nullptr;
     uint64_t keep = kPoolKeep;
-    if (cudaMemPoolCreate(&p, &props) != cudaSuccess) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) {
       cudaGetLastError();
       return nullptr;
     }
-    cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+    const bool made = cudaMemPoolCreate(&p, &props) == cudaSuccess;
+    if (made) cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+    else cudaGetLastError();
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (!made) return nullptr;
     pools[dev] = p;
   }
   return pools[dev];
