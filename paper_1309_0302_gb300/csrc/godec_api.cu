@@ -1526,25 +1526,6 @@ godec_status godec_get_L(godec_ctx* c, float* U, float* sigma, float* V, int32_t
   return GODEC_OK;
 }
 
-// The residual pass in its dump mode on the current factors: R, or L alone.
-static void dump_pass(godec_ctx* c, float* out, int64_t ldo, bool l_only) {
-  launch_lsplit(c->U, c->V, c->sigma, c->p.m, c->p.n, c->RP, c->r, c->ctl->zscale, c->LA, c->LB, c->st);
-  ResidTcLaunch rl{};
-  rl.ra.X = c->X;
-  rl.ra.m = c->p.m;
-  rl.ra.n = c->p.n;
-  rl.ra.ctl = c->ctl;
-  rl.mapX = c->tmap[5];
-  rl.mapA = c->tmap[6];
-  rl.mapB = c->tmap[7];
-  rl.zscale = c->ctl->zscale;
-  rl.dump = out;
-  rl.ldd = ldo;
-  rl.dump_l = l_only ? 1 : 0;
-  rl.nsm = c->nsm_dev;   // alone on the device, whatever the problem's budget
-  launch_resid_tc(rl, c->st);
-}
-
 godec_status godec_get_L_dense(godec_ctx* c, float* L, int64_t ldl) {
   if (!c) return GODEC_ERR_ARG;
   if (!L || ldl < c->p.n) return fail(c, GODEC_ERR_ARG, "godec_get_L_dense: L must be non-NULL with ldl >= n");
@@ -1552,9 +1533,7 @@ godec_status godec_get_L_dense(godec_ctx* c, float* L, int64_t ldl) {
   godec_status s = read_ctl(c, &h);
   if (s) return s;
   if (h.iter == 0) return fail(c, GODEC_ERR_STATE, "no iteration has run yet");
-  // up to rank 8 float32 fmas err less, at about the same time; above, the tensor cores
-  if (c->r <= kDenseSmall) launch_dense_small(c->U, c->V, c->sigma, c->p.m, c->p.n, c->RP, c->r, L, ldl, c->st);
-  else dump_pass(c, L, ldl, true);
+  launch_dense(c->U, c->sigma, c->V, c->RP, c->p.m, c->p.n, c->r, L, ldl, c->st);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(c->st));
   return GODEC_OK;
@@ -1569,7 +1548,20 @@ godec_status godec_residual(godec_ctx* c, float* R, int64_t ldr) {
   godec_status s = read_ctl(c, &h);
   if (s) return s;
   if (h.iter < 1) return fail(c, GODEC_ERR_STATE, "no iteration has run yet");
-  dump_pass(c, R, ldr, false);
+  launch_lsplit(c->U, c->V, c->sigma, c->p.m, c->p.n, c->RP, c->r, c->ctl->zscale, c->LA, c->LB, c->st);
+  ResidTcLaunch rl{};
+  rl.ra.X = c->X;
+  rl.ra.m = c->p.m;
+  rl.ra.n = c->p.n;
+  rl.ra.ctl = c->ctl;
+  rl.mapX = c->tmap[5];
+  rl.mapA = c->tmap[6];
+  rl.mapB = c->tmap[7];
+  rl.zscale = c->ctl->zscale;
+  rl.dump = R;
+  rl.ldd = ldr;
+  rl.nsm = c->nsm_dev;   // alone on the device, whatever the problem's budget
+  launch_resid_tc(rl, c->st);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(c->st));
   return GODEC_OK;

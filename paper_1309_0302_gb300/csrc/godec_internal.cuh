@@ -322,15 +322,13 @@ struct ResidTcLaunch {
   const void* mapB;        // over B (n x 128 halves), box 64 x 64
   const float* zscale;     // {s_Z, 1/s_Z}
   float* dump;             // non-null: write R densely (row stride ldd) instead of selecting
-  int dump_l;              // ... or L alone
   int64_t ldd;
   int nsm;
 };
 void launch_resid_tc(const ResidTcLaunch& l, cudaStream_t st);
-// L = U diag(sigma) V^T densely, r <= kDenseSmall.
-constexpr int kDenseSmall = 8;
-void launch_dense_small(const float* U, const float* V, const float* sigma, int64_t m, int64_t n, int RP, int r, float* L,
-                        int64_t ldl, cudaStream_t st);
+// L (m x n, row stride ldl) = U diag(sigma) V^T, U and V with rows of RP (k_dense.cu).
+void launch_dense(const float* U, const float* sigma, const float* V, int RP, int64_t m, int64_t n, int r, float* L,
+                  int64_t ldl, cudaStream_t st);
 cudaError_t prepare_resid_kernels();
 
 struct SelectArgs {

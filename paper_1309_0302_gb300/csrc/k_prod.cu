@@ -145,20 +145,6 @@ __device__ __forceinline__ void load_block(void* dst, const CUtensorMap* map, ui
         : "memory");
 }
 
-// Packed pairs of float32 (two fmas per instruction).
-using f32x2 = uint64_t;
-__device__ __forceinline__ f32x2 pack2(float a, float b) {
-  f32x2 d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
-  return d;
-}
-__device__ __forceinline__ void unpack2(f32x2 d, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(d));
-}
-__device__ __forceinline__ void fma2(f32x2& d, f32x2 a, f32x2 b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
-}
-
 // Gram partial Y^T Y of the tile in Ps (128 rows, row stride LD) by the completion threads
 // (u = 0 .. 255): the upper triangle of 8 x 8 blocks, each as two 4 x 8 halves, SPL adjacent
 // lanes per half (lane sp takes the rows sp mod SPL), summed by a reduce-scatter over those

@@ -16,10 +16,8 @@
 // 4096-bin histogram of the top key bits (full mode) or the candidates with key >= guess
 // (candidate mode), the float64 sums of R^2, and the non-finite check.  Bound: HBM, 4 m n
 // bytes of X; a candidate pass at 10^4 x 10^4, r = 50 takes 112 us (floor 60 us), the rest
-// is the epilogue's issue rate.  A dump mode writes R densely, or L alone (godec_get_L_dense: bound by
-// the 4 m n bytes written; 10^4 x 10^4, r = 50: 562 us before as float32 fmas on the CUDA
-// cores).  Candidates are staged
-// per warp in shared memory (the histogram's space) and written out with one global
+// is the epilogue's issue rate.  A dump mode writes R densely.  Candidates are staged per warp in
+// shared memory (the histogram's space) and written out with one global
 // atomic per full buffer, so no tile waits on a contended atomic.
 //
 // Warps: 0 TMA producer of the X tiles, 18 TMA producer of the B and A tiles (the MMA's
@@ -78,7 +76,6 @@ struct RTArgs {
   long long k;              // selecting for the k largest (-1: the caller ends the pass itself)
   const float* zscale;      // zscale[1] = 1 / s_Z
   float* dump;              // dump mode when non-null: R into dump (row stride ldd)
-  int dump_l;               // dump mode writes L = X - R instead (X is not read)
   int64_t ldd;
 };
 
@@ -179,7 +176,7 @@ k_resid_tc(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUt
       uint32_t phx = 0;
       int64_t nx = 0;
       const uint64_t pol = policy_evict_first();
-      for (int64_t g = a.dump_l ? g1 : g0; g < g1 && !s_err; ++g) {
+      for (int64_t g = g0; g < g1 && !s_err; ++g) {
         if (!mbar_wait(&xempty[sx], phx ^ 1u, kRWait)) { rtimeout(ctl, &s_err); break; }
         // both boxes always: columns past n (and rows past m) are zero-filled, and so are
         // the rows of A and B past m and n, which makes R exactly 0 there
@@ -272,7 +269,6 @@ k_resid_tc(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUt
     const int f4b = (cq & 1) * 4;           // this quarter's first float4 in its 128-byte box row
     const uint32_t tlane = (uint32_t)(q4 * 32) << 16;
     const float zinv = a.zscale[1], zlo = zinv * kLoInv;
-    const bool vec4 = a.dump && (a.ldd & 3) == 0 && (reinterpret_cast<uintptr_t>(a.dump) & 15) == 0;
     // candidate iff key >= max(guess, 1); for a non-NaN value that is |R| >= gf (a NaN
     // fails the compare, lands in the sum and is caught there)
     const float gf = __uint_as_float(guess > 1u ? guess : 1u);
@@ -307,7 +303,7 @@ k_resid_tc(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUt
     for (int64_t g = g0; g < g1; ++g) {
       if (__any_sync(0xffffffffu, s_err != 0)) break;
       const int b = ai % kAcc;
-      if (!wwait(&accfull[b], (uint32_t)((ai / kAcc) & 1), lane) || (!a.dump_l && !wwait(&xfull[sx], phx, lane))) {
+      if (!wwait(&accfull[b], (uint32_t)((ai / kAcc) & 1), lane) || !wwait(&xfull[sx], phx, lane)) {
         if (lane == 0) rtimeout(ctl, &s_err);
         break;
       }
@@ -402,23 +398,6 @@ k_resid_tc(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUt
             if (key) atomicAdd(&hist[key >> kD1Shift], 1u);
           }
         }
-      } else if (a.dump_l) {   // L: a thread writes 64 contiguous bytes of its row
-        const int64_t i = ib * RM + row, j0 = jb * RNC + cq * kECols;
-        float* d = a.dump + i * a.ldd + j0;
-        float l[kECols];
-#pragma unroll
-        for (int q = 0; q < kECols; ++q) l[q] = fmaf(vl[q], zlo, vh[q] * zinv);
-        if (i < m) {
-          if (vec4 && j0 + kECols <= n) {
-#pragma unroll
-            for (int u = 0; u < kECols / 4; ++u)
-              *reinterpret_cast<float4*>(d + 4 * u) = make_float4(l[4 * u], l[4 * u + 1], l[4 * u + 2], l[4 * u + 3]);
-          } else {
-#pragma unroll
-            for (int q = 0; q < kECols; ++q)
-              if (j0 + q < n) d[q] = l[q];
-          }
-        }
       } else {   // dump
         const int64_t i = ib * RM + row, j0 = jb * RNC + cq * kECols;
 #pragma unroll
@@ -501,47 +480,6 @@ __global__ void k_lsplit(const float* __restrict__ U, const float* __restrict__ 
   }
 }
 
-// Dense L = U diag(sigma) V^T for r <= RT <= 8: float32 fmas, a thread keeps four rows of V in
-// registers and takes eight rows of U from shared memory.  Bound: the 4 m n bytes written.  At
-// these ranks the fmas are the more exact side (error against 64 bits 4.4e-8 against 1.2e-7 on the
-// tensor cores at r = 3, 5.5e-8 against 1.1e-7 at r = 6).  A call at
-// 76800 x 1000, r = 3: 186 -> 156 us; at 38400 x 600, r = 6: 86 -> 106 us; 16 columns of registers
-// (r = 16 at 10^4 x 10^4: 206 -> 818 us) are too many, so the line is at 8.
-template <int RT>
-__global__ void __launch_bounds__(256)
-k_dense_small(const float* __restrict__ U, const float* __restrict__ V, const float* __restrict__ sigma, int64_t m,
-              int64_t n, int RP, int r, float* __restrict__ L, int64_t ldl, int vec) {
-  constexpr int TM = 64;
-  __shared__ float sU[TM][RT];
-  const int64_t i0 = (int64_t)blockIdx.x * TM;
-  for (int e = threadIdx.x; e < TM * RT; e += 256) {
-    const int i = e / RT, l = e % RT;
-    sU[i][l] = (i0 + i < m && l < r) ? U[(i0 + i) * RP + l] * sigma[l] : 0.f;
-  }
-  __syncthreads();
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  for (int64_t j = (int64_t)blockIdx.y * 128 + tx * 4; j < n; j += (int64_t)gridDim.y * 128) {
-    float v[4][RT];
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-      for (int l = 0; l < RT; ++l) v[q][l] = (j + q < n && l < r) ? V[(j + q) * RP + l] : 0.f;
-    for (int i = ty; i < TM && i0 + i < m; i += 8) {
-      float a[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-      for (int l = 0; l < RT; ++l) {
-        const float u = sU[i][l];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) a[q] = fmaf(u, v[q][l], a[q]);
-      }
-      float* o = L + (i0 + i) * ldl + j;
-      if (vec && j + 4 <= n) *reinterpret_cast<float4*>(o) = make_float4(a[0], a[1], a[2], a[3]);
-      else
-        for (int q = 0; q < 4 && j + q < n; ++q) o[q] = a[q];
-    }
-  }
-}
-
 }  // namespace
 
 cudaError_t prepare_resid_kernels() {
@@ -558,15 +496,6 @@ void launch_lsplit(const float* U, const float* V, const float* sigma, int64_t m
                                                           skip);
 }
 
-void launch_dense_small(const float* U, const float* V, const float* sigma, int64_t m, int64_t n, int RP, int r, float* L,
-                        int64_t ldl, cudaStream_t st) {
-  const int vec = ldl % 4 == 0 && reinterpret_cast<uintptr_t>(L) % 16 == 0;
-  const int64_t cols = (n + 127) / 128;
-  const dim3 grid((unsigned)((m + 63) / 64), (unsigned)(cols < 65535 ? cols : 65535));
-  if (r <= 4) k_dense_small<4><<<grid, 256, 0, st>>>(U, V, sigma, m, n, RP, r, L, ldl, vec);
-  else k_dense_small<8><<<grid, 256, 0, st>>>(U, V, sigma, m, n, RP, r, L, ldl, vec);
-}
-
 void launch_resid_tc(const ResidTcLaunch& l, cudaStream_t st) {
   RTArgs a;
   a.m = l.ra.m;
@@ -580,7 +509,6 @@ void launch_resid_tc(const ResidTcLaunch& l, cudaStream_t st) {
   a.k = l.ra.k;
   a.zscale = l.zscale;
   a.dump = l.dump;
-  a.dump_l = l.dump_l;
   a.ldd = l.ldd;
   const int64_t T = ((a.m + RM - 1) / RM) * ((a.n + RNC - 1) / RNC);
   const int G = (int)(T < l.nsm ? T : l.nsm);

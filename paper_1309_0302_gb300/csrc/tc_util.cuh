@@ -255,6 +255,20 @@ __device__ __forceinline__ void tmem_ld8x4(uint32_t ta, uint32_t tb, float* va, 
   }
 }
 
+// Packed pairs of float32 (two fmas per instruction).
+using f32x2 = uint64_t;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ __forceinline__ void unpack2(f32x2 d, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(d));
+}
+__device__ __forceinline__ void fma2(f32x2& d, f32x2 a, f32x2 b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+
 // Programmatic dependent launch: wait until the preceding kernel of the stream has
 // completed and its memory is visible (returns at once when this launch has no
 // programmatic dependency), and let the next kernel of the stream start its prologue
