@@ -180,7 +180,8 @@ godec_status godec_get_S(godec_ctx* ctx, int64_t* idx, float* val, int64_t cap, 
  * Algorithm 1 thresholds, eq. raw_lss), computed by the same tensor-core kernel and
  * arithmetic as the S-step's residual pass.
  *   R : device, m x ldr float32, ldr >= n.
- * GODEC_ERR_STATE before the first iteration.  Synchronises the stream.
+ * GODEC_ERR_STATE before the first iteration; GODEC_ERR_TIMEOUT (R incomplete) when one of
+ * the kernel's bounded waits gave up.  Synchronises the stream.
  */
 godec_status godec_residual(godec_ctx* ctx, float* R, int64_t ldr);
 
@@ -290,6 +291,13 @@ godec_status godec_profile(godec_ctx* ctx, int32_t n_iter, double* ms, int64_t* 
  * polls out of range.
  */
 godec_status godec_check_timeout(godec_ctx* ctx, uint32_t polls);
+
+/*
+ * The first half of it: queue the wait and return without a look at the result, as a wait of
+ * a kernel in flight would end.  The next call on the context that runs iterations or the
+ * residual reports it (GODEC_ERR_TIMEOUT).
+ */
+godec_status godec_queue_timeout(godec_ctx* ctx, uint32_t polls);
 
 /*
  * The launches of the last iteration that godec_profile ran, in enqueue order:

@@ -72,6 +72,7 @@ def _declare(lib):
         "godec_profile": ([_P, C.c_int32, f64p, i64p, f64p], C.c_int),
         "godec_profile_trace": ([_P, C.c_int32, i32p, i32p, f32p, f32p, i32p], C.c_int),
         "godec_check_timeout": ([_P, C.c_uint32], C.c_int),
+        "godec_queue_timeout": ([_P, C.c_uint32], C.c_int),
         "godec_hard_threshold": ([_P, C.c_int64, C.c_int64, C.c_int64, C.c_int64, _P, _P, C.c_int64, i64p, _P],
                                  C.c_int),
         "godec_copy_rows": ([_P, C.c_int64, C.c_int64, C.c_int64, _P, C.c_int64, _P], C.c_int),
@@ -220,6 +221,10 @@ class GoDec:
         """Run the timeout self-test (godec_check_timeout): raises GodecError with
         status 5 (GODEC_ERR_TIMEOUT) when the bounded wait gives up, as it must."""
         _check(library().godec_check_timeout(self._h, C.c_uint32(polls)), "godec_check_timeout", self._h)
+
+    def queue_timeout(self, polls: int = 1000) -> None:
+        """Queue that wait without a look at the result (godec_queue_timeout)."""
+        _check(library().godec_queue_timeout(self._h, C.c_uint32(polls)), "godec_queue_timeout", self._h)
 
     def info(self) -> dict:
         inf = GodecInfo()

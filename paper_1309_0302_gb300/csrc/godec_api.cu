@@ -1412,14 +1412,19 @@ godec_status godec_solve(godec_ctx* c, int32_t* iters, double* rel_err) {
   return GODEC_OK;
 }
 
-godec_status godec_check_timeout(godec_ctx* c, uint32_t polls) {
+godec_status godec_queue_timeout(godec_ctx* c, uint32_t polls) {
   if (!c) return GODEC_ERR_ARG;
   if (polls < 1 || polls > (1u << 20)) return fail(c, GODEC_ERR_ARG, "polls must be in 1 .. 2^20");
   launch_wait_check(c->ctl, polls, c->st);
   CK(cudaGetLastError());
-  Ctl h;
-  godec_status s = read_ctl(c, &h);
+  return GODEC_OK;
+}
+
+godec_status godec_check_timeout(godec_ctx* c, uint32_t polls) {
+  godec_status s = godec_queue_timeout(c, polls);
   if (s) return s;
+  Ctl h;
+  if ((s = read_ctl(c, &h))) return s;
   if (h.abort) return handle_abort(c, h);
   return fail(c, GODEC_ERR_STATE, "the self-test wait completed, which nothing should make it do");
 }
@@ -1563,8 +1568,8 @@ godec_status godec_residual(godec_ctx* c, float* R, int64_t ldr) {
   rl.nsm = c->nsm_dev;   // alone on the device, whatever the problem's budget
   launch_resid_tc(rl, c->st);
   CK(cudaGetLastError());
-  CK(cudaStreamSynchronize(c->st));
-  return GODEC_OK;
+  if ((s = read_ctl(c, &h))) return s;
+  return h.timeout ? handle_abort(c, h) : GODEC_OK;   // a wait that gave up left tiles of R unwritten
 }
 
 godec_status godec_get_S(godec_ctx* c, int64_t* idx, float* val, int64_t cap, int64_t* nnz) {
