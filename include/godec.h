@@ -241,12 +241,22 @@ godec_status godec_run_host(const godec_params* params, const float* X_host,
  * split of both operands (float32-level accuracy, about 1e-7 relative); one
  * extra read of Z finds the power-of-two scale that keeps it in float16 range.
  * The call allocates its scratch on `stream` and frees it before returning
- * (stream-ordered), and does not synchronise.
+ * (stream-ordered), and does not synchronise.  Rows of the result that a bounded wait of
+ * the kernel which gave up left unfinished are NaN (there is no status to report it by).
  */
 godec_status godec_mul_ZB(const float* Z, int64_t m, int64_t n, int64_t ldz,
                           const float* B, int32_t r, float* Y, void* stream);
 godec_status godec_mul_ZtC(const float* Z, int64_t m, int64_t n, int64_t ldz,
                            const float* C, int32_t r, float* W, void* stream);
+
+/*
+ * Self-test of that: godec_mul_ZB (trans 0) or godec_mul_ZtC with the loads of the first of
+ * the kernel's blocks withheld, so that its waits run out (after about 40 ms).  The rows that
+ * block had a share of, from row 0 on in whole blocks of 128, become NaN; the others are as the
+ * product gives them.
+ */
+godec_status godec_mul_check_timeout(const float* Z, int64_t m, int64_t n, int64_t ldz, const float* B,
+                                     int32_t r, float* Y, int32_t trans, void* stream);
 
 /*
  * Copy an m x n float32 matrix to another row stride: src (device, any row stride lds >= n)
@@ -333,7 +343,8 @@ godec_status godec_profile_trace(godec_ctx* ctx, int32_t cap, int32_t* cls, int3
  * backward sweep (slower, m n floats).  Scratch is
  * allocated and freed on `stream` (stream-ordered); the call does not synchronise.
  * Float32 arithmetic with the float32-accurate tensor-core products; the sparse products
- * accumulate with float atomics (results may differ in the last bits between runs).
+ * accumulate with float atomics (results may differ in the last bits between runs).  A
+ * bounded wait of a product that gave up leaves NaN in dX, as for godec_mul_ZB.
  * GODEC_ERR_ARG on invalid arguments, GODEC_ERR_OOM when scratch cannot be allocated.
  */
 godec_status godec_backward(const float* X, int64_t m, int64_t n, int64_t ldx, const float* A1, int32_t r,

@@ -80,6 +80,7 @@ def _declare(lib):
         "godec_backward": ([_P, C.c_int64, C.c_int64, C.c_int64, _P, C.c_int32, C.c_int32, C.POINTER(_P), i64p,
                             _P, _P, C.c_int32, _P, C.c_int64, _P, C.c_int64, C.c_int32, _P], C.c_int),
         "godec_mul_ZtC": ([_P, C.c_int64, C.c_int64, C.c_int64, _P, C.c_int32, _P, _P], C.c_int),
+        "godec_mul_check_timeout": ([_P, C.c_int64, C.c_int64, C.c_int64, _P, C.c_int32, _P, C.c_int32, _P], C.c_int),
         "godec_batch_init": ([C.POINTER(_P), C.c_int32, C.POINTER(GodecParams), C.POINTER(_P), C.POINTER(_P),
                               C.c_int32, _P], C.c_int),
         "godec_batch_iterate": ([_P, C.c_int32], C.c_int),

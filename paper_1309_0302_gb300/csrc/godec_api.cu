@@ -1751,7 +1751,7 @@ godec_status godec_hard_threshold(const float* R, int64_t m, int64_t n, int64_t 
 
 // ---- streaming primitives ----------------------------------------------------------------
 static godec_status mul_common(const float* Z, int64_t m, int64_t n, int64_t ldz, const float* B, int32_t r,
-                               float* Y, void* stream, int trans) {
+                               float* Y, void* stream, int trans, int withhold = -1) {
   if (!Z || !B || !Y || m < 1 || n < 1 || ldz < n || (ldz * 4) % 16 || r < 1 || r > GODEC_MAX_RANK ||
       (reinterpret_cast<uintptr_t>(Z) & 15)) {
     snprintf(g_static_err, sizeof(g_static_err), "godec_mul: invalid argument");
@@ -1817,6 +1817,7 @@ static godec_status mul_common(const float* Z, int64_t m, int64_t n, int64_t ldz
     l.zscale = sc;
     l.pend = reinterpret_cast<int*>(mem + o_pend);
     l.trans = trans;
+    l.withhold = withhold;
     if (trans) launch_prod_split(l, st);
     else launch_prod_tc(l, st);
     e = cudaGetLastError();
@@ -1851,6 +1852,11 @@ godec_status godec_mul_ZB(const float* Z, int64_t m, int64_t n, int64_t ldz, con
 godec_status godec_mul_ZtC(const float* Z, int64_t m, int64_t n, int64_t ldz, const float* C, int32_t r,
                            float* W, void* stream) {
   return mul_common(Z, m, n, ldz, C, r, W, stream, 1);
+}
+
+godec_status godec_mul_check_timeout(const float* Z, int64_t m, int64_t n, int64_t ldz, const float* B, int32_t r,
+                                     float* Y, int32_t trans, void* stream) {
+  return mul_common(Z, m, n, ldz, B, r, Y, stream, trans != 0, 0);
 }
 
 // ---- GreBsmo (Sec. 3.2.1, Algorithm 2) --------------------------------------------------

@@ -247,8 +247,10 @@ struct TcLaunch {
   int trans;               // launch_prod_split: the product with Z^T (mapA's boxes have 64 rows, else 128)
   int half_a;              // launch_prod_split: the h halves alone
   int* pend;               // launch_prod_tc: G x geom.maxpend ints of scratch
-  Ctl* ctl;
+  Ctl* ctl;                // launch_prod_split, nullable; without one (and in launch_prod_tc) the
+                           // output rows of tiles that a timeout left unfinished become NaN
   int pdl = 0;             // programmatic dependent launch on the preceding kernel of the stream
+  int withhold = -1;       // self-test (without ctl): the CTA whose loads are not issued
   int z_prefetch = 0;      // the preceding kernels leave Zsrc unchanged: its first stages may be
                            // loaded before the wait on them (with pdl)
 };

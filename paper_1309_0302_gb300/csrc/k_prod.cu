@@ -41,8 +41,9 @@
 // owner), 2-3 spare, 4-7 epilogue, 8-15 completion.  The MMA warp runs its loop with all
 // lanes (uniform operands stay in uniform registers) and issues from one elected lane; with
 // the loop on a single lane its issue rate, about 1400 cycles a stage, was the limit.  Every
-// wait is bounded and ends early when another role gave up; a timeout sets ctl->timeout,
-// and the CTA drains its copies and MMAs and returns.
+// wait is bounded and ends early when another role gave up; a timeout sets ctl->timeout (without
+// a control block: makes the output rows of the CTA's tiles NaN), and the CTA drains its copies
+// and MMAs and returns.
 #include <cuda.h>
 #include <cuda_fp16.h>
 
@@ -97,6 +98,8 @@ struct PArgs {
   const float* zscale;      // {s_Z, 1 / s_Z} (nullable: 1)
   float* gram_part;         // nullable: tiles x RP x RP
   int z_prefetch;           // Z's first stages may be loaded before the programmatic wait
+  uint32_t limit;           // polls after which a wait gives up
+  int withhold;             // self-test: the CTA whose loads are not issued (-1: none)
   Ctl* ctl;
 };
 
@@ -111,8 +114,8 @@ __device__ __forceinline__ void p_timeout(Ctl* ctl, volatile int* s_err) {
 }
 
 // Bounded wait that also ends (false) when another role of the CTA has given up.
-__device__ __forceinline__ bool p_wait(uint64_t* bar, uint32_t parity, Ctl* ctl, volatile int* s_err) {
-  for (uint32_t i = 0; i < kPWait; ++i) {
+__device__ __forceinline__ bool p_wait(uint64_t* bar, uint32_t parity, uint32_t limit, Ctl* ctl, volatile int* s_err) {
+  for (uint32_t i = 0; i < limit; ++i) {
     if (mbar_wait(bar, parity, 1)) return true;
     if (*s_err) return false;
   }
@@ -340,6 +343,7 @@ k_prod_split(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
   constexpr int kAccCols = RPp <= 32 ? 64 : 128, kAcc = 512 / kAccCols;
   constexpr uint32_t kA = HALF ? 16384 : 32768;
   const int NS = a.ns;
+  const uint32_t limit = a.limit;
   Ctl* ctl = a.ctl;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -417,9 +421,10 @@ k_prod_split(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
       int pb = (int)(g0 % ks), s = 0;   // K stage of the skinny tile
       uint32_t ph = 0;
       int i = 0;
-      for (; i < nst; ++i) {
+      const int loads = c == a.withhold ? 0 : nst;
+      for (; i < loads; ++i) {
         if (i >= npre) {
-          if (!p_wait(&empty[s], ph ^ 1u, ctl, &s_err)) break;
+          if (!p_wait(&empty[s], ph ^ 1u, limit, ctl, &s_err)) break;
           load_a(s);
         }
         tma_load_2d(sm + (size_t)s * stage + kA, &mapB, &full[s], pb * BK, 0);
@@ -455,11 +460,11 @@ k_prod_split(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
       if (n > kChunk) n = kChunk;
       if (n > left) n = left;
       const int b = ch & (kAcc - 1);
-      if (!__all_sync(0xffffffffu, p_wait(&accempty[b], (uint32_t)(((ch / kAcc) & 1) ^ 1), ctl, &s_err))) break;
+      if (!__all_sync(0xffffffffu, p_wait(&accempty[b], (uint32_t)(((ch / kAcc) & 1) ^ 1), limit, ctl, &s_err))) break;
       const uint32_t dcol = tbase + (uint32_t)(b * kAccCols);
       bool ok = true;
       for (int e = 0; e < n; ++e) {
-        ok = __all_sync(0xffffffffu, p_wait(&full[s], ph, ctl, &s_err));
+        ok = __all_sync(0xffffffffu, p_wait(&full[s], ph, limit, ctl, &s_err));
         if (!ok) break;
         tc_fence_after();
         const uint64_t so = (uint64_t)((uint32_t)s * (stage >> 4));
@@ -500,7 +505,7 @@ k_prod_split(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
     int ch = 0, pushed = 0;
     auto push = [&](int v) {   // one thread
       const int k = pushed % kQ;
-      if (!p_wait(&qempty[k], (uint32_t)(((pushed / kQ) & 1) ^ 1), ctl, &s_err)) return;
+      if (!p_wait(&qempty[k], (uint32_t)(((pushed / kQ) & 1) ^ 1), limit, ctl, &s_err)) return;
       s_q[k] = v;
       mbar_arrive(&qfull[k]);
       ++pushed;
@@ -520,7 +525,7 @@ k_prod_split(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
       for (; g < tend; g = (g + kChunk < tend) ? g + kChunk : tend, ++ch) {
         if (failed) continue;                // keep the loop count; nothing more to read
         const int b = ch & (kAcc - 1);
-        if (!__all_sync(0xffffffffu, p_wait(&accfull[b], (uint32_t)((ch / kAcc) & 1), ctl, &s_err))) {
+        if (!__all_sync(0xffffffffu, p_wait(&accfull[b], (uint32_t)((ch / kAcc) & 1), limit, ctl, &s_err))) {
           failed = true;
           continue;
         }
@@ -570,7 +575,7 @@ k_prod_split(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
     const float zi = a.zscale ? a.zscale[1] : 1.f;
     for (int k = 0;; ++k) {
       const int q = k & (kQ - 1);
-      if (u == 0) s_go = p_wait(&qfull[q], (uint32_t)((k / kQ) & 1), ctl, &s_err) ? s_q[q] : -1;
+      if (u == 0) s_go = p_wait(&qfull[q], (uint32_t)((k / kQ) & 1), limit, ctl, &s_err) ? s_q[q] : -1;
       named_sync(2, kHelpers);
       const int64_t tt = s_go;
       if (tt < 0) break;
@@ -586,6 +591,7 @@ k_prod_split(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ C
     tc_fence_after();
     tmem_dealloc(tbase, 512);
   }
+  if (s_err && !ctl && a.out) poison_tiles(a.out, a.oc, a.rows, g0 / ks, (g1 - 1) / ks, tid, kPThreads);
 }
 
 template <int RPp, bool TR, bool HALF>
@@ -682,6 +688,8 @@ void launch_prod_split(const TcLaunch& l, cudaStream_t st) {
   a.zscale = l.zscale;
   a.gram_part = l.gram_mode ? static_cast<float*>(l.gram_part) : nullptr;
   a.z_prefetch = l.z_prefetch;
+  a.limit = l.withhold >= 0 ? kTestPolls : kPWait;
+  a.withhold = l.withhold;
   a.ctl = l.ctl;
   if (l.trans) launch_dir<true>(l, a, st);
   else launch_dir<false>(l, a, st);

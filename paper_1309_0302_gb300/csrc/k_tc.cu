@@ -42,7 +42,8 @@
 // refilled) and cpdone -> converters -> tfull (after the skinny tile's bfull too) -> MMA
 // -> sfree -> the stage slot and the skinny TMA slot.  The MMA issuer waits once and
 // commits once per stage.
-// Every wait is bounded; a timeout sets ctl->timeout and the CTA drains and exits.
+// Every wait is bounded; a CTA that gives up drains, makes the output rows of the tiles it had
+// a share of NaN (the calls do not synchronise and have no status to give) and exits.
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cudaTypedefs.h>
@@ -91,18 +92,11 @@ struct TcArgs {
   const float* zscale;      // {s_Z, 1 / s_Z} (nullable: 1)
   int* pend;                // G x maxpend: tiles each CTA completes, deferred to its end
   int maxpend;
-  Ctl* ctl;
+  uint32_t limit;           // polls after which a wait of the pipeline gives up
+  int withhold;             // self-test: the CTA whose matrix loads are not issued (-1: none)
 };
 
 __device__ __forceinline__ int64_t cta_of(int64_t g, int64_t S, int G) { return ((g + 1) * (int64_t)G - 1) / S; }
-
-__device__ __forceinline__ void note_timeout(Ctl* ctl, volatile int* s_err) {
-  *s_err = 1;
-  if (ctl) {
-    ctl->timeout = 1;
-    ctl->abort = 1;
-  }
-}
 
 // cvt.rn.f16x2: first source goes to the upper half, so element k sits in bits 0-15.
 __device__ __forceinline__ uint32_t pack_h2(float even, float odd) {
@@ -168,7 +162,7 @@ __device__ void tile_finish(const TcArgs& a, int64_t t, int nseg, int u, int nth
 // skinny-operand stages are one 64-column float16 box.
 template <bool IS_A>
 __device__ void produce(const CUtensorMap* map, unsigned char* ring, int nslot, size_t slot_bytes, uint32_t box_bytes,
-                        uint64_t* fullb, uint64_t* emptyb, int64_t g0, int64_t g1, int64_t ks, Ctl* ctl,
+                        uint64_t* fullb, uint64_t* emptyb, int64_t g0, int64_t g1, int64_t ks, uint32_t limit,
                         volatile int* s_err) {
   int64_t t = g0 / ks, kst = g0 % ks, issued = 0;
   int s = 0;
@@ -177,7 +171,7 @@ __device__ void produce(const CUtensorMap* map, unsigned char* ring, int nslot, 
   // leaves L2 to the skinny operand (read by every CTA) and the partial slots
   const uint64_t pol = policy_evict_first();
   for (int64_t g = g0; g < g1 && !*s_err; ++g) {
-    if (!mbar_wait(&emptyb[s], ph ^ 1u, kWaitLimit)) { note_timeout(ctl, s_err); break; }
+    if (!mbar_wait(&emptyb[s], ph ^ 1u, limit)) { *s_err = 1; break; }
     unsigned char* dst = ring + (size_t)s * slot_bytes;
     if (IS_A) {
       // both boxes always: columns at and past K are zero-filled
@@ -194,14 +188,14 @@ __device__ void produce(const CUtensorMap* map, unsigned char* ring, int nslot, 
   }
   // Every copy issued has landed before the CTA may exit (immediate in the normal case).
   for (int64_t j = (issued > nslot ? issued - nslot : 0); j < issued; ++j)
-    if (!mbar_wait(&fullb[(int)(j % nslot)], (uint32_t)((j / nslot) & 1), kWaitLimit)) note_timeout(ctl, s_err);
+    if (!mbar_wait(&fullb[(int)(j % nslot)], (uint32_t)((j / nslot) & 1), kWaitLimit)) *s_err = 1;
 }
 
 // Warp-uniform bounded wait: lane 0 polls, the warp follows (__syncwarp orders the
 // other lanes' later accesses after lane 0's acquire).
-__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int lane) {
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int lane, uint32_t limit) {
   int ok = 1;
-  if (lane == 0) ok = mbar_wait(bar, parity, kWaitLimit) ? 1 : 0;
+  if (lane == 0) ok = mbar_wait(bar, parity, limit) ? 1 : 0;
   ok = __shfl_sync(0xffffffffu, ok, 0);
   __syncwarp();
   return ok != 0;
@@ -210,7 +204,7 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int la
 template <int RPp>
 __global__ void __launch_bounds__(kThreads, 1)
 k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, TcArgs a) {
-  Ctl* ctl = a.ctl;
+  const uint32_t limit = a.limit;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   unsigned char* sA = sm + kOffA;
@@ -248,10 +242,7 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
   }
   if (warp == 1) tmem_alloc(&tmem_base, kTmemCols);
   if (tid == 0) {
-    // Iteration already abandoned, or Z outgrew its scale in the last S-step (the caller
-    // rescales it): do nothing, and make the rest of the iteration skip too.
-    s_err = (ctl && (ctl->abort || ctl->range_err)) ? 2 : 0;
-    if (ctl && ctl->range_err) ctl->abort = 1;
+    s_err = 0;
     s_npend = 0;
     s_zi = a.zscale ? a.zscale[1] : 1.f;
   }
@@ -262,12 +253,12 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
 
   if (warp == 0) {
     // ---------------- TMA producer: Zsrc tiles ----------------
-    if (lane == 0)
-      produce<true>(&mapA, sA, NA, kStageA, (uint32_t)kBoxA, afull, aempty, g0, g1, ks, ctl, &s_err);
+    if (lane == 0 && c != a.withhold)
+      produce<true>(&mapA, sA, NA, kStageA, (uint32_t)kBoxA, afull, aempty, g0, g1, ks, limit, &s_err);
   } else if (warp == 14) {
     // ---------------- TMA producer: skinny-operand tiles ----------------
     if (lane == 0)
-      produce<false>(&mapB, sB, NS, kStageB, (uint32_t)(2 * a.RP * BK * 2), bfull, sfree, g0, g1, ks, ctl,
+      produce<false>(&mapB, sB, NS, kStageB, (uint32_t)(2 * a.RP * BK * 2), bfull, sfree, g0, g1, ks, limit,
                      &s_err);
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
@@ -285,12 +276,12 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
         if (n > kChunk) n = kChunk;
         if (n > g1 - g) n = g1 - g;
         const int b = ch & 1;
-        if (!mbar_wait(&accempty[b], (uint32_t)(((ch >> 1) & 1) ^ 1), kWaitLimit)) { note_timeout(ctl, &s_err); break; }
+        if (!mbar_wait(&accempty[b], (uint32_t)(((ch >> 1) & 1) ^ 1), limit)) { s_err = 1; break; }
         tc_fence_after();
         const uint32_t dcol = tbase + (uint32_t)(b * 128);
         uint32_t acc = 0;
         for (int64_t e = 0; e < n; ++e) {
-          if (!mbar_wait(&tfull[st], ph, kWaitLimit)) { note_timeout(ctl, &s_err); break; }
+          if (!mbar_wait(&tfull[st], ph, limit)) { s_err = 1; break; }
           tc_fence_after();
           const uint64_t db = sdesc_k128(sB + (size_t)st * kStageB);
           // slot columns: [h of K 0..31 | l of K 0..31 | h of K 32..63 | l of K 32..63], 16 each
@@ -314,7 +305,7 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
         if (kst == ks) kst = 0;
       }
       mma_commit(&mma_done);
-      if (!mbar_wait(&mma_done, 0, kWaitLimit)) note_timeout(ctl, &s_err);
+      if (!mbar_wait(&mma_done, 0, kWaitLimit)) s_err = 1;
     }
   } else if (warp == 15) {
     // ---------------- copier: landed Zsrc stage -> its TMEM stage slot ----------------
@@ -323,8 +314,8 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
       uint32_t pha = 0, ph = 0;
       int64_t n = 0;
       for (int64_t g = g0; g < g1 && !s_err; ++g) {
-        if (!mbar_wait(&afull[sa], pha, kWaitLimit) || !mbar_wait(&sfree[st], ph ^ 1u, kWaitLimit)) {
-          note_timeout(ctl, &s_err);
+        if (!mbar_wait(&afull[sa], pha, limit) || !mbar_wait(&sfree[st], ph ^ 1u, limit)) {
+          s_err = 1;
           break;
         }
         tc_fence_after();
@@ -343,7 +334,7 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
       }
       // the last copies have finished reading shared memory and writing TMEM
       for (int64_t j = (n > NS ? n - NS : 0); j < n; ++j)
-        if (!mbar_wait(&cpdone[(int)(j % NS)], (uint32_t)((j / NS) & 1), kWaitLimit)) note_timeout(ctl, &s_err);
+        if (!mbar_wait(&cpdone[(int)(j % NS)], (uint32_t)((j / NS) & 1), kWaitLimit)) s_err = 1;
     }
   } else if (warp < 2 + kConvWarps) {
     // ---------------- converters: float32 stage in TMEM -> packed (h1, h2) in place ----------------
@@ -354,8 +345,8 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
     uint32_t ph = 0;
     for (int64_t g = g0; g < g1; ++g) {
       if (__any_sync(0xffffffffu, s_err != 0)) break;
-      if (!warp_wait(&cpdone[st], ph, lane)) {
-        if (lane == 0) note_timeout(ctl, &s_err);
+      if (!warp_wait(&cpdone[st], ph, lane, limit)) {
+        if (lane == 0) s_err = 1;
         break;
       }
       tc_fence_after();
@@ -378,8 +369,8 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
       tmem_wait_st();
       tc_fence_before();
       // the skinny tile of this stage has landed too: the MMA issuer waits on tfull alone
-      if (!warp_wait(&bfull[st], ph, lane)) {
-        if (lane == 0) note_timeout(ctl, &s_err);
+      if (!warp_wait(&bfull[st], ph, lane, limit)) {
+        if (lane == 0) s_err = 1;
         break;
       }
       if (lane == 0) mbar_arrive(&tfull[st]);
@@ -409,8 +400,8 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
       for (; g < tend; g = (g + kChunk < tend) ? g + kChunk : tend, ++ch) {
         if (failed) continue;                // keep the loop count; nothing more to read
         const int b = ch & 1;
-        if (!__all_sync(0xffffffffu, mbar_wait(&accfull[b], (uint32_t)((ch >> 1) & 1), kWaitLimit))) {
-          if (lane == 0) note_timeout(ctl, &s_err);
+        if (!__all_sync(0xffffffffu, mbar_wait(&accfull[b], (uint32_t)((ch >> 1) & 1), limit))) {
+          if (lane == 0) s_err = 1;
           failed = true;
           continue;
         }
@@ -448,7 +439,7 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
       if (s_last) {
         if (et == 0) {
           if (npend < a.maxpend) a.pend[(int64_t)c * a.maxpend + npend] = (int)t;
-          else if (ctl) ctl->abort = 1;   // cannot happen with the host's bound; never skip silently
+          else s_err = 1;   // cannot happen with the host's bound; never skip silently
         }
         ++npend;
       }
@@ -470,6 +461,7 @@ k_prod_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
     const int nseg = (int)(cta_of((t + 1) * ks - 1, S, G) - c_first + 1);
     tile_finish(a, t, nseg, tid, kThreads, s_csc, s_zi);
   }
+  if (s_err) poison_tiles(a.out, a.oc, a.rows, g0 / ks, (g1 - 1) / ks, tid, kThreads);
 }
 
 // Column c of a row-major rows x RP operand B -> rows c and RP + c of the split
@@ -710,7 +702,8 @@ void launch_prod_tc(const TcLaunch& l, cudaStream_t st) {
   a.zscale = l.zscale;
   a.pend = l.pend;
   a.maxpend = l.geom.maxpend;
-  a.ctl = l.ctl;
+  a.limit = l.withhold >= 0 ? kTestPolls : kWaitLimit;
+  a.withhold = l.withhold;
   const CUtensorMap& A = *reinterpret_cast<const CUtensorMap*>(l.mapA);
   const CUtensorMap& B = *reinterpret_cast<const CUtensorMap*>(l.mapB);
   switch (tc_rpp(l.RP)) {

@@ -255,6 +255,17 @@ __device__ __forceinline__ void tmem_ld8x4(uint32_t ta, uint32_t tb, float* va, 
   }
 }
 
+// The polls of a self-test's waits (about 40 ms).
+constexpr uint32_t kTestPolls = 20000;
+
+// A product without a control block cannot report a wait that gave up: the rows of row tiles t0
+// .. t1 (128 rows) of its output become NaN.  A CTA does it for the tiles it had a share of: a
+// tile is left unfinished only by a CTA that gave up before its share or its completion of it.
+__device__ __forceinline__ void poison_tiles(float* out, int oc, int64_t rows, int64_t t0, int64_t t1, int u, int nthr) {
+  const int64_t i1 = (t1 + 1) * 128 < rows ? (t1 + 1) * 128 : rows;
+  for (int64_t e = t0 * 128 * oc + u; e < i1 * oc; e += nthr) out[e] = __int_as_float(0x7fffffff);
+}
+
 // Packed pairs of float32 (two fmas per instruction).
 using f32x2 = uint64_t;
 __device__ __forceinline__ f32x2 pack2(float a, float b) {
