@@ -95,7 +95,8 @@ typedef struct godec_params {
 /* The chain's first projection (X - S) A1 (Algorithm 1's L-step; A1 is fixed for the run)
    is formed either by streaming X - S like the other products (the default,
    GODEC_FLAG_DENSE_FIRST), or, with GODEC_FLAG_SPARSE_FIRST, as X A1 - S A1 with X A1
-   computed once per godec_init / godec_reset and S A1 summed over the k entries of S.
+   computed once per godec_init / godec_reset and S A1 summed over the k entries of S (a
+   second array of about 4*m*n bytes holds the values of S at their positions).
    The second reads S at random positions: on GB300 its kernel is faster only for sparse
    S (k below about m n / 200), and over whole iterations its rounding made the lagged
    normalisers' alarm trip more often on the inputs measured.  Both flags set:
@@ -184,6 +185,14 @@ godec_status godec_get_S(godec_ctx* ctx, int64_t* idx, float* val, int64_t cap, 
  * the kernel's bounded waits gave up.  Synchronises the stream.
  */
 godec_status godec_residual(godec_ctx* ctx, float* R, int64_t ldr);
+
+/*
+ * (X - S) A1 of the current state as GODEC_FLAG_SPARSE_FIRST forms it, X A1 - S A1, row by row
+ * in column order (testing).
+ *   P : device, m x r_eff float32.
+ * GODEC_ERR_STATE on a context without that flag.  Synchronises the stream.
+ */
+godec_status godec_first_projection(godec_ctx* ctx, float* P);
 
 /* State after the last committed iteration t: its objective
    ||X - L_t - S_t||_F^2 (E_t^2 of Appendix I), |Omega| and bookkeeping. */

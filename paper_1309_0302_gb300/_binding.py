@@ -63,6 +63,7 @@ def _declare(lib):
         "godec_get_L_dense": ([_P, _P, C.c_int64], C.c_int),
         "godec_get_S": ([_P, _P, _P, C.c_int64, i64p], C.c_int),
         "godec_residual": ([_P, _P, C.c_int64], C.c_int),
+        "godec_first_projection": ([_P, _P], C.c_int),
         "godec_get_info": ([_P, C.POINTER(GodecInfo)], C.c_int),
         "godec_destroy": ([_P], None),
         "godec_last_error": ([_P], C.c_char_p),
@@ -295,6 +296,13 @@ class GoDec:
         R = torch.empty((m, n), dtype=torch.float32, device=self._X.device)
         _check(library().godec_residual(self._h, _ptr(R), n), "godec_residual", self._h)
         return R
+
+    def first_projection(self):
+        """(X - S) A1 (m, r_eff) as the sparse first projection forms it (FLAG_SPARSE_FIRST)."""
+        torch = _torch()
+        P = torch.empty((self.m, self.info()["r_eff"]), dtype=torch.float32, device=self._X.device)
+        _check(library().godec_first_projection(self._h, _ptr(P)), "godec_first_projection", self._h)
+        return P
 
 
 def naive_columns(m: int, n: int, r: int) -> int:

@@ -157,6 +157,7 @@ struct godec_ctx {
   unsigned* cmax = nullptr;            // column maxima of an operand being split
   float* XA1 = nullptr;                // m x RP: X A1, the cached part of the first projection (null: the
                                        // first product streams Z)
+  float* Sd = nullptr;                 // with it: m x ldz, S's values at the positions of its support
   long long* S_idx[2] = {nullptr, nullptr};
   float* S_val[2] = {nullptr, nullptr};
   int idx_bits = 1;
@@ -598,8 +599,7 @@ void enqueue_lstep(godec_ctx* c, bool fast) {
       const bool sp = i == 0 && c->XA1;
       if (sp)
         PROF(c, 11, c->st,
-             launch_sproj(c->XA1, c->A1, RP, c->X, c->p.ldx, c->Z, c->ldz, m, n, c->sbits, c->sbits_words, c->ctl,
-                          c->P, c->st));
+             launch_sproj(c->XA1, c->A1, RP, c->Sd, c->ldz, m, n, c->sbits, c->sbits_words, c->ctl, c->P, c->st));
       if (fast && sp) {
         apply(c, c->P, rows, sT(0, i), sT(1, i), nullptr, c->gscr, nextB);
         fork_side(c);
@@ -668,6 +668,7 @@ EmitArgs z_args(godec_ctx* c) {
   ea.Z = c->Z;
   ea.ldz = c->ldz;
   ea.zscale = c->ctl->zscale;
+  ea.Sd = c->Sd;
   ea.max_nnz = c->p.k;
   ea.sbits = c->sbits;
   ea.sbits_words = c->sbits_words;
@@ -1257,7 +1258,10 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
   // alarm trips more often with it (8 against 2 in 36 iterations), which costs more than
   // it saves, so streaming stays the default.
   const bool sparse_first = (p->flags & GODEC_FLAG_SPARSE_FIRST) != 0;
-  if (A1 && !greb && !c->naive && !c->lingo && !c->half && sparse_first) want(&c->XA1, (size_t)m * RP);
+  if (A1 && !greb && !c->naive && !c->lingo && !c->half && sparse_first) {
+    want(&c->XA1, (size_t)m * RP);
+    want(&c->Sd, (size_t)m * c->ldz);
+  }
   want(&c->P, (size_t)mx * RP);
   want(&c->Q1, (size_t)m * RP);
   want(&c->Q2, (size_t)n * RP);
@@ -1570,6 +1574,25 @@ godec_status godec_residual(godec_ctx* c, float* R, int64_t ldr) {
   CK(cudaGetLastError());
   if ((s = read_ctl(c, &h))) return s;
   return h.timeout ? handle_abort(c, h) : GODEC_OK;   // a wait that gave up left tiles of R unwritten
+}
+
+godec_status godec_first_projection(godec_ctx* c, float* P) {
+  if (!c) return GODEC_ERR_ARG;
+  if (!P) return fail(c, GODEC_ERR_ARG, "godec_first_projection: P must be non-NULL");
+  if (!c->XA1) return fail(c, GODEC_ERR_STATE, "godec_first_projection needs a context with GODEC_FLAG_SPARSE_FIRST");
+  Ctl h;
+  godec_status s;
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    launch_sproj(c->XA1, c->A1, c->RP, c->Sd, c->ldz, c->p.m, c->p.n, c->sbits, c->sbits_words, c->ctl, c->P, c->st);
+    CK(cudaGetLastError());
+    if ((s = read_ctl(c, &h))) return s;
+    if (!h.abort) break;
+    if ((s = handle_abort(c, h))) return s;   // Z outgrew its scale in the last S-step: brought back first
+  }
+  launch_unpad_copy(c->P, c->p.m, c->RP, P, c->r, c->st);
+  CK(cudaGetLastError());
+  CK(cudaStreamSynchronize(c->st));
+  return GODEC_OK;
 }
 
 godec_status godec_get_S(godec_ctx* c, int64_t* idx, float* val, int64_t cap, int64_t* nnz) {

@@ -56,9 +56,6 @@ __device__ __forceinline__ void zs_put(__half* Z, int64_t i, int64_t j, int64_t 
   Z[o] = h;
   Z[o + 64] = l;
 }
-__device__ __forceinline__ float zs_get(const __half* Z, int64_t o) {
-  return fmaf(__half2float(Z[o + 64]), 1.f / 2048.f, __half2float(Z[o]));
-}
 
 // Row and column of a linear index (idx = i n + j): a float estimate of the quotient,
 // refined once from the remainder and then corrected exactly in integers (no 64-bit
@@ -183,11 +180,10 @@ void launch_apply(const float* P, int64_t rows, int RP, const float* T0, const f
 
 // First projection of the chain from the cached X A1 (k_sproj.cu): P = X A1 - S A1 (m x RP,
 // row stride RP; XA1 and A1 likewise), S read on its support (bitmap ctl->cur of sbits,
-// `words` words per bitmap) as X - Z / s_Z; each row's entries are subtracted in column
-// order.  Like the product, it abandons the iteration when Z is flagged out of range.
-void launch_sproj(const float* XA1, const float* A1, int RP, const float* X, int64_t ldx, const void* Z, int64_t ldz,
-                  int64_t m, int64_t n, const unsigned* sbits, long long words, Ctl* ctl, float* P,
-                  cudaStream_t st);
+// `words` words per bitmap) from Sd (row stride lds); each row's entries are subtracted in
+// column order.  Like the product, it abandons the iteration when Z is flagged out of range.
+void launch_sproj(const float* XA1, const float* A1, int RP, const float* Sd, int64_t lds, int64_t m, int64_t n,
+                  const unsigned* sbits, long long words, Ctl* ctl, float* P, cudaStream_t st);
 
 // Tensor-core streaming product (k_tc.cu).
 struct TcGeom {
@@ -369,6 +365,7 @@ struct EmitArgs {
   void* Z;                 // the split working copy
   int64_t ldz;
   const float* zscale;     // Z is stored scaled by zscale[0]
+  float* Sd;               // S's values at their positions (row stride ldz, nullable), for k_sproj
   long long max_nnz;       // bound on the support of S (k): the z-update grid
   unsigned* sbits;         // two bitmaps of m n bits (nullable), sbits_words words apart: bitmap
   long long sbits_words;   // `cur` holds the support of the committed S, the other one is clear.

@@ -567,7 +567,9 @@ __global__ void k_z_update(EmitArgs a) {
     const long long idx = a.S_idx[cb][e];
     long long i, j;
     split_idx(idx, a.n, ninv, i, j);
-    z_write(a, i, j, a.X[i * a.ldx + j] - a.S_val[cb][e], zs, bad);
+    const float v = a.S_val[cb][e];
+    z_write(a, i, j, a.X[i * a.ldx + j] - v, zs, bad);
+    if (a.Sd) a.Sd[i * a.ldz + j] = v;
   }
   z_flag(ctl, bad);
 }

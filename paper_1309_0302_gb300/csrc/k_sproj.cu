@@ -6,8 +6,9 @@
 // tensor-core product over X, and each iteration subtracts S A1, k r multiply-adds,
 // instead of streaming the m x n matrix Z.
 //
-// S is read on its support bitmap (bit i n + j for entry (i, j)) as X - Z / s_Z: Z holds
-// (X - S) s_Z on the support, so this is the value the product over Z would have used.
+// S is read on its support bitmap (bit i n + j for entry (i, j)) from a dense m x lds array
+// that holds its values there (and nothing elsewhere): the float32 values themselves, where
+// X - Z / s_Z would carry the 2^-23 of Z's split.
 // Each row is handled by 16 lanes (two rows per warp, four columns of A1 per lane): the
 // row's bitmap words are staged in shared memory in one round trip and expanded into a
 // list of columns in increasing order, the entries' values gathered together, and the A1
@@ -30,9 +31,8 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
 }
 
 __global__ void __launch_bounds__(SP_WARPS * 32, 18)   // 36 warps, 72 rows per SM
-k_sproj(const float* __restrict__ XA1, const float* __restrict__ A1, int RP, const float* __restrict__ X, int64_t ldx,
-        const __half* __restrict__ Z, int64_t ldz, int64_t m, int64_t n, const unsigned* __restrict__ sbits,
-        long long words, Ctl* __restrict__ ctl, float* __restrict__ P) {
+k_sproj(const float* __restrict__ XA1, const float* __restrict__ A1, int RP, const float* __restrict__ Sd, int64_t lds,
+        int64_t m, int64_t n, const unsigned* __restrict__ sbits, long long words, Ctl* __restrict__ ctl, float* __restrict__ P) {
   __shared__ unsigned s_w[SP_WARPS * 2][SP_WCAP];
   __shared__ int s_j[SP_WARPS * 2][SP_CAP];
   __shared__ float s_v[SP_WARPS * 2][SP_CAP];
@@ -50,14 +50,12 @@ k_sproj(const float* __restrict__ XA1, const float* __restrict__ A1, int RP, con
   const bool live = i < m;
   const bool colok = live && 4 * hl < RP;   // RP is a multiple of 8: float4 columns
   const unsigned* B = sbits + (size_t)ctl->cur * (size_t)words;
-  const float zi = ctl->zscale[1];
   float4 acc = colok ? *reinterpret_cast<const float4*>(XA1 + i * RP + 4 * hl) : make_float4(0.f, 0.f, 0.f, 0.f);
   const int64_t b0 = i * n, b1 = b0 + n;   // the row's bits [b0, b1)
   const int64_t w0 = b0 >> 5;
   const int64_t nw = live ? ((b1 - 1) >> 5) - w0 + 1 : 0;
   const int64_t nwmax = n / 32 + 2;         // bound on nw for every row (uniform)
-  const float* Xr = X + (live ? i : 0) * ldx;
-  const int64_t zr = (live ? i : 0);
+  const float* Sr = Sd + (live ? i : 0) * lds;
   int* lj = s_j[slot];
   float* lv = s_v[slot];
   // Applies the nl listed entries of this row (called by the whole warp).
@@ -65,21 +63,16 @@ k_sproj(const float* __restrict__ XA1, const float* __restrict__ A1, int RP, con
     __syncwarp();
     const int cm = max(nl, __shfl_xor_sync(full, nl, 16));
     for (int u0 = 0; u0 < cm; u0 += 16 * 8) {   // S on the entries, 8 gathers in flight per lane
-      float xv[8], zv[8];
+      float v[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int e = u0 + 16 * u + hl;
-        xv[u] = zv[u] = 0.f;
-        if (e < nl) {
-          const int j = lj[e];
-          xv[u] = Xr[j];
-          zv[u] = zs_get(Z, zs_at(zr, j, ldz));
-        }
+        v[u] = e < nl ? Sr[lj[e]] : 0.f;
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int e = u0 + 16 * u + hl;
-        if (e < nl) lv[e] = xv[u] - zv[u] * zi;
+        if (e < nl) lv[e] = v[u];
       }
     }
     __syncwarp();
@@ -166,12 +159,10 @@ k_sproj(const float* __restrict__ XA1, const float* __restrict__ A1, int RP, con
 
 }  // namespace
 
-void launch_sproj(const float* XA1, const float* A1, int RP, const float* X, int64_t ldx, const void* Z, int64_t ldz,
-                  int64_t m, int64_t n, const unsigned* sbits, long long words, Ctl* ctl, float* P,
-                  cudaStream_t st) {
+void launch_sproj(const float* XA1, const float* A1, int RP, const float* Sd, int64_t lds, int64_t m, int64_t n,
+                  const unsigned* sbits, long long words, Ctl* ctl, float* P, cudaStream_t st) {
   const unsigned grid = (unsigned)((m + 2 * SP_WARPS - 1) / (2 * SP_WARPS));
-  k_sproj<<<grid, SP_WARPS * 32, 0, st>>>(XA1, A1, RP, X, ldx, static_cast<const __half*>(Z), ldz, m, n, sbits,
-                                          words, ctl, P);
+  k_sproj<<<grid, SP_WARPS * 32, 0, st>>>(XA1, A1, RP, Sd, lds, m, n, sbits, words, ctl, P);
 }
 
 }  // namespace godec
