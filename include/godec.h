@@ -268,6 +268,14 @@ godec_status godec_mul_check_timeout(const float* Z, int64_t m, int64_t n, int64
                                      int32_t r, float* Y, int32_t trans, void* stream);
 
 /*
+ * godec_mul_*, godec_hard_threshold and godec_backward take their scratch from a memory pool of
+ * the library's own, one per device, which keeps up to 256 MB of it between calls.  This call
+ * gives back to the device what the current device's pool keeps and no call in flight uses
+ * (synchronise first).  A context's memory is not part of it: godec_destroy frees all of that.
+ */
+godec_status godec_trim_scratch(void);
+
+/*
  * Copy an m x n float32 matrix to another row stride: src (device, any row stride lds >= n)
  * to dst (device, 16-byte aligned, ldd >= n, ldd*4 a multiple of 16 bytes; columns n .. ldd-1
  * are left as they are).  What a caller whose rows are not 16-byte aligned does before the

@@ -76,6 +76,7 @@ def _declare(lib):
         "godec_queue_timeout": ([_P, C.c_uint32], C.c_int),
         "godec_hard_threshold": ([_P, C.c_int64, C.c_int64, C.c_int64, C.c_int64, _P, _P, C.c_int64, i64p, _P],
                                  C.c_int),
+        "godec_trim_scratch": ([], C.c_int),
         "godec_copy_rows": ([_P, C.c_int64, C.c_int64, C.c_int64, _P, C.c_int64, _P], C.c_int),
         "godec_mul_ZB": ([_P, C.c_int64, C.c_int64, C.c_int64, _P, C.c_int32, _P, _P], C.c_int),
         "godec_backward": ([_P, C.c_int64, C.c_int64, C.c_int64, _P, C.c_int32, C.c_int32, C.POINTER(_P), i64p,
@@ -502,6 +503,12 @@ def hard_threshold(R, k: int, stream=None):
                                         C.byref(nnz), _stream_ptr(stream))
     _check(st, "godec_hard_threshold")
     return idx[: nnz.value], val[: nnz.value]
+
+
+def trim_scratch() -> None:
+    """Give back to the device the scratch (up to 256 MB) that the library keeps between calls of
+    mul_ZB, mul_ZtC, hard_threshold and backward on the current device."""
+    _check(library().godec_trim_scratch(), "godec_trim_scratch")
 
 
 def mul_ZB(Z, B, stream=None):

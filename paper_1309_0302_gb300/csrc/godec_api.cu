@@ -36,12 +36,12 @@ namespace {
 // stream work, so it is exempted from the capture's check, which would end the capture.
 constexpr int kPoolDevices = 64;
 constexpr uint64_t kPoolKeep = 256ull << 20;
-cudaMemPool_t scratch_pool(int dev) {
+cudaMemPool_t scratch_pool(int dev, bool create = true) {
   static std::mutex mu;
   static cudaMemPool_t pools[kPoolDevices] = {};
   if (dev < 0 || dev >= kPoolDevices) return nullptr;
   std::lock_guard<std::mutex> lock(mu);
-  if (!pools[dev]) {
+  if (!pools[dev] && create) {
     cudaMemPoolProps props{};
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
@@ -61,6 +61,12 @@ cudaMemPool_t scratch_pool(int dev) {
     pools[dev] = p;
   }
   return pools[dev];
+}
+
+// What the pool keeps and no call in flight uses goes back to the device.
+cudaError_t trim_pool(int dev) {
+  cudaMemPool_t pool = scratch_pool(dev, false);
+  return pool ? cudaMemPoolTrimTo(pool, 0) : cudaSuccess;
 }
 }
 
@@ -1315,7 +1321,11 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
   {
     const size_t total = c->arena_bytes;
     c->arena_bytes = 0;
-    CKI(cudaMalloc(reinterpret_cast<void**>(&c->arena), total));
+    if (cudaMalloc(reinterpret_cast<void**>(&c->arena), total) != cudaSuccess) {
+      cudaGetLastError();   // once more without what the scratch pool keeps
+      trim_pool(c->dev);
+      CKI(cudaMalloc(reinterpret_cast<void**>(&c->arena), total));
+    }
     c->arena_bytes = total;
     for (auto& q : plan) *q.first = c->arena + q.second;
   }
@@ -1848,6 +1858,15 @@ static godec_status mul_common(const float* Z, int64_t m, int64_t n, int64_t ldz
   cudaFreeAsync(mem, st);
   if (e != cudaSuccess) return out(GODEC_ERR_CUDA, cudaGetErrorString(e));
   return GODEC_OK;
+}
+
+godec_status godec_trim_scratch(void) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = trim_pool(dev);
+  if (e == cudaSuccess) return GODEC_OK;
+  snprintf(g_static_err, sizeof(g_static_err), "godec_trim_scratch: %s", cudaGetErrorString(e));
+  return GODEC_ERR_CUDA;
 }
 
 godec_status godec_copy_rows(const float* src, int64_t m, int64_t n, int64_t lds, float* dst, int64_t ldd, void* stream) {
