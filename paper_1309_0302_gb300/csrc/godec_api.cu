@@ -173,6 +173,7 @@ struct godec_ctx {
   int graph_nodes = 0;
   int exact_direct = 3;       // exact iterations still launched directly before a graph of them is captured
   int fast_run = 0;           // fast iterations since the start or the last alarm
+  int seen_iter = 0;          // iterations completed when the control block was last read (0 after a reset)
   bool need_exact = true;
   int exact_left = 0;   // exact iterations still owed after an alarm of the lagged normalisers
   int backoff = 1;      // exact iterations owed at the next alarm (doubles while alarms repeat)
@@ -841,6 +842,7 @@ godec_status build_graph(godec_ctx* c, int mode) {
 godec_status read_ctl(godec_ctx* c, Ctl* h) {
   CK(cudaMemcpyAsync(h, c->ctl, offsetof(Ctl, hist), cudaMemcpyDeviceToHost, c->st));
   CK(cudaStreamSynchronize(c->st));
+  c->seen_iter = h->iter;
   return GODEC_OK;
 }
 
@@ -910,6 +912,7 @@ void refresh_z(godec_ctx* c, double* sumsq) {
 godec_status reset_state(godec_ctx* c, bool sync = true) {
   c->r = c->p.r;   // captured graphs stay: buffers and geometry are the same, and graph_r tells a rank drop
   c->fast_run = 0;
+  c->seen_iter = 0;
   c->rank_drops = 0;
   c->need_exact = true;
   c->exact_left = 0;
@@ -1564,9 +1567,9 @@ godec_status godec_residual(godec_ctx* c, float* R, int64_t ldr) {
     return GODEC_ERR_ARG;
   }
   Ctl h;
-  godec_status s = read_ctl(c, &h);
-  if (s) return s;
-  if (h.iter < 1) return fail(c, GODEC_ERR_STATE, "no iteration has run yet");
+  godec_status s = GODEC_OK;
+  if (c->seen_iter < 1 && (s = read_ctl(c, &h))) return s;
+  if (c->seen_iter < 1) return fail(c, GODEC_ERR_STATE, "no iteration has run yet");
   launch_lsplit(c->U, c->V, c->sigma, c->p.m, c->p.n, c->RP, c->r, c->ctl->zscale, c->LA, c->LB, c->st);
   ResidTcLaunch rl{};
   rl.ra.X = c->X;
