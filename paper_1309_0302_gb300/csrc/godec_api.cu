@@ -124,11 +124,10 @@ struct godec_ctx {
   // bt2[1] by odd products (read by even ones, K = n), bt2[2] holds A1 (read by product 0).
   void* bt2 = nullptr;
   int64_t ldb = 0;
-  int RPp = 0;
   float* cs = nullptr;                 // [2][RP] output factors: A1's column scales, 1 / kSkinnyScale
-  // tensor maps: 0 Z for Z B, 1 Z for Z^T C, 2-4 bt2[0..2], 5 X, 6-7 Lsplit A, B; 13-14
-  // bt2[3] over K = n and K = m (8-12 unused)
-  alignas(64) unsigned char tmap[16][128];
+  // tensor maps: 0 Z for Z B, 1 Z for Z^T C, 2-4 bt2[0..2], 5 X, 6-7 Lsplit A, B; 8-9
+  // bt2[3] over K = n and K = m
+  alignas(64) unsigned char tmap[10][128];
   // precision form: float32 correction scratch
   float *RA = nullptr, *RB = nullptr, *Wa = nullptr, *Wb = nullptr, *Qa = nullptr, *Qb = nullptr, *Qtmp = nullptr;
   float *Rf = nullptr, *cs_ref = nullptr;
@@ -467,7 +466,7 @@ void refine(godec_ctx* c) {
   l.ctl = c->ctl;
   split_operand(c, c->V, n);
   l.mapA = c->tmap[0];
-  l.mapB = c->tmap[13];
+  l.mapB = c->tmap[8];
   l.rows = m;
   l.K = n;
   l.geom = c->tg[0];
@@ -476,7 +475,7 @@ void refine(godec_ctx* c) {
   split_operand(c, c->U, m);
   l.trans = 1;
   l.mapA = c->tmap[1];
-  l.mapB = c->tmap[14];
+  l.mapB = c->tmap[9];
   l.rows = n;
   l.K = m;
   l.geom = c->tg[1];
@@ -683,7 +682,7 @@ EmitArgs z_args(godec_ctx* c) {
 }
 
 // S-step of one iteration (Algorithm 1, eq. raw_lss) on the current L factors.
-void enqueue_sstep(godec_ctx* c, int r) {
+void enqueue_sstep(godec_ctx* c) {
   const int64_t m = c->p.m, n = c->p.n;
   cudaStream_t st = c->st;
   ResidualArgs ra{};
@@ -691,11 +690,6 @@ void enqueue_sstep(godec_ctx* c, int r) {
   ra.m = m;
   ra.n = n;
   ra.ldx = c->p.ldx;
-  ra.U = c->U;
-  ra.sigma = c->sigma;
-  ra.V = c->V;
-  ra.r = r;
-  ra.RP = c->RP;
   ra.ctl = c->ctl;
   ra.cand_key = c->cand_key;
   ra.cand_idx = c->cand_idx;
@@ -759,7 +753,7 @@ void greb_prod(godec_ctx* c, bool even, int map_b, const float* cscale, float* o
 void greb_apply_D(godec_ctx* c, int ri, int p, const float* B, float* out) {
   const int RP = c->RP;
   split_operand(c, B, c->p.n);
-  greb_prod(c, true, 13, c->cs_ref, out, 0, 0);
+  greb_prod(c, true, 8, c->cs_ref, out, 0, 0);
   if (ri > 0) {
     launch_cross_gram(c->Q2, RP, ri, B, RP, p, c->p.n, c->rf_part, kRefineParts, c->rf_C, RP, c->st, &c->ctl->abort);
     launch_tall_small_d(c->Q1, RP, ri, c->rf_C, RP, 0, p, c->p.m, -1.f, 1.f, out, RP, c->st, &c->ctl->abort);
@@ -770,7 +764,7 @@ void greb_apply_D(godec_ctx* c, int ri, int p, const float* B, float* out) {
 void greb_apply_Dt(godec_ctx* c, int ri, int p, const float* Y, float* out) {
   const int RP = c->RP;
   split_operand(c, Y, c->p.m);
-  greb_prod(c, false, 14, c->cs_ref, out, 0, 0);
+  greb_prod(c, false, 9, c->cs_ref, out, 0, 0);
   if (ri > 0) {
     launch_cross_gram(c->Q1, RP, ri, Y, RP, p, c->p.m, c->rf_part, kRefineParts, c->rf_C, RP, c->st, &c->ctl->abort);
     launch_tall_small_d(c->Q2, RP, ri, c->rf_C, RP, 0, p, c->p.n, -1.f, 1.f, out, RP, c->st, &c->ctl->abort);
@@ -806,11 +800,11 @@ void enqueue_naive_lstep(godec_ctx* c) {
 void enqueue_iteration(godec_ctx* c, bool fast) {
   if (c->naive) {
     enqueue_naive_lstep(c);
-    enqueue_sstep(c, c->r);
+    enqueue_sstep(c);
     return;
   }
   enqueue_lstep(c, fast);
-  enqueue_sstep(c, c->r);
+  enqueue_sstep(c);
 }
 
 godec_status build_graph(godec_ctx* c, int mode) {
@@ -1279,7 +1273,6 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
   want(&c->sigma, (size_t)RP);
   want(&c->Um, rr);
   want(&c->Vm, rr);
-  c->RPp = tc_rpp(RP);
   c->ldb = (mx + 7) / 8 * 8;
   want(reinterpret_cast<unsigned short**>(&c->bt2), (size_t)4 * 2 * RP * c->ldb);
   want(&c->cs, (size_t)2 * RP);
@@ -1348,8 +1341,8 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
                     make_tmap_f16(c->tmap[3], bt2(c, 1), 2 * RP, n, c->ldb, 2 * RP) &&
                     make_tmap_f16(c->tmap[4], bt2(c, 2), 2 * RP, n, c->ldb, 2 * RP);
     const bool ok3 = !(c->half || greb || c->naive || c->lingo) ||
-                     (make_tmap_f16(c->tmap[13], bt2(c, 3), 2 * RP, n, c->ldb, 2 * RP) &&
-                      make_tmap_f16(c->tmap[14], bt2(c, 3), 2 * RP, m, c->ldb, 2 * RP));
+                     (make_tmap_f16(c->tmap[8], bt2(c, 3), 2 * RP, n, c->ldb, 2 * RP) &&
+                      make_tmap_f16(c->tmap[9], bt2(c, 3), 2 * RP, m, c->ldb, 2 * RP));
     if (!ok || !ok3) {
       fail(c, GODEC_ERR_CUDA, "tensor map encoding failed");
       return bail(GODEC_ERR_CUDA);
@@ -1964,8 +1957,6 @@ static void greb_sstep(godec_ctx* c, int ri, unsigned guess, const float* U, flo
   rl.ra.m = m;
   rl.ra.n = n;
   rl.ra.ldx = c->p.ldx;
-  rl.ra.r = ri;
-  rl.ra.RP = RP;
   rl.ra.pass = 0;
   rl.ra.ctl = c->ctl;
   rl.ra.cand_key = c->cand_key;
@@ -2638,8 +2629,8 @@ godec_status batch_iterate(godec_batch* b, int n_iter) {
   for (size_t i = 0; i < P; ++i) {
     out[i] = b->hctl[i].abort ? 1 : 0;
     before[i] = b->hctl[i].iter;
-    // a rank drop, a candidate buffer grown, a new budget or a reset: the captured
-    // graph holds stale sizes or pointers of that problem
+    // a rank drop, a candidate buffer grown or a new budget: the captured graph holds
+    // stale sizes or pointers of that problem
     rebuild = rebuild || b->graph_r[i] != b->ctx[i]->r || b->graph_epoch[i] != b->ctx[i]->graph_epoch;
   }
   if (rebuild && (s = build_batch_graph(b))) return s;

@@ -145,8 +145,8 @@ struct Ctl {
 // Kernel launchers (defined in the .cu files).  All take the context stream.
 // --------------------------------------------------------------------------------
 
-// Streaming product Y = Zsrc B (Zsrc rows x K row-major with stride ld, B K x RP)
-// with split-K partials; the last CTA of each 128-row tile sums the partials (split
+// The no-allocation product's streaming kernel (k_stream.cu): Y = Zsrc B (Zsrc rows x K
+// row-major with stride ld, B K x RP) with split-K partials; the last CTA of each 128-row tile sums the partials (split
 // order), right-multiplies by Tn (RP x RP, nullable), writes `out` (rows x RP) and the
 // tile's Gram partial (gram_mode 0 none, 1 float, 2 exact products in double-float).
 struct ProdArgs {
@@ -294,10 +294,6 @@ void launch_svd(const float* Ra, const float* Rb, const float* Rapp0, const floa
 struct ResidualArgs {
   const float* X;
   int64_t m, n, ldx;
-  const float* U;          // m x RP (orthonormal columns)
-  const float* sigma;      // RP
-  const float* V;          // n x RP
-  int r, RP;
   int pass;                // 0, 1, 2
   Ctl* ctl;
   unsigned* cand_key;

@@ -1,9 +1,8 @@
 // Gram partials of the 128-row tiles of a chain product's float32 output, for the rank
 // test's exactly accumulated Gram of P = Z Q2 on the fast path: nothing on the critical path
-// needs it, so it runs on the rank test's own stream (whose kernels have the GPU's few
-// spare SMs to themselves while the chain goes on) instead of in the product's tile
-// completion, where the double-float accumulation takes ~20 us.  Same partial layout as
-// the product's own (tile t at t RP RP), summed by k_gram_sum.
+// needs it, so it runs on the rank test's own stream, on the SMs that the products of the
+// chain leave free.  The exact path takes it too, and the sparse first projection its float
+// form.  Same partial layout as the product's own Gram (tile t at t RP RP), summed by k_gram_sum.
 #include "godec_internal.cuh"
 #include "gram_tile.cuh"
 

@@ -8,8 +8,8 @@
 // halves: 64 of h (K zero-padded to 64) then 64 of l.  Per 128 x 64 tile of R:
 //   D[:, 0:128]  = A_h [B_h; B_l]^T      (N = 128, K = 64)
 //   D[:, 64:128] += A_l B_h^T           (N = 64)
-// so L = (D[:, :64] + 2^-11 D[:, 64:]) / s_Z to float32 accuracy (the dropped A_l B_l
-// term is 2^-24 relative).  s_Z, the scale of the working copy of X - S, bounds
+// so L = (D[:, :64] + 2^-11 D[:, 64:]) / s_Z to float32 accuracy (a term's two pairs are
+// off by 2^-23 each at most and the dropped A_l B_l by 2^-22).  s_Z, the scale of the working copy of X - S, bounds
 // sigma s_Z and keeps A and B inside the float16 range.
 //
 // The epilogue forms R from the accumulator and the X tile (TMA-staged), and takes a
@@ -261,7 +261,7 @@ k_resid_tc(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUt
     }
   } else {
     // ---------------- epilogue ----------------
-    // Each thread owns one row and 32 columns of the tile: R = X - (D_h + 2^-11 D_l) / s_Z,
+    // Each thread owns one row and 16 columns of the tile: R = X - (D_h + 2^-11 D_l) / s_Z,
     // formed with two FMAs (1 / s_Z is a power of two, so the scaled terms are exact).
     const int w = warp - 2;
     const int q4 = warp & 3, cq = w >> 2;   // TMEM lane quarter; column quarter of the tile

@@ -90,7 +90,7 @@ __device__ void after_pass(Ctl* ctl, int pass, int mode, long long k, unsigned l
     if (go) {
       __threadfence();
       ctl->done_ctas = 0u;
-      go = !__ldcg(&ctl->abort);   // by one thread: the rank test may set it at any time
+      go = !__ldcg(&ctl->abort);   // by one thread: a wait of this pass that gave up sets it
     }
     s_last_pass = go;
   }
