@@ -97,9 +97,8 @@ typedef struct godec_params {
    GODEC_FLAG_DENSE_FIRST), or, with GODEC_FLAG_SPARSE_FIRST, as X A1 - S A1 with X A1
    computed once per godec_init / godec_reset and S A1 summed over the k entries of S (a
    second array of about 4*m*n bytes holds the values of S at their positions).
-   The second reads S at random positions: on GB300 its kernel is faster only for sparse
-   S (k below about m n / 200), and over whole iterations its rounding made the lagged
-   normalisers' alarm trip more often on the inputs measured.  Both flags set:
+   The second reads S at random positions: on GB300 an iteration is faster with it only for
+   sparse S (by 1 % at k = m n / 1000, level near m n / 300).  Both flags set:
    GODEC_ERR_ARG.  Plain form only: the precision form, GreBsmo, naive GoDec, LinGoDec and
    MSE training always stream. */
 #define GODEC_FLAG_SPARSE_FIRST 8

@@ -1255,11 +1255,10 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
   want(&c->A1_orig, (size_t)n * RP);
   // plain GoDec with a given test matrix, on request: its first projection subtracts S A1
   // from a cached X A1 (the other forms change A1 or X between L-steps, or stream
-  // half of Z).  The cost of S A1 grows with k at about the rate of random reads from HBM;
-  // at m = n = 10^4 it matches the 94 us product near k = m n / 200 and saves 40 us at
-  // k = m n / 1000, but over whole iterations at k = m n / 1000 the lagged normalisers'
-  // alarm trips more often with it (8 against 2 in 36 iterations), which costs more than
-  // it saves, so streaming stays the default.
+  // half of Z).  The cost of S A1 and of keeping S's values at their positions grows with k at
+  // about the rate of random accesses to HBM: at m = n = 10^4 an iteration takes 1.467 ms
+  // against 1.483 streamed at k = m n / 1000, 1.572 against 1.559 at k = m n / 200, so
+  // streaming is the default.
   const bool sparse_first = (p->flags & GODEC_FLAG_SPARSE_FIRST) != 0;
   if (A1 && !greb && !c->naive && !c->lingo && !c->half && sparse_first) {
     want(&c->XA1, (size_t)m * RP);
