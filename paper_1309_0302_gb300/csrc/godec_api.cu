@@ -241,12 +241,16 @@ godec_status fail(godec_ctx* c, godec_status s, const char* fmt, ...) {
   return s;
 }
 
+// A CUDA error is reported once: left behind as the last error, the next call that looks for
+// errors of its own launches (this library's or the application's) would report it again.
 #define CK(call)                                                                          \
   do {                                                                                    \
     cudaError_t e_ = (call);                                                              \
-    if (e_ != cudaSuccess)                                                                \
+    if (e_ != cudaSuccess) {                                                              \
+      cudaGetLastError();                                                                 \
       return fail(c, e_ == cudaErrorMemoryAllocation ? GODEC_ERR_OOM : GODEC_ERR_CUDA,    \
                   "%s: %s", #call, cudaGetErrorString(e_));                              \
+    }                                                                                     \
   } while (0)
 
 int round_up(int v, int a) { return (v + a - 1) / a * a; }
@@ -1201,6 +1205,7 @@ static godec_status init_ctx(godec_ctx** out, const godec_params* p, const float
   do {                                                                                       \
     cudaError_t e_ = (call);                                                                 \
     if (e_ != cudaSuccess) {                                                                 \
+      cudaGetLastError();                                                                    \
       fail(c, GODEC_ERR_CUDA, "%s: %s", #call, cudaGetErrorString(e_));                      \
       return bail(e_ == cudaErrorMemoryAllocation ? GODEC_ERR_OOM : GODEC_ERR_CUDA);         \
     }                                                                                        \

@@ -57,6 +57,7 @@ struct Scratch {
   T* get(size_t elems) {
     void* p = nullptr;
     if (!ok || scratch_alloc(&p, std::max<size_t>(elems, 1) * sizeof(T), dev, st) != cudaSuccess) {
+      cudaGetLastError();   // reported by the call's status, not again by a later launch
       ok = false;
       return nullptr;
     }
