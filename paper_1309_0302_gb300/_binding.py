@@ -293,9 +293,8 @@ class GoDec:
     def residual(self):
         """Dense R = X - L_t (m, n) as a CUDA float32 tensor, from the S-step's kernel."""
         torch = _torch()
-        m, n = self._X.shape
-        R = torch.empty((m, n), dtype=torch.float32, device=self._X.device)
-        _check(library().godec_residual(self._h, _ptr(R), n), "godec_residual", self._h)
+        R = torch.empty((self.m, self.n), dtype=torch.float32, device=self._X.device)
+        _check(library().godec_residual(self._h, _ptr(R), self.n), "godec_residual", self._h)
         return R
 
     def first_projection(self):
